@@ -100,7 +100,7 @@ struct wash_ctx {
     int x_self = -1;
     void *x_row[2] = {nullptr, nullptr};
     int x_dtype[2] = {0, 0};
-    uint32_t *x_mask = nullptr;            // a byte per group, whole warp tiles
+    uint32_t *x_mask = nullptr;            // a word per four groups, whole warp tiles
     uint32_t *x_warp_total = nullptr;      // [x_blocks * kExchangeWarps][N + 1]
     uint32_t *x_block_total = nullptr;     // [x_blocks][N + 1]
     uint32_t x_wtiles = 0, x_blocks = 0;

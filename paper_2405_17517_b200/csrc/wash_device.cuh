@@ -28,6 +28,21 @@ __device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint3
     return Philox4{c0, c1, c2, c3};
 }
 
+// Bit j of the result = (w[j] < thr), for a thr of at least 1.  A word is compared by the carry of
+// word + (2^32 - thr), which an addition shifts into the mask: two additions a word.  A compare and
+// a select a word cost the pipe that Philox's XORs fill (2^27 mask words: 92.5 -> 86.3 us; the
+// blocks alone take 80.1).
+template <int COUNT>
+__device__ __forceinline__ uint32_t pack_below(const uint32_t (&w)[COUNT], uint32_t thr)
+{
+    const uint32_t minus_thr = 0u - thr;
+    uint32_t out = 0;   // bit set: word >= thr
+#pragma unroll
+    for (int j = COUNT - 1; j >= 0; --j)
+        asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %1, %2;\n\taddc.u32 %0, %0, %0;\n\t}" : "+r"(out) : "r"(w[j]), "r"(minus_thr));
+    return ~out & (COUNT < 32 ? (1u << COUNT) - 1u : 0xFFFFFFFFu);
+}
+
 // ---- element types -------------------------------------------------------------------
 // A "group" is 4 consecutive elements: 16 bytes of fp32, 8 bytes of bf16.  Values are
 // carried as raw bits (uint32 per element, bf16 in the low half).
@@ -143,13 +158,13 @@ __device__ __forceinline__ uint32_t group_value(const typename T::vec (&v)[CAP],
 __device__ __forceinline__ void publish_block_stats(unsigned long long *stats, StatSlot *slots, uint32_t selected, uint32_t moved)
 {
     if (!stats) return;
-    if (!__syncthreads_or(selected != 0)) return;   // most blocks have nothing to report at small p
+    if (!__syncthreads_or((selected | moved) != 0)) return;   // most blocks have nothing to report at small p
     __shared__ uint32_t block_sum[2];
     if (threadIdx.x == 0) block_sum[0] = block_sum[1] = 0;
     __syncthreads();
     selected = __reduce_add_sync(0xFFFFFFFFu, selected);
     moved = __reduce_add_sync(0xFFFFFFFFu, moved);
-    if ((threadIdx.x & 31) == 0 && selected) {
+    if ((threadIdx.x & 31) == 0 && (selected | moved)) {   // a value may be moved by another warp than the one that drew its coordinate
         atomicAdd(&block_sum[0], selected);
         atomicAdd(&block_sum[1], moved);
     }
@@ -179,21 +194,6 @@ __device__ __forceinline__ GroupInfo find_group(const PopView &pop, uint32_t g, 
     while (s < last && g >= __ldg(&pop.seg[s].group_end)) ++s;
     const uint4 lo = __ldg(reinterpret_cast<const uint4 *>(pop.seg + s));       // begin, end, tensor, cgroup_begin
     const uint4 hi = __ldg(reinterpret_cast<const uint4 *>(pop.seg + s) + 1);   // numel, -, thr
-    return group_info(lo, hi, g, s, status);
-}
-
-// As find_group, for a caller that visits groups in increasing order: `cursor` is the
-// segment of the previous group (or any segment not after g's) and is advanced; `seg`
-// may be a copy of the table in shared memory.
-__device__ __forceinline__ GroupInfo find_group_forward(const SegEntry *seg, int n_seg, uint32_t &cursor, uint32_t g,
-                                                        uint32_t *status)
-{
-    const uint32_t last = static_cast<uint32_t>(n_seg) - 1u;
-    uint32_t s = cursor;
-    while (s < last && g >= seg[s].group_end) ++s;
-    cursor = s;
-    const uint4 lo = reinterpret_cast<const uint4 *>(seg + s)[0];
-    const uint4 hi = reinterpret_cast<const uint4 *>(seg + s)[1];
     return group_info(lo, hi, g, s, status);
 }
 

@@ -7,19 +7,19 @@
 // another device).  After all workers have sent, each one copies its slots into its model.
 //
 // Work is cut into warp tiles of 128 groups (512 coordinates: a lane owns four consecutive
-// groups, so its four Philox draws overlap and its four mask bytes move as one word).  A
+// groups, so its four Philox draws overlap and their masks move as one word).  A
 // warp owns a contiguous range of warp tiles and visits them in order, which turns "the
 // slot of a coordinate" into a running count: no per-tile offsets are stored, only one
 // total per warp and per block, and the kernels need no block-wide barrier inside the loop.
-//   plan     draws the mask and, for selected coordinates, the permutation; writes a byte per
-//            group (low nibble: selected coordinates, high nibble: those whose new value comes
+//   plan     draws the mask and, for selected coordinates, the permutation; writes a word per
+//            four groups (low half: selected coordinates, high half: those whose new value comes
 //            from another worker) and, per warp and per block, how many slots of every
 //            worker's buffer its range takes (+ the selected count)
 //   send     adds up the totals of the blocks and warps before it (its first slots), then
 //            replays its range: redraws the permutations of the selected coordinates, numbers
 //            every worker's slots with warp votes and stores this worker's value where
 //            pi_i(n) is this worker
-//   receive  the same replay for its own buffer only, from the high nibbles: no draw at all
+//   receive  the same replay for its own buffer only, from the high halves: no draw at all
 // The plan reads no model data; send and receive touch only selected coordinates.
 // All three kernels must be launched with the same grid (n_blocks).
 #include "wash_device.cuh"
@@ -57,15 +57,13 @@ __device__ __forceinline__ void routes_of(const ExchangeArgs &a, uint32_t elem, 
 }
 
 // first and one-past-last warp tile of this warp (the n_wtiles tiles are dealt out evenly,
-// in order, to the grid's warps), and the cursor into the segment table for the first
-__device__ __forceinline__ void warp_range(const ExchangeArgs &a, uint32_t *t0, uint32_t *t1, uint32_t *cursor)
+// in order, to the grid's warps)
+__device__ __forceinline__ void warp_range(const ExchangeArgs &a, uint32_t *t0, uint32_t *t1)
 {
     const uint64_t range = blockIdx.x * kExchangeWarps + (threadIdx.x >> 5);
     const uint64_t ranges = static_cast<uint64_t>(a.n_blocks) * kExchangeWarps;
     *t0 = static_cast<uint32_t>(range * a.n_wtiles / ranges);
     *t1 = static_cast<uint32_t>((range + 1) * a.n_wtiles / ranges);
-    const uint32_t g = *t0 * kExchangeTileGroups;
-    *cursor = (*t0 < *t1 && g < a.pop.n_groups) ? __ldg(a.pop.tile_first + (g >> kTileShift)) : 0u;
 }
 
 __global__ void __launch_bounds__(kXThreads, kExchangeBlocksPerSm) exchange_plan_kernel(const __grid_constant__ ExchangeArgs a)
@@ -77,8 +75,8 @@ __global__ void __launch_bounds__(kXThreads, kExchangeBlocksPerSm) exchange_plan
     const int n_models = a.pop.N, columns = n_models + 1;
     for (int col = lane; col < columns; col += 32) s_count[warp][col] = 0;
     __syncwarp();
-    uint32_t t0, t1, cursor;
-    warp_range(a, &t0, &t1, &cursor);
+    uint32_t t0, t1;
+    warp_range(a, &t0, &t1);
     uint32_t head = 0, tail = 0;   // ring positions served / queued so far
     const uint32_t range_elem = 4u * kExchangeTileGroups * t0;   // first row element of the warp's range (rows are shorter than 2^32)
     // one round: lane j takes entry head + j; counts every worker's slots and marks the
@@ -92,19 +90,15 @@ __global__ void __launch_bounds__(kXThreads, kExchangeBlocksPerSm) exchange_plan
             for (unsigned long long left = need; left; left &= left - 1ull) atomicAdd(&s_count[warp][__ffsll(static_cast<long long>(left)) - 1], 1u);
             atomicAdd(&s_count[warp][n_models], 1u);
             if ((need >> a.self) & 1ull) {
-                const uint32_t g = elem >> 2;   // byte g % 4 of word g / 4, bit 4 + c
-                atomicOr(&a.mask[g >> 2], 16u << ((elem & 3u) + 8u * (g & 3u)));
+                atomicOr(&a.mask[elem >> 4], 0x10000u << (elem & 15u));
             }
         }
         __syncwarp();
         head += count;
     };
-    LaneSegment ls{1, 0, 0, 0, 0};
-    const uint32_t whole_tiles = a.pop.n_groups / kExchangeTileGroups;   // tiles with all 128 groups inside the row
+    LaneSegment ls;
     for (uint32_t t = t0; t < t1; ++t) {
-        const uint32_t g0 = t * kExchangeTileGroups + 4u * lane;   // rows are shorter than 2^32 elements: no wrap
-        uint32_t sel4 = 0;
-        if (!(t < whole_tiles && lane_masks_fast(a, g0, ls, &sel4))) sel4 = lane_masks_general(a, g0, ls, cursor);
+        const uint32_t sel4 = lane_masks(a, t * kExchangeTileGroups + 4u * lane, a.pop.n_groups, ls);   // rows are shorter than 2^32 elements: no wrap
         a.mask[static_cast<size_t>(t) * 32u + lane] = sel4;
         if (__any_sync(kFull, sel4 != 0)) {
             tail = ring_append(s_ring[warp], tail, sel4, t - t0);   // orders the mask stores before the rounds' atomics, too
@@ -161,8 +155,8 @@ __global__ void __launch_bounds__(kXThreads) exchange_send_kernel(const __grid_c
         for (uint32_t w = 0; w < warp; ++w) sum += a.warp_total[static_cast<size_t>(blockIdx.x * kExchangeWarps + w) * columns + col];
         run[h] = sum;
     }
-    uint32_t t0, t1, cursor;
-    warp_range(a, &t0, &t1, &cursor);
+    uint32_t t0, t1;
+    warp_range(a, &t0, &t1);
     uint32_t head = 0, tail = 0;
     const uint32_t range_elem = 4u * kExchangeTileGroups * t0;
     // one round: lane j takes entry head + j (coordinate order along the lanes); the warp votes
@@ -196,7 +190,7 @@ __global__ void __launch_bounds__(kXThreads) exchange_send_kernel(const __grid_c
         head += count;
     };
     for (uint32_t t = t0; t < t1; ++t) {
-        const uint32_t sel4 = a.mask[static_cast<size_t>(t) * 32u + lane] & 0x0F0F0F0Fu;
+        const uint32_t sel4 = a.mask[static_cast<size_t>(t) * 32u + lane] & 0xFFFFu;
         if (!__any_sync(kFull, sel4 != 0)) continue;
         tail = ring_append(s_ring[warp], tail, sel4, t - t0);
         while (tail - head >= 32u) serve(32u);
@@ -228,19 +222,18 @@ __global__ void __launch_bounds__(kXThreads) exchange_receive_kernel(const __gri
 #pragma unroll
     for (int w = 0; w < kExchangeWarps; ++w) run += s_part[w];
     for (uint32_t w = 0; w < warp; ++w) run += a.warp_total[static_cast<size_t>(blockIdx.x * kExchangeWarps + w) * columns + a.self];
-    uint32_t t0, t1, cursor;
-    warp_range(a, &t0, &t1, &cursor);
+    uint32_t t0, t1;
+    warp_range(a, &t0, &t1);
     const void *src[2] = {a.row[0] ? a.staging[0][a.self] : nullptr, a.row[1] ? a.staging[1][a.self] : nullptr};
     for (uint32_t t = t0; t < t1; ++t) {
-        const uint32_t take4 = (a.mask[static_cast<size_t>(t) * 32u + lane] >> 4) & 0x0F0F0F0Fu;
+        const uint32_t take4 = a.mask[static_cast<size_t>(t) * 32u + lane] >> 16;
         if (!__any_sync(kFull, take4 != 0)) continue;
         uint32_t total = 0;
         uint32_t slot = run + warp_exclusive_scan(__popc(take4), &total);
         run += total;
         const long long lane_elem = 4ll * (static_cast<long long>(t) * kExchangeTileGroups + 4u * lane);
         for (uint32_t left = take4; left; left &= left - 1u, ++slot) {
-            const int bit = __ffs(left) - 1;   // byte q = bit / 8, coordinate c = bit % 8
-            const long long elem = lane_elem + 4 * (bit >> 3) + (bit & 7);
+            const long long elem = lane_elem + __ffs(left) - 1;
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 if (!a.row[k]) continue;

@@ -111,8 +111,8 @@ struct ExchangeArgs {
     uint32_t n_blocks;            // grid of all three kernels; its warps share the warp tiles evenly, in order
     PhiloxKeys keys;
     uint32_t step_lo, step_hi8;
-    uint32_t *mask;               // [n_wtiles * 32] a word per lane = its four groups' bytes; low nibble of a byte:
-                                  // selected coordinates, high nibble: those this worker receives
+    uint32_t *mask;               // [n_wtiles * 32] a word per lane, a nibble per group; low half:
+                                  // selected coordinates, high half: those this worker receives
     uint32_t *warp_total;         // [n_blocks * kExchangeWarps][N + 1]: column n = slots of worker n's buffer the
                                   // warp's range takes; column N = selected coordinates
     uint32_t *block_total;        // [n_blocks][N + 1] the same per block

@@ -1,15 +1,26 @@
 // Sparse shuffle (WASH_MODE_SPARSE): the mask is drawn first, without touching the stacks, and
 // only the selected coordinates are loaded, permuted and stored -- the paper's point that a
-// step moves p d values, not d, carried onto one GPU.  The kernel is bound by the integer
-// pipes (one Philox block per 4 coordinates), not by memory.
+// step moves p d values, not d, carried onto one GPU.
 //
-// Work is cut into warp tiles (wash_warp_tiles.cuh): a lane draws the masks of four consecutive
-// groups at once; a warp walks a contiguous range of tiles, queues the selected coordinates in
-// a ring in shared memory and serves them 32 at a time, one per lane, so that the permutation
-// draws and the N loads of a coordinate run on full warps although selected coordinates are
-// rare and scattered.  The exchange is in place: a lane first loads the coordinate's N values
-// into its column of shared memory, then stores the ones that move.
+// A block walks a contiguous range of warp tiles (wash_warp_tiles.cuh), its warps taking turns.
+// The selected coordinates of all its warps go to one queue in shared memory; when the range is
+// done (or the queue full) the block serves the queue: a thread per coordinate draws the
+// permutation, then a thread per (coordinate, model) pair moves one value, so that neither step
+// runs on a few lanes of every warp and all the loads of a set are in flight at once.
+//
+// The exchange is in place: a warp loads all values of its set of coordinates before it stores
+// the first of them.
+//
+// Two bounds.  The mask: one Philox block per 4 coordinates on the integer pipes (2^27 coordinates:
+// 80 us for the blocks alone, 86 us with the compares, this kernel 100 us at N = 2, p = 1e-4).  The
+// values: DRAM serves about 45e9 scattered 4-byte loads a second, 22e9 scattered stores and 20e9 pairs
+// of both (measured, one access per 800 bytes), so [N][P] cannot go below 1 us per 20 000 moved
+// values and stack: cfg4 (1.8e6 values in both stacks) 90 us by that figure, 81 us here -- neighbouring
+// coordinates of a model share DRAM pages.  With a queue per warp, served at the end of the warp's
+// range by a lane per coordinate, the same launches took (before -> now): cfg2 21.2 -> 16.4 us, cfg3
+// 70.9 -> 59.1, cfg4 89.1 -> 81.4, cfg1 8.2 -> 6.2, 2^27 coordinates N = 2 at p = 1e-3 119 -> 107 us.
 #pragma once
+#include <cmath>
 #include "wash_device.cuh"
 #include "wash_launch.cuh"
 #include "wash_warp_tiles.cuh"
@@ -17,86 +28,128 @@
 
 namespace wash {
 
-constexpr int kSparseWarps = 8;
+constexpr int kSparseWarps = 4;
 constexpr int kSparseThreads = 32 * kSparseWarps;
+constexpr int kSparsePairs = 4;      // (coordinate, model) pairs a lane has in flight
+constexpr double kSparsePerBlock = 16.0;   // selected coordinates a block expects, at least
+
+// entries of the queue: a permutation of up to 16 models stays in its entry (8 bytes), a larger one
+// takes N bytes beside it
+__host__ __device__ constexpr uint32_t sparse_queue_capacity(int n_models) { return n_models <= 32 ? 512u : 256u; }
 
 struct SparseArgs {
     ShuffleArgs s;
-    uint32_t n_wtiles;   // warp tiles in [group_lo, group_hi)
-    uint32_t n_blocks;   // grid; its warps share the warp tiles evenly, in order
+    uint32_t n_wtiles;      // warp tiles in [group_lo, group_hi)
+    uint32_t per_block, extra;   // tiles of a block: per_block, one more in the first `extra` blocks
+    uint32_t in_set;        // coordinates whose N values a warp moves at a time: 32 * kSparsePairs / N
+    uint32_t inverse;       // 2^16 / d, rounded up, for the division of a pair's number (below 128) by in_set ([N][P]) or N ([P][N])
 };
 
 template <class TA, class TB, int LAYOUT>
-__global__ void __launch_bounds__(kSparseThreads, 4) shuffle_sparse_kernel(const __grid_constant__ SparseArgs p)
+__global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_sparse_kernel(const __grid_constant__ SparseArgs p)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ uint32_t s_count;
     constexpr bool kHasB = TB::kCode != kDtypeNone;
     const ShuffleArgs &a = p.s;
     const int n_models = a.pop.N;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    // [a ring per warp][a column of N words per thread][a column of N bytes per thread, N > 16]
-    uint32_t *ring = reinterpret_cast<uint32_t *>(smem_raw) + warp * kXRing;
-    uint32_t *s_col = reinterpret_cast<uint32_t *>(smem_raw) + kSparseWarps * kXRing + threadIdx.x;
-    uint8_t *s_perm = smem_raw + 4u * (kSparseWarps * kXRing + static_cast<uint32_t>(n_models) * kSparseThreads) + threadIdx.x;
+    const uint32_t capacity = sparse_queue_capacity(n_models);
+    // [entry: {coordinate within its tensor, tensor}, then the packed permutation][entry: row element,
+    // counted from the first element of the block's range][byte n of entry e at n * capacity + e, N > 16]
+    uint2 *q_key = reinterpret_cast<uint2 *>(smem_raw);
+    uint32_t *q_elem = reinterpret_cast<uint32_t *>(q_key + capacity);
+    uint8_t *q_bytes = reinterpret_cast<uint8_t *>(q_elem + capacity);
+    if (threadIdx.x == 0) s_count = 0;
 
-    // this warp's tiles: t0 .. t1-1, tile t = groups group_lo + 128 t ..
-    const uint64_t range = blockIdx.x * kSparseWarps + warp, ranges = static_cast<uint64_t>(p.n_blocks) * kSparseWarps;
-    const uint32_t t0 = static_cast<uint32_t>(range * p.n_wtiles / ranges), t1 = static_cast<uint32_t>((range + 1) * p.n_wtiles / ranges);
-    const uint64_t range_group = static_cast<uint64_t>(a.group_lo) + static_cast<uint64_t>(t0) * kWarpTileGroups;
-    uint32_t cursor = (t0 < t1 && range_group < a.group_hi) ? __ldg(a.pop.tile_first + (range_group >> kTileShift)) : 0u;
+    const uint32_t t_first = blockIdx.x * p.per_block + min(blockIdx.x, p.extra);
+    const uint32_t t_end = t_first + p.per_block + (blockIdx.x < p.extra ? 1u : 0u);
+    const uint32_t block_group = a.group_lo + t_first * kWarpTileGroups;
+    const long long block_elem = 4ll * static_cast<long long>(block_group);
 
-    uint32_t selected = 0, moved = 0, head = 0, tail = 0;
-    // one round: lane j takes entry head + j
-    auto serve = [&](uint32_t count) {
-        if (lane < count) {
-            const long long e = 4ll * static_cast<long long>(range_group) + ring[(head + lane) % kXRing];
-            const GroupInfo gi = find_group(a.pop, static_cast<uint32_t>(e >> 2), a.status);
-            const uint32_t coord = 4u * gi.cgroup + static_cast<uint32_t>(e & 3);
-            uint64_t perm = 0;
-            if (n_models <= 16) perm = draw_permutation_packed(n_models, coord, gi.tensor_id, a.step_lo, a.step_hi8, a.keys);
-            else draw_permutation_u8(s_perm, kSparseThreads, n_models, coord, gi.tensor_id, a.step_lo, a.step_hi8, a.keys);
-            // nibble n of `perm` (N <= 16) or byte n of the column is the model whose value model n takes
-            auto source_of = [&](int n, uint64_t rest) -> int {
-                return n_models <= 16 ? static_cast<int>(static_cast<uint32_t>(rest) & 15u) : static_cast<int>(s_perm[n * kSparseThreads]);
-            };
-            // all N old values first (the exchange is in place), then the moved ones back
-            for (int n = 0; n < n_models; ++n) s_col[n * kSparseThreads] = TA::load_elem(a.a, elem_index<LAYOUT>(a.pop, n, e));
-            uint64_t rest = perm;
-            for (int n = 0; n < n_models; ++n, rest >>= 4) {
-                const int src = source_of(n, rest);
-                if (src == n) continue;
-                TA::store_elem(a.a, elem_index<LAYOUT>(a.pop, n, e), s_col[src * kSparseThreads]);
-                ++moved;
-            }
-            if constexpr (kHasB) {
-                for (int n = 0; n < n_models; ++n) s_col[n * kSparseThreads] = TB::load_elem(a.b, elem_index<LAYOUT>(a.pop, n, e));
-                rest = perm;
-                for (int n = 0; n < n_models; ++n, rest >>= 4) {
-                    const int src = source_of(n, rest);
-                    if (src != n) TB::store_elem(a.b, elem_index<LAYOUT>(a.pop, n, e), s_col[src * kSparseThreads]);
+    __syncthreads();
+
+    uint32_t selected = 0, moved = 0;
+    LaneSegment ls;
+    uint32_t t = t_first + warp, sel = 0, sel_g0 = 0;   // sel: coordinates of the lane's last tile that are not queued yet; sel_g0: its first group there
+    for (;;) {
+        for (;;) {
+            if (sel) {
+                uint32_t pos = atomicAdd(&s_count, static_cast<uint32_t>(__popc(sel)));
+                for (; sel && pos < capacity; sel &= sel - 1u, ++pos) {
+                    const uint32_t bit = static_cast<uint32_t>(__ffs(sel) - 1), g = sel_g0 + (bit >> 2), c = bit & 3u;
+                    if (g - ls.begin < ls.end - ls.begin) q_key[pos] = make_uint2(4u * (g + ls.cgroup_off) + c, ls.tensor);
+                    else {
+                        const GroupInfo gi = find_group(a.pop, g, a.status);
+                        q_key[pos] = make_uint2(4u * gi.cgroup + c, gi.tensor_id);
+                    }
+                    q_elem[pos] = 4u * (sel_g0 - block_group) + bit;
                 }
             }
+            if (sel || t >= t_end) break;   // the queue is full, or the range is done (lane by lane: nothing in this loop needs the warp together)
+            sel_g0 = a.group_lo + t * kWarpTileGroups + 4u * lane;
+            sel = lane_masks(a, sel_g0, a.group_hi, ls);
+            t += kSparseWarps;
+        }
+        const bool again = __syncthreads_or(sel != 0 || t < t_end);   // (orders the queue's entries, too)
+        const uint32_t count = min(s_count, capacity);
+        for (uint32_t e = threadIdx.x; e < count; e += kSparseThreads) {
+            const uint2 key = q_key[e];
+            if (n_models <= 16) {
+                const uint64_t packed = draw_permutation_packed(n_models, key.x, key.y, a.step_lo, a.step_hi8, a.keys);
+                q_key[e] = make_uint2(static_cast<uint32_t>(packed), static_cast<uint32_t>(packed >> 32));
+            } else draw_permutation_u8(q_bytes + e, static_cast<int>(capacity), n_models, key.x, key.y, a.step_lo, a.step_hi8, a.keys);
             ++selected;
         }
-        __syncwarp();
-        head += count;
-    };
-    LaneSegment ls{1, 0, 0, 0, 0};
-    const uint32_t whole_tiles = (a.group_hi - a.group_lo) / kWarpTileGroups;   // tiles with all 128 groups inside the range
-    for (uint32_t t = t0; t < t1; ++t) {
-        uint32_t sel4 = 0;
-        const uint32_t g0 = a.group_lo + t * kWarpTileGroups + 4u * lane;   // meaningful (no wrap) when t < whole_tiles
-        if (!(t < whole_tiles && lane_masks_fast(a, g0, ls, &sel4))) {
-            const uint64_t g0_wide = static_cast<uint64_t>(a.group_lo) + static_cast<uint64_t>(t) * kWarpTileGroups + 4u * lane;
-            // ranges end on multiples of 4 groups: a lane's groups are all inside or all outside
-            if (g0_wide < a.group_hi) sel4 = lane_masks_general(a, static_cast<uint32_t>(g0_wide), ls, cursor);
+        __syncthreads();
+        // the lane's pairs of a set: [N][P] takes neighbouring coordinates of one model side by side,
+        // [P][N] the models of one coordinate
+        uint32_t pair_entry[kSparsePairs], pair_model[kSparsePairs];
+#pragma unroll
+        for (int k = 0; k < kSparsePairs; ++k) {
+            const uint32_t i = lane + 32u * k, outer = (i * p.inverse) >> 16;
+            const uint32_t inner = i - outer * (LAYOUT == kLayoutNP ? p.in_set : static_cast<uint32_t>(n_models));
+            pair_entry[k] = LAYOUT == kLayoutNP ? inner : outer;
+            pair_model[k] = LAYOUT == kLayoutNP ? outer : inner;
+            if (pair_model[k] >= static_cast<uint32_t>(n_models) || pair_entry[k] >= p.in_set) pair_entry[k] = 0xFFFFu;   // no pair
         }
-        if (__any_sync(kFull, sel4 != 0)) {
-            tail = ring_append(ring, tail, sel4, t - t0);
-            while (tail - head >= 32u) serve(32u);
+        for (uint32_t first = warp * p.in_set; first < count; first += kSparseWarps * p.in_set) {
+            const uint32_t left = count - first;
+            uint32_t va[kSparsePairs], vb[kSparsePairs];
+            long long out[kSparsePairs];
+#pragma unroll
+            for (int k = 0; k < kSparsePairs; ++k) {
+                out[k] = -1;
+                if (pair_entry[k] < left) {
+                    const uint32_t e = first + pair_entry[k], n = pair_model[k];
+                    uint32_t src;
+                    if (n_models <= 16) {
+                        const uint2 packed = q_key[e];
+                        src = ((n < 8 ? packed.x : packed.y) >> (4u * (n & 7u))) & 15u;
+                    } else src = q_bytes[n * capacity + e];
+                    if (src != n) {
+                        const long long elem = block_elem + q_elem[e];
+                        const long long in = elem_index<LAYOUT>(a.pop, static_cast<int>(src), elem);
+                        out[k] = elem_index<LAYOUT>(a.pop, static_cast<int>(n), elem);
+                        va[k] = TA::load_elem(a.a, in);
+                        if constexpr (kHasB) vb[k] = TB::load_elem(a.b, in);
+                    }
+                }
+            }
+            __syncwarp();   // every value of the set is loaded before the first is overwritten
+#pragma unroll
+            for (int k = 0; k < kSparsePairs; ++k) {
+                if (out[k] < 0) continue;
+                TA::store_elem(a.a, out[k], va[k]);
+                if constexpr (kHasB) TB::store_elem(a.b, out[k], vb[k]);
+                ++moved;
+            }
         }
+        if (!again) break;
+        __syncthreads();   // the queue is free
+        if (threadIdx.x == 0) s_count = 0;
+        __syncthreads();
     }
-    if (tail != head) serve(tail - head);
     publish_block_stats(a.stats, a.stat_slots, selected, moved);
 }
 
@@ -107,30 +160,32 @@ cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchSha
     SparseArgs p;
     p.s = args;
     p.n_wtiles = (args.group_hi - args.group_lo + kWarpTileGroups - 1) / kWarpTileGroups;
-    const size_t n = static_cast<size_t>(args.pop.N);
-    const size_t smem = 4 * (static_cast<size_t>(kSparseWarps) * kXRing + n * kSparseThreads) + (n > 16 ? n * kSparseThreads : 0);
+    const size_t smem = sparse_queue_capacity(args.pop.N) * (12 + (args.pop.N > 16 ? static_cast<size_t>(args.pop.N) : 0));
     auto kernel = args.pop.layout == kLayoutNP ? shuffle_sparse_kernel<TA, TB, kLayoutNP> : shuffle_sparse_kernel<TA, TB, kLayoutPN>;
     KernelFit fit;
     cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), kSparseThreads, smem, &fit);
     if (err != cudaSuccess) return err;
     if (fit.occupancy < 1) return cudaErrorLaunchOutOfResources;
-    // one resident wave of blocks, fewer for short rows; the warps share the tiles evenly
     const uint32_t resident = static_cast<uint32_t>(shape.sm_count > 0 ? shape.sm_count : 148) * static_cast<uint32_t>(fit.occupancy);
+    // Grid: enough blocks that one expects kSparsePerBlock selected coordinates, in several waves, so
+    // that one wave's (memory-bound) serving overlaps the next one's (multiply-bound) mask; but a warp
+    // keeps a few tiles, or a block's start, barriers and end weigh more than its mask, and a resident
+    // wave is the least.  Measured with 8 / 16 / 32 / 64 per block: cfg3 61.3 / 60.9 / 66.1 / 68.7 us, cfg4
+    // 82.3 / 82.3 / 86.2 / 96.3 us, 2^27 coordinates N = 2 at p = 1e-3 131 / 119 / 117 / 120 us; with 1 / 2 / 3 / 4 tiles a
+    // warp: five ResNet-50 models at p = 0.05 -> 0 60.7 / 51.2 / 49.7 / 51.2 us, eight of 2^25 at p = 0.01 98.2 / 98.6 /
+    // 101.7 / 104.0 us, [P][N] 69.6 / 53.3 / 49.3 / 49.2 us.
+    const double expected = static_cast<double>(args.expected_share) * 4.0 * static_cast<double>(args.group_hi - args.group_lo);
+    const double by_tiles = static_cast<double>(p.n_wtiles) / (kSparseWarps * (args.pop.layout == kLayoutNP ? 2 : 3));
+    uint32_t grid = static_cast<uint32_t>(fmin(expected / kSparsePerBlock, by_tiles));
+    if (grid < resident) grid = resident;
     const uint32_t want = (p.n_wtiles + kSparseWarps - 1) / kSparseWarps;
-    // Grid: one resident wave when a warp expects few selected coordinates; up to four waves when it
-    // expects many.  A warp serves its queue in full rounds and once at the end of its range, so with
-    // one wave every warp reaches its (latency-bound) last round at the same time, after the
-    // (multiply-bound) mask; with shorter ranges in several waves the block scheduler overlaps one
-    // wave's serving with the next one's mask and evens out ranges that select unequally (per-layer p).
-    // Measured (1 / 2 / 4 waves): cfg2 21.3 / 26.6 / 35.7 us at 2.4 coordinates a warp, cfg3 77.3 / 71.0 /
-    // 75.6 us at 11, cfg4 104.1 / 94.4 / 89.4 us at 27.  A warp keeps at least two tiles.
-    const double per_warp = static_cast<double>(args.expected_share) * 4.0 * static_cast<double>(args.group_hi - args.group_lo) /
-                            (static_cast<double>(resident) * kSparseWarps);
-    uint32_t waves = per_warp <= 8.0 ? 1u : (per_warp <= 20.0 ? 2u : 4u);
-    while (waves > 1 && p.n_wtiles < 2ull * waves * resident * kSparseWarps) waves >>= 1;
-    const uint32_t cap = resident * waves;
-    p.n_blocks = want < cap ? want : cap;
-    kernel<<<p.n_blocks, kSparseThreads, smem, stream>>>(p);
+    if (grid > want) grid = want;
+    p.per_block = p.n_wtiles / grid;
+    p.extra = p.n_wtiles % grid;
+    p.in_set = 32u * kSparsePairs / static_cast<uint32_t>(args.pop.N);
+    const uint32_t divisor = args.pop.layout == kLayoutNP ? p.in_set : static_cast<uint32_t>(args.pop.N);
+    p.inverse = (65536u + divisor - 1u) / divisor;
+    kernel<<<grid, kSparseThreads, smem, stream>>>(p);
     count_launch();
     return cudaGetLastError();
 }

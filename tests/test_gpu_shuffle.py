@@ -154,6 +154,22 @@ def test_sparse_mode_and_launch_shapes_give_the_same_bits(N):
     ref.close()
 
 
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("N,numel,p", [(2, [511], 1.0), (5, [512], 1.0), (5, [2049], 1.0), (16, [6143, 2], 1.0), (17, [2047, 4100], 1.0),
+                                       (32, [8192], 0.3), (33, [2100], 1.0), (64, [5000, 3], 0.9), (2, [3_000_001], 0.9), (10, [400_009], 0.002)])
+def test_sparse_queue_at_its_edges(N, numel, p, layout):
+    """One, two and several warp tiles per block; a queue that overflows within a tile (a block queues 512
+    coordinates, 256 above 32 models) and is served several times; sets that leave pairs without a coordinate."""
+    c = Case(N, numel, layout, "f32", "bf16" if N in (5, 17) else None, seed=N)
+    B.wash_set_mode(c.gpu.ctx, B.WASH_MODE_SPARSE)
+    call = B.wash_shuffle if c.host_opt is None else B.wash_shuffle_both
+    call(c.gpu.ctx, 6, p, None, seed=12, stats=c.stats_dev)
+    want = oracle.shuffle(c.ora, c.host, p, seed=12, step=6, stack2=c.host_opt)
+    c.assert_equal("N=%d numel=%s p=%g layout=%d" % (N, numel, p, layout))
+    assert c.gpu_stats() == tuple(want)
+    c.close()
+
+
 def test_edge_cases_p0_p1_single_element_and_padding():
     # p = 0: identity, nothing written; p = 1: everything selected
     c = Case(4, [1], 0, seed=1)
