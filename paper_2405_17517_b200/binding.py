@@ -52,7 +52,8 @@ def load() -> ctypes.CDLL:
                           "(there is no fallback path)" % LIB_PATH)
     L = ctypes.CDLL(LIB_PATH)
     vp, i32, i64, u64, dbl = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_uint64, ctypes.c_double
-    i64p, u32p, dblp = ctypes.POINTER(i64), ctypes.POINTER(ctypes.c_uint32), ctypes.POINTER(dbl)
+    i64p, u32p = ctypes.POINTER(i64), ctypes.POINTER(ctypes.c_uint32)
+    dblp = vp     # an array's address: making a typed pointer object costs more than the call's own checks
     L.wash_create.argtypes = [ctypes.POINTER(vp), i32, i32, i64p, i32, i32]
     L.wash_create_segments.argtypes = [ctypes.POINTER(vp), i32, i32, i64p, u32p, i64p, i32, i32]
     L.wash_destroy.argtypes = [vp]
@@ -88,7 +89,7 @@ def load() -> ctypes.CDLL:
 
 
 def _check(rc: int) -> None:
-    if rc != WASH_OK:
+    if rc:
         raise WashError(rc, load().wash_last_error().decode())
 
 
@@ -101,7 +102,7 @@ def _dbl_or_null(a):
     if a is None:
         return None, None
     arr = np.ascontiguousarray(a, dtype=np.float64)
-    return arr, arr.ctypes.data_as(ctypes.POINTER(ctypes.c_double))
+    return arr, arr.__array_interface__["data"][0]
 
 
 def _ptr(x) -> Optional[int]:
@@ -117,10 +118,20 @@ def _ptr(x) -> Optional[int]:
     raise TypeError("cannot take the address of %r" % type(x))
 
 
+_current_raw_stream = None
+
+
 def _stream(stream) -> Optional[int]:
+    """The caller's stream; None = the current stream of the current device.  That one is asked for by
+    its address: a torch.cuda.Stream object costs 4.7 us to make, as much as two kernel launches."""
+    global _current_raw_stream
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream or None
+        if _current_raw_stream is None:
+            import torch
+            torch.cuda.init()
+            _current_raw_stream = (torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+        raw, device = _current_raw_stream
+        return raw(device()) or None
     if isinstance(stream, int):
         return stream or None
     return stream.cuda_stream or None
