@@ -258,7 +258,8 @@ int shuffle_impl(wash_ctx *ctx, int which, uint64_t step, double p, const double
                              (elem_bytes(a_dtype) + (b ? elem_bytes(b_dtype) : 0));
         const double kernel_ns = bytes / 6000.0 + 2000.0;
         const double reporting_blocks = std::fmin(ctx->expected_selected, static_cast<double>(ctx->n_groups) / 64.0);
-        args.stat_slots = (2.0 * reporting_blocks / kernel_ns > 0.35) ? ctx->stat_slots_dev : nullptr;
+        args.stat_slots = ctx->stat_slots_dev;
+        args.stats_direct = 2.0 * reporting_blocks / kernel_ns <= 0.35;
         // WASH_MODE_AUTO: the expected share of selected coordinates decides
         if (ctx->mode == WASH_MODE_AUTO) {
             double coordinates = 0.0;
@@ -285,10 +286,10 @@ int shuffle_impl(wash_ctx *ctx, int which, uint64_t step, double p, const double
         if (ctx->shape.blocks_per_sm == -3) args.early = true;
         if (sq) {   // the statistic is gathered by the streaming kernel only
             mode = WASH_MODE_STREAM;
-            args.stat_slots = ctx->stat_slots_dev;
+            args.stats_direct = false;
             args.sq = *sq;
         }
-        if (mode == WASH_MODE_SPARSE) args.stat_slots = nullptr;   // one wave of large blocks: a few hundred atomics at most
+        if (mode == WASH_MODE_SPARSE) args.stats_direct = true;   // blocks that each serve a few dozen coordinates and more, spread over the launch
     }
     args.status = ctx->status_dev;
     bool supported = false;

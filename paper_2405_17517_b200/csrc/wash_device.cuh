@@ -175,6 +175,32 @@ __device__ __forceinline__ void publish_block_stats(unsigned long long *stats, S
     atomicAdd(dst + 1, static_cast<unsigned long long>(block_sum[1]));
 }
 
+// The same for a resident grid of one-warp blocks, without the flush kernel: the last block to
+// report to a slot moves the slot's totals on and zeroes the slot.  Two levels, because a few
+// thousand blocks that end together would queue up at one address (1-2 ns each).
+__device__ __forceinline__ void publish_warp_stats(unsigned long long *stats, StatSlot *slots, uint32_t selected, uint32_t moved)
+{
+    if (!stats) return;
+    selected = __reduce_add_sync(0xFFFFFFFFu, selected);
+    moved = __reduce_add_sync(0xFFFFFFFFu, moved);
+    if (threadIdx.x != 0) return;
+    StatSlot *slot = slots + blockIdx.x % kStatSlots;
+    if (selected) {
+        atomicAdd(&slot->selected, static_cast<unsigned long long>(selected));
+        atomicAdd(&slot->moved, static_cast<unsigned long long>(moved));
+    }
+    __threadfence();
+    const unsigned long long sharers = (gridDim.x - blockIdx.x % kStatSlots + kStatSlots - 1) / kStatSlots;
+    if (atomicAdd(&slot->blocks, 1ull) + 1ull != sharers) return;
+    __threadfence();
+    slot->blocks = 0;
+    const unsigned long long s = atomicExch(&slot->selected, 0ull), m = atomicExch(&slot->moved, 0ull);
+    if (s) {
+        atomicAdd(stats, s);
+        atomicAdd(stats + 1, m);
+    }
+}
+
 // ---- which segment does group g belong to ---------------------------------------------
 struct GroupInfo {
     uint32_t tensor_id;

@@ -107,9 +107,11 @@ cudaError_t launch_philox_probe(unsigned long long n_blocks, uint64_t seed, uint
     return cudaGetLastError();
 }
 
+// *flush: the kernel leaves its counters in the partial-sum slots
 static cudaError_t launch_shuffle_kernel(const ShuffleArgs &args, int a_dtype, int b_dtype, int mode,
-                                         const LaunchShape &shape, cudaStream_t stream, bool *supported)
+                                         const LaunchShape &shape, cudaStream_t stream, bool *supported, bool *flush)
 {
+    *flush = args.stats && !args.stats_direct;
     if (mode == kModeSparse) return launch_shuffle_sparse(args, a_dtype, b_dtype, shape, stream, supported);
     // Two streaming kernels.  A group of all models (both stacks) of at most kLoopMaxGroupBytes goes to the
     // resident-warp kernel, whose instruction count per group is a fraction of the one-trip kernel's, unless
@@ -123,15 +125,19 @@ static cudaError_t launch_shuffle_kernel(const ShuffleArgs &args, int a_dtype, i
     if (per_group > kLoopMaxGroupBytes && per_group <= kLoopWideGroupBytes) loop = args.expected_share >= kLoopWideShareLo && args.expected_share <= kLoopWideShareHi;
     if (shape.blocks_per_sm == -4) loop = true;
     if (shape.blocks_per_sm == -5 || args.sq.slots || args.early) loop = false;
-    if (loop) return launch_shuffle_stream_loop(args, a_dtype, b_dtype, shape, stream, supported);
+    if (loop) {
+        *flush = false;
+        return launch_shuffle_stream_loop(args, a_dtype, b_dtype, shape, stream, supported);
+    }
     return launch_shuffle_stream(args, a_dtype, b_dtype, shape, stream, supported);
 }
 
 cudaError_t launch_shuffle(const ShuffleArgs &args, int a_dtype, int b_dtype, int mode,
                            const LaunchShape &shape, cudaStream_t stream, bool *supported)
 {
-    cudaError_t err = launch_shuffle_kernel(args, a_dtype, b_dtype, mode, shape, stream, supported);
-    if (err != cudaSuccess || !*supported || !args.stats || !args.stat_slots) return err;
+    bool flush = false;
+    cudaError_t err = launch_shuffle_kernel(args, a_dtype, b_dtype, mode, shape, stream, supported, &flush);
+    if (err != cudaSuccess || !*supported || !flush) return err;
     flush_stats_kernel<<<1, kStatSlots, 0, stream>>>(args.stat_slots, args.stats);
     count_launch();
     return cudaGetLastError();

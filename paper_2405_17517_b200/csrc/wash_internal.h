@@ -29,7 +29,9 @@ static_assert(sizeof(SegEntry) == 32, "SegEntry must stay 32 bytes");
 // to dominate the kernel once most blocks have a selected coordinate.
 constexpr int kStatSlots = 256;
 struct StatSlot {
-    unsigned long long selected, moved, blocks, reserved;
+    unsigned long long selected, moved;
+    unsigned long long blocks;   // resident-warp streaming kernel: blocks that have reported
+    unsigned long long reserved;
 };
 
 struct PopView {
@@ -79,7 +81,8 @@ struct ShuffleArgs {
     PhiloxKeys keys;              // from the seed
     uint32_t step_lo, step_hi8;   // step & 0xFFFFFFFF, (step >> 32) << 8
     unsigned long long *stats;    // device-accessible {selected, moved} or nullptr
-    StatSlot *stat_slots;         // device, kStatSlots zeroed entries (left zeroed by every launch), or nullptr
+    StatSlot *stat_slots;         // device, kStatSlots zeroed entries (left zeroed by every launch)
+    bool stats_direct = false;    // few blocks report: they add to `stats` themselves (kernels that need a flush kernel otherwise)
     uint32_t *status;             // device status word
     SqArgs sq;                    // consensus distance of the first stack (streaming kernel only)
     uint32_t pn_pad = 0;          // streaming kernel, [P][N]: elements of padding after a group in the shared-memory image (0 or 4)
@@ -130,14 +133,16 @@ cudaError_t launch_exchange_receive(const ExchangeArgs &args, cudaStream_t strea
 enum ReduceOp { kOpEma = 0, kOpAverage = 1, kOpPapaAll = 2, kOpConsensus = 3 };
 
 // The resident-warp streaming kernel takes groups (all models, both stacks) of up to 48 bytes -- fp32 N = 2, 3;
-// bf16 N <= 6 -- when at most 30 % of the coordinates are expected to be selected.  Measured on 2^27 coordinates
-// against the one-trip kernel: 32 bytes 0.73-0.93 of its time, 48 bytes 0.89-0.98, 64 bytes 0.97-1.12.
+// bf16 N <= 6 -- when at most 30 % of the coordinates are expected to be selected, and two groups per lane instead of four
+// below kLoopNarrowShare (see its launcher).  Against the one-trip kernel, 2^25 coordinates: 32 bytes 0.6-0.9 of its time.
 constexpr size_t kLoopMaxGroupBytes = 48;
-constexpr float kLoopMaxShare = 0.3f;
-// Groups of 49 to 64 bytes go to it only for an expected selection between 0.7 % and 5 %: measured at 1 % and 3 %
-// it takes 0.89-0.97 of the one-trip kernel's time (both layouts), at 0.3 % 1.01-1.03, at 10 % 0.93 in [P][N] but 1.20 in [N][P].
+constexpr size_t kLoopFourMaxGroupBytes = 128;
+constexpr float kLoopMaxShare = 0.3f, kLoopNarrowShare = 0.0007f;
+// Groups of 49 to 64 bytes go to it for an expected selection between 0.3 % and 5 %, where serving weighs most.  Time
+// against what was launched before (the one-trip kernel; from 0.7 % to 5 % this one with two groups per lane) at p = 0.1 / 0.3 / 0.6 / 2 / 5 / 10 %: fp32 N = 4 [N][P] 1.12 0.96 0.88 0.89 0.95 1.05, [P][N] 1.08 0.98 0.80
+// 0.71 0.86 0.96; two fp32 stacks of N = 2 1.11 0.98 0.75 0.77 0.99 1.07; bf16 N = 8 1.06 0.94 0.74 0.74 0.76 0.79.
 constexpr size_t kLoopWideGroupBytes = 64;
-constexpr float kLoopWideShareLo = 0.007f, kLoopWideShareHi = 0.05f;
+constexpr float kLoopWideShareLo = 0.003f, kLoopWideShareHi = 0.05f;
 
 struct LaunchShape {
     int threads;         // 0 = default

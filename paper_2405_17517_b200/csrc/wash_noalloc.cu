@@ -75,6 +75,7 @@ extern "C" int wash_shuffle_noalloc(int32_t N, int32_t n_tensors, const int64_t 
     // row geometry, the same rule as wash_create: tensors start on multiples of 8 elements
     std::vector<SegEntry> seg(static_cast<size_t>(n_tensors));
     long long cur = 0;
+    double coordinates = 0.0, expected = 0.0;
     for (int t = 0; t < n_tensors; ++t) {
         const long long d = numel[t];
         if (d <= 0 || d >= (1ll << 32)) return fail(WASH_ERR_ARG, "numel[t] must be in (0, 2^32)");
@@ -90,6 +91,8 @@ extern "C" int wash_shuffle_noalloc(int32_t N, int32_t n_tensors, const int64_t 
         e.numel = static_cast<uint32_t>(d);
         e.reserved = 0;
         e.thr = static_cast<uint64_t>(std::floor(pt * 4294967296.0));
+        coordinates += static_cast<double>(d);
+        expected += static_cast<double>(d) * pt;
     }
     const long long padded_P = cur;
     if (n_elems != static_cast<int64_t>(N) * padded_P) return fail(WASH_ERR_ARG, "n_elems must equal N * padded_P");
@@ -162,6 +165,7 @@ extern "C" int wash_shuffle_noalloc(int32_t N, int32_t n_tensors, const int64_t 
             args.stats = reinterpret_cast<unsigned long long *>(stats);
             args.stat_slots = slots_dev;
             args.status = nullptr;
+            args.expected_share = static_cast<float>(expected / coordinates);
             const wash::LaunchShape shape{0, 0, sm_count};
             bool supported = false;
             err = wash::launch_shuffle(args, dtype, wash::kDtypeNone, wash::kModeStream, shape, stream, &supported);

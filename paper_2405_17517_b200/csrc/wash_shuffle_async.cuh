@@ -723,7 +723,7 @@ __global__ void __launch_bounds__(256, EARLY ? 3 : 5) shuffle_async_kernel(const
                                        g_first + static_cast<uint64_t>(i) * T_, sel[i], gi[i], selected, moved);
         }
     }
-    publish_block_stats(a.stats, a.stat_slots, selected, moved);
+    publish_block_stats(a.stats, a.stats_direct ? nullptr : a.stat_slots, selected, moved);
 }
 
 template <class TA, class TB, int G>

@@ -12,7 +12,15 @@
 // trips.  Tiles are dealt round-robin over the blocks, so the blocks resident at one moment read
 // neighbouring addresses.
 //
-// The image of a stage is the one-trip kernel's block image with T = 32 (the block is one warp,
+// Serving costs a hundred issue slots and more on a mostly idle warp however few coordinates it
+// serves (a permutation is a Philox block and a chain of swaps), so it is done once a tile for the
+// G groups of every lane together: the tile's selected coordinates are listed and dealt to the
+// lanes 32 at a time.  Bound: HBM up to p = 1e-3, issue slots above it.  N = 2, fp32, 2^27 coordinates
+// (before: two groups per lane, served one after the other, and a flush kernel for the counters):
+// p = 1e-2 390 -> 245 us, 1e-3 206 -> 203; 2^25 coordinates: p = 0.1 134 -> 95, 0.02 125 -> 71; one model
+// step of N = 3, 2^20 coordinates 12.3 -> 8.3.
+//
+// An image of a stage is the one-trip kernel's block image with T = 32 (the block is one warp,
 // so every helper of that kernel -- copies, serving, padding rule -- is used as it is).
 #pragma once
 #define WASH_SERVING_ONLY
@@ -95,19 +103,36 @@ __device__ __forceinline__ void fetch_full_tile_f32(uint32_t image, uint32_t ima
     }
 }
 
-template <class TA, class TB, int LAYOUT, int G, int S>
-__global__ void __launch_bounds__(32, 32) shuffle_loop_kernel(const __grid_constant__ ShuffleArgs a)
+// The tile's selected coordinates, listed as owner lane * 4G + bit, where bit 4 i + c stands for
+// coordinate c of the lane's group of image i.  `sel` has at most 4G bits.  Returns their number.
+template <int G>
+__device__ __forceinline__ uint32_t list_selected(uint16_t *list, uint32_t sel)
+{
+    const uint32_t lane = threadIdx.x;
+    uint32_t total = 0;
+    for (uint32_t owners = __ballot_sync(0xFFFFFFFFu, sel != 0); owners; owners = __ballot_sync(0xFFFFFFFFu, sel != 0)) {
+        if (sel) list[total + __popc(owners & ((1u << lane) - 1u))] = static_cast<uint16_t>(lane * (4 * G) + __ffs(sel) - 1);
+        sel &= sel - 1u;
+        total += __popc(owners);
+    }
+    __syncwarp();
+    return total;
+}
+
+template <class TA, class TB, int LAYOUT, int G>
+__global__ void __launch_bounds__(32, G == 2 ? 32 : 28) shuffle_loop_kernel(const __grid_constant__ ShuffleArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr bool kHasB = TB::kCode != kDtypeNone;
     constexpr uint32_t T_ = 32;   // the launch has one warp per block
     const int n_models = a.pop.N;
+    const uint32_t lane = threadIdx.x;
     const size_t group_elems = LAYOUT == kLayoutPN ? pn_group_elems(n_models, a.pn_pad) : 4u * static_cast<size_t>(n_models);
     const uint32_t a_bytes = static_cast<uint32_t>(group_elems * T_ * TA::kBytes);
     const uint32_t b_bytes = kHasB ? static_cast<uint32_t>(group_elems * T_ * TB::kBytes) : 0u;
     const uint32_t stage_bytes = G * (a_bytes + b_bytes);
-    uint8_t *s_list = smem_raw + S * stage_bytes;   // 128 bytes: the warp's list of selected coordinates
-    uint8_t *s_perm = s_list + 128 + threadIdx.x;   // a column [n][T] of bytes, used when N > 16
+    uint16_t *s_list = reinterpret_cast<uint16_t *>(smem_raw + 2 * stage_bytes);   // the tile's selected coordinates
+    uint8_t *s_perm = smem_raw + 2 * stage_bytes + 2 * T_ * 4 * G + lane;          // a column [n][T] of bytes, used when N > 16
 
     // group indices fit 32 bits (the table holds them so); a tile index therefore too
     const uint32_t n_tiles = static_cast<uint32_t>((a.group_hi - a.group_lo + T_ * G - 1) / (T_ * G));
@@ -125,7 +150,7 @@ __global__ void __launch_bounds__(32, 32) shuffle_loop_kernel(const __grid_const
             if constexpr (kHasB && TB::kBytes == 4) fetch_full_tile_f32<LAYOUT, G>(image_a + a_bytes, a_bytes + b_bytes, a.b, a.pop, g_first, n_models);
         }
         if (tile < n_tiles && !(tile < full_tiles && linear && kFastA && kFastB)) {
-#pragma unroll
+#pragma unroll 1
             for (int i = 0; i < G; ++i) {
                 const uint64_t g_block = static_cast<uint64_t>(g_first) + static_cast<uint64_t>(i) * T_;
                 if (g_block >= a.group_hi) break;
@@ -142,85 +167,95 @@ __global__ void __launch_bounds__(32, 32) shuffle_loop_kernel(const __grid_const
     uint32_t selected = 0, moved = 0, stage = 0;
     SegCache sc{0, 0, 0, 0, 0, 0, 0, 0, 0};
     uint32_t tile = blockIdx.x;
-    // S - 1 tiles in flight ahead of the one that is served; beyond the last tile (also when the
-    // index wraps) a fetch copies nothing
-    uint32_t ahead = tile, ahead_stage = 0;
-#pragma unroll
-    for (int k = 0; k < S - 1; ++k) {
-        fetch(ahead, ahead_stage);
-        ahead = ahead + gridDim.x >= ahead ? ahead + gridDim.x : n_tiles;
-        ahead_stage = ahead_stage + 1 == S ? 0 : ahead_stage + 1;
-    }
-    for (; tile < n_tiles; tile += gridDim.x, stage = stage + 1 == S ? 0 : stage + 1) {
-        fetch(ahead, ahead_stage);
-        ahead = ahead + gridDim.x >= ahead ? ahead + gridDim.x : n_tiles;
-        ahead_stage = ahead_stage + 1 == S ? 0 : ahead_stage + 1;
+    fetch(tile, 0);
+    for (; tile < n_tiles; tile += gridDim.x, stage ^= 1u) {
+        const uint32_t next = tile + gridDim.x;
+        fetch(next >= tile ? next : n_tiles, stage ^ 1u);   // beyond the last tile (also when the index wraps) a fetch copies nothing
         const uint32_t g_first = group_lo + tile * (T_ * G);
-        uint32_t sel[G];
-        GroupInfo gi[G];
+        uint32_t sel = 0;   // bit 4 i + c: coordinate c of group g_first + 32 i + lane
         // the usual tile: full, every lane's G groups whole and in the segment of its previous
         // group, thresholds that the mask words decide -- then nothing is looked up or predicated
-        const uint32_t local = g_first + threadIdx.x - sc.begin;
-        const bool plain = tile < full_tiles && __all_sync(0xFFFFFFFFu, local < sc.plain && local + (G - 1) * T_ < sc.plain);
-        if (plain) {
+        const uint32_t local = g_first + lane - sc.begin;
+        if (tile < full_tiles && __all_sync(0xFFFFFFFFu, local < sc.plain && local + (G - 1) * T_ < sc.plain)) {
+            uint32_t w[4 * G];
 #pragma unroll
             for (int i = 0; i < G; ++i) {
-                gi[i].seg = sc.seg;
-                gi[i].tensor_id = sc.tensor_id;
-                gi[i].cgroup = sc.cgroup_begin + local + i * T_;
-                gi[i].valid = 4;
-                gi[i].thr = sc.thr_lo;
-                const Philox4 w = philox4x32_10(gi[i].cgroup, sc.tensor_id, a.step_lo, a.step_hi8, a.keys);
-                sel[i] = (w.x < sc.thr_lo ? 1u : 0u) | (w.y < sc.thr_lo ? 2u : 0u) | (w.z < sc.thr_lo ? 4u : 0u) | (w.w < sc.thr_lo ? 8u : 0u);
+                const Philox4 block = philox4x32_10(sc.cgroup_begin + local + i * T_, sc.tensor_id, a.step_lo, a.step_hi8, a.keys);
+                w[4 * i] = block.x;
+                w[4 * i + 1] = block.y;
+                w[4 * i + 2] = block.z;
+                w[4 * i + 3] = block.w;
             }
+            sel = pack_below(w, sc.thr_lo);
         } else {
-#pragma unroll
+#pragma unroll 1
             for (int i = 0; i < G; ++i) {
-                sel[i] = 0;
-                gi[i] = GroupInfo{0, 0, 0, 0, 0};
-                const uint64_t g = static_cast<uint64_t>(g_first) + static_cast<uint64_t>(i) * T_ + threadIdx.x;
-                if (g < a.group_hi) {
-                    gi[i] = find_group_cached(a.pop, sc, static_cast<uint32_t>(g), a.status);
-                    if (gi[i].thr != 0 && gi[i].valid != 0) {
-                        uint32_t m = 0xFu;   // a threshold of 2^32 selects whatever the word is
-                        if ((gi[i].thr >> 32) == 0) {
-                            const Philox4 w = philox4x32_10(gi[i].cgroup, gi[i].tensor_id, a.step_lo, a.step_hi8, a.keys);
-                            const uint32_t thr_lo = static_cast<uint32_t>(gi[i].thr);
-                            m = (w.x < thr_lo ? 1u : 0u) | (w.y < thr_lo ? 2u : 0u) | (w.z < thr_lo ? 4u : 0u) | (w.w < thr_lo ? 8u : 0u);
-                        }
-                        sel[i] = m & ((1u << gi[i].valid) - 1u);
-                    }
+                const uint64_t g = static_cast<uint64_t>(g_first) + static_cast<uint64_t>(i) * T_ + lane;
+                if (g >= a.group_hi) break;
+                const GroupInfo gi = find_group_cached(a.pop, sc, static_cast<uint32_t>(g), a.status);
+                if (gi.thr == 0 || gi.valid == 0) continue;
+                uint32_t m = 0xFu;   // a threshold of 2^32 selects whatever the word is
+                if ((gi.thr >> 32) == 0) {
+                    const Philox4 w = philox4x32_10(gi.cgroup, gi.tensor_id, a.step_lo, a.step_hi8, a.keys);
+                    const uint32_t thr_lo = static_cast<uint32_t>(gi.thr);
+                    m = (w.x < thr_lo ? 1u : 0u) | (w.y < thr_lo ? 2u : 0u) | (w.z < thr_lo ? 4u : 0u) | (w.w < thr_lo ? 8u : 0u);
                 }
+                sel |= (m & ((1u << gi.valid) - 1u)) << (4 * i);
             }
         }
-        uint32_t any = 0;
-#pragma unroll
-        for (int i = 0; i < G; ++i) any |= sel[i];
-        cp_async_wait_all_but_latest<S - 1>();   // this tile's copies; the next tiles' stay in flight
+        cp_async_wait_all_but_latest<1>();   // this tile's copies; the next tile's stay in flight
         __syncwarp();
-        if (__any_sync(0xFFFFFFFFu, any != 0)) {
-#pragma unroll
+        if (!__any_sync(0xFFFFFFFFu, sel != 0)) continue;
+        const unsigned char *images = smem_raw + stage * stage_bytes;
+        const uint32_t count = __reduce_add_sync(0xFFFFFFFFu, __popc(sel));
+        if (n_models <= 16 && count >= kDenseMinSelected * G) {
+            // every lane serves its own groups, those that are whole; the others go to the list below
+#pragma unroll 1
             for (int i = 0; i < G; ++i) {
-                const unsigned char *image_a = smem_raw + stage * stage_bytes + i * (a_bytes + b_bytes);
-                serve_tile<TA, TB, LAYOUT>(a, image_a, image_a + a_bytes, s_list, s_perm,
-                                           static_cast<uint64_t>(g_first) + static_cast<uint64_t>(i) * T_, sel[i], gi[i], selected, moved);
+                const uint32_t mine = (sel >> (4 * i)) & 15u;
+                if (!mine) continue;
+                const uint32_t g = g_first + i * T_ + lane;
+                const GroupInfo gi = find_group_cached(a.pop, sc, g, a.status);
+                if (gi.valid != 4) continue;
+                sel &= ~(15u << (4 * i));
+                const unsigned char *image_a = images + i * (a_bytes + b_bytes);
+                if (n_models <= 8) serve_group_dense<TA, TB, LAYOUT, uint32_t>(a, image_a, image_a + a_bytes, g - lane, mine, gi, selected, moved);
+                else serve_group_dense<TA, TB, LAYOUT, uint64_t>(a, image_a, image_a + a_bytes, g - lane, mine, gi, selected, moved);
             }
-            __syncwarp();   // the stage is overwritten by the copies the next trip starts
         }
+        // the selected coordinates of all G images, 32 at a time, one per lane
+        const uint32_t total = list_selected<G>(s_list, sel);
+        for (uint32_t first = lane; first < total; first += 32) {
+            const uint32_t entry = s_list[first], owner = entry / (4 * G), i = (entry / 4) % G, c = entry & 3u;
+            const uint32_t g = g_first + i * T_ + owner;
+            uint32_t cgroup = sc.cgroup_begin + (g - sc.begin), tensor = sc.tensor_id;
+            if (g - sc.begin >= sc.end - sc.begin) {   // another lane's tensor
+                const GroupInfo gi = find_group(a.pop, g, a.status);
+                cgroup = gi.cgroup;
+                tensor = gi.tensor_id;
+            }
+            uint64_t perm = 0;
+            if (n_models <= 16) perm = draw_permutation_packed(n_models, 4u * cgroup + c, tensor, a.step_lo, a.step_hi8, a.keys);
+            else draw_permutation_u8(s_perm, T_, n_models, 4u * cgroup + c, tensor, a.step_lo, a.step_hi8, a.keys);
+            const unsigned char *image_a = images + i * (a_bytes + b_bytes);
+            move_coordinate<TA, TB, LAYOUT>(a, image_a, image_a + a_bytes, s_perm, perm, owner, c, g - owner, moved);
+            ++selected;
+        }
+        __syncwarp();   // the stage is overwritten by the copies the next trip starts
     }
     cp_async_wait_all();
-    publish_block_stats(a.stats, a.stat_slots, selected, moved);
+    publish_warp_stats(a.stats, a.stat_slots, selected, moved);
 }
 
-template <class TA, class TB, int G, int S>
+template <class TA, class TB, int G>
 cudaError_t launch_shuffle_loop_tiles(const ShuffleArgs &args, const LaunchShape &shape, cudaStream_t stream)
 {
     constexpr bool kHasB = TB::kCode != kDtypeNone;
     const size_t group_elems = 4 * static_cast<size_t>(args.pop.N) + (args.pop.layout == kLayoutPN ? args.pn_pad : 0);
     const size_t image = group_elems * (TA::kBytes + (kHasB ? TB::kBytes : 0)) * 32;
-    const size_t smem = (S * G * image + 128 + (args.pop.N > 16 ? 32 * static_cast<size_t>(args.pop.N) : 0) + 15) & ~static_cast<size_t>(15);
+    const size_t smem = (2 * G * image + 2 * 32 * 4 * G + (args.pop.N > 16 ? 32 * static_cast<size_t>(args.pop.N) : 0) + 15) & ~static_cast<size_t>(15);
     const bool np = args.pop.layout == kLayoutNP;
-    auto kernel = np ? shuffle_loop_kernel<TA, TB, kLayoutNP, G, S> : shuffle_loop_kernel<TA, TB, kLayoutPN, G, S>;
+    auto kernel = np ? shuffle_loop_kernel<TA, TB, kLayoutNP, G> : shuffle_loop_kernel<TA, TB, kLayoutPN, G>;
     KernelFit fit;
     cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), 32, smem, &fit);
     if (err != cudaSuccess) return err;
@@ -238,11 +273,15 @@ cudaError_t launch_shuffle_loop_tiles(const ShuffleArgs &args, const LaunchShape
 template <class TA, class TB>
 cudaError_t launch_shuffle_loop_typed(const ShuffleArgs &args, const LaunchShape &shape, cudaStream_t stream)
 {
-    // Two groups per lane and tile, two stages.  Measured on 2^27 coordinates (N = 2, fp32, p = 1e-4 .. 0.1):
-    // one group per lane leaves too few bytes in flight (0.215 against 0.174 ms at p = 1e-4), four make a
-    // trip that serves anything long and cost resident warps (0.294 against 0.217 ms at p = 1e-3), a third
-    // stage changes nothing (0.226 against 0.219 ms).
-    return launch_shuffle_loop_tiles<TA, TB, 2, 2>(args, shape, stream);
+    // Four groups per lane and tile, or two when less than kLoopNarrowShare of the coordinates is expected to
+    // be selected: then a trip is short, and more resident warps (32 against 24 on an SM at N = 2) matter more than the
+    // serving that four groups share.  Measured (N = 2, fp32, 2^27 coordinates, four / two): p = 1e-4 191 / 176 us, 1e-3
+    // 207 / 201, 1e-2 244 / 310; 2^25 coordinates, p = 3e-4 54.1 / 51.5, 1e-3 58.0 / 59.3, 0.1 95.2 / 98.7.  A third stage
+    // costs resident warps and was slower everywhere (p = 1e-2 334 us with two groups).
+    // (A forced launch may bring groups of any size: beyond kLoopFourMaxGroupBytes four of them leave too few warps.)
+    const size_t per_group = static_cast<size_t>(args.pop.N) * 4 * (TA::kBytes + TB::kBytes);
+    if (args.expected_share < kLoopNarrowShare || per_group > kLoopFourMaxGroupBytes) return launch_shuffle_loop_tiles<TA, TB, 2>(args, shape, stream);
+    return launch_shuffle_loop_tiles<TA, TB, 4>(args, shape, stream);
 }
 
 inline cudaError_t launch_shuffle_loop(const ShuffleArgs &args, int a_dtype, int b_dtype, const LaunchShape &shape,

@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_spa
         if (threadIdx.x == 0) s_count = 0;
         __syncthreads();
     }
-    publish_block_stats(a.stats, a.stat_slots, selected, moved);
+    publish_block_stats(a.stats, a.stats_direct ? nullptr : a.stat_slots, selected, moved);
 }
 
 template <class TA, class TB>

@@ -170,6 +170,27 @@ def test_sparse_queue_at_its_edges(N, numel, p, layout):
     c.close()
 
 
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("N,numel,p,dtype,opt", [
+    (2, [509], 0.3, "f32", None), (2, [512], 0.3, "f32", None), (3, [513, 8], 0.2, "f32", None), (3, [255, 256, 257, 1024], 0.02, "bf16", None),
+    (2, [2_000_003], 0.01, "f32", None), (3, [2_400_000, 9, 700_000], 0.0002, "f32", None), (2, [1_500_001], 1.0, "f32", None),
+    (4, [900_001, 77], 0.02, "f32", None), (2, [700_001], 0.3, "f32", "f32"), (10, [300_001], 0.6, "f32", None), (17, [40_001], 0.3, "bf16", "f32")])
+def test_resident_warp_kernel_serves_a_tiles_groups_together(N, numel, p, dtype, opt, layout):
+    """The small-group streaming kernel: tiles of 128 and of 64 groups (below 0.07 % expected selection), ragged and
+    single tiles, tensors that end inside a tile, lists of more than 32 coordinates, tiles selected in full."""
+    c = Case(N, numel, layout, dtype, opt, seed=N)
+    B.wash_set_launch(c.gpu.ctx, 0, -4)
+    call = B.wash_shuffle if opt is None else B.wash_shuffle_both
+    tot = [0, 0]
+    for step in (0, 1):     # twice: the counters' slots must be left zeroed
+        call(c.gpu.ctx, step, p, None, seed=31, stats=c.stats_dev)
+        s = oracle.shuffle(c.ora, c.host, p, seed=31, step=step, stack2=c.host_opt)
+        tot[0] += s[0]; tot[1] += s[1]
+    c.assert_equal("N=%d numel=%s p=%g layout=%d" % (N, numel, p, layout))
+    assert c.gpu_stats() == tuple(tot)
+    c.close()
+
+
 def test_edge_cases_p0_p1_single_element_and_padding():
     # p = 0: identity, nothing written; p = 1: everything selected
     c = Case(4, [1], 0, seed=1)
