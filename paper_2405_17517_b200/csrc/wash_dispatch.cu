@@ -11,6 +11,7 @@ WASH_N_LIST(WASH_DECL)
 #undef WASH_DECL
 cudaError_t launch_shuffle_sparse(const ShuffleArgs &, int, int, const LaunchShape &, cudaStream_t, bool *);
 cudaError_t launch_shuffle_stream(const ShuffleArgs &, int, int, const LaunchShape &, cudaStream_t, bool *);
+cudaError_t launch_shuffle_stream_wide(const ShuffleArgs &, int, int, const LaunchShape &, cudaStream_t, bool *);
 cudaError_t launch_shuffle_stream_loop(const ShuffleArgs &, int, int, const LaunchShape &, cudaStream_t, bool *);
 cudaError_t launch_reduce_n0(const ReduceArgs &, int, int, int, const LaunchShape &, cudaStream_t, bool *);
 
@@ -113,10 +114,11 @@ static cudaError_t launch_shuffle_kernel(const ShuffleArgs &args, int a_dtype, i
 {
     *flush = args.stats && !args.stats_direct;
     if (mode == kModeSparse) return launch_shuffle_sparse(args, a_dtype, b_dtype, shape, stream, supported);
-    // Two streaming kernels.  A group of all models (both stacks) of at most kLoopMaxGroupBytes goes to the
+    // Three streaming kernels.  A group of all models (both stacks) of at most kLoopMaxGroupBytes goes to the
     // resident-warp kernel, whose instruction count per group is a fraction of the one-trip kernel's, unless
     // most coordinates are expected to be served (there the one-trip kernel measured 6 % faster); larger
-    // groups, the consensus statistic and the early flavour stay with the one-trip kernel.
+    // groups, the consensus statistic and the early flavour stay with the one-trip kernel; populations of more
+    // than 16 models have a one-trip kernel of their own from kWideMinShare on, until the early flavour takes over.
     // blocks_per_sm of wash_set_launch: -4 forces the resident-warp kernel, -5 the one-trip kernel.
     const size_t elem_a = a_dtype == kDtypeF32 ? 4 : a_dtype == kDtypeBF16 ? 2 : 0, elem_b = b_dtype == kDtypeF32 ? 4 : b_dtype == kDtypeBF16 ? 2 : 0;
     const size_t per_group = static_cast<size_t>(args.pop.N) * 4 * (elem_a + elem_b);
@@ -124,11 +126,12 @@ static cudaError_t launch_shuffle_kernel(const ShuffleArgs &args, int a_dtype, i
     // 64-byte groups (fp32 N = 4, two fp32 stacks of N = 2, bf16 N = 8): only where serving weighs most
     if (per_group > kLoopMaxGroupBytes && per_group <= kLoopWideGroupBytes) loop = args.expected_share >= kLoopWideShareLo && args.expected_share <= kLoopWideShareHi;
     if (shape.blocks_per_sm == -4) loop = true;
-    if (shape.blocks_per_sm == -5 || args.sq.slots || args.early) loop = false;
+    if (shape.blocks_per_sm == -5 || args.sq.slots || args.early || args.pop.N > 16) loop = false;
     if (loop) {
         *flush = false;
         return launch_shuffle_stream_loop(args, a_dtype, b_dtype, shape, stream, supported);
     }
+    if (args.pop.N > 16 && !args.early && args.expected_share >= kWideMinShare) return launch_shuffle_stream_wide(args, a_dtype, b_dtype, shape, stream, supported);
     return launch_shuffle_stream(args, a_dtype, b_dtype, shape, stream, supported);
 }
 

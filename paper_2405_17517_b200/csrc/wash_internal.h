@@ -86,6 +86,7 @@ struct ShuffleArgs {
     uint32_t *status;             // device status word
     SqArgs sq;                    // consensus distance of the first stack (streaming kernel only)
     uint32_t pn_pad = 0;          // streaming kernel, [P][N]: elements of padding after a group in the shared-memory image (0 or 4)
+    uint32_t pair_inverse = 0;    // streaming kernel, N > 16: 2^20 / N, rounded up (i / N = i * pair_inverse >> 20 for i < 2080; set by its launcher)
     bool early = false;           // streaming kernel: the flavour that draws permutations while the copies are in flight
     float expected_share = 0.f;   // share of the coordinates the call's probabilities select, in expectation (sizes the sparse kernel's grid)
 };
@@ -143,6 +144,11 @@ constexpr float kLoopMaxShare = 0.3f, kLoopNarrowShare = 0.0007f;
 // 0.71 0.86 0.96; two fp32 stacks of N = 2 1.11 0.98 0.75 0.77 0.99 1.07; bf16 N = 8 1.06 0.94 0.74 0.74 0.76 0.79.
 constexpr size_t kLoopWideGroupBytes = 64;
 constexpr float kLoopWideShareLo = 0.003f, kLoopWideShareHi = 0.05f;
+
+// N > 16: below this expected selection the one-trip kernel's own serving (a single coordinate of a warp served by the
+// whole warp) is as good (N = 20 .. 64, p = 1e-3: 0.97-1.03 of the wide kernel's time; N = 17 in bf16 26.6 against 27.6 us for
+// 4.0 M coordinates); at 1 % the wide kernel takes 0.65-0.99 of its time.
+constexpr float kWideMinShare = 0.003f;
 
 struct LaunchShape {
     int threads;         // 0 = default

@@ -132,7 +132,6 @@ __global__ void __launch_bounds__(32, G == 2 ? 32 : 28) shuffle_loop_kernel(cons
     const uint32_t b_bytes = kHasB ? static_cast<uint32_t>(group_elems * T_ * TB::kBytes) : 0u;
     const uint32_t stage_bytes = G * (a_bytes + b_bytes);
     uint16_t *s_list = reinterpret_cast<uint16_t *>(smem_raw + 2 * stage_bytes);   // the tile's selected coordinates
-    uint8_t *s_perm = smem_raw + 2 * stage_bytes + 2 * T_ * 4 * G + lane;          // a column [n][T] of bytes, used when N > 16
 
     // group indices fit 32 bits (the table holds them so); a tile index therefore too
     const uint32_t n_tiles = static_cast<uint32_t>((a.group_hi - a.group_lo + T_ * G - 1) / (T_ * G));
@@ -208,7 +207,7 @@ __global__ void __launch_bounds__(32, G == 2 ? 32 : 28) shuffle_loop_kernel(cons
         if (!__any_sync(0xFFFFFFFFu, sel != 0)) continue;
         const unsigned char *images = smem_raw + stage * stage_bytes;
         const uint32_t count = __reduce_add_sync(0xFFFFFFFFu, __popc(sel));
-        if (n_models <= 16 && count >= kDenseMinSelected * G) {
+        if (count >= kDenseMinSelected * G) {
             // every lane serves its own groups, those that are whole; the others go to the list below
 #pragma unroll 1
             for (int i = 0; i < G; ++i) {
@@ -234,11 +233,9 @@ __global__ void __launch_bounds__(32, G == 2 ? 32 : 28) shuffle_loop_kernel(cons
                 cgroup = gi.cgroup;
                 tensor = gi.tensor_id;
             }
-            uint64_t perm = 0;
-            if (n_models <= 16) perm = draw_permutation_packed(n_models, 4u * cgroup + c, tensor, a.step_lo, a.step_hi8, a.keys);
-            else draw_permutation_u8(s_perm, T_, n_models, 4u * cgroup + c, tensor, a.step_lo, a.step_hi8, a.keys);
+            const uint64_t perm = draw_permutation_packed(n_models, 4u * cgroup + c, tensor, a.step_lo, a.step_hi8, a.keys);
             const unsigned char *image_a = images + i * (a_bytes + b_bytes);
-            move_coordinate<TA, TB, LAYOUT>(a, image_a, image_a + a_bytes, s_perm, perm, owner, c, g - owner, moved);
+            move_coordinate<TA, TB, LAYOUT>(a, image_a, image_a + a_bytes, nullptr, perm, owner, c, g - owner, moved);
             ++selected;
         }
         __syncwarp();   // the stage is overwritten by the copies the next trip starts
@@ -253,7 +250,7 @@ cudaError_t launch_shuffle_loop_tiles(const ShuffleArgs &args, const LaunchShape
     constexpr bool kHasB = TB::kCode != kDtypeNone;
     const size_t group_elems = 4 * static_cast<size_t>(args.pop.N) + (args.pop.layout == kLayoutPN ? args.pn_pad : 0);
     const size_t image = group_elems * (TA::kBytes + (kHasB ? TB::kBytes : 0)) * 32;
-    const size_t smem = (2 * G * image + 2 * 32 * 4 * G + (args.pop.N > 16 ? 32 * static_cast<size_t>(args.pop.N) : 0) + 15) & ~static_cast<size_t>(15);
+    const size_t smem = (2 * G * image + 2 * 32 * 4 * G + 15) & ~static_cast<size_t>(15);
     const bool np = args.pop.layout == kLayoutNP;
     auto kernel = np ? shuffle_loop_kernel<TA, TB, kLayoutNP, G> : shuffle_loop_kernel<TA, TB, kLayoutPN, G>;
     KernelFit fit;

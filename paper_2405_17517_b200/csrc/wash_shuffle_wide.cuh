@@ -1,0 +1,160 @@
+// Streaming shuffle for populations of more than 16 models: the one-trip kernel's copies and block
+// image (wash_shuffle_async.cuh), its serving arranged for permutations that fit no register.
+//
+// Shared memory (35 KB a block of 64 threads at N = 32 in fp32) leaves six blocks on an SM, so a block's
+// life from its first copy to its last store decides the bandwidth, and registers are free.  What a
+// selected coordinate costs is kept off that path: the warp lists its coordinates and draws the first
+// 32 permutations while the copies are in flight, the Philox blocks dealt to all lanes
+// (draw_permutations_by_warp); after the wait a lane per (coordinate, model) pair moves one value,
+// which in [P][N] is one 128-byte store per coordinate.  Before, one lane drew a coordinate's eight blocks one
+// after the other and moved its N values in a loop, all after the wait.  N = 32, fp32, 2^24 coordinates, [P][N],
+// p = 0.01 / 0.03 / 0.1: 376 / 500 / 681 -> 334 / 373 / 482 us (reading and writing alone 331 / 338 / 361); [N][P] 415 / 599 / 753 ->
+// 408 / 544 / 632 us; N = 20, bf16 + fp32, [P][N], p = 0.25: 1221 -> 678 us.
+#pragma once
+#define WASH_SERVING_ONLY
+#include "wash_shuffle_async.cuh"
+
+namespace wash {
+
+// [N][P]: up to this many coordinates of a round are moved by a lane per (coordinate, model) pair, more by a lane
+// per coordinate: the models of a coordinate share a bank of the image.  N = 32, 2^24 coordinates: p = 0.01 (1.3
+// coordinates a warp) 408 us by pairs, 422 by coordinates; p = 0.1 (12.8) 1155 / 627 us.
+constexpr uint32_t kWidePairsMax = 6;
+
+// What a (coordinate, model) pair's lane does: model n takes the value of model src.
+template <class TA, class TB, int LAYOUT>
+__device__ __forceinline__ void move_value(const ShuffleArgs &a, const unsigned char *image_a, const unsigned char *image_b, uint64_t g_block,
+                                           uint32_t t_owner, uint32_t c, uint32_t n, uint32_t src)
+{
+    constexpr bool kHasB = TB::kCode != kDtypeNone;
+    const int n_models = a.pop.N;
+    const long long out = elem_index<LAYOUT>(a.pop, static_cast<int>(n), 4ll * static_cast<long long>(g_block + t_owner) + c);
+    TA::store_elem(a.a, out, image_value<TA, LAYOUT>(image_a, n_models, a.pn_pad, t_owner, static_cast<int>(src), static_cast<int>(c)));
+    if constexpr (kHasB) TB::store_elem(a.b, out, image_value<TB, LAYOUT>(image_b, n_models, a.pn_pad, t_owner, static_cast<int>(src), static_cast<int>(c)));
+}
+
+template <class TA, class TB, int LAYOUT, bool STAT>
+__global__ void __launch_bounds__(64, 6) shuffle_wide_kernel(const __grid_constant__ ShuffleArgs a)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    constexpr bool kHasB = TB::kCode != kDtypeNone;
+    const int n_models = a.pop.N;
+    const uint32_t T_ = blockDim.x, lane = threadIdx.x & 31u, warp_base = threadIdx.x & ~31u;
+    // the images of the two stacks, the warps' lists, 32 permutations per warp
+    const size_t group_elems = LAYOUT == kLayoutPN ? pn_group_elems(n_models, a.pn_pad) : 4u * static_cast<size_t>(n_models);
+    unsigned char *image_a = smem_raw, *image_b = image_a + group_elems * T_ * TA::kBytes;
+    uint8_t *list = image_b + (kHasB ? group_elems * T_ * TB::kBytes : 0) + 4 * warp_base;   // 128 bytes a warp: owner lane * 4 + coordinate slot
+    uint32_t *s_perm = reinterpret_cast<uint32_t *>(image_b + (kHasB ? group_elems * T_ * TB::kBytes : 0) + 4 * T_) + warp_base * wide_pitch(n_models);
+
+    const uint64_t g_block = a.group_lo + static_cast<uint64_t>(blockIdx.x) * T_;
+    const uint32_t in_block = static_cast<uint32_t>(min(static_cast<uint64_t>(T_), a.group_hi - g_block));
+    async_fetch<TA, LAYOUT>(smem_addr(image_a), a.a, a.pop, g_block, in_block, n_models, a.pn_pad);
+    if constexpr (kHasB) async_fetch<TB, LAYOUT>(smem_addr(image_b), a.b, a.pop, g_block, in_block, n_models, a.pn_pad);
+
+    uint32_t selected = 0, moved = 0, sel = 0;
+    GroupInfo gi{0, 0, 0, 0, 0};
+    if (threadIdx.x < in_block) {
+        gi = find_group(a.pop, static_cast<uint32_t>(g_block + threadIdx.x), a.status);
+        if (gi.thr != 0 && gi.valid != 0) {
+            uint32_t m = 0xFu;   // a threshold of 2^32 selects whatever the word is
+            if ((gi.thr >> 32) == 0) {
+                const Philox4 w = philox4x32_10(gi.cgroup, gi.tensor_id, a.step_lo, a.step_hi8, a.keys);
+                const uint32_t thr_lo = static_cast<uint32_t>(gi.thr);
+                m = (w.x < thr_lo ? 1u : 0u) | (w.y < thr_lo ? 2u : 0u) | (w.z < thr_lo ? 4u : 0u) | (w.w < thr_lo ? 8u : 0u);
+            }
+            sel = m & ((1u << gi.valid) - 1u);   // coordinates beyond the tensor's end do not exist
+        }
+    }
+    // the warp's selected coordinates, and the first 32 permutations, while the copies are in flight
+    uint32_t total = 0;
+    for (uint32_t left = sel, owners; (owners = __ballot_sync(0xFFFFFFFFu, left != 0)) != 0; left &= left - 1u) {
+        if (left) list[total + __popc(owners & ((1u << lane) - 1u))] = static_cast<uint8_t>(lane * 4 + __ffs(left) - 1);
+        total += __popc(owners);
+    }
+    __syncwarp();
+    uint32_t entry = 0;
+    auto draw = [&](uint32_t first, uint32_t count) {
+        entry = lane < count ? list[first + lane] : 0u;
+        const uint32_t owner = entry >> 2;
+        const uint32_t cgroup = __shfl_sync(0xFFFFFFFFu, gi.cgroup, owner), tensor = __shfl_sync(0xFFFFFFFFu, gi.tensor_id, owner);
+        draw_permutations_by_warp(s_perm, n_models, count, 4u * cgroup + (entry & 3u), tensor, a.step_lo, a.step_hi8, a.keys);
+    };
+    if (total) draw(0, min(32u, total));
+    cp_async_wait_all();
+    if (LAYOUT == kLayoutPN) __syncthreads();   // a group's bytes were copied by threads of other warps
+    else __syncwarp();
+    if constexpr (STAT) consensus_tile<TA, LAYOUT>(a, image_a, gi, threadIdx.x < in_block);
+
+    for (uint32_t first = 0; first < total; first += 32) {
+        const uint32_t count = min(32u, total - first);
+        if (first) draw(first, count);
+        if (lane < count) ++selected;
+        if (LAYOUT == kLayoutPN || count <= kWidePairsMax) {
+            // a lane per (coordinate, model) pair, the models of a coordinate side by side
+            const uint32_t pairs = count * static_cast<uint32_t>(n_models);
+            for (uint32_t base = 0; base < pairs; base += 32) {
+                const uint32_t i = base + lane, l = min((i * a.pair_inverse) >> 20, count - 1u), n = i - l * static_cast<uint32_t>(n_models);
+                const uint32_t its_entry = __shfl_sync(0xFFFFFFFFu, entry, l);
+                if (i >= pairs) continue;
+                const uint32_t src = reinterpret_cast<const uint8_t *>(s_perm + l * wide_pitch(n_models))[n];
+                if (src == n) continue;
+                move_value<TA, TB, LAYOUT>(a, image_a, image_b, g_block, warp_base + (its_entry >> 2), its_entry & 3u, n, src);
+                ++moved;
+            }
+        } else if (lane < count) {
+            // a lane per coordinate: the models of a coordinate lie a whole row apart here, and in one bank of the image
+            const uint8_t *perm = reinterpret_cast<const uint8_t *>(s_perm + lane * wide_pitch(n_models));
+#pragma unroll 4
+            for (int n = 0; n < n_models; ++n) {
+                const uint32_t src = perm[n];
+                if (src == static_cast<uint32_t>(n)) continue;
+                move_value<TA, TB, LAYOUT>(a, image_a, image_b, g_block, warp_base + (entry >> 2), entry & 3u, n, src);
+                ++moved;
+            }
+        }
+        __syncwarp();   // the permutations are overwritten by the next round
+    }
+    publish_block_stats(a.stats, a.stats_direct ? nullptr : a.stat_slots, selected, moved);
+}
+
+template <class TA, class TB>
+cudaError_t launch_shuffle_wide_typed(const ShuffleArgs &call, const LaunchShape &shape, cudaStream_t stream)
+{
+    constexpr bool kHasB = TB::kCode != kDtypeNone;
+    ShuffleArgs args = call;
+    args.pair_inverse = ((1u << 20) + static_cast<uint32_t>(args.pop.N) - 1u) / static_cast<uint32_t>(args.pop.N);
+    const size_t group_elems = 4 * static_cast<size_t>(args.pop.N) + (args.pop.layout == kLayoutPN ? args.pn_pad : 0);
+    const size_t per_thread = group_elems * (TA::kBytes + (kHasB ? TB::kBytes : 0)) + 4 + 4 * wide_pitch(args.pop.N);
+    int threads = shape.threads > 0 ? (shape.threads >= 64 ? 64 : 32) : 64;
+    while (threads > 32 && per_thread * threads > 44 * 1024) threads >>= 1;   // five blocks and more on an SM
+    const size_t smem = (per_thread * threads + 15) & ~static_cast<size_t>(15);
+    const bool np = args.pop.layout == kLayoutNP;
+    auto kernel = np ? shuffle_wide_kernel<TA, TB, kLayoutNP, false> : shuffle_wide_kernel<TA, TB, kLayoutPN, false>;
+    if (args.sq.slots) kernel = np ? shuffle_wide_kernel<TA, TB, kLayoutNP, true> : shuffle_wide_kernel<TA, TB, kLayoutPN, true>;
+    KernelFit fit;
+    cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), threads, smem, &fit);
+    if (err != cudaSuccess) return err;
+    if (fit.occupancy < 1) return cudaErrorLaunchOutOfResources;
+    const uint64_t grid = (static_cast<uint64_t>(args.group_hi - args.group_lo) + threads - 1) / threads;
+    if (grid == 0) return cudaSuccess;
+    if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+    kernel<<<static_cast<unsigned>(grid), threads, smem, stream>>>(args);
+    count_launch();
+    return cudaGetLastError();
+}
+
+inline cudaError_t launch_shuffle_wide(const ShuffleArgs &args, int a_dtype, int b_dtype, const LaunchShape &shape,
+                                       cudaStream_t stream, bool *supported)
+{
+    *supported = true;
+    if (a_dtype == kDtypeF32 && b_dtype == kDtypeNone) return launch_shuffle_wide_typed<F32, NoStack>(args, shape, stream);
+    if (a_dtype == kDtypeBF16 && b_dtype == kDtypeNone) return launch_shuffle_wide_typed<BF16, NoStack>(args, shape, stream);
+    if (a_dtype == kDtypeF32 && b_dtype == kDtypeF32) return launch_shuffle_wide_typed<F32, F32>(args, shape, stream);
+    if (a_dtype == kDtypeBF16 && b_dtype == kDtypeF32) return launch_shuffle_wide_typed<BF16, F32>(args, shape, stream);
+    if (a_dtype == kDtypeBF16 && b_dtype == kDtypeBF16) return launch_shuffle_wide_typed<BF16, BF16>(args, shape, stream);
+    if (a_dtype == kDtypeF32 && b_dtype == kDtypeBF16) return launch_shuffle_wide_typed<F32, BF16>(args, shape, stream);
+    *supported = false;
+    return cudaSuccess;
+}
+
+}  // namespace wash

@@ -191,6 +191,22 @@ def test_resident_warp_kernel_serves_a_tiles_groups_together(N, numel, p, dtype,
     c.close()
 
 
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("N,numel,p,dtype,opt", [
+    (17, [30_001], 0.01, "f32", None), (18, [127, 1, 130, 4000], 0.1, "bf16", None), (20, [50_003], 0.25, "bf16", "f32"),
+    (32, [40_009], 0.1, "f32", None), (33, [255, 9000], 0.2, "f32", None), (63, [20_001], 0.05, "f32", "bf16"), (64, [12_345], 0.28, "f32", "f32")])
+def test_wide_population_kernel(N, numel, p, dtype, opt, layout):
+    """The streaming kernel of N > 16: permutations of 17 to 64 entries (last Philox block full and partly used), rounds
+    of up to 32 and several rounds per warp, few and many coordinates in [N][P] (a lane per pair / per coordinate)."""
+    c = Case(N, numel, layout, dtype, opt, seed=N)
+    call = B.wash_shuffle if opt is None else B.wash_shuffle_both
+    call(c.gpu.ctx, 3, p, None, seed=77, stats=c.stats_dev)
+    want = oracle.shuffle(c.ora, c.host, p, seed=77, step=3, stack2=c.host_opt)
+    c.assert_equal("N=%d numel=%s p=%g layout=%d" % (N, numel, p, layout))
+    assert c.gpu_stats() == tuple(want)
+    c.close()
+
+
 def test_edge_cases_p0_p1_single_element_and_padding():
     # p = 0: identity, nothing written; p = 1: everything selected
     c = Case(4, [1], 0, seed=1)
