@@ -101,7 +101,6 @@ struct wash_ctx {
     void *x_row[2] = {nullptr, nullptr};
     int x_dtype[2] = {0, 0};
     uint32_t *x_mask = nullptr;            // a word per four groups, whole warp tiles
-    uint32_t *x_warp_total = nullptr;      // [x_blocks * kExchangeWarps][N + 1]
     uint32_t *x_block_total = nullptr;     // [x_blocks][N + 1]
     uint32_t x_wtiles = 0, x_blocks = 0;
     void **x_staging[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // [parity][stack]: device array of N pointers
@@ -127,7 +126,6 @@ void release(wash_ctx *ctx)
     if (ctx->sq_slots_dev) cudaFree(ctx->sq_slots_dev);
     if (ctx->avg_dev) cudaFree(ctx->avg_dev);
     if (ctx->x_mask) cudaFree(ctx->x_mask);
-    if (ctx->x_warp_total) cudaFree(ctx->x_warp_total);
     if (ctx->x_block_total) cudaFree(ctx->x_block_total);
     for (auto &set : ctx->x_staging)
         for (void **ptrs : set)
@@ -749,7 +747,6 @@ int exchange_args(wash_ctx *ctx, wash::ExchangeArgs *out)
     a.step_lo = static_cast<uint32_t>(ctx->x_step);
     a.step_hi8 = static_cast<uint32_t>(ctx->x_step >> 32) << 8;
     a.mask = ctx->x_mask;
-    a.warp_total = ctx->x_warp_total;
     a.block_total = ctx->x_block_total;
     const int parity = static_cast<int>(ctx->x_step & 1u);
     for (int k = 0; k < 2; ++k) {
@@ -792,8 +789,9 @@ int wash_exchange_bind(wash_ctx *ctx, int32_t self, int32_t stack, int32_t dtype
     if (!ctx->x_mask) {
         DeviceGuard guard(ctx->device);
         if (guard.err != cudaSuccess) return cuda_fail(guard.err, "cudaSetDevice");
-        // the grid: kExchangeBlocksPerSm blocks per SM, fewer for short rows; its
-        // warps share the warp tiles evenly
+        // the grid, whose blocks share the warp tiles evenly: a resident wave of the plan kernel, fewer blocks for
+        // short rows (more waves made the totals that every block adds up cost more than they saved: 25.6 M
+        // coordinates, N = 5, one / two / three waves 50.6 / 55.1 / 53.1 us a step)
         const uint32_t wtiles = (ctx->n_groups + wash::kExchangeTileGroups - 1) / wash::kExchangeTileGroups;
         const uint32_t max_blocks = static_cast<uint32_t>(ctx->shape.sm_count > 0 ? ctx->shape.sm_count : 148) * static_cast<uint32_t>(wash::kExchangeBlocksPerSm);
         const uint32_t want = (wtiles + wash::kExchangeWarps - 1) / wash::kExchangeWarps;
@@ -801,13 +799,10 @@ int wash_exchange_bind(wash_ctx *ctx, int32_t self, int32_t stack, int32_t dtype
         const size_t columns = static_cast<size_t>(ctx->N) + 1;
         cudaError_t err;
         if ((err = cudaMalloc(&ctx->x_mask, sizeof(uint32_t) * 32u * static_cast<size_t>(wtiles))) != cudaSuccess ||
-            (err = cudaMalloc(&ctx->x_warp_total, sizeof(uint32_t) * columns * blocks * wash::kExchangeWarps)) != cudaSuccess ||
             (err = cudaMalloc(&ctx->x_block_total, sizeof(uint32_t) * columns * blocks)) != cudaSuccess) {
             cudaGetLastError();
             if (ctx->x_mask) cudaFree(ctx->x_mask);
-            if (ctx->x_warp_total) cudaFree(ctx->x_warp_total);
             ctx->x_mask = nullptr;
-            ctx->x_warp_total = nullptr;
             return fail(WASH_ERR_ALLOC, "device allocation of the exchange tables failed: %s", cudaGetErrorString(err));
         }
         ctx->x_wtiles = wtiles;

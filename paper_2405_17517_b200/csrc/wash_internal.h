@@ -104,22 +104,17 @@ struct ReduceArgs {
 // One model per device (wash_exchange_*): the row is one model of a population of pop.N.
 constexpr int kExchangeTileGroups = 128;   // a warp tile (wash_warp_tiles.cuh): 32 lanes x 4 groups = 512 coordinates
 constexpr int kExchangeWarps = 8;          // warps per block of the exchange kernels
-#ifndef WASH_EXCHANGE_BLOCKS_PER_SM
-#define WASH_EXCHANGE_BLOCKS_PER_SM 4
-#endif
-constexpr int kExchangeBlocksPerSm = WASH_EXCHANGE_BLOCKS_PER_SM;   // grid of the exchange kernels = this many blocks per SM (what the plan kernel fits)
+constexpr int kExchangeBlocksPerSm = 4;    // resident blocks of the plan kernel on an SM
 struct ExchangeArgs {
     PopView pop;
     int self;                     // this worker's index in the population
     uint32_t n_wtiles;            // ceil(n_groups / kExchangeTileGroups)
-    uint32_t n_blocks;            // grid of all three kernels; its warps share the warp tiles evenly, in order
+    uint32_t n_blocks;            // grid of all three kernels; its blocks share the warp tiles evenly, in order
     PhiloxKeys keys;
     uint32_t step_lo, step_hi8;
     uint32_t *mask;               // [n_wtiles * 32] a word per lane, a nibble per group; low half:
                                   // selected coordinates, high half: those this worker receives
-    uint32_t *warp_total;         // [n_blocks * kExchangeWarps][N + 1]: column n = slots of worker n's buffer the
-                                  // warp's range takes; column N = selected coordinates
-    uint32_t *block_total;        // [n_blocks][N + 1] the same per block
+    uint32_t *block_total;        // [n_blocks][N + 1]: column n = slots of worker n's buffer the block's range takes; column N = selected coordinates
     void *row[2];                 // this worker's model: parameters, optimizer state (nullptr: absent)
     int dtype[2];
     void *const *staging[2];      // per stack: device array of N pointers, entry n = worker n's staging buffer

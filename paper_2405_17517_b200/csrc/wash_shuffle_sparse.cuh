@@ -34,7 +34,7 @@ constexpr int kSparsePairs = 4;      // (coordinate, model) pairs a lane has in 
 constexpr double kSparsePerBlock = 16.0;   // selected coordinates a block expects, at least
 
 // entries of the queue: a permutation of up to 16 models stays in its entry (8 bytes), a larger one
-// takes N bytes beside it
+// takes wide_pitch(N) words beside it
 __host__ __device__ constexpr uint32_t sparse_queue_capacity(int n_models) { return n_models <= 32 ? 512u : 256u; }
 
 struct SparseArgs {
@@ -56,10 +56,10 @@ __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_spa
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint32_t capacity = sparse_queue_capacity(n_models);
     // [entry: {coordinate within its tensor, tensor}, then the packed permutation][entry: row element,
-    // counted from the first element of the block's range][byte n of entry e at n * capacity + e, N > 16]
+    // counted from the first element of the block's range][N > 16: byte n of entry e's permutation at word e * wide_pitch(N)]
     uint2 *q_key = reinterpret_cast<uint2 *>(smem_raw);
     uint32_t *q_elem = reinterpret_cast<uint32_t *>(q_key + capacity);
-    uint8_t *q_bytes = reinterpret_cast<uint8_t *>(q_elem + capacity);
+    uint32_t *q_wide = q_elem + capacity;
     if (threadIdx.x == 0) s_count = 0;
 
     const uint32_t t_first = blockIdx.x * p.per_block + min(blockIdx.x, p.extra);
@@ -93,13 +93,20 @@ __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_spa
         }
         const bool again = __syncthreads_or(sel != 0 || t < t_end);   // (orders the queue's entries, too)
         const uint32_t count = min(s_count, capacity);
-        for (uint32_t e = threadIdx.x; e < count; e += kSparseThreads) {
-            const uint2 key = q_key[e];
-            if (n_models <= 16) {
+        if (n_models <= 16) {
+            for (uint32_t e = threadIdx.x; e < count; e += kSparseThreads) {
+                const uint2 key = q_key[e];
                 const uint64_t packed = draw_permutation_packed(n_models, key.x, key.y, a.step_lo, a.step_hi8, a.keys);
                 q_key[e] = make_uint2(static_cast<uint32_t>(packed), static_cast<uint32_t>(packed >> 32));
-            } else draw_permutation_u8(q_bytes + e, static_cast<int>(capacity), n_models, key.x, key.y, a.step_lo, a.step_hi8, a.keys);
-            ++selected;
+                ++selected;
+            }
+        } else {
+            for (uint32_t first = warp * 32u; first < count; first += kSparseThreads) {
+                const uint32_t in_round = min(32u, count - first);
+                const uint2 key = q_key[first + min(lane, in_round - 1u)];
+                draw_permutations_by_warp(q_wide + first * wide_pitch(n_models), n_models, in_round, key.x, key.y, a.step_lo, a.step_hi8, a.keys);
+                if (lane < in_round) ++selected;
+            }
         }
         __syncthreads();
         // the lane's pairs of a set: [N][P] takes neighbouring coordinates of one model side by side,
@@ -126,7 +133,7 @@ __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_spa
                     if (n_models <= 16) {
                         const uint2 packed = q_key[e];
                         src = ((n < 8 ? packed.x : packed.y) >> (4u * (n & 7u))) & 15u;
-                    } else src = q_bytes[n * capacity + e];
+                    } else src = reinterpret_cast<const uint8_t *>(q_wide + e * wide_pitch(n_models))[n];
                     if (src != n) {
                         const long long elem = block_elem + q_elem[e];
                         const long long in = elem_index<LAYOUT>(a.pop, static_cast<int>(src), elem);
@@ -160,7 +167,7 @@ cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchSha
     SparseArgs p;
     p.s = args;
     p.n_wtiles = (args.group_hi - args.group_lo + kWarpTileGroups - 1) / kWarpTileGroups;
-    const size_t smem = sparse_queue_capacity(args.pop.N) * (12 + (args.pop.N > 16 ? static_cast<size_t>(args.pop.N) : 0));
+    const size_t smem = sparse_queue_capacity(args.pop.N) * (12 + (args.pop.N > 16 ? 4 * static_cast<size_t>(wide_pitch(args.pop.N)) : 0));
     auto kernel = args.pop.layout == kLayoutNP ? shuffle_sparse_kernel<TA, TB, kLayoutNP> : shuffle_sparse_kernel<TA, TB, kLayoutPN>;
     KernelFit fit;
     cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), kSparseThreads, smem, &fit);

@@ -120,25 +120,4 @@ __device__ __forceinline__ uint32_t warp_exclusive_scan(uint32_t mine, uint32_t 
     return upto - mine;
 }
 
-// The selected coordinates of a warp's range are few and scattered: serving each where it is
-// found would leave 31 lanes idle.  Instead the warp queues them, in coordinate order, as
-// row elements in a ring in shared memory and serves them 32 at a time, one per lane.
-constexpr uint32_t kXRing = 1024;   // entries; a warp tile adds at most 512, a round removes 32
-
-// appends the lane's selected coordinates of the warp's tile number t_rel (counted from the first
-// tile of the warp's range); an entry is the coordinate's row element counted from the first
-// element of that range.  sel4: a nibble per group.
-__device__ __forceinline__ uint32_t ring_append(uint32_t *ring, uint32_t tail, uint32_t sel4, uint32_t t_rel)
-{
-    const uint32_t lane = threadIdx.x & 31u;
-    uint32_t total = 0;
-    uint32_t pos = tail + warp_exclusive_scan(__popc(sel4), &total);
-    const uint32_t elem0 = 4u * (t_rel * kWarpTileGroups + 4u * lane);
-    for (uint32_t left = sel4; left; left &= left - 1u, ++pos) {
-        ring[pos % kXRing] = elem0 + static_cast<uint32_t>(__ffs(left) - 1);
-    }
-    __syncwarp();
-    return tail + total;
-}
-
 }  // namespace wash

@@ -297,3 +297,22 @@ def test_bench_arm_with_two_ranks_on_one_device():
     assert line["counts_match_oracle"] is True
     expect = line["expected_values_per_rank_per_step"]
     assert abs(line["values_received_per_rank_per_step"] - expect) < 6 * expect ** 0.5
+
+
+@pytest.mark.parametrize("N,numel,p_layer", [
+    (3, [6_000_011, 5, 260_000], [0.02, 1.0, 1.0]),      # several chunks of mask words per block; lists that fill up and are served in parts
+    (2, [8193, 8191, 16_384], [0.9, 0.5, 0.0]),          # rows of a few chunks, one of them empty
+    (33, [40_003], [0.7])])                              # permutations drawn by whole warps, partly filled ones among them
+def test_lists_of_a_block_reproduce_the_population_shuffle(N, numel, p_layer):
+    w = Workers(N, numel, seed=N)
+    w.step(5, 0.0, p_layer, seed=8)
+    sel, moved = oracle.shuffle(w.ora, w.host[0], p_layer, seed=8, step=5)
+    w.check()
+    assert (to_host_bits(w.dev[0]) == bits(w.host[0])).all()
+    need, _ = oracle.exchange_counts(w.ora, p_layer, seed=8, step=5)
+    for n in range(N):
+        g_need, g_sel = B.wash_exchange_counts(w.ctx[n], N)
+        assert g_need == need.tolist() and g_sel == sel
+    st = w.stats.cpu().numpy()
+    assert (st[:, 0] == sel).all() and st[:, 1].sum() == moved
+    w.close()
