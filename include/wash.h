@@ -123,14 +123,14 @@ int wash_bind(wash_ctx *ctx, int32_t stack, int32_t dtype, void *dev_ptr, int64_
 int wash_set_mode(wash_ctx *ctx, int32_t mode);
 
 /* Launch shape override for tuning: threads per block (multiple of 32 in 32..256;
- * 0 = each kernel's default) and grid style: blocks_per_sm == 0 each kernel's default,
- * > 0 a persistent grid of SM count x min(blocks_per_sm, resident blocks per SM) blocks
- * that stride over the groups, < 0 one group of 4 coordinates per thread.  For
- * WASH_MODE_STREAM blocks_per_sm = 1 or 2 fixes the number of groups a thread takes
+ * 0 = each kernel's default; a kernel built for fewer takes what it can) and, in
+ * blocks_per_sm, the kernel of a streaming shuffle (0: by the rules below; the dense
+ * operators and WASH_MODE_SPARSE ignore it).  blocks_per_sm = 1 or 2 fixes the number of groups a thread takes
  * (default: 2 when a group of all models is at most 64 bytes, else 1); blocks_per_sm = -2 / -3
  * forces the streaming kernel's lean / early flavour (early draws the permutations while the
  * stack's copies are in flight and serves populations of more than 16 models densely; by
- * default it is launched for N > 16 when the call's probabilities select 30 % or more);
+ * default it is launched for N > 16 when the call's probabilities select 30 % or more; from
+ * 0.3 % to there populations of more than 16 models have a kernel of their own);
  * blocks_per_sm = -4 / -5 forces (N <= 16) / excludes the streaming kernel for small groups (a
  * resident grid of warps walking tiles through two shared-memory stages; by default
  * it is launched when a group of all models of both stacks is at most 48 bytes and the

@@ -2,15 +2,12 @@
 
     python -m paper_2405_17517_b200.build [--force] [--verbose]
 
-wash_inst.cu (the dense operators) is compiled once per population size listed in
-csrc/wash_nlist.h (plus once for run-time N); the objects are compiled in parallel and
-linked with the C ABI into paper_2405_17517_b200/libwash.so.
+The translation units are compiled in parallel and linked into paper_2405_17517_b200/libwash.so.
 """
 from __future__ import annotations
 
 import concurrent.futures as cf
 import os
-import re
 import shutil
 import subprocess
 import sys
@@ -21,6 +18,9 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libwash.so")
 
+UNITS = ("wash_shuffle", "wash_shuffle_loop", "wash_shuffle_wide", "wash_shuffle_sparse", "wash_reduce_f32", "wash_reduce_bf16", "wash_exchange",
+         "wash_dispatch", "wash_noalloc", "wash_api")   # slowest first
+
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
 
@@ -30,13 +30,6 @@ def _nvcc() -> str:
         if cand and os.path.exists(cand):
             return cand
     raise RuntimeError("nvcc not found: libwash.so cannot be built")
-
-
-def population_sizes() -> list[int]:
-    with open(os.path.join(CSRC, "wash_nlist.h")) as f:
-        text = f.read()
-    line = [ln for ln in text.splitlines() if ln.startswith("#define WASH_N_LIST")][0]
-    return [int(x) for x in re.findall(r"X\((\d+)\)", line.split("WASH_N_LIST(X)")[1])]
 
 
 def _sources_mtime() -> float:
@@ -61,12 +54,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if not force and not is_stale():
         return LIB
     os.makedirs(BUILD, exist_ok=True)
-    jobs = [(os.path.join(CSRC, "wash_api.cu"), os.path.join(BUILD, "wash_api.o"), [], verbose),
-            (os.path.join(CSRC, "wash_dispatch.cu"), os.path.join(BUILD, "wash_dispatch.o"), [], verbose)]
-    for name in ("wash_noalloc", "wash_shuffle", "wash_shuffle_sparse", "wash_shuffle_loop", "wash_shuffle_wide", "wash_exchange"):
-        jobs.append((os.path.join(CSRC, name + ".cu"), os.path.join(BUILD, name + ".o"), [], verbose))
-    for n in [0] + population_sizes():
-        jobs.append((os.path.join(CSRC, "wash_inst.cu"), os.path.join(BUILD, "wash_inst_n%d.o" % n), ["-DWASH_N=%d" % n], verbose))
+    jobs = [(os.path.join(CSRC, name + ".cu"), os.path.join(BUILD, name + ".o"), [], verbose) for name in UNITS]
     workers = max(1, min(len(jobs), os.cpu_count() or 1))
     objs = []
     with cf.ThreadPoolExecutor(workers) as pool:

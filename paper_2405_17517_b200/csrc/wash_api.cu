@@ -86,7 +86,7 @@ struct wash_ctx {
     uint32_t *status_dev = nullptr;
     wash_stats *stats_dev = nullptr;       // for wash_step_host
     wash::StatSlot *stat_slots_dev = nullptr;
-    double *sq_slots_dev = nullptr;        // partial sums of wash_shuffle_consensus, allocated on first use, zero between calls
+    double *sq_slots_dev = nullptr;        // partial sums of the consensus distances, zero between calls; behind stat_slots_dev in its allocation
     double expected_selected = 0.0;        // sum over tensors of numel * thr / 2^32, for the current thresholds
     void *avg_dev = nullptr;               // for wash_step_host, allocated on first use
     size_t avg_bytes = 0;
@@ -123,7 +123,6 @@ void release(wash_ctx *ctx)
     if (ctx->status_dev) cudaFree(ctx->status_dev);
     if (ctx->stats_dev) cudaFree(ctx->stats_dev);
     if (ctx->stat_slots_dev) cudaFree(ctx->stat_slots_dev);
-    if (ctx->sq_slots_dev) cudaFree(ctx->sq_slots_dev);
     if (ctx->avg_dev) cudaFree(ctx->avg_dev);
     if (ctx->x_mask) cudaFree(ctx->x_mask);
     if (ctx->x_block_total) cudaFree(ctx->x_block_total);
@@ -298,8 +297,8 @@ int shuffle_impl(wash_ctx *ctx, int which, uint64_t step, double p, const double
     return WASH_OK;
 }
 
-int reduce_impl(wash_ctx *ctx, int op, int stack, void *out, int out_dtype, float alpha, int tensor_lo,
-                int tensor_hi, double *sq_out, void *stream_v, uint32_t group_lo = 0, uint32_t group_hi = 0xFFFFFFFFu)
+int reduce_impl(wash_ctx *ctx, int op, int stack, void *out, int out_dtype, float alpha, void *stream_v,
+                uint32_t group_lo = 0, uint32_t group_hi = 0xFFFFFFFFu)
 {
     if (!ctx) return fail(WASH_ERR_ARG, "ctx is NULL");
     if (stack != WASH_STACK_PARAMS && stack != WASH_STACK_OPT) return fail(WASH_ERR_ARG, "stack must be 0 or 1");
@@ -315,12 +314,9 @@ int reduce_impl(wash_ctx *ctx, int op, int stack, void *out, int out_dtype, floa
     args.out = out;
     args.alpha = alpha;
     args.one_minus_alpha = 1.0f - alpha;
-    args.group_lo = ctx->seg_host[static_cast<size_t>(tensor_lo)].group_begin;
-    args.group_hi = ctx->seg_host[static_cast<size_t>(tensor_hi) - 1].group_end;
-    if (group_lo > args.group_lo) args.group_lo = group_lo;   // optional narrowing to a range of groups
-    if (group_hi < args.group_hi) args.group_hi = group_hi;
+    args.group_lo = group_lo;   // optional narrowing to a range of groups
+    args.group_hi = group_hi < ctx->n_groups ? group_hi : ctx->n_groups;
     if (args.group_lo >= args.group_hi) return WASH_OK;
-    args.sq_out = sq_out;
     args.status = ctx->status_dev;
     bool supported = false;
     cudaError_t err = wash::launch_reduce(args, op, ctx->stack_dtype[stack], out_dtype, ctx->shape, stream, &supported);
@@ -395,11 +391,12 @@ int wash_create_segments(wash_ctx **out, int32_t N, int32_t n_segments, const in
     if (err != cudaSuccess) { delete ctx; return cuda_fail(err, "cudaDeviceGetAttribute"); }
     ctx->shape.sm_count = sm_count;
     const size_t seg_bytes = sizeof(SegEntry) * static_cast<size_t>(n_segments);
+    const size_t slot_bytes = sizeof(wash::StatSlot) * wash::kStatSlots + sizeof(double) * wash::kSqSlots * wash::kMaxSqRanges * static_cast<size_t>(N);
     if ((err = cudaMalloc(&ctx->seg_dev, seg_bytes)) != cudaSuccess ||
         (err = cudaMalloc(&ctx->tile_first_dev, sizeof(uint32_t) * ctx->n_tiles)) != cudaSuccess ||
         (err = cudaMalloc(&ctx->status_dev, sizeof(uint32_t))) != cudaSuccess ||
         (err = cudaMalloc(&ctx->stats_dev, sizeof(wash_stats))) != cudaSuccess ||
-        (err = cudaMalloc(&ctx->stat_slots_dev, sizeof(wash::StatSlot) * wash::kStatSlots)) != cudaSuccess) {
+        (err = cudaMalloc(&ctx->stat_slots_dev, slot_bytes)) != cudaSuccess) {
         release(ctx);
         cudaGetLastError();
         return fail(WASH_ERR_ALLOC, "device allocation failed: %s", cudaGetErrorString(err));
@@ -415,10 +412,11 @@ int wash_create_segments(wash_ctx **out, int32_t N, int32_t n_segments, const in
     if ((err = cudaMemcpy(ctx->tile_first_dev, tile_first.data(), sizeof(uint32_t) * ctx->n_tiles, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (err = cudaMemset(ctx->status_dev, 0, sizeof(uint32_t))) != cudaSuccess ||
         (err = cudaMemset(ctx->stats_dev, 0, sizeof(wash_stats))) != cudaSuccess ||
-        (err = cudaMemset(ctx->stat_slots_dev, 0, sizeof(wash::StatSlot) * wash::kStatSlots)) != cudaSuccess) {
+        (err = cudaMemset(ctx->stat_slots_dev, 0, slot_bytes)) != cudaSuccess) {
         release(ctx);
         return cuda_fail(err, "table upload");
     }
+    ctx->sq_slots_dev = reinterpret_cast<double *>(ctx->stat_slots_dev + wash::kStatSlots);
     *out = ctx;
     return WASH_OK;
 }
@@ -521,18 +519,6 @@ int wash_shuffle_consensus(wash_ctx *ctx, int32_t stacks, uint64_t step, double 
     for (int r = n_ranges + 1; r <= wash::kMaxSqRanges; ++r) sq.seg_bound[r] = sq.seg_bound[n_ranges];
     sq.n_ranges = n_ranges;
     sq.inv_n = 1.0 / static_cast<double>(ctx->N);
-    if (!ctx->sq_slots_dev) {
-        DeviceGuard guard(ctx->device);
-        if (guard.err != cudaSuccess) return cuda_fail(guard.err, "cudaSetDevice");
-        const size_t bytes = sizeof(double) * wash::kSqSlots * wash::kMaxSqRanges * static_cast<size_t>(ctx->N);
-        cudaError_t err = cudaMalloc(&ctx->sq_slots_dev, bytes);
-        if (err != cudaSuccess) {
-            cudaGetLastError();
-            ctx->sq_slots_dev = nullptr;
-            return fail(WASH_ERR_ALLOC, "device allocation of the consensus partial sums failed: %s", cudaGetErrorString(err));
-        }
-        if ((err = cudaMemset(ctx->sq_slots_dev, 0, bytes)) != cudaSuccess) return cuda_fail(err, "cudaMemset(consensus partial sums)");
-    }
     sq.slots = ctx->sq_slots_dev;
     return shuffle_impl(ctx, stacks, step, p, p_layer, seed, stream, stats, 0, 0xFFFFFFFFu, &sq, dev_sq_out);
 }
@@ -541,7 +527,7 @@ int papa_ema(wash_ctx *ctx, int32_t stack, float alpha, void *stream)
 {
     if (!(alpha > 0.0f && alpha < 1.0f)) return fail(WASH_ERR_ARG, "alpha is %g, must be in (0,1)", (double)alpha);
     if (!ctx) return fail(WASH_ERR_ARG, "ctx is NULL");
-    return reduce_impl(ctx, wash::kOpEma, stack, nullptr, WASH_F32, alpha, 0, ctx->n_seg, nullptr, stream);
+    return reduce_impl(ctx, wash::kOpEma, stack, nullptr, WASH_F32, alpha, stream);
 }
 
 int population_average(wash_ctx *ctx, int32_t stack, void *dev_out, int32_t out_dtype, void *stream)
@@ -549,22 +535,47 @@ int population_average(wash_ctx *ctx, int32_t stack, void *dev_out, int32_t out_
     if (!ctx) return fail(WASH_ERR_ARG, "ctx is NULL");
     if (!dev_out || (reinterpret_cast<uintptr_t>(dev_out) & 15)) return fail(WASH_ERR_ARG, "dev_out must be a 16-byte aligned device pointer");
     if (out_dtype != WASH_F32 && out_dtype != WASH_BF16) return fail(WASH_ERR_ARG, "unknown out_dtype %d", out_dtype);
-    return reduce_impl(ctx, wash::kOpAverage, stack, dev_out, out_dtype, 0.0f, 0, ctx->n_seg, nullptr, stream);
+    return reduce_impl(ctx, wash::kOpAverage, stack, dev_out, out_dtype, 0.0f, stream);
 }
 
 int papa_all(wash_ctx *ctx, int32_t stack, void *stream)
 {
     if (!ctx) return fail(WASH_ERR_ARG, "ctx is NULL");
-    return reduce_impl(ctx, wash::kOpPapaAll, stack, nullptr, WASH_F32, 0.0f, 0, ctx->n_seg, nullptr, stream);
+    return reduce_impl(ctx, wash::kOpPapaAll, stack, nullptr, WASH_F32, 0.0f, stream);
 }
 
-int wash_consensus_sq(wash_ctx *ctx, int32_t stack, int32_t tensor_lo, int32_t tensor_hi, double *dev_sq_out, void *stream)
+int wash_consensus_sq(wash_ctx *ctx, int32_t stack, int32_t tensor_lo, int32_t tensor_hi, double *dev_sq_out, void *stream_v)
 {
     if (!ctx) return fail(WASH_ERR_ARG, "ctx is NULL");
     if (!dev_sq_out) return fail(WASH_ERR_ARG, "dev_sq_out is NULL");
     if (tensor_lo < 0 || tensor_hi > ctx->n_seg || tensor_lo > tensor_hi) return fail(WASH_ERR_ARG, "tensor range [%d, %d) is not within [0, %d]", tensor_lo, tensor_hi, ctx->n_seg);
     if (tensor_lo == tensor_hi) return WASH_OK;
-    return reduce_impl(ctx, wash::kOpConsensus, stack, nullptr, WASH_F32, 0.0f, tensor_lo, tensor_hi, dev_sq_out, stream);
+    if (stack != WASH_STACK_PARAMS && stack != WASH_STACK_OPT) return fail(WASH_ERR_ARG, "stack must be 0 or 1");
+    if (!ctx->stack_ptr[stack]) return fail(WASH_ERR_STATE, "stack %d is not bound", stack);
+    DeviceGuard guard(ctx->device);
+    if (guard.err != cudaSuccess) return cuda_fail(guard.err, "cudaSetDevice");
+    cudaStream_t stream = static_cast<cudaStream_t>(stream_v);
+    int rc = ensure_table(ctx, stream);
+    if (rc != WASH_OK) return rc;
+    // the streaming shuffle's statistic with nothing selected
+    wash::ShuffleArgs args = {};
+    args.pop = view_of(ctx);
+    args.a = ctx->stack_ptr[stack];
+    args.group_lo = ctx->seg_host[static_cast<size_t>(tensor_lo)].group_begin;
+    args.group_hi = ctx->seg_host[static_cast<size_t>(tensor_hi) - 1].group_end;
+    args.stat_slots = ctx->stat_slots_dev;
+    args.status = ctx->status_dev;
+    for (int r = 0; r <= wash::kMaxSqRanges; ++r) args.sq.seg_bound[r] = static_cast<uint32_t>(r ? tensor_hi : tensor_lo);
+    args.sq.n_ranges = 1;
+    args.sq.inv_n = 1.0 / static_cast<double>(ctx->N);
+    args.sq.slots = ctx->sq_slots_dev;
+    args.measure_only = true;
+    bool supported = false;
+    cudaError_t err = wash::launch_shuffle(args, ctx->stack_dtype[stack], wash::kDtypeNone, wash::kModeStream, ctx->shape, stream, &supported);
+    if (err == cudaSuccess && supported) err = wash::launch_sq_flush(args.sq, ctx->N, dev_sq_out, stream);
+    if (err != cudaSuccess) return cuda_fail(err, "consensus kernel launch");
+    if (!supported) return fail(WASH_ERR_UNSUPPORTED, "no kernel for dtype %d", ctx->stack_dtype[stack]);
+    return WASH_OK;
 }
 
 int wash_step_host(wash_ctx *ctx, int32_t ops, void *host_params, void *host_opt, void *host_avg, uint64_t step,
@@ -656,11 +667,11 @@ int wash_step_host(wash_ctx *ctx, int32_t ops, void *host_params, void *host_opt
                     if (rc != WASH_OK) return rc;
                 }
                 if (ops & WASH_OP_EMA) {
-                    rc = reduce_impl(ctx, wash::kOpEma, WASH_STACK_PARAMS, nullptr, WASH_F32, alpha, 0, ctx->n_seg, nullptr, stream, g0, g1);
+                    rc = reduce_impl(ctx, wash::kOpEma, WASH_STACK_PARAMS, nullptr, WASH_F32, alpha, stream, g0, g1);
                     if (rc != WASH_OK) return rc;
                 }
                 if (ops & WASH_OP_AVERAGE) {
-                    rc = reduce_impl(ctx, wash::kOpAverage, WASH_STACK_PARAMS, ctx->avg_dev, pd, 0.0f, 0, ctx->n_seg, nullptr, stream, g0, g1);
+                    rc = reduce_impl(ctx, wash::kOpAverage, WASH_STACK_PARAMS, ctx->avg_dev, pd, 0.0f, stream, g0, g1);
                     if (rc != WASH_OK) return rc;
                 }
                 if ((err = cudaEventRecord(ev_done[k], stream)) != cudaSuccess || (err = cudaStreamWaitEvent(ctx->copy_out, ev_done[k], 0)) != cudaSuccess)

@@ -1,19 +1,16 @@
-// Chooses the kernel instantiation for a population size.
+// Chooses the shuffle kernel of a call, and the small kernels beside them.
 #include <atomic>
 #include "wash_internal.h"
 #include "wash_device.cuh"
-#include "wash_nlist.h"
 
 namespace wash {
 
-#define WASH_DECL(n) cudaError_t launch_reduce_n##n(const ReduceArgs &, int, int, int, const LaunchShape &, cudaStream_t, bool *);
-WASH_N_LIST(WASH_DECL)
-#undef WASH_DECL
+cudaError_t launch_reduce_f32(const ReduceArgs &, int, int, const LaunchShape &, cudaStream_t);
+cudaError_t launch_reduce_bf16(const ReduceArgs &, int, int, const LaunchShape &, cudaStream_t);
 cudaError_t launch_shuffle_sparse(const ShuffleArgs &, int, int, const LaunchShape &, cudaStream_t, bool *);
 cudaError_t launch_shuffle_stream(const ShuffleArgs &, int, int, const LaunchShape &, cudaStream_t, bool *);
 cudaError_t launch_shuffle_stream_wide(const ShuffleArgs &, int, int, const LaunchShape &, cudaStream_t, bool *);
 cudaError_t launch_shuffle_stream_loop(const ShuffleArgs &, int, int, const LaunchShape &, cudaStream_t, bool *);
-cudaError_t launch_reduce_n0(const ReduceArgs &, int, int, int, const LaunchShape &, cudaStream_t, bool *);
 
 static std::atomic<uint64_t> g_launches{0};
 void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
@@ -55,22 +52,27 @@ __global__ void __launch_bounds__(kStatSlots) flush_stats_kernel(StatSlot *slots
 }
 
 // Adds the kSqSlots partial copies of the [range][model] table of squared distances into the
-// caller's array and leaves the slots zeroed for the next launch.
-__global__ void __launch_bounds__(256) sq_flush_kernel(double *slots, int count, double *out)
+// caller's array and leaves the slots zeroed for the next launch.  A warp per entry, a lane per two
+// copies (a thread that went through the copies of an entry one after the other took 64 round trips).
+__global__ void __launch_bounds__(1024) sq_flush_kernel(double *slots, int count, double *out)
 {
-    for (int j = threadIdx.x; j < count; j += blockDim.x) {
-        double s = 0.0;
-        for (int k = 0; k < kSqSlots; ++k) {
-            s += slots[k * count + j];
-            slots[k * count + j] = 0.0;
-        }
-        out[j] += s;
+    static_assert(kSqSlots == 64, "two copies per lane");
+    const int lane = threadIdx.x & 31;
+    for (int j = threadIdx.x >> 5; j < count; j += blockDim.x >> 5) {
+        double *lo = slots + lane * count + j, *hi = lo + 32 * count;
+        double s = *lo + *hi;
+        *lo = 0.0;
+        *hi = 0.0;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, d);
+        if (lane == 0) out[j] += s;
     }
 }
 
 cudaError_t launch_sq_flush(const SqArgs &sq, int N, double *out, cudaStream_t stream)
 {
-    sq_flush_kernel<<<1, 256, 0, stream>>>(sq.slots, sq.n_ranges * N, out);
+    const int entries = sq.n_ranges * N;
+    sq_flush_kernel<<<1, entries < 32 ? 32 * entries : 1024, 0, stream>>>(sq.slots, entries, out);
     count_launch();
     return cudaGetLastError();
 }
@@ -146,16 +148,12 @@ cudaError_t launch_shuffle(const ShuffleArgs &args, int a_dtype, int b_dtype, in
     return cudaGetLastError();
 }
 
-cudaError_t launch_reduce(const ReduceArgs &args, int op, int dtype, int out_dtype,
-                          const LaunchShape &shape, cudaStream_t stream, bool *supported)
+cudaError_t launch_reduce(const ReduceArgs &args, int op, int dtype, int out_dtype, const LaunchShape &shape,
+                          cudaStream_t stream, bool *supported)
 {
-    switch (args.pop.N) {
-#define WASH_CASE(n) case n: return launch_reduce_n##n(args, op, dtype, out_dtype, shape, stream, supported);
-        WASH_N_LIST(WASH_CASE)
-#undef WASH_CASE
-    default:
-        return launch_reduce_n0(args, op, dtype, out_dtype, shape, stream, supported);
-    }
+    *supported = (dtype == kDtypeF32 || dtype == kDtypeBF16) && (out_dtype == kDtypeF32 || out_dtype == kDtypeBF16);
+    if (!*supported) return cudaSuccess;
+    return dtype == kDtypeF32 ? launch_reduce_f32(args, op, out_dtype, shape, stream) : launch_reduce_bf16(args, op, out_dtype, shape, stream);
 }
 
 }  // namespace wash

@@ -85,6 +85,7 @@ struct ShuffleArgs {
     bool stats_direct = false;    // few blocks report: they add to `stats` themselves (kernels that need a flush kernel otherwise)
     uint32_t *status;             // device status word
     SqArgs sq;                    // consensus distance of the first stack (streaming kernel only)
+    bool measure_only = false;    // with sq: nothing is selected
     uint32_t pn_pad = 0;          // streaming kernel, [P][N]: elements of padding after a group in the shared-memory image (0 or 4)
     uint32_t pair_inverse = 0;    // streaming kernel, N > 16: 2^20 / N, rounded up (i / N = i * pair_inverse >> 20 for i < 2080; set by its launcher)
     bool early = false;           // streaming kernel: the flavour that draws permutations while the copies are in flight
@@ -96,8 +97,7 @@ struct ReduceArgs {
     void *stack;                  // device stack (read; written by EMA / papa_all)
     void *out;                    // average row (device) or nullptr
     float alpha, one_minus_alpha;
-    uint32_t group_lo, group_hi;  // range of groups to process
-    double *sq_out;               // consensus: N doubles (device) or nullptr
+    uint32_t group_lo, group_hi;  // range of groups to process (both even: whole units of 8 elements)
     uint32_t *status;
 };
 
@@ -126,7 +126,7 @@ cudaError_t launch_exchange_plan(const ExchangeArgs &args, cudaStream_t stream);
 cudaError_t launch_exchange_send(const ExchangeArgs &args, cudaStream_t stream);
 cudaError_t launch_exchange_receive(const ExchangeArgs &args, cudaStream_t stream);
 
-enum ReduceOp { kOpEma = 0, kOpAverage = 1, kOpPapaAll = 2, kOpConsensus = 3 };
+enum ReduceOp { kOpEma = 0, kOpAverage = 1, kOpPapaAll = 2 };
 
 // The resident-warp streaming kernel takes groups (all models, both stacks) of up to 48 bytes -- fp32 N = 2, 3;
 // bf16 N <= 6 -- when at most 30 % of the coordinates are expected to be selected, and two groups per lane instead of four
@@ -147,7 +147,7 @@ constexpr float kWideMinShare = 0.003f;
 
 struct LaunchShape {
     int threads;         // 0 = default
-    int blocks_per_sm;   // <= 0: one group per thread; > 0: persistent grid, that many blocks per SM
+    int blocks_per_sm;   // streaming shuffle: which kernel (wash_set_launch)
     int sm_count;
 };
 

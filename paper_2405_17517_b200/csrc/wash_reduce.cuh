@@ -1,162 +1,414 @@
-// The dense comparison operators, each one fused pass over the stack:
+// The dense comparison operators, each one pass over the stack:
 //   kOpEma       PAPA's EMA, Eq. 1:  x_n <- alpha x_n + (1 - alpha) m
 //   kOpAverage   the averaged model (output of Algorithm 1): out <- m
 //   kOpPapaAll   PAPA-all / DART: x_n <- m
-//   kOpConsensus squared distances to the consensus (Eq. 2 / Eq. 5 / Fig. 2)
 // with m = (((x_0 + x_1) + x_2) + ...)/N in binary32, each operation rounded once
 // (explicit _rn intrinsics: the compiler may neither fuse nor reorder them).
 //
-// A thread owns one group of 4 coordinates for all N models, as in the shuffle.
+// The unit of work is 16 bytes of every model: 4 coordinates in fp32, 8 in bf16 (tensors start on
+// multiples of 8 elements, so a unit never straddles two).  [N][P] keeps a unit's N vectors in registers
+// where N is small (unrolled per N); larger populations and [P][N] stage them in shared memory by
+// cp.async with N a run-time value, sum them from there and, for the operators that write the stack,
+// read them once more from there.
+// Bound: HBM, except bf16 [P][N], which has two values a word to widen, round and check for NaN and is bound
+// by issue slots (N = 32 249 us where the bytes take 164).  Before, a thread held four coordinates of every model (8-byte
+// vectors in bf16, values of [P][N] picked out of registers), and populations not in a list of unrolled sizes went
+// through local memory: EMA N = 8 bf16 ResNet-50 141 -> 133 us, [P][N] 233 -> 160; N = 7 fp32, 2^24 coordinates 671 -> 142, N = 31 [P][N],
+// 2^23 coordinates 1740 -> 311; average of N = 13, fp32 ResNet-50 1029 -> 206.
 #pragma once
-#include "wash_device.cuh"
-#include "wash_launch.cuh"
+#define WASH_SERVING_ONLY
+#include "wash_shuffle_async.cuh"
 
 namespace wash {
 
-template <int N, class T, class TOUT, int LAYOUT, int OP>
-__global__ void __launch_bounds__(256) reduce_kernel(const __grid_constant__ ReduceArgs a)
-{
-    constexpr int kCap = N > 0 ? N : kMaxN;
-    const int n_models = N > 0 ? N : a.pop.N;
-    const float inv_count = static_cast<float>(n_models);
-    double acc[OP == kOpConsensus ? kCap : 1];
-    if constexpr (OP == kOpConsensus) {
-#pragma unroll
-        for (int n = 0; n < kCap; ++n) acc[n] = 0.0;
+template <class T>
+struct Unit {
+    static constexpr int kElems = 16 / T::kBytes;
+    static constexpr uint32_t kGroups = kElems / 4;
+    // element q of a vector, widened to binary32
+    static __device__ __forceinline__ float get(const uint4 &v, int q)
+    {
+        const uint32_t w = T::kBytes == 4 ? (q == 0 ? v.x : q == 1 ? v.y : q == 2 ? v.z : v.w)
+                                          : (q < 2 ? v.x : q < 4 ? v.y : q < 6 ? v.z : v.w);
+        if (T::kBytes == 4) return __uint_as_float(w);
+        return __uint_as_float((q & 1) ? w & 0xFFFF0000u : w << 16);
     }
-    const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
-    for (uint64_t g = a.group_lo + static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x; g < a.group_hi; g += stride) {
-        typename T::vec v[kCap];
-        if constexpr (N > 0) {
-#pragma unroll
-            for (int j = 0; j < N; ++j) v[j] = T::load_group(group_vec_ptr<T, LAYOUT>(a.stack, a.pop, g, j));
-        } else {
-            for (int j = 0; j < n_models; ++j) v[j] = T::load_group(group_vec_ptr<T, LAYOUT>(a.stack, a.pop, g, j));
+    static __device__ __forceinline__ uint4 pack(const float (&r)[kElems])
+    {
+        if constexpr (T::kBytes == 4) return make_uint4(__float_as_uint(r[0]), __float_as_uint(r[1]), __float_as_uint(r[2]), __float_as_uint(r[3]));
+        else return make_uint4(BF16::pair_from_floats(r[0], r[1]), BF16::pair_from_floats(r[2], r[3]), BF16::pair_from_floats(r[4], r[5]), BF16::pair_from_floats(r[6], r[7]));
+    }
+    // coordinates that exist among the unit's elements (a tensor may end inside it; the rest is padding)
+    static __device__ __forceinline__ int valid(const PopView &pop, uint64_t unit, uint32_t *status)
+    {
+        const uint32_t g = static_cast<uint32_t>(unit) * kGroups;
+        uint32_t s = __ldg(pop.tile_first + (g >> kTileShift));
+        const uint32_t last = static_cast<uint32_t>(pop.n_seg) - 1u;
+        while (s < last && g >= __ldg(&pop.seg[s].group_end)) ++s;
+        const uint4 lo = __ldg(reinterpret_cast<const uint4 *>(pop.seg + s));   // begin, end, tensor, cgroup_begin
+        if (g < lo.x || g >= lo.y) {   // table inconsistent with the row: report, touch nothing
+            if (status) atomicOr(status, 1u);
+            return 0;
         }
-        const GroupInfo gi = find_group(a.pop, static_cast<uint32_t>(g), a.status);
-        if (gi.valid == 0) continue;
+        const long long left = static_cast<long long>(__ldg(&pop.seg[s].numel)) - 4ll * (g - lo.x);
+        return left >= kElems ? kElems : (left > 0 ? static_cast<int>(left) : 0);
+    }
+};
 
-        if constexpr (OP == kOpConsensus) {
+// One unit of the average row: m of its coordinates.
+template <class T, class TOUT>
+__device__ __forceinline__ void store_average(const ReduceArgs &a, uint64_t unit, int valid, const float (&m)[Unit<T>::kElems])
+{
+    constexpr int kElems = Unit<T>::kElems;
+    const long long e0 = static_cast<long long>(unit) * kElems;
+    if (valid == kElems) {
+        char *out = static_cast<char *>(a.out) + e0 * TOUT::kBytes;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                if (c >= gi.valid) break;
-                double sum = 0.0;
+        for (int q = 0; q < kElems; q += 4) TOUT::store_group(out + q * TOUT::kBytes, TOUT::pack_floats(m[q], m[q + 1], m[q + 2], m[q + 3]));
+    } else {
 #pragma unroll
-                for (int n = 0; n < kCap; ++n)
-                    if (n < n_models) sum += static_cast<double>(T::to_float(group_value<T, LAYOUT, kCap>(v, n_models, n, c)));
-                const double mean = sum / static_cast<double>(n_models);
+        for (int q = 0; q < kElems; ++q)
+            if (q < valid) TOUT::store_elem(a.out, e0 + q, TOUT::from_float(m[q]));
+    }
+}
+
+// [N][P], a thread per unit, its N vectors in registers, all loads in flight at once.
+template <class T, class TOUT, int OP, int N>
+__global__ void __launch_bounds__(256) regs_np_kernel(const __grid_constant__ ReduceArgs a)
+{
+    constexpr int kElems = Unit<T>::kElems;
+    const uint64_t unit = a.group_lo / Unit<T>::kGroups + static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (unit * Unit<T>::kGroups >= a.group_hi) return;
+    const size_t row = static_cast<size_t>(a.pop.padded_P) * T::kBytes;
+    char *out = static_cast<char *>(a.stack) + unit * 16;
+    uint4 v[N];
 #pragma unroll
-                for (int n = 0; n < kCap; ++n)
-                    if (n < n_models) {
-                        const double d = static_cast<double>(T::to_float(group_value<T, LAYOUT, kCap>(v, n_models, n, c))) - mean;
-                        acc[n] += d * d;
-                    }
-            }
-            continue;
-        } else {
-            // consensus m of the 4 coordinates, binary32, terms in model order
-            float m[4];
+    for (int n = 0; n < N; ++n) v[n] = F32::load_group(out + n * row);
+    const int valid = Unit<T>::valid(a.pop, unit, a.status);
+    if (valid == 0) return;
+    float m[kElems];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                float s = T::to_float(group_value<T, LAYOUT, kCap>(v, n_models, 0, c));
+    for (int q = 0; q < kElems; ++q) {
+        m[q] = Unit<T>::get(v[0], q);
 #pragma unroll
-                for (int n = 1; n < kCap; ++n)
-                    if (n < n_models) s = __fadd_rn(s, T::to_float(group_value<T, LAYOUT, kCap>(v, n_models, n, c)));
-                m[c] = __fdiv_rn(s, inv_count);
-            }
-            if constexpr (OP == kOpAverage) {
-                const long long e0 = 4ll * static_cast<long long>(g);
-                if (gi.valid == 4) {
-                    TOUT::store_group(static_cast<char *>(a.out) + e0 * TOUT::kBytes, TOUT::pack_floats(m[0], m[1], m[2], m[3]));
-                } else {
+        for (int n = 1; n < N; ++n) m[q] = __fadd_rn(m[q], Unit<T>::get(v[n], q));
+        m[q] = __fdiv_rn(m[q], static_cast<float>(N));
+        if (OP == kOpEma) m[q] = __fmul_rn(a.one_minus_alpha, m[q]);
+    }
+    if constexpr (OP == kOpAverage) store_average<T, TOUT>(a, unit, valid, m);
+    else if (valid == kElems) {
+        const uint4 all = Unit<T>::pack(m);   // PAPA-all: every model's vector
 #pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        if (c < gi.valid) TOUT::store_elem(a.out, e0 + c, TOUT::from_float(m[c]));
-                }
-            } else {
-                // new value of (model n, coordinate c)
-                auto updated = [&](int n, int c) -> float {
-                    if constexpr (OP == kOpPapaAll) return m[c];
-                    const float x = T::to_float(group_value<T, LAYOUT, kCap>(v, n_models, n, c));
-                    return __fadd_rn(__fmul_rn(a.alpha, x), __fmul_rn(a.one_minus_alpha, m[c]));
-                };
-                if (gi.valid == 4) {
+        for (int n = 0; n < N; ++n, out += row) {
+            if constexpr (OP == kOpPapaAll) *reinterpret_cast<uint4 *>(out) = all;
+            else {
+                float r[kElems];
 #pragma unroll
-                    for (int j = 0; j < kCap; ++j) {
-                        if (j >= n_models) break;
-                        float r[4];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            // element q of vector j is (model n, coordinate c):
-                            const int n = LAYOUT == kLayoutNP ? j : (4 * j + q) % n_models;
-                            const int c = LAYOUT == kLayoutNP ? q : (4 * j + q) / n_models;
-                            r[q] = updated(n, c);
-                        }
-                        T::store_group(group_vec_ptr<T, LAYOUT>(a.stack, a.pop, g, j), T::pack_floats(r[0], r[1], r[2], r[3]));
-                    }
-                } else {
-                    const long long e0 = 4ll * static_cast<long long>(g);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        if (c >= gi.valid) break;
-#pragma unroll
-                        for (int n = 0; n < kCap; ++n)
-                            if (n < n_models) T::store_elem(a.stack, elem_index<LAYOUT>(a.pop, n, e0 + c), T::from_float(updated(n, c)));
-                    }
-                }
+                for (int q = 0; q < kElems; ++q) r[q] = __fadd_rn(__fmul_rn(a.alpha, Unit<T>::get(v[n], q)), m[q]);
+                *reinterpret_cast<uint4 *>(out) = Unit<T>::pack(r);
             }
         }
-    }
-    if constexpr (OP == kOpConsensus) {
-        // warp sums, then one atomic per warp and model
+    } else {
 #pragma unroll
-        for (int n = 0; n < kCap; ++n) {
-            if (n >= n_models) break;
-            double s = acc[n];
+        for (int n = 0; n < N; ++n, out += row) {
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, off);
-            if ((threadIdx.x & 31) == 0 && s != 0.0) atomicAdd(a.sq_out + n, s);
+            for (int q = 0; q < kElems; ++q)
+                if (q < valid) T::store_elem(out, q, T::from_float(OP == kOpPapaAll ? m[q] : __fadd_rn(__fmul_rn(a.alpha, Unit<T>::get(v[n], q)), m[q])));
         }
     }
 }
 
-template <int N, class T, class TOUT, int OP>
+// [N][P], any N: a thread stages the vectors of `per_thread` <= 4 units,
+// blockDim.x apart, and reads nobody else's, so the kernel has no barrier.  Image: vector n of unit u at [u][n][thread].
+template <class T, class TOUT, int OP>
+__global__ void __launch_bounds__(64, 20) staged_np_kernel(const __grid_constant__ ReduceArgs a, int per_thread)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    constexpr int kElems = Unit<T>::kElems;
+    const int n_models = a.pop.N;
+    const uint32_t T_ = blockDim.x;
+    const size_t row = static_cast<size_t>(a.pop.padded_P) * T::kBytes;
+    const uint64_t first = a.group_lo / Unit<T>::kGroups + static_cast<uint64_t>(blockIdx.x) * T_ * per_thread + threadIdx.x;
+    const uint64_t unit_hi = a.group_hi / Unit<T>::kGroups;
+    char *stack = static_cast<char *>(a.stack);
+    uint32_t dst = smem_addr(smem_raw) + threadIdx.x * 16;
+    for (int u = 0; u < per_thread; ++u) {
+        const uint64_t unit = first + static_cast<uint64_t>(u) * T_;
+        if (unit >= unit_hi) break;
+        const char *src = stack + unit * 16;
+#pragma unroll 4
+        for (int n = 0; n < n_models; ++n, src += row, dst += T_ * 16) cp_async<16>(dst, src);
+    }
+    uint32_t valids = 0;   // four bits per unit
+    for (int u = 0; u < per_thread; ++u) {
+        const uint64_t unit = first + static_cast<uint64_t>(u) * T_;
+        if (unit >= unit_hi) break;
+        valids |= static_cast<uint32_t>(Unit<T>::valid(a.pop, unit, a.status)) << (4 * u);
+    }
+    cp_async_wait_all();
+    const uint4 *image = reinterpret_cast<const uint4 *>(smem_raw) + threadIdx.x;
+    const float count = static_cast<float>(n_models);
+    for (int u = 0; u < per_thread; ++u, image += n_models * T_) {
+        const int valid = static_cast<int>((valids >> (4 * u)) & 15u);
+        if (valid == 0) continue;
+        const uint64_t unit = first + static_cast<uint64_t>(u) * T_;
+        float m[kElems];
+        {
+            const uint4 v = image[0];
+#pragma unroll
+            for (int q = 0; q < kElems; ++q) m[q] = Unit<T>::get(v, q);
+        }
+#pragma unroll 4
+        for (int n = 1; n < n_models; ++n) {
+            const uint4 v = image[n * T_];
+#pragma unroll
+            for (int q = 0; q < kElems; ++q) m[q] = __fadd_rn(m[q], Unit<T>::get(v, q));
+        }
+#pragma unroll
+        for (int q = 0; q < kElems; ++q) {
+            m[q] = __fdiv_rn(m[q], count);
+            if (OP == kOpEma) m[q] = __fmul_rn(a.one_minus_alpha, m[q]);
+        }
+        char *out = stack + unit * 16;
+        if constexpr (OP == kOpAverage) store_average<T, TOUT>(a, unit, valid, m);
+        else if (valid == kElems) {
+            const uint4 all = Unit<T>::pack(m);   // PAPA-all: every model's vector
+#pragma unroll 2
+            for (int n = 0; n < n_models; ++n, out += row) {
+                if constexpr (OP == kOpPapaAll) *reinterpret_cast<uint4 *>(out) = all;
+                else {
+                    const uint4 v = image[n * T_];
+                    float r[kElems];
+#pragma unroll
+                    for (int q = 0; q < kElems; ++q) r[q] = __fadd_rn(__fmul_rn(a.alpha, Unit<T>::get(v, q)), m[q]);
+                    *reinterpret_cast<uint4 *>(out) = Unit<T>::pack(r);
+                }
+            }
+        } else {
+            for (int n = 0; n < n_models; ++n, out += row) {
+                const uint4 v = image[n * T_];
+#pragma unroll
+                for (int q = 0; q < kElems; ++q)
+                    if (q < valid) T::store_elem(out, q, T::from_float(OP == kOpPapaAll ? m[q] : __fadd_rn(__fmul_rn(a.alpha, Unit<T>::get(v, q)), m[q])));
+            }
+        }
+    }
+}
+
+// [P][N], all three operators.  A unit's values are N contiguous vectors, element f = (coordinate f / N, model
+// f % N); a warp copies the vectors of its 32 * per_thread units in the order they lie, a lane sums and
+// updates its own units' vectors where they are in shared memory (a unit takes an odd number of vectors
+// there, N or N + 1, so that the lanes fall into different banks), and the warp copies them back in the
+// order they lie.
+// kN: the population size if it is below the number of elements in a vector (a vector may then hold
+// several coordinates' ends, which only unrolled code can place cheaply), else 0.
+template <class T, class TOUT, int OP, int kN>
+__global__ void __launch_bounds__(64, 16) dense_pn_kernel(const __grid_constant__ ReduceArgs a, int per_thread)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    constexpr int kElems = Unit<T>::kElems;
+    const uint32_t N = kN ? kN : static_cast<uint32_t>(a.pop.N), pitch = N | 1u;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    uint4 *image = reinterpret_cast<uint4 *>(smem_raw) + static_cast<size_t>(warp) * 32u * per_thread * pitch;
+    const uint64_t unit_hi = a.group_hi / Unit<T>::kGroups;
+    const uint64_t first = a.group_lo / Unit<T>::kGroups + (static_cast<uint64_t>(blockIdx.x) * (blockDim.x >> 5) + warp) * 32u * per_thread;
+    if (first >= unit_hi) return;   // (no barrier below covers more than the warp)
+    const uint32_t units = static_cast<uint32_t>(min(static_cast<uint64_t>(32u * per_thread), unit_hi - first));
+    uint4 *stack = static_cast<uint4 *>(a.stack) + first * N;
+    const uint32_t dq = 32u / N, dr = 32u - dq * N;
+    // vector k is vector j = k % N of unit k / N; the pair is advanced without dividing again
+    {
+        uint32_t unit = lane / N, j = lane - unit * N;
+        const uint32_t base = smem_addr(image);
+        for (uint32_t k = lane; k < units * N; k += 32) {
+            cp_async<16>(base + (unit * pitch + j) * 16u, stack + k);
+            unit += dq;
+            j += dr;
+            if (j >= N) { j -= N; ++unit; }
+        }
+    }
+    uint32_t valids = 0;
+    for (int u = 0; u < per_thread; ++u)
+        if (32u * u + lane < units) valids |= static_cast<uint32_t>(Unit<T>::valid(a.pop, first + 32u * u + lane, a.status)) << (4 * u);
+    cp_async_wait_all();
+    __syncwarp();
+    const float count = static_cast<float>(N);
+    for (int u = 0; u < per_thread; ++u) {
+        const int valid = static_cast<int>((valids >> (4 * u)) & 15u);
+        uint4 *mine = image + (32u * u + lane) * pitch;
+        if (valid) {
+            float m[kElems];   // run-time N: the finished coordinates are shifted through m
+            uint32_t n = 0;
+            auto finished = [&](float s) -> float {
+                const float mean = __fdiv_rn(s, count);
+                return OP == kOpEma ? __fmul_rn(a.one_minus_alpha, mean) : mean;
+            };
+            auto shift = [&]() {
+#pragma unroll
+                for (int i = 0; i + 1 < kElems; ++i) m[i] = m[i + 1];
+            };
+            if constexpr (kN != 0) {
+#pragma unroll
+                for (int j = 0; j < kN; ++j) {
+                    const uint4 v = mine[j];
+#pragma unroll
+                    for (int q = 0; q < kElems; ++q) {
+                        const int f = j * kElems + q, c = f / kN;
+                        m[c] = f % kN == 0 ? Unit<T>::get(v, q) : __fadd_rn(m[c], Unit<T>::get(v, q));
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < kElems; ++c) m[c] = finished(m[c]);
+            } else {
+                float s = 0.f;
+                for (uint32_t j = 0; j < N; ++j) {
+                    const uint4 v = mine[j];
+                    if (n + kElems <= N) {   // one coordinate's values
+                        s = n == 0 ? Unit<T>::get(v, 0) : __fadd_rn(s, Unit<T>::get(v, 0));
+#pragma unroll
+                        for (int q = 1; q < kElems; ++q) s = __fadd_rn(s, Unit<T>::get(v, q));
+                        n += kElems;
+                        if (n == N) {
+                            n = 0;
+                            shift();
+                            m[kElems - 1] = finished(s);
+                        }
+                    } else {                 // the end of one, the beginning of the next
+                        const uint32_t rest = N - n;
+#pragma unroll
+                        for (int q = 0; q < kElems; ++q) {
+                            if (q == static_cast<int>(rest)) {
+                                shift();
+                                m[kElems - 1] = finished(s);
+                                s = Unit<T>::get(v, q);
+                            } else s = __fadd_rn(s, Unit<T>::get(v, q));
+                        }
+                        n = kElems - rest;
+                    }
+                }
+            }
+            if constexpr (OP == kOpAverage) store_average<T, TOUT>(a, first + 32u * u + lane, valid, m);
+            else if (valid == kElems) {
+                auto updated = [&](const uint4 &v, int q, float mean) -> float {
+                    return OP == kOpPapaAll ? mean : __fadd_rn(__fmul_rn(a.alpha, Unit<T>::get(v, q)), mean);
+                };
+                if constexpr (kN != 0) {
+#pragma unroll
+                    for (int j = 0; j < kN; ++j) {
+                        const uint4 v = mine[j];
+                        float r[kElems];
+#pragma unroll
+                        for (int q = 0; q < kElems; ++q) r[q] = updated(v, q, m[(j * kElems + q) / kN]);
+                        mine[j] = Unit<T>::pack(r);
+                    }
+                } else {
+                    for (uint32_t j = 0; j < N; ++j) {
+                        const uint4 v = mine[j];
+                        float r[kElems];
+                        const uint32_t rest = N - n;   // elements of the current coordinate left; at least one
+#pragma unroll
+                        for (int q = 0; q < kElems; ++q) r[q] = updated(v, q, static_cast<uint32_t>(q) < rest ? m[0] : m[1]);
+                        n += kElems;
+                        if (n >= N) {
+                            n -= N;
+                            shift();
+                        }
+                        mine[j] = Unit<T>::pack(r);
+                    }
+                }
+            } else {   // a tensor's ragged end: its padding is not written
+                n = 0;
+                for (uint32_t f = 0; f < static_cast<uint32_t>(valid) * N; ++f) {
+                    const float x = T::to_float(T::load_elem(mine, f));
+                    T::store_elem(stack + (static_cast<size_t>(32u * u) + lane) * N, f, T::from_float(OP == kOpPapaAll ? m[0] : __fadd_rn(__fmul_rn(a.alpha, x), m[0])));
+                    if (++n == N) {
+                        n = 0;
+                        shift();
+                    }
+                }
+            }
+        }
+        if constexpr (OP != kOpAverage) {
+            const uint32_t whole = __ballot_sync(0xFFFFFFFFu, valid == kElems);   // (orders the lanes' updates, too)
+            uint32_t unit = lane / N, j = lane - unit * N;
+            for (uint32_t k = lane; k < 32u * N; k += 32) {
+                if ((whole >> unit) & 1u) stack[static_cast<size_t>(32u * u) * N + k] = image[(32u * u + unit) * pitch + j];
+                unit += dq;
+                j += dr;
+                if (j >= N) { j -= N; ++unit; }
+            }
+        }
+    }
+}
+
+// Units a thread stages: small populations take several, so that enough bytes are in flight.
+inline int units_per_thread(int N) { return N <= 2 ? 4 : (N <= 5 ? 2 : 1); }
+
+template <class K>
+cudaError_t launch_dense(K kernel, const ReduceArgs &args, uint64_t units, int per_thread, size_t bytes_per_unit, const LaunchShape &shape, cudaStream_t stream)
+{
+    int threads = shape.threads > 0 && shape.threads < 64 ? 32 : 64;
+    while (threads > 32 && bytes_per_unit * per_thread * threads > 44 * 1024) threads >>= 1;   // five blocks and more on an SM
+    const size_t smem = bytes_per_unit * per_thread * threads;
+    KernelFit fit;
+    cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), threads, smem, &fit);
+    if (err != cudaSuccess) return err;
+    if (fit.occupancy < 1) return cudaErrorLaunchOutOfResources;
+    const uint64_t per_block = static_cast<uint64_t>(threads) * per_thread, grid = (units + per_block - 1) / per_block;
+    if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+    kernel<<<static_cast<unsigned>(grid), threads, smem, stream>>>(args, per_thread);
+    count_launch();
+    return cudaGetLastError();
+}
+
+// [N][P]: the largest population whose vectors are kept in registers.  Measured (registers / staged): average,
+// fp32, N = 3 78 / 82 us, N = 10 162 / 164, N = 20 (ResNet-18) 136 / 139; EMA, fp32, N = 5 71 / 74, N = 10 309 / 313, 131072 coordinates of
+// N = 16 4.6 / 6.1, N = 32 equal; EMA, bf16, 2^25 coordinates N = 2 49 / 59, ResNet-50
+// N = 5 94 / 87, N = 8 156 / 133 (few resident warps); PAPA-all, bf16, N = 8 129 / 132.
+template <class T>
+constexpr int regs_max_models(int op) { return op == kOpAverage ? 32 : (T::kBytes == 4 ? 16 : (op == kOpEma ? 3 : 8)); }
+
+template <class T, class TOUT, int OP, int N>
+cudaError_t launch_regs_n(const ReduceArgs &args, uint64_t units, const LaunchShape &shape, cudaStream_t stream)
+{
+    if constexpr (N < regs_max_models<T>(OP))
+        if (args.pop.N > N) return launch_regs_n<T, TOUT, OP, N + 1>(args, units, shape, stream);
+    const unsigned threads = shape.threads > 0 ? static_cast<unsigned>(shape.threads) : 256u;
+    const uint64_t grid = (units + threads - 1) / threads;
+    if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+    regs_np_kernel<T, TOUT, OP, N><<<static_cast<unsigned>(grid), threads, 0, stream>>>(args);
+    count_launch();
+    return cudaGetLastError();
+}
+
+template <class T, class TOUT, int OP>
 cudaError_t launch_reduce_typed(const ReduceArgs &args, const LaunchShape &shape, cudaStream_t stream)
 {
-    const uint64_t items = args.group_hi > args.group_lo ? args.group_hi - args.group_lo : 0;
-    if (args.pop.layout == kLayoutNP)
-        return launch_grid_stride(reduce_kernel<N, T, TOUT, kLayoutNP, OP>, args, items, 0, shape, stream);
-    return launch_grid_stride(reduce_kernel<N, T, TOUT, kLayoutPN, OP>, args, items, 0, shape, stream);
-}
-
-template <int N>
-cudaError_t launch_reduce_n(const ReduceArgs &args, int op, int dtype, int out_dtype, const LaunchShape &shape,
-                            cudaStream_t stream, bool *supported)
-{
-    *supported = true;
-    const bool f32 = dtype == kDtypeF32, bf16 = dtype == kDtypeBF16;
-    if (!f32 && !bf16) { *supported = false; return cudaSuccess; }
-    switch (op) {
-    case kOpEma:
-        return f32 ? launch_reduce_typed<N, F32, F32, kOpEma>(args, shape, stream)
-                   : launch_reduce_typed<N, BF16, BF16, kOpEma>(args, shape, stream);
-    case kOpPapaAll:
-        return f32 ? launch_reduce_typed<N, F32, F32, kOpPapaAll>(args, shape, stream)
-                   : launch_reduce_typed<N, BF16, BF16, kOpPapaAll>(args, shape, stream);
-    case kOpConsensus:
-        return f32 ? launch_reduce_typed<N, F32, F32, kOpConsensus>(args, shape, stream)
-                   : launch_reduce_typed<N, BF16, BF16, kOpConsensus>(args, shape, stream);
-    case kOpAverage:
-        if (f32 && out_dtype == kDtypeF32) return launch_reduce_typed<N, F32, F32, kOpAverage>(args, shape, stream);
-        if (f32 && out_dtype == kDtypeBF16) return launch_reduce_typed<N, F32, BF16, kOpAverage>(args, shape, stream);
-        if (bf16 && out_dtype == kDtypeF32) return launch_reduce_typed<N, BF16, F32, kOpAverage>(args, shape, stream);
-        if (bf16 && out_dtype == kDtypeBF16) return launch_reduce_typed<N, BF16, BF16, kOpAverage>(args, shape, stream);
-        break;
-    default:
-        break;
+    const uint64_t units = args.group_hi > args.group_lo ? (args.group_hi - args.group_lo) / Unit<T>::kGroups : 0;
+    if (units == 0) return cudaSuccess;
+    const int N = args.pop.N;
+    if (args.pop.layout == kLayoutPN) {
+        const int per_thread = units_per_thread(N);
+        const size_t bytes = static_cast<size_t>(N | 1) * 16;
+        if constexpr (Unit<T>::kElems == 4) {
+            switch (N) {
+            case 2: return launch_dense(dense_pn_kernel<T, TOUT, OP, 2>, args, units, per_thread, bytes, shape, stream);
+            case 3: return launch_dense(dense_pn_kernel<T, TOUT, OP, 3>, args, units, per_thread, bytes, shape, stream);
+            }
+        } else {
+            switch (N) {
+            case 2: return launch_dense(dense_pn_kernel<T, TOUT, OP, 2>, args, units, per_thread, bytes, shape, stream);
+            case 3: return launch_dense(dense_pn_kernel<T, TOUT, OP, 3>, args, units, per_thread, bytes, shape, stream);
+            case 4: return launch_dense(dense_pn_kernel<T, TOUT, OP, 4>, args, units, per_thread, bytes, shape, stream);
+            case 5: return launch_dense(dense_pn_kernel<T, TOUT, OP, 5>, args, units, per_thread, bytes, shape, stream);
+            case 6: return launch_dense(dense_pn_kernel<T, TOUT, OP, 6>, args, units, per_thread, bytes, shape, stream);
+            case 7: return launch_dense(dense_pn_kernel<T, TOUT, OP, 7>, args, units, per_thread, bytes, shape, stream);
+            }
+        }
+        return launch_dense(dense_pn_kernel<T, TOUT, OP, 0>, args, units, per_thread, bytes, shape, stream);
     }
-    *supported = false;
-    return cudaSuccess;
+    if (N <= regs_max_models<T>(OP)) return launch_regs_n<T, TOUT, OP, 2>(args, units, shape, stream);
+    return launch_dense(staged_np_kernel<T, TOUT, OP>, args, units, units_per_thread(N), static_cast<size_t>(N) * 16, shape, stream);
 }
 
 }  // namespace wash

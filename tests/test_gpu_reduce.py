@@ -282,3 +282,27 @@ def test_host_step_average_requested_on_a_later_call():
         assert (havg.numpy().view(np.uint32) == want_avg.view(np.uint32)).all()
     B.wash_check(c.gpu.ctx)
     c.close()
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("N,numel,dtype", [
+    (2, [7, 2049], "f32"), (3, [4099], "bf16"), (4, [2051, 9], "bf16"), (5, [6001], "bf16"), (6, [1, 3000], "bf16"), (7, [5003], "bf16"),
+    (9, [4097], "bf16"), (11, [3001, 8], "f32"), (16, [2050], "f32"), (17, [2999, 5], "f32"), (31, [1031], "bf16"), (33, [515], "bf16"), (64, [1025], "bf16"),
+    (8, [300_007], "bf16"), (13, [200_003], "f32")])
+def test_dense_operators_of_every_kernel(N, numel, dtype, layout):
+    """Registers and shared memory ([N][P]), unrolled and run-time population sizes ([P][N]: below and above the elements
+    of a vector), one to four units per thread, ragged last units, several blocks."""
+    c = Case(N, numel, layout, dtype, seed=N + 7)
+    B.papa_ema(c.gpu.ctx, B.WASH_STACK_PARAMS, 0.9)
+    oracle.papa_ema(c.ora, c.host, 0.9)
+    c.assert_equal("ema N=%d %s layout=%d" % (N, dtype, layout))       # same operations in the same order: the same bits, padding too
+    for tdt, ndt, code in ((torch.float32, np.float32, B.WASH_F32), (torch.bfloat16, np.uint16, B.WASH_BF16)):
+        out = torch.zeros(c.P, dtype=tdt, device="cuda")
+        want = np.zeros(c.P, dtype=ndt)
+        B.population_average(c.gpu.ctx, B.WASH_STACK_PARAMS, out, code)
+        oracle.population_average(c.ora, c.host, want)
+        assert (to_host_bits(out) == bits(want)).all()
+    B.papa_all(c.gpu.ctx, B.WASH_STACK_PARAMS)
+    oracle.papa_all(c.ora, c.host)
+    c.assert_equal("papa_all N=%d %s layout=%d" % (N, dtype, layout))
+    c.close()
