@@ -237,6 +237,8 @@ enum wash_step_ops { WASH_OP_SHUFFLE = 1, WASH_OP_EMA = 2, WASH_OP_AVERAGE = 4 }
  * of the parameter dtype) to host_avg (may be NULL unless WASH_OP_AVERAGE), and waits
  * for the stream.  host_stats (may be NULL) receives this call's counters.  The
  * device stacks must be bound; they serve as staging and hold the results too.
+ * A step that only shuffles and moves few values stores them into the host buffers as the
+ * kernels run, when the buffers are pinned and mapped, and does not copy the stacks back.
  * Populations of 2^20 coordinates per model and more are processed in eight coordinate
  * ranges on two internal copy streams, so that the copy in of one range, the kernels on
  * the previous one and the copy out of the one before overlap; the result is the same. */

@@ -8,6 +8,7 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "../../include/wash.h"
@@ -41,6 +42,11 @@ int cuda_fail(cudaError_t err, const char *what)
 
 constexpr int kSlots = 4;   // pinned staging slots for table uploads
 constexpr double kEarlyShare = 0.3;   // expected share of selected coordinates from which the streaming kernel's early flavour is launched (N > 16)
+// wash_step_host: up to this expected selection the moved values are stored into the caller's mapped buffers, above it the
+// stacks are copied back.  A scattered store over PCIe took 0.87 ns a value ([P][N]: the N values of a coordinate share one), the
+// copy back, beside the copy in, 11-22 ps: five ResNet-18 models with momentum 10.9 ms a step copied, 8.37 / 9.07 / 10.98 ms
+// stored at p = 0.001 / 0.01 / 0.03 (the copy in alone 8.1); bf16 + fp32 12.8, 12.2 / 15.6 at 0.01 / 0.03; [P][N], N = 8 3.75, 3.06 / 3.67 at 0.01 / 0.1.
+constexpr double kMirrorShare = 0.012;
 constexpr int kPipeChunks = 32;   // wash_step_host cuts a large population into at most this many coordinate ranges
 
 // makes `device` current for the lifetime of the guard
@@ -159,6 +165,32 @@ wash::PopView view_of(const wash_ctx *ctx)
 
 size_t elem_bytes(int dtype) { return dtype == WASH_BF16 ? 2 : 4; }
 
+// The device's address of a host buffer of elements if the whole of it lies in one allocation that the
+// device can write (pinned, mapped, not read-only), else nullptr.
+void *mapped_host(void *ptr, size_t bytes, int dtype)
+{
+    if (reinterpret_cast<uintptr_t>(ptr) % elem_bytes(dtype)) return nullptr;   // copies take any address, stores do not
+    cudaPointerAttributes attr;
+    unsigned flags = 0;
+    if (cudaPointerGetAttributes(&attr, ptr) != cudaSuccess || attr.type != cudaMemoryTypeHost || !attr.devicePointer ||
+        cudaHostGetFlags(&flags, ptr) != cudaSuccess || (flags & cudaHostRegisterReadOnly)) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    void *entry = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPoint("cuPointerGetAttribute", &entry, cudaEnableDefault, &found) != cudaSuccess || found != cudaDriverEntryPointSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    const auto get = reinterpret_cast<CUresult (*)(void *, CUpointer_attribute, CUdeviceptr)>(entry);
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(ptr);
+    if (get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) != CUDA_SUCCESS || get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) != CUDA_SUCCESS) return nullptr;
+    return at >= start && bytes <= size && at - start <= size - bytes ? attr.devicePointer : nullptr;
+}
+
 // floor(p * 2^32) for p in [0, 1]; the product is exact in binary64
 uint64_t threshold_of(double p) { return static_cast<uint64_t>(std::floor(p * 4294967296.0)); }
 
@@ -212,7 +244,7 @@ int ensure_table(wash_ctx *ctx, cudaStream_t stream)
 // which: 0 = parameters, 1 = optimizer state, 2 = both
 int shuffle_impl(wash_ctx *ctx, int which, uint64_t step, double p, const double *p_layer, uint64_t seed,
                  void *stream_v, wash_stats *stats, uint32_t group_lo = 0, uint32_t group_hi = 0xFFFFFFFFu,
-                 const wash::SqArgs *sq = nullptr, double *sq_out = nullptr)
+                 const wash::SqArgs *sq = nullptr, double *sq_out = nullptr, void *mirror_a = nullptr, void *mirror_b = nullptr)
 {
     if (!ctx) return fail(WASH_ERR_ARG, "ctx is NULL");
     if (step >> 56) return fail(WASH_ERR_ARG, "step must be below 2^56");
@@ -285,6 +317,11 @@ int shuffle_impl(wash_ctx *ctx, int which, uint64_t step, double p, const double
             mode = WASH_MODE_STREAM;
             args.stats_direct = false;
             args.sq = *sq;
+        }
+        if (mirror_a) {   // moved values go to host memory as well: the kernel that touches nothing else
+            mode = WASH_MODE_SPARSE;
+            args.mirror_a = mirror_a;
+            args.mirror_b = mirror_b;
         }
         if (mode == WASH_MODE_SPARSE) args.stats_direct = true;   // blocks that each serve a few dozen coordinates and more, spread over the launch
     }
@@ -609,6 +646,20 @@ int wash_step_host(wash_ctx *ctx, int32_t ops, void *host_params, void *host_opt
     }
     int rc;
     wash_stats st = {0, 0};
+    // A step that only shuffles changes few of the caller's values: when both buffers can be written by the
+    // device, the moved values are stored into them and the stacks are not copied back.
+    void *mirror_p = nullptr, *mirror_o = nullptr;
+    if (ops == WASH_OP_SHUFFLE || ops == (WASH_OP_SHUFFLE | WASH_OP_AVERAGE)) {
+        double coordinates = 0.0, expected = 0.0;
+        for (int s = 0; s < ctx->n_seg; ++s) {
+            coordinates += static_cast<double>(ctx->numel[s]);
+            expected += static_cast<double>(ctx->numel[s]) * (p_layer ? p_layer[s] : p);
+        }
+        if (expected <= kMirrorShare * coordinates * (ctx->layout == WASH_LAYOUT_PN ? std::fmin(ctx->N, 5.0) : 1.0)) {
+            mirror_p = mapped_host(host_params, p_bytes, pd);
+            if (mirror_p && host_opt && !(mirror_o = mapped_host(host_opt, o_bytes, ctx->stack_dtype[WASH_STACK_OPT]))) mirror_p = nullptr;
+        }
+    }
     // Large populations go through in kPipeChunks coordinate ranges so that the copy of one
     // range to the device, the kernels on the previous one and the copy of the one before
     // back to the host overlap (the PCIe link is full duplex, and the draws are keyed by
@@ -663,7 +714,7 @@ int wash_step_host(wash_ctx *ctx, int32_t ops, void *host_params, void *host_opt
                 if ((err = cudaEventRecord(ev_in[k], ctx->copy_in)) != cudaSuccess || (err = cudaStreamWaitEvent(stream, ev_in[k], 0)) != cudaSuccess)
                     return cuda_fail(err, "pipeline event");
                 if (ops & WASH_OP_SHUFFLE) {
-                    rc = shuffle_impl(ctx, host_opt ? 2 : 0, step, p, p_layer, seed, stream, ctx->stats_dev, g0, g1);
+                    rc = shuffle_impl(ctx, host_opt ? 2 : 0, step, p, p_layer, seed, stream, ctx->stats_dev, g0, g1, nullptr, nullptr, mirror_p, mirror_o);
                     if (rc != WASH_OK) return rc;
                 }
                 if (ops & WASH_OP_EMA) {
@@ -676,9 +727,9 @@ int wash_step_host(wash_ctx *ctx, int32_t ops, void *host_params, void *host_opt
                 }
                 if ((err = cudaEventRecord(ev_done[k], stream)) != cudaSuccess || (err = cudaStreamWaitEvent(ctx->copy_out, ev_done[k], 0)) != cudaSuccess)
                     return cuda_fail(err, "pipeline event");
-                if ((err = copy_range(host_params, ctx->stack_ptr[WASH_STACK_PARAMS], pd, e0, count, cudaMemcpyDeviceToHost, ctx->copy_out)) != cudaSuccess)
+                if (!mirror_p && (err = copy_range(host_params, ctx->stack_ptr[WASH_STACK_PARAMS], pd, e0, count, cudaMemcpyDeviceToHost, ctx->copy_out)) != cudaSuccess)
                     return cuda_fail(err, "copy of a parameter range to the host");
-                if (host_opt && (err = copy_range(host_opt, ctx->stack_ptr[WASH_STACK_OPT], od, e0, count, cudaMemcpyDeviceToHost, ctx->copy_out)) != cudaSuccess)
+                if (host_opt && !mirror_p && (err = copy_range(host_opt, ctx->stack_ptr[WASH_STACK_OPT], od, e0, count, cudaMemcpyDeviceToHost, ctx->copy_out)) != cudaSuccess)
                     return cuda_fail(err, "copy of an optimizer-state range to the host");
                 if ((ops & WASH_OP_AVERAGE) &&
                     (err = cudaMemcpyAsync(static_cast<char *>(host_avg) + e0 * elem_bytes(pd), static_cast<char *>(ctx->avg_dev) + e0 * elem_bytes(pd),
@@ -711,7 +762,7 @@ int wash_step_host(wash_ctx *ctx, int32_t ops, void *host_params, void *host_opt
         return cuda_fail(err, "copy of the optimizer-state stack to the device");
     if (ops & WASH_OP_SHUFFLE) {
         if ((err = cudaMemsetAsync(ctx->stats_dev, 0, sizeof(wash_stats), stream)) != cudaSuccess) return cuda_fail(err, "cudaMemsetAsync(stats)");
-        rc = shuffle_impl(ctx, host_opt ? 2 : 0, step, p, p_layer, seed, stream, ctx->stats_dev);
+        rc = shuffle_impl(ctx, host_opt ? 2 : 0, step, p, p_layer, seed, stream, ctx->stats_dev, 0, 0xFFFFFFFFu, nullptr, nullptr, mirror_p, mirror_o);
         if (rc != WASH_OK) return rc;
     }
     if (ops & WASH_OP_EMA) {
@@ -725,9 +776,9 @@ int wash_step_host(wash_ctx *ctx, int32_t ops, void *host_params, void *host_opt
         rc = population_average(ctx, WASH_STACK_PARAMS, ctx->avg_dev, pd, stream);
         if (rc != WASH_OK) return rc;
     }
-    if ((err = cudaMemcpyAsync(host_params, ctx->stack_ptr[WASH_STACK_PARAMS], p_bytes, cudaMemcpyDeviceToHost, stream)) != cudaSuccess)
+    if (!mirror_p && (err = cudaMemcpyAsync(host_params, ctx->stack_ptr[WASH_STACK_PARAMS], p_bytes, cudaMemcpyDeviceToHost, stream)) != cudaSuccess)
         return cuda_fail(err, "copy of the parameter stack to the host");
-    if (host_opt && (err = cudaMemcpyAsync(host_opt, ctx->stack_ptr[WASH_STACK_OPT], o_bytes, cudaMemcpyDeviceToHost, stream)) != cudaSuccess)
+    if (host_opt && !mirror_p && (err = cudaMemcpyAsync(host_opt, ctx->stack_ptr[WASH_STACK_OPT], o_bytes, cudaMemcpyDeviceToHost, stream)) != cudaSuccess)
         return cuda_fail(err, "copy of the optimizer-state stack to the host");
     if ((ops & WASH_OP_AVERAGE) && (err = cudaMemcpyAsync(host_avg, ctx->avg_dev, avg_bytes, cudaMemcpyDeviceToHost, stream)) != cudaSuccess)
         return cuda_fail(err, "copy of the average to the host");

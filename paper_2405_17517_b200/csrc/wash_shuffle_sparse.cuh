@@ -45,7 +45,8 @@ struct SparseArgs {
     uint32_t inverse;       // 2^16 / d, rounded up, for the division of a pair's number (below 128) by in_set ([N][P]) or N ([P][N])
 };
 
-template <class TA, class TB, int LAYOUT>
+// MIRROR: the moved values go to a second copy of the stacks as well (wash_step_host: the caller's buffers).
+template <class TA, class TB, int LAYOUT, bool MIRROR>
 __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_sparse_kernel(const __grid_constant__ SparseArgs p)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -149,6 +150,10 @@ __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_spa
                 if (out[k] < 0) continue;
                 TA::store_elem(a.a, out[k], va[k]);
                 if constexpr (kHasB) TB::store_elem(a.b, out[k], vb[k]);
+                if constexpr (MIRROR) {
+                    TA::store_elem(a.mirror_a, out[k], va[k]);
+                    if constexpr (kHasB) TB::store_elem(a.mirror_b, out[k], vb[k]);
+                }
                 ++moved;
             }
         }
@@ -168,7 +173,9 @@ cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchSha
     p.s = args;
     p.n_wtiles = (args.group_hi - args.group_lo + kWarpTileGroups - 1) / kWarpTileGroups;
     const size_t smem = sparse_queue_capacity(args.pop.N) * (12 + (args.pop.N > 16 ? 4 * static_cast<size_t>(wide_pitch(args.pop.N)) : 0));
-    auto kernel = args.pop.layout == kLayoutNP ? shuffle_sparse_kernel<TA, TB, kLayoutNP> : shuffle_sparse_kernel<TA, TB, kLayoutPN>;
+    const bool np = args.pop.layout == kLayoutNP;
+    auto kernel = np ? shuffle_sparse_kernel<TA, TB, kLayoutNP, false> : shuffle_sparse_kernel<TA, TB, kLayoutPN, false>;
+    if (args.mirror_a) kernel = np ? shuffle_sparse_kernel<TA, TB, kLayoutNP, true> : shuffle_sparse_kernel<TA, TB, kLayoutPN, true>;
     KernelFit fit;
     cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), kSparseThreads, smem, &fit);
     if (err != cudaSuccess) return err;

@@ -306,3 +306,27 @@ def test_dense_operators_of_every_kernel(N, numel, dtype, layout):
     oracle.papa_all(c.ora, c.host)
     c.assert_equal("papa_all N=%d %s layout=%d" % (N, dtype, layout))
     c.close()
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("N,numel,dtype,opt,p", [
+    (3, [5000, 7, 300], "f32", "f32", 0.01), (5, [1_100_003, 9], "bf16", "f32", 0.004), (4, [1_300_001], "f32", None, 0.01), (20, [60_001], "f32", "bf16", 0.009)])
+def test_host_step_into_pinned_buffers(N, numel, dtype, opt, p, layout):
+    """Pinned buffers and few selected coordinates: the moved values are stored into the host buffers by the kernel
+    (in one piece and in ranges); buffers that lie inside a larger allocation, at an odd element."""
+    c = Case(N, numel, layout, dtype, opt, seed=N)
+    pinned = []
+    for h in [c.host] + ([c.host_opt] if opt else []):
+        flat = torch.from_numpy(h.reshape(-1).view(np.int16 if h.dtype == np.uint16 else np.int32))
+        buf = torch.full((flat.numel() + 5,), 0x55, dtype=flat.dtype, pin_memory=True)
+        buf[1:-4] = flat
+        pinned.append(buf)
+    views = [b[1:-4] for b in pinned]
+    got = B.wash_step_host(c.gpu.ctx, B.WASH_OP_SHUFFLE, views[0], views[1] if opt else None, None, 9, p, None, 41)
+    want = oracle.shuffle(c.ora, c.host, p, seed=41, step=9, stack2=c.host_opt)
+    assert got == tuple(want)
+    c.assert_equal("device stacks")
+    for v, b, h in zip(views, pinned, [c.host, c.host_opt]):
+        assert (v.numpy().view(bits(h).dtype) == bits(h)).all()
+        assert b[0] == 0x55 and (b[-4:] == 0x55).all()
+    c.close()
