@@ -2,6 +2,7 @@
 #include <atomic>
 #include "wash_internal.h"
 #include "wash_device.cuh"
+#include "wash_launch.cuh"
 
 namespace wash {
 
@@ -21,6 +22,8 @@ uint64_t launch_count() { return g_launches.load(std::memory_order_relaxed); }
 // compare-and-swap loops and cost this one-block kernel 20 us when 256 threads contended.)
 __global__ void __launch_bounds__(kStatSlots) flush_stats_kernel(StatSlot *slots, unsigned long long *stats)
 {
+    let_next_start();
+    await_previous();
     __shared__ unsigned long long part[2][kStatSlots / 32];
     unsigned long long sel = slots[threadIdx.x].selected, mov = slots[threadIdx.x].moved;
     if (sel) {
@@ -56,6 +59,8 @@ __global__ void __launch_bounds__(kStatSlots) flush_stats_kernel(StatSlot *slots
 // copies (a thread that went through the copies of an entry one after the other took 64 round trips).
 __global__ void __launch_bounds__(1024) sq_flush_kernel(double *slots, int count, double *out)
 {
+    let_next_start();
+    await_previous();
     static_assert(kSqSlots == 64, "two copies per lane");
     const int lane = threadIdx.x & 31;
     for (int j = threadIdx.x >> 5; j < count; j += blockDim.x >> 5) {
@@ -72,9 +77,7 @@ __global__ void __launch_bounds__(1024) sq_flush_kernel(double *slots, int count
 cudaError_t launch_sq_flush(const SqArgs &sq, int N, double *out, cudaStream_t stream)
 {
     const int entries = sq.n_ranges * N;
-    sq_flush_kernel<<<1, entries < 32 ? 32 * entries : 1024, 0, stream>>>(sq.slots, entries, out);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(sq_flush_kernel, 1, entries < 32 ? 32 * entries : 1024, 0, stream, sq.slots, entries, out);
 }
 
 // Nothing but the mask's Philox blocks: four blocks per thread (four independent chains, as in the
@@ -143,9 +146,7 @@ cudaError_t launch_shuffle(const ShuffleArgs &args, int a_dtype, int b_dtype, in
     bool flush = false;
     cudaError_t err = launch_shuffle_kernel(args, a_dtype, b_dtype, mode, shape, stream, supported, &flush);
     if (err != cudaSuccess || !*supported || !flush) return err;
-    flush_stats_kernel<<<1, kStatSlots, 0, stream>>>(args.stat_slots, args.stats);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(flush_stats_kernel, 1, kStatSlots, 0, stream, args.stat_slots, args.stats);
 }
 
 cudaError_t launch_reduce(const ReduceArgs &args, int op, int dtype, int out_dtype, const LaunchShape &shape,

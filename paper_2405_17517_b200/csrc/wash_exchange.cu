@@ -88,6 +88,8 @@ constexpr uint32_t kPlanQueue = 1024;
 __global__ void __launch_bounds__(kXThreads, kExchangeBlocksPerSm) exchange_plan_kernel(const __grid_constant__ ExchangeArgs a)
 {
     extern __shared__ uint32_t s_perm_all[];   // 32 * wide_pitch(N) words per warp when N > 16, else nothing
+    let_next_start();
+    await_previous();
     __shared__ uint2 q_key[kPlanQueue];       // {coordinate within its tensor, tensor}
     __shared__ uint32_t q_elem[kPlanQueue];   // row element (rows are shorter than 2^32)
     __shared__ uint32_t s_total[kMaxN + 1], s_count;
@@ -210,6 +212,8 @@ __device__ __forceinline__ uint32_t fill_list(const ExchangeArgs &a, CoordList &
 
 __global__ void __launch_bounds__(kXThreads) exchange_send_kernel(const __grid_constant__ ExchangeArgs a)
 {
+    let_next_start();
+    await_previous();
     extern __shared__ uint32_t s_perm_all[];
     __shared__ CoordList list;
     __shared__ uint32_t s_base[kMaxN], s_votes[kExchangeWarps][kMaxN];
@@ -286,6 +290,8 @@ __global__ void __launch_bounds__(kXThreads) exchange_send_kernel(const __grid_c
 
 __global__ void __launch_bounds__(kXThreads) exchange_receive_kernel(const __grid_constant__ ExchangeArgs a)
 {
+    let_next_start();
+    await_previous();
     __shared__ CoordList list;
     __shared__ uint32_t s_part[kExchangeWarps];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
@@ -344,9 +350,7 @@ cudaError_t launch_exchange_plan(const ExchangeArgs &args, cudaStream_t stream)
     size_t smem = 0;
     cudaError_t err = perm_smem(args, reinterpret_cast<const void *>(exchange_plan_kernel), &smem);
     if (err != cudaSuccess) return err;
-    exchange_plan_kernel<<<args.n_blocks, kXThreads, smem, stream>>>(args);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(exchange_plan_kernel, args.n_blocks, kXThreads, smem, stream, args);
 }
 
 cudaError_t launch_exchange_send(const ExchangeArgs &args, cudaStream_t stream)
@@ -355,17 +359,13 @@ cudaError_t launch_exchange_send(const ExchangeArgs &args, cudaStream_t stream)
     size_t smem = 0;
     cudaError_t err = perm_smem(args, reinterpret_cast<const void *>(exchange_send_kernel), &smem);
     if (err != cudaSuccess) return err;
-    exchange_send_kernel<<<args.n_blocks, kXThreads, smem, stream>>>(args);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(exchange_send_kernel, args.n_blocks, kXThreads, smem, stream, args);
 }
 
 cudaError_t launch_exchange_receive(const ExchangeArgs &args, cudaStream_t stream)
 {
     if (args.n_blocks == 0) return cudaSuccess;
-    exchange_receive_kernel<<<args.n_blocks, kXThreads, 0, stream>>>(args);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(exchange_receive_kernel, args.n_blocks, kXThreads, 0, stream, args);
 }
 
 }  // namespace wash

@@ -1,4 +1,5 @@
-// How many blocks of a kernel fit an SM, looked up once per launch shape.
+// Launching a kernel in the chain of a stream, and how many blocks of one fit an SM (looked up once per
+// launch shape).
 #pragma once
 #include <cstdint>
 #include <map>
@@ -8,6 +9,33 @@
 #include "wash_internal.h"
 
 namespace wash {
+
+// Kernels of this library are launched with the programmatic-serialization attribute: a launch need not
+// wait until the kernel before it in the stream has drained, its blocks may start as that one's
+// last blocks run.  In return every kernel calls await_previous() before it touches anything that an
+// earlier kernel may write or read -- which waits until the kernels before it are complete and their
+// writes visible -- and let_next_start() at its beginning.  A kernel of another library before or
+// after ours, or a copy between two kernels, is ordered as always.
+__device__ __forceinline__ void await_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... Params, class... Args>
+cudaError_t launch_chained(void (*kernel)(Params...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, const Args &...args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t config = {};
+    config.gridDim = dim3(grid);
+    config.blockDim = dim3(threads);
+    config.dynamicSmemBytes = smem;
+    config.stream = stream;
+    config.attrs = &attr;
+    config.numAttrs = 1;
+    cudaError_t err = cudaLaunchKernelEx(&config, kernel, static_cast<Params>(args)...);
+    if (err == cudaSuccess) count_launch();
+    return err;
+}
 
 struct KernelFit {
     int occupancy;   // resident blocks per SM at (threads, smem)

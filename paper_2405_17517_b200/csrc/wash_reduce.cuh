@@ -76,6 +76,8 @@ __device__ __forceinline__ void store_average(const ReduceArgs &a, uint64_t unit
 template <class T, class TOUT, int OP, int N>
 __global__ void __launch_bounds__(256) regs_np_kernel(const __grid_constant__ ReduceArgs a)
 {
+    let_next_start();
+    await_previous();
     constexpr int kElems = Unit<T>::kElems;
     const uint64_t unit = a.group_lo / Unit<T>::kGroups + static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (unit * Unit<T>::kGroups >= a.group_hi) return;
@@ -123,6 +125,8 @@ __global__ void __launch_bounds__(256) regs_np_kernel(const __grid_constant__ Re
 template <class T, class TOUT, int OP>
 __global__ void __launch_bounds__(64, 20) staged_np_kernel(const __grid_constant__ ReduceArgs a, int per_thread)
 {
+    let_next_start();
+    await_previous();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr int kElems = Unit<T>::kElems;
     const int n_models = a.pop.N;
@@ -205,6 +209,8 @@ __global__ void __launch_bounds__(64, 20) staged_np_kernel(const __grid_constant
 template <class T, class TOUT, int OP, int kN>
 __global__ void __launch_bounds__(64, 16) dense_pn_kernel(const __grid_constant__ ReduceArgs a, int per_thread)
 {
+    let_next_start();
+    await_previous();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr int kElems = Unit<T>::kElems;
     const uint32_t N = kN ? kN : static_cast<uint32_t>(a.pop.N), pitch = N | 1u;
@@ -356,9 +362,7 @@ cudaError_t launch_dense(K kernel, const ReduceArgs &args, uint64_t units, int p
     if (fit.occupancy < 1) return cudaErrorLaunchOutOfResources;
     const uint64_t per_block = static_cast<uint64_t>(threads) * per_thread, grid = (units + per_block - 1) / per_block;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    kernel<<<static_cast<unsigned>(grid), threads, smem, stream>>>(args, per_thread);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(kernel, static_cast<unsigned>(grid), threads, smem, stream, args, per_thread);
 }
 
 // [N][P]: the largest population whose vectors are kept in registers.  Measured (registers / staged): average,
@@ -376,9 +380,7 @@ cudaError_t launch_regs_n(const ReduceArgs &args, uint64_t units, const LaunchSh
     const unsigned threads = shape.threads > 0 ? static_cast<unsigned>(shape.threads) : 256u;
     const uint64_t grid = (units + threads - 1) / threads;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    regs_np_kernel<T, TOUT, OP, N><<<static_cast<unsigned>(grid), threads, 0, stream>>>(args);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(regs_np_kernel<T, TOUT, OP, N>, static_cast<unsigned>(grid), threads, 0, stream, args);
 }
 
 template <class T, class TOUT, int OP>

@@ -644,6 +644,8 @@ __device__ __forceinline__ void consensus_tile(const ShuffleArgs &a, const unsig
 template <class TA, class TB, int LAYOUT, int G, bool STAT, bool EARLY>
 __global__ void __launch_bounds__(256, EARLY ? 3 : 5) shuffle_async_kernel(const __grid_constant__ ShuffleArgs a)
 {
+    let_next_start();
+    await_previous();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr bool kHasB = TB::kCode != kDtypeNone;
     const int n_models = a.pop.N;
@@ -755,9 +757,7 @@ cudaError_t launch_shuffle_async_tiles(const ShuffleArgs &args, const LaunchShap
     const uint64_t grid = (static_cast<uint64_t>(args.group_hi - args.group_lo) + per_block - 1) / per_block;
     if (grid == 0) return cudaSuccess;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    kernel<<<static_cast<unsigned>(grid), threads, smem, stream>>>(args);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(kernel, static_cast<unsigned>(grid), threads, smem, stream, args);
 }
 
 template <class TA, class TB>

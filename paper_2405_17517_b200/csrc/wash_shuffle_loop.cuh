@@ -122,6 +122,8 @@ __device__ __forceinline__ uint32_t list_selected(uint16_t *list, uint32_t sel)
 template <class TA, class TB, int LAYOUT, int G>
 __global__ void __launch_bounds__(32, G == 2 ? 32 : 28) shuffle_loop_kernel(const __grid_constant__ ShuffleArgs a)
 {
+    let_next_start();
+    await_previous();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr bool kHasB = TB::kCode != kDtypeNone;
     constexpr uint32_t T_ = 32;   // the launch has one warp per block
@@ -262,9 +264,7 @@ cudaError_t launch_shuffle_loop_tiles(const ShuffleArgs &args, const LaunchShape
     if (n_tiles == 0) return cudaSuccess;
     const uint64_t resident = static_cast<uint64_t>(shape.sm_count > 0 ? shape.sm_count : 148) * fit.occupancy;
     const uint64_t grid = n_tiles < resident ? n_tiles : resident;
-    kernel<<<static_cast<unsigned>(grid), 32, smem, stream>>>(args);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(kernel, static_cast<unsigned>(grid), 32, smem, stream, args);
 }
 
 template <class TA, class TB>

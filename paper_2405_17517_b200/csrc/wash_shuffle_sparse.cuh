@@ -49,6 +49,7 @@ struct SparseArgs {
 template <class TA, class TB, int LAYOUT, bool MIRROR>
 __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_sparse_kernel(const __grid_constant__ SparseArgs p)
 {
+    let_next_start();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ uint32_t s_count;
     constexpr bool kHasB = TB::kCode != kDtypeNone;
@@ -94,6 +95,7 @@ __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_spa
         }
         const bool again = __syncthreads_or(sel != 0 || t < t_end);   // (orders the queue's entries, too)
         const uint32_t count = min(s_count, capacity);
+        await_previous();   // the masks read nothing but the tables; the stacks come now
         if (n_models <= 16) {
             for (uint32_t e = threadIdx.x; e < count; e += kSparseThreads) {
                 const uint2 key = q_key[e];
@@ -199,9 +201,7 @@ cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchSha
     p.in_set = 32u * kSparsePairs / static_cast<uint32_t>(args.pop.N);
     const uint32_t divisor = args.pop.layout == kLayoutNP ? p.in_set : static_cast<uint32_t>(args.pop.N);
     p.inverse = (65536u + divisor - 1u) / divisor;
-    kernel<<<grid, kSparseThreads, smem, stream>>>(p);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(kernel, grid, kSparseThreads, smem, stream, p);
 }
 
 inline cudaError_t launch_shuffle_sparse_tiles(const ShuffleArgs &args, int a_dtype, int b_dtype, const LaunchShape &shape,

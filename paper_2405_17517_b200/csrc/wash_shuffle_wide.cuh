@@ -36,6 +36,8 @@ __device__ __forceinline__ void move_value(const ShuffleArgs &a, const unsigned 
 template <class TA, class TB, int LAYOUT, bool STAT>
 __global__ void __launch_bounds__(64, 6) shuffle_wide_kernel(const __grid_constant__ ShuffleArgs a)
 {
+    let_next_start();
+    await_previous();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr bool kHasB = TB::kCode != kDtypeNone;
     const int n_models = a.pop.N;
@@ -138,9 +140,7 @@ cudaError_t launch_shuffle_wide_typed(const ShuffleArgs &call, const LaunchShape
     const uint64_t grid = (static_cast<uint64_t>(args.group_hi - args.group_lo) + threads - 1) / threads;
     if (grid == 0) return cudaSuccess;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    kernel<<<static_cast<unsigned>(grid), threads, smem, stream>>>(args);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(kernel, static_cast<unsigned>(grid), threads, smem, stream, args);
 }
 
 inline cudaError_t launch_shuffle_wide(const ShuffleArgs &args, int a_dtype, int b_dtype, const LaunchShape &shape,

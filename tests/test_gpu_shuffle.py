@@ -432,3 +432,64 @@ def test_random_configurations_match_oracle(seed):
         assert c.gpu_stats() == tuple(tot), what
         B.wash_check(c.gpu.ctx)
         c.close()
+
+
+@pytest.mark.parametrize("captured", [False, True], ids=["stream", "graph"])
+def test_calls_that_follow_each_other_at_once(captured):
+    """Kernels are launched so that one may start while the one before it ends: a chain of calls on shared stacks with
+    other kernels, copies and changes of the probabilities (a table upload) in between must see every result before it,
+    launched on a side stream and replayed from a graph (no upload there: the probabilities stay)."""
+    N, numel = 5, [120_001, 64, 30_003]
+    c = Case(N, numel, 0, "f32", "f32", seed=3)
+    avg = torch.zeros(c.P, dtype=torch.float32, device="cuda")
+    seen, scale = [torch.zeros_like(avg) for _ in range(4)], torch.full((1,), 0.5, device="cuda")
+
+    def chain(stream):
+        for i in range(4):
+            B.wash_set_mode(c.gpu.ctx, (B.WASH_MODE_SPARSE, B.WASH_MODE_STREAM)[i & 1])
+            p = 0.05 if captured else (0.05, 0.05, 0.2, 0.01)[i]
+            B.wash_shuffle_both(c.gpu.ctx, i, p, None, seed=4, stream=stream, stats=c.stats_dev)
+            B.wash_shuffle(c.gpu.ctx, 100 + i, p, None, seed=4, stream=stream, stats=c.stats_dev)
+            B.papa_ema(c.gpu.ctx, B.WASH_STACK_PARAMS, 0.75, stream=stream)
+            if i == 2:
+                c.dev.mul_(scale)                              # another library's kernel between two of ours
+            B.population_average(c.gpu.ctx, B.WASH_STACK_PARAMS, avg, B.WASH_F32, stream=stream)
+            seen[i].copy_(avg)
+
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    repeats = 1
+    if captured:
+        B.wash_shuffle(c.gpu.ctx, 7, 0.05, None, seed=4, stream=s)      # the table is uploaded before the capture
+        oracle.shuffle(c.ora, c.host, 0.05, seed=4, step=7)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            chain(s)
+        torch.cuda.current_stream().wait_stream(s)
+        repeats = 3
+        for _ in range(repeats):
+            g.replay()
+    else:
+        with torch.cuda.stream(s):
+            chain(s)
+    torch.cuda.synchronize()
+    tot, want = [0, 0], np.zeros(c.P, dtype=np.float32)
+    for _ in range(repeats):
+        for i in range(4):
+            p = 0.05 if captured else (0.05, 0.05, 0.2, 0.01)[i]
+            for st in (oracle.shuffle(c.ora, c.host, p, seed=4, step=i, stack2=c.host_opt), oracle.shuffle(c.ora, c.host, p, seed=4, step=100 + i)):
+                tot[0] += st[0]; tot[1] += st[1]
+            oracle.papa_ema(c.ora, c.host, 0.75)
+            if i == 2:
+                c.host *= np.float32(0.5)
+            oracle.population_average(c.ora, c.host, want)
+            got = to_host_bits(seen[i])
+            if repeats == 1:
+                assert (got == bits(want)).all(), i
+    assert (to_host_bits(seen[3]) == bits(want)).all()
+    got, h = to_host_bits(c.dev), bits(c.host)
+    finite = ~np.isnan(c.host.reshape(-1))
+    assert (got[finite] == h[finite]).all()
+    assert (to_host_bits(c.dev_opt) == bits(c.host_opt)).all()
+    assert c.gpu_stats() == tuple(tot)
+    c.close()
