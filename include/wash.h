@@ -61,12 +61,13 @@ enum wash_mode {
                              per-thread asynchronous copies (cp.async).  Default.            */
     WASH_MODE_SPARSE = 1, /* draws the mask first; touches only selected coordinates          */
     WASH_MODE_AUTO = 2             /* SPARSE when the call's probabilities select, in expectation,
-                                      less than a share of the coordinates that depends on layout
-                                      and N, else STREAM.  [N][padded_P]: max(3 %, 35 % / N);
-                                      [padded_P][N]: 30 % up to N = 8, 10 % above (the measured
+                                      less than a share of the coordinates that depends on layout,
+                                      N and the number of stacks, else STREAM.  [N][padded_P]:
+                                      60 % / N for one stack, 35 % / N for two, 18 % at most;
+                                      [padded_P][N]: 13 % to 40 %, growing with N (the measured
                                       crossovers on B200: in the second layout the N values of a
                                       coordinate share a DRAM access; a small population leaves
-                                      the streaming kernel bound by issue slots)                 */
+                                      the streaming kernels bound by issue slots)                */
 };
 
 #define WASH_MAX_N 64            /* largest population                                     */
@@ -129,7 +130,7 @@ int wash_set_mode(wash_ctx *ctx, int32_t mode);
  * (default: 2 when a group of all models is at most 64 bytes, else 1); blocks_per_sm = -2 / -3
  * forces the streaming kernel's lean / early flavour (early draws the permutations while the
  * stack's copies are in flight and serves populations of more than 16 models densely; by
- * default it is launched for N > 16 when the call's probabilities select 30 % or more; from
+ * default it is launched for N > 16 when the call's probabilities select 70 % or more; from
  * 0.3 % to there populations of more than 16 models have a kernel of their own);
  * blocks_per_sm = -4 / -5 forces (N <= 16) / excludes the streaming kernel for small groups (a
  * resident grid of warps walking tiles through two shared-memory stages; by default

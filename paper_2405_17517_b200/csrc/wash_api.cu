@@ -41,7 +41,10 @@ int cuda_fail(cudaError_t err, const char *what)
 }
 
 constexpr int kSlots = 4;   // pinned staging slots for table uploads
-constexpr double kEarlyShare = 0.3;   // expected share of selected coordinates from which the streaming kernel's early flavour is launched (N > 16)
+// Expected share of selected coordinates from which the streaming kernel's early flavour is launched (N > 16) instead of the
+// wide kernel.  2^24 coordinates, fp32, N = 32, wide / early at 50 / 70 / 100 %: [N][P] 559 / 647, 693 / 690, 895 / 665 us; [P][N] 659 / 960, 838 / 867,
+// 1092 / 848; N = 17 crosses at 60 %, N = 64 and two stacks at 70-90 %.
+constexpr double kEarlyShare = 0.7;
 // wash_step_host: up to this expected selection the moved values are stored into the caller's mapped buffers, above it the
 // stacks are copied back.  A scattered store over PCIe took 0.87 ns a value ([P][N]: the N values of a coordinate share one), the
 // copy back, beside the copy in, 11-22 ps: five ResNet-18 models with momentum 10.9 ms a step copied, 8.37 / 9.07 / 10.98 ms
@@ -194,6 +197,22 @@ void *mapped_host(void *ptr, size_t bytes, int dtype)
 // floor(p * 2^32) for p in [0, 1]; the product is exact in binary64
 uint64_t threshold_of(double p) { return static_cast<uint64_t>(std::floor(p * 4294967296.0)); }
 
+// WASH_MODE_AUTO: the expected share of selected coordinates up to which the sparse kernel is launched.  Serving a
+// coordinate costs it a scattered DRAM access and store per model and stack in [N][P], a few neighbouring ones for
+// all N models in [P][N]; the streaming kernels pay for the stack's bytes and, in small populations, for issue slots.
+// Measured crossovers (2^24-2^25 coordinates):
+//   [N][P]  one stack   fp32 N = 2 18 %, 3 14 %, 4 15 %, 5 12 %, 8 6 %, 12 5 %, 16 4.7 %, 20 5 %, 32 2 %; bf16 18, 16, 19, 11, 15, 10, 7.5, 3, 1 %
+//           two stacks  fp32 N = 2 20 %, 5 6 %, 16 3 %, 32 1.8 %; bf16 + fp32 21, 5, 2.8, 1.3 %
+//   [P][N]  one stack   fp32 N = 2 14 %, 3 13 %, 4 15 %, 5 15 %, 8 17 %, 12 20 %, 16 40 %, 20 35 %, 32 above 50 %; bf16 13, 12, 19, 27, 28, 38, 48, 20, 33 %
+//           two stacks  fp32 N = 2 23 %, 5 20 %, 16 and 32 above 50 %; bf16 + fp32 20, 30, above 50 %
+double sparse_share(int layout, int N, bool two_stacks, bool bf16)
+{
+    if (layout == WASH_LAYOUT_NP) return std::fmin(0.18, (two_stacks ? 0.35 : 0.6) / N);
+    if (N <= 3) return two_stacks ? 0.2 : 0.13;
+    if (N < 16) return two_stacks || bf16 ? 0.2 : 0.16;
+    return bf16 && !two_stacks ? (N == 16 ? 0.4 : 0.2) : 0.4;
+}
+
 // Brings the device copy of the segment table up to date with the call's
 // probabilities (uploaded, in stream order, only when they changed).
 int sync_table(wash_ctx *ctx, double p, const double *p_layer, cudaStream_t stream)
@@ -293,11 +312,7 @@ int shuffle_impl(wash_ctx *ctx, int which, uint64_t step, double p, const double
         if (ctx->mode == WASH_MODE_AUTO) {
             double coordinates = 0.0;
             for (int s = 0; s < ctx->n_seg; ++s) coordinates += static_cast<double>(ctx->seg_host[s].numel);
-            // measured crossovers of the two kernels (fp32, 2^25-2^26 coordinates): serving a coordinate costs a
-            // 128-byte DRAM access per model and stack in [N][P], one or two for all N models in [P][N]; and a
-            // small population leaves the streaming kernel bound by issue slots, not by the stack's bytes.
-            // [N][P]: N = 2 17 %, 4 10 %, 8 4 %, 16 2.5 %, 32 3-5 %; [P][N]: N <= 8 above 30 %, 16 10 %, 32 12 %
-            const double share = ctx->layout == WASH_LAYOUT_PN ? (ctx->N <= 8 ? 0.30 : 0.10) : std::fmax(0.03, 0.35 / ctx->N);
+            const double share = sparse_share(ctx->layout, ctx->N, b != nullptr, a_dtype == wash::kDtypeBF16);
             mode = ctx->expected_selected < share * coordinates ? WASH_MODE_SPARSE : WASH_MODE_STREAM;
         }
         double coordinates = 0.0;
@@ -309,7 +324,7 @@ int shuffle_impl(wash_ctx *ctx, int which, uint64_t step, double p, const double
         // The streaming kernel's early flavour (permutations drawn while the copies are in flight, dense
         // serving for N > 16) costs registers and, for N > 16, three more permutation columns of shared
         // memory per thread: measured, it pays only for large populations of which most coordinates are
-        // served (N = 32, p = 1: 15.7 -> 10.4 ms, [P][N] 29.8 -> 13.3 ms; slower by 0-15 % everywhere else).
+        // served (kEarlyShare).
         args.early = ctx->N > 16 && ctx->expected_selected >= kEarlyShare * coordinates;
         if (ctx->shape.blocks_per_sm == -2) args.early = false;   // tuning override (wash_set_launch)
         if (ctx->shape.blocks_per_sm == -3) args.early = true;
