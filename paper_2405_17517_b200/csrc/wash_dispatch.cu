@@ -113,23 +113,42 @@ cudaError_t launch_philox_probe(unsigned long long n_blocks, uint64_t seed, uint
     return cudaGetLastError();
 }
 
+// Whether the resident-warp kernel takes a launch whose groups have `per_group` bytes over all models.  It does up
+// to kLoopMaxGroupBytes while at most kLoopMaxShare is expected to be selected; larger groups only where serving, which it
+// does once per four groups of a lane, weighs most against its fewer resident warps.  Its time over the one-trip
+// kernel's, 2^24 coordinates, at 0.3 / 0.5 / 1 / 2 / 5 / 8 / 12 %:
+//   64 bytes  fp32 N = 4  [N][P] .97 .89 .81 .83 .94 1.01 1.06   [P][N] .97 .87 .72 .66 .75 .87 .94   (two stacks of N = 2 alike)
+//             bf16 N = 8  [N][P] .94 .80 .65 .70 .76 .77 .87     [P][N] .97 .89 .78 .71 .91 1.11 1.23
+//   80        fp32 N = 5  [N][P] .89 .90 .89 .91 1.01 1.09 1.16  [P][N] .88 .87 .78 .73 .80 .92 1.05
+//             bf16 N = 10 [N][P] 1.08 .98 .80 .81 .81 .81 .95    [P][N] 1.20 1.08 .88 .74 .85 1.06 1.19
+//   96        bf16 N = 12 [N][P] 1.18 1.04 .85 .86 .85 .88 1.03  [P][N] 1.30 1.17 .97 .90 1.07 1.28 1.28
+//             two fp32 stacks of N = 3 [N][P] 1.01 1.02 1.02 1.07 1.10 1.14 1.19  [P][N] 1.03 .99 .90 .90 1.07 1.15 1.19
+//   128       fp32 N = 8  [P][N] 1.15 1.12 .97 .82 .92 1.05 1.21
+static bool resident_warps_pay(size_t per_group, int layout, bool bf16, bool two_stacks, float share)
+{
+    const bool np = layout == kLayoutNP, one_bf16 = bf16 && !two_stacks;
+    if (per_group <= kLoopMaxGroupBytes) return share <= kLoopMaxShare;
+    if (per_group <= 64) return share >= 0.003f && share <= (one_bf16 ? (np ? 0.12f : 0.06f) : (np ? 0.07f : 0.12f));
+    if (per_group > 96) return false;
+    if (two_stacks) return !np && share >= 0.008f && share <= 0.03f;
+    if (bf16) return np ? share >= 0.008f && share <= 0.1f : share >= 0.01f && share <= 0.04f;
+    return np ? share >= 0.004f && share <= 0.025f : share >= 0.006f && share <= 0.08f;
+}
+
 // *flush: the kernel leaves its counters in the partial-sum slots
 static cudaError_t launch_shuffle_kernel(const ShuffleArgs &args, int a_dtype, int b_dtype, int mode,
                                          const LaunchShape &shape, cudaStream_t stream, bool *supported, bool *flush)
 {
     *flush = args.stats && !args.stats_direct;
     if (mode == kModeSparse) return launch_shuffle_sparse(args, a_dtype, b_dtype, shape, stream, supported);
-    // Three streaming kernels.  A group of all models (both stacks) of at most kLoopMaxGroupBytes goes to the
-    // resident-warp kernel, whose instruction count per group is a fraction of the one-trip kernel's, unless
-    // most coordinates are expected to be served (there the one-trip kernel measured 6 % faster); larger
+    // Three streaming kernels.  Small groups of all models (both stacks) go to the resident-warp kernel, whose
+    // instruction count per group is a fraction of the one-trip kernel's (resident_warps_pay); larger
     // groups, the consensus statistic and the early flavour stay with the one-trip kernel; populations of more
     // than 16 models have a one-trip kernel of their own from kWideMinShare on, until the early flavour takes over.
     // blocks_per_sm of wash_set_launch: -4 forces the resident-warp kernel, -5 the one-trip kernel.
     const size_t elem_a = a_dtype == kDtypeF32 ? 4 : a_dtype == kDtypeBF16 ? 2 : 0, elem_b = b_dtype == kDtypeF32 ? 4 : b_dtype == kDtypeBF16 ? 2 : 0;
     const size_t per_group = static_cast<size_t>(args.pop.N) * 4 * (elem_a + elem_b);
-    bool loop = per_group <= kLoopMaxGroupBytes && args.expected_share <= kLoopMaxShare;
-    // 64-byte groups (fp32 N = 4, two fp32 stacks of N = 2, bf16 N = 8): only where serving weighs most
-    if (per_group > kLoopMaxGroupBytes && per_group <= kLoopWideGroupBytes) loop = args.expected_share >= kLoopWideShareLo && args.expected_share <= kLoopWideShareHi;
+    bool loop = resident_warps_pay(per_group, args.pop.layout, a_dtype == kDtypeBF16, b_dtype != kDtypeNone, args.expected_share);
     if (shape.blocks_per_sm == -4) loop = true;
     if (shape.blocks_per_sm == -5 || args.sq.slots || args.early || args.pop.N > 16) loop = false;
     if (loop) {

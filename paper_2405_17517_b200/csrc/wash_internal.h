@@ -136,12 +136,6 @@ enum ReduceOp { kOpEma = 0, kOpAverage = 1, kOpPapaAll = 2 };
 constexpr size_t kLoopMaxGroupBytes = 48;
 constexpr size_t kLoopFourMaxGroupBytes = 128;
 constexpr float kLoopMaxShare = 0.3f, kLoopNarrowShare = 0.0007f;
-// Groups of 49 to 64 bytes go to it for an expected selection between 0.3 % and 5 %, where serving weighs most.  Time
-// against what was launched before (the one-trip kernel; from 0.7 % to 5 % this one with two groups per lane) at p = 0.1 / 0.3 / 0.6 / 2 / 5 / 10 %: fp32 N = 4 [N][P] 1.12 0.96 0.88 0.89 0.95 1.05, [P][N] 1.08 0.98 0.80
-// 0.71 0.86 0.96; two fp32 stacks of N = 2 1.11 0.98 0.75 0.77 0.99 1.07; bf16 N = 8 1.06 0.94 0.74 0.74 0.76 0.79.
-constexpr size_t kLoopWideGroupBytes = 64;
-constexpr float kLoopWideShareLo = 0.003f, kLoopWideShareHi = 0.05f;
-
 // N > 16: below this expected selection the one-trip kernel's own serving (a single coordinate of a warp served by the
 // whole warp) is as good (N = 20 .. 64, p = 1e-3: 0.97-1.03 of the wide kernel's time; N = 17 in bf16 26.6 against 27.6 us for
 // 4.0 M coordinates); at 1 % the wide kernel takes 0.65-0.99 of its time.

@@ -434,6 +434,18 @@ def test_random_configurations_match_oracle(seed):
         c.close()
 
 
+@pytest.mark.parametrize("N,dtype,opt,layout,p", [(5, "f32", None, 1, 0.01), (6, "f32", None, 0, 0.01), (12, "bf16", None, 0, 0.03), (10, "bf16", None, 1, 0.02),
+                                                  (3, "f32", "f32", 1, 0.01), (8, "bf16", None, 0, 0.1), (4, "f32", None, 1, 0.1)])
+def test_groups_of_49_to_96_bytes_by_default(N, dtype, opt, layout, p):
+    c = Case(N, [260_003, 17, 9000], layout, dtype, opt, seed=N)
+    call = B.wash_shuffle if opt is None else B.wash_shuffle_both
+    call(c.gpu.ctx, 2, p, None, seed=6, stats=c.stats_dev)
+    want = oracle.shuffle(c.ora, c.host, p, seed=6, step=2, stack2=c.host_opt)
+    c.assert_equal("N=%d" % N)
+    assert c.gpu_stats() == tuple(want)
+    c.close()
+
+
 @pytest.mark.parametrize("captured", [False, True], ids=["stream", "graph"])
 def test_calls_that_follow_each_other_at_once(captured):
     """Kernels are launched so that one may start while the one before it ends: a chain of calls on shared stacks with
