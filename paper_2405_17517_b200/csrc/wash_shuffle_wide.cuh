@@ -119,6 +119,99 @@ __global__ void __launch_bounds__(64, 6) shuffle_wide_kernel(const __grid_consta
     publish_block_stats(a.stats, a.stats_direct ? nullptr : a.stat_slots, selected, moved);
 }
 
+// [P][N] with a group of all models of kWideSplitBytes and more: two threads to a group, the block's selected
+// coordinates in one list shared evenly by its warps.  Six blocks of 35 KB hold twice the warps that way,
+// each with half the copies, draws and moves.  N = 32, fp32, 2^23 coordinates, p = 0.03 / 0.1 / 0.25: 197 / 246 / 410 us by the kernel
+// above, 192 / 233 / 404; N = 24, bf16 + fp32, p = 0.25 436 / 386; N = 64, fp32, p = 0.1 632 / 542.  Smaller groups (N = 20, fp32, p = 0.1
+// 145 / 165 us) and [N][P] (N = 20 200 / 202, N = 17 bf16 103 / 162) lose more by the block's barriers.
+constexpr size_t kWideSplitBytes = 512;
+constexpr uint32_t kWideRound = 16;   // coordinates of a warp's round
+template <class TA, class TB>
+__global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_constant__ ShuffleArgs a)
+{
+    let_next_start();
+    await_previous();
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ uint32_t s_count;
+    constexpr int LAYOUT = kLayoutPN;
+    constexpr bool kHasB = TB::kCode != kDtypeNone;
+    const int n_models = a.pop.N;
+    const uint32_t groups = blockDim.x / 2u, lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    // the images of the two stacks, the block's list {coordinate within its tensor, tensor} and where it lies (group * 4 +
+    // coordinate slot), kWideRound permutations per warp
+    const uint32_t group_elems = pn_group_elems(n_models, a.pn_pad);
+    unsigned char *image_a = smem_raw, *image_b = image_a + group_elems * groups * TA::kBytes;
+    uint2 *s_key = reinterpret_cast<uint2 *>(image_b + (kHasB ? group_elems * groups * TB::kBytes : 0));
+    uint32_t *s_perm = reinterpret_cast<uint32_t *>(s_key + 4 * groups) + warp * kWideRound * wide_pitch(n_models);
+    uint8_t *s_entry = reinterpret_cast<uint8_t *>(reinterpret_cast<uint32_t *>(s_key + 4 * groups) + warps * kWideRound * wide_pitch(n_models));
+
+    const uint64_t g_block = a.group_lo + static_cast<uint64_t>(blockIdx.x) * groups;
+    const uint32_t in_block = static_cast<uint32_t>(min(static_cast<uint64_t>(groups), a.group_hi - g_block));
+    async_fetch<TA, LAYOUT>(smem_addr(image_a), a.a, a.pop, g_block, in_block, n_models, a.pn_pad);
+    if constexpr (kHasB) async_fetch<TB, LAYOUT>(smem_addr(image_b), a.b, a.pop, g_block, in_block, n_models, a.pn_pad);
+    if (threadIdx.x == 0) s_count = 0;
+    __syncthreads();
+
+    uint32_t selected = 0, moved = 0;
+    if (threadIdx.x < in_block) {
+        const GroupInfo gi = find_group(a.pop, static_cast<uint32_t>(g_block + threadIdx.x), a.status);
+        if (gi.thr != 0 && gi.valid != 0) {
+            uint32_t m = 0xFu;   // a threshold of 2^32 selects whatever the word is
+            if ((gi.thr >> 32) == 0) {
+                const Philox4 w = philox4x32_10(gi.cgroup, gi.tensor_id, a.step_lo, a.step_hi8, a.keys);
+                const uint32_t thr_lo = static_cast<uint32_t>(gi.thr);
+                m = (w.x < thr_lo ? 1u : 0u) | (w.y < thr_lo ? 2u : 0u) | (w.z < thr_lo ? 4u : 0u) | (w.w < thr_lo ? 8u : 0u);
+            }
+            m &= (1u << gi.valid) - 1u;   // coordinates beyond the tensor's end do not exist
+            if (m) {
+                uint32_t pos = atomicAdd(&s_count, static_cast<uint32_t>(__popc(m)));
+                for (; m; m &= m - 1u, ++pos) {
+                    const uint32_t c = static_cast<uint32_t>(__ffs(m) - 1);
+                    s_key[pos] = make_uint2(4u * gi.cgroup + c, gi.tensor_id);
+                    s_entry[pos] = static_cast<uint8_t>(4u * threadIdx.x + c);
+                }
+            }
+        }
+    }
+    __syncthreads();
+    const uint32_t total = s_count;
+    // a round gives every warp up to kWideRound coordinates, as evenly as they go
+    uint32_t mine = 0, count = 0;
+    auto deal = [&](uint32_t first) {
+        const uint32_t left = total - first, share = min(kWideRound, (left + warps - 1u) / warps);
+        mine = first + warp * share;
+        count = mine < total ? min(share, total - mine) : 0u;
+        if (count) {
+            const uint2 key = s_key[mine + min(lane, count - 1u)];
+            draw_permutations_by_warp(s_perm, n_models, count, key.x, key.y, a.step_lo, a.step_hi8, a.keys);
+        }
+        return share * warps;
+    };
+    // the first round's permutations are drawn while the copies are in flight
+    uint32_t step = total ? deal(0) : 0u;
+    cp_async_wait_all();
+    __syncthreads();   // a group's bytes were copied by threads of other warps
+    for (uint32_t first = 0; first < total; first += step) {
+        if (first) step = deal(first);
+        if (lane < count) ++selected;
+        // a lane per (coordinate, model) pair, the models of a coordinate side by side
+        const uint32_t pairs = count * static_cast<uint32_t>(n_models);
+        for (uint32_t i = lane; i < pairs; i += 32) {
+            const uint32_t l = (i * a.pair_inverse) >> 20, n = i - l * static_cast<uint32_t>(n_models);
+            const uint32_t src = reinterpret_cast<const uint8_t *>(s_perm + l * wide_pitch(n_models))[n];
+            if (src == n) continue;
+            const uint32_t entry = s_entry[mine + l], g = entry >> 2, c = entry & 3u;
+            const long long out = elem_index<LAYOUT>(a.pop, static_cast<int>(n), 4ll * static_cast<long long>(g_block + g) + c);
+            const uint32_t from = g * group_elems + c * static_cast<uint32_t>(n_models) + src;
+            TA::store_elem(a.a, out, TA::load_elem(image_a, from));
+            if constexpr (kHasB) TB::store_elem(a.b, out, TB::load_elem(image_b, from));
+            ++moved;
+        }
+        __syncwarp();   // the permutations are overwritten by the next round
+    }
+    publish_block_stats(a.stats, a.stats_direct ? nullptr : a.stat_slots, selected, moved);
+}
+
 template <class TA, class TB>
 cudaError_t launch_shuffle_wide_typed(const ShuffleArgs &call, const LaunchShape &shape, cudaStream_t stream)
 {
@@ -127,6 +220,20 @@ cudaError_t launch_shuffle_wide_typed(const ShuffleArgs &call, const LaunchShape
     args.pair_inverse = ((1u << 20) + static_cast<uint32_t>(args.pop.N) - 1u) / static_cast<uint32_t>(args.pop.N);
     const size_t group_elems = 4 * static_cast<size_t>(args.pop.N) + (args.pop.layout == kLayoutPN ? args.pn_pad : 0);
     const size_t per_thread = group_elems * (TA::kBytes + (kHasB ? TB::kBytes : 0)) + 4 + 4 * wide_pitch(args.pop.N);
+    if (args.pop.layout == kLayoutPN && !args.sq.slots && 4 * static_cast<size_t>(args.pop.N) * (TA::kBytes + TB::kBytes) >= kWideSplitBytes) {
+        // the images, the list (keys and places of every coordinate) and kWideRound permutations per warp
+        const size_t per_group = group_elems * (TA::kBytes + (kHasB ? TB::kBytes : 0)) + 4 * 8 + 4 + 4 * wide_pitch(args.pop.N);
+        const uint32_t groups = per_group * 64 > 44 * 1024 ? 32 : 64;   // five blocks and more on an SM
+        const size_t smem = (per_group * groups + 15) & ~static_cast<size_t>(15);
+        KernelFit fit;
+        cudaError_t err = kernel_fit(reinterpret_cast<const void *>(shuffle_wide_pn_kernel<TA, TB>), 2 * static_cast<int>(groups), smem, &fit);
+        if (err != cudaSuccess) return err;
+        if (fit.occupancy < 1) return cudaErrorLaunchOutOfResources;
+        const uint64_t grid = (static_cast<uint64_t>(args.group_hi - args.group_lo) + groups - 1) / groups;
+        if (grid == 0) return cudaSuccess;
+        if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+        return launch_chained(shuffle_wide_pn_kernel<TA, TB>, static_cast<unsigned>(grid), 2 * groups, smem, stream, args);
+    }
     int threads = shape.threads > 0 ? (shape.threads >= 64 ? 64 : 32) : 64;
     while (threads > 32 && per_thread * threads > 44 * 1024) threads >>= 1;   // five blocks and more on an SM
     const size_t smem = (per_thread * threads + 15) & ~static_cast<size_t>(15);

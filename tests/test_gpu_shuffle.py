@@ -194,7 +194,7 @@ def test_resident_warp_kernel_serves_a_tiles_groups_together(N, numel, p, dtype,
 @pytest.mark.parametrize("layout", [0, 1])
 @pytest.mark.parametrize("N,numel,p,dtype,opt", [
     (17, [30_001], 0.01, "f32", None), (18, [127, 1, 130, 4000], 0.1, "bf16", None), (20, [50_003], 0.25, "bf16", "f32"),
-    (32, [40_009], 0.1, "f32", None), (33, [255, 9000], 0.2, "f32", None), (63, [20_001], 0.05, "f32", "bf16"), (64, [12_345], 0.28, "f32", "f32")])
+    (32, [40_009], 0.1, "f32", None), (32, [253, 4, 3000], 0.65, "f32", None), (24, [30_011], 0.03, "bf16", "f32"), (33, [255, 9000], 0.2, "f32", None), (63, [20_001], 0.05, "f32", "bf16"), (64, [12_345], 0.28, "f32", "f32")])
 def test_wide_population_kernel(N, numel, p, dtype, opt, layout):
     """The streaming kernel of N > 16: permutations of 17 to 64 entries (last Philox block full and partly used), rounds
     of up to 32 and several rounds per warp, few and many coordinates in [N][P] (a lane per pair / per coordinate)."""
