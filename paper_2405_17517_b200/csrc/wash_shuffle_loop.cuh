@@ -20,6 +20,12 @@
 // p = 1e-2 390 -> 245 us, 1e-3 206 -> 203; 2^25 coordinates: p = 0.1 134 -> 95, 0.02 125 -> 71; one model
 // step of N = 3, 2^20 coordinates 12.3 -> 8.3.
 //
+// As issue slots bound it, the tile kernel is also compiled for each population of 2 to 5 models, whose copies,
+// swap chains and row addresses then need no loop control or multiplications (run-time N -> compiled in: N = 2,
+// 2^27 coordinates p = 1e-2 236 -> 216 us, 1e-3 205 -> 195; 2^25 coordinates: N = 2 [P][N] p = 0.1 94.0 -> 81.0, N = 3
+// p = 1e-2 85.4 -> 82.4 (bf16 78.6 -> 70.4), N = 4 bf16 88.9 -> 79.9, N = 5 144.7 -> 137.9; N = 3, 2^20 7.49 -> 7.07).
+// Larger populations move more bytes for the same control.
+//
 // An image of a stage is the one-trip kernel's block image with T = 32 (the block is one warp,
 // so every helper of that kernel -- copies, serving, padding rule -- is used as it is).
 #pragma once
@@ -119,15 +125,18 @@ __device__ __forceinline__ uint32_t list_selected(uint16_t *list, uint32_t sel)
     return total;
 }
 
-template <class TA, class TB, int LAYOUT, int G>
+// kN: the population size where it is compiled in (the helpers read it from the arguments: the assumption reaches
+// them), 0 = run-time N.
+template <class TA, class TB, int LAYOUT, int G, int kN>
 __global__ void __launch_bounds__(32, G == 2 ? 32 : 28) shuffle_loop_kernel(const __grid_constant__ ShuffleArgs a)
 {
+    if constexpr (kN != 0) __builtin_assume(a.pop.N == kN);
     let_next_start();
     await_previous();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr bool kHasB = TB::kCode != kDtypeNone;
     constexpr uint32_t T_ = 32;   // the launch has one warp per block
-    const int n_models = a.pop.N;
+    const int n_models = kN ? kN : a.pop.N;
     const uint32_t lane = threadIdx.x;
     const size_t group_elems = LAYOUT == kLayoutPN ? pn_group_elems(n_models, a.pn_pad) : 4u * static_cast<size_t>(n_models);
     const uint32_t a_bytes = static_cast<uint32_t>(group_elems * T_ * TA::kBytes);
@@ -246,7 +255,7 @@ __global__ void __launch_bounds__(32, G == 2 ? 32 : 28) shuffle_loop_kernel(cons
     publish_warp_stats(a.stats, a.stat_slots, selected, moved);
 }
 
-template <class TA, class TB, int G>
+template <class TA, class TB, int G, int kN>
 cudaError_t launch_shuffle_loop_tiles(const ShuffleArgs &args, const LaunchShape &shape, cudaStream_t stream)
 {
     constexpr bool kHasB = TB::kCode != kDtypeNone;
@@ -254,7 +263,7 @@ cudaError_t launch_shuffle_loop_tiles(const ShuffleArgs &args, const LaunchShape
     const size_t image = group_elems * (TA::kBytes + (kHasB ? TB::kBytes : 0)) * 32;
     const size_t smem = (2 * G * image + 2 * 32 * 4 * G + 15) & ~static_cast<size_t>(15);
     const bool np = args.pop.layout == kLayoutNP;
-    auto kernel = np ? shuffle_loop_kernel<TA, TB, kLayoutNP, G> : shuffle_loop_kernel<TA, TB, kLayoutPN, G>;
+    auto kernel = np ? shuffle_loop_kernel<TA, TB, kLayoutNP, G, kN> : shuffle_loop_kernel<TA, TB, kLayoutPN, G, kN>;
     KernelFit fit;
     cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), 32, smem, &fit);
     if (err != cudaSuccess) return err;
@@ -277,8 +286,15 @@ cudaError_t launch_shuffle_loop_typed(const ShuffleArgs &args, const LaunchShape
     // costs resident warps and was slower everywhere (p = 1e-2 334 us with two groups).
     // (A forced launch may bring groups of any size: beyond kLoopFourMaxGroupBytes four of them leave too few warps.)
     const size_t per_group = static_cast<size_t>(args.pop.N) * 4 * (TA::kBytes + TB::kBytes);
-    if (args.expected_share < kLoopNarrowShare || per_group > kLoopFourMaxGroupBytes) return launch_shuffle_loop_tiles<TA, TB, 2>(args, shape, stream);
-    return launch_shuffle_loop_tiles<TA, TB, 4>(args, shape, stream);
+    if (args.expected_share < kLoopNarrowShare || per_group > kLoopFourMaxGroupBytes)
+        return launch_shuffle_loop_tiles<TA, TB, 2, 0>(args, shape, stream);
+    switch (args.pop.N) {
+    case 2: return launch_shuffle_loop_tiles<TA, TB, 4, 2>(args, shape, stream);
+    case 3: return launch_shuffle_loop_tiles<TA, TB, 4, 3>(args, shape, stream);
+    case 4: return launch_shuffle_loop_tiles<TA, TB, 4, 4>(args, shape, stream);
+    case 5: return launch_shuffle_loop_tiles<TA, TB, 4, 5>(args, shape, stream);
+    default: return launch_shuffle_loop_tiles<TA, TB, 4, 0>(args, shape, stream);
+    }
 }
 
 inline cudaError_t launch_shuffle_loop(const ShuffleArgs &args, int a_dtype, int b_dtype, const LaunchShape &shape,

@@ -243,6 +243,24 @@ def test_last_layer_untouched_and_schedules_agree_with_oracle():
     c.close()
 
 
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("dtype,opt", [("f32", None), ("bf16", None), ("bf16", "f32")])
+@pytest.mark.parametrize("N", [2, 3, 4, 5, 6])
+def test_resident_warp_kernel_for_each_compiled_population(N, dtype, opt, layout):
+    """Populations of 2 to 5 models have kernels of their own and 6 the one that reads N at run time: rare and common
+    selection, a tensor selected in full, a ragged last tile."""
+    numel = [150_001, 3, 127, 40_000]
+    c = Case(N, numel, layout, dtype, opt, seed=N)
+    B.wash_set_launch(c.gpu.ctx, 0, -4)
+    p = [0.02, 0.5, 1.0, 0.4]
+    call = B.wash_shuffle if opt is None else B.wash_shuffle_both
+    call(c.gpu.ctx, 3, 0.5, p, seed=8, stats=c.stats_dev)
+    want = oracle.shuffle(c.ora, c.host, p, seed=8, step=3, stack2=c.host_opt)
+    c.assert_equal("N=%d layout=%d" % (N, layout))
+    assert c.gpu_stats() == tuple(want)
+    c.close()
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("N", [2, 4])
 def test_resident_warp_kernel_with_a_padded_coordinate_major_image(N, dtype):
