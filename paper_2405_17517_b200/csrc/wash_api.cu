@@ -253,6 +253,16 @@ int sync_table(wash_ctx *ctx, double p, const double *p_layer, cudaStream_t stre
     return WASH_OK;
 }
 
+// [P][N] with the distance to the consensus: every thread reads its whole group from the shared-memory image, so an
+// even population is padded against bank conflicts whatever is selected (ResNet-18, fp32: N = 12 566 -> 232 us, N = 32
+// 2896 -> 711; N = 4 and 2^25 coordinates 531 -> 142, some of it from the compiled N).  Two models' groups of two vectors
+// conflict two ways only and the padding would cost half as many bytes again (fp32 with
+// momentum, 2^25 coordinates: 209 us without, 239 with).
+uint32_t sq_pad(const wash_ctx *ctx)
+{
+    return ctx->layout == WASH_LAYOUT_PN && ctx->N > 2 && !(ctx->N & 1) ? 4u : 0u;
+}
+
 int ensure_table(wash_ctx *ctx, cudaStream_t stream)
 {
     if (ctx->seg_uploaded) return WASH_OK;
@@ -332,6 +342,7 @@ int shuffle_impl(wash_ctx *ctx, int which, uint64_t step, double p, const double
             mode = WASH_MODE_STREAM;
             args.stats_direct = false;
             args.sq = *sq;
+            args.pn_pad = sq_pad(ctx);
         }
         if (mirror_a) {   // moved values go to host memory as well: the kernel that touches nothing else
             mode = WASH_MODE_SPARSE;
@@ -622,6 +633,7 @@ int wash_consensus_sq(wash_ctx *ctx, int32_t stack, int32_t tensor_lo, int32_t t
     args.sq.inv_n = 1.0 / static_cast<double>(ctx->N);
     args.sq.slots = ctx->sq_slots_dev;
     args.measure_only = true;
+    args.pn_pad = sq_pad(ctx);
     bool supported = false;
     cudaError_t err = wash::launch_shuffle(args, ctx->stack_dtype[stack], wash::kDtypeNone, wash::kModeStream, ctx->shape, stream, &supported);
     if (err == cudaSuccess && supported) err = wash::launch_sq_flush(args.sq, ctx->N, dev_sq_out, stream);

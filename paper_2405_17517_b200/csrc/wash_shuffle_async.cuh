@@ -568,14 +568,49 @@ __device__ __forceinline__ void image_group(const unsigned char *image, int n_mo
 // before it serve.  Called by all threads of the block; `exists`: the thread has a group in this
 // tile.  WHOLE: every lane of the warp has a whole group of one and the same range (the usual
 // case, decided by the caller with one vote), so nothing is predicated per coordinate.
-template <class T, int LAYOUT, bool WHOLE>
+// kN: the population size where it is compiled in (2 to 8), else 0.  Issue slots, conversions to binary64 and the
+// warp sums bound this part, not memory.  With a compiled N the group is read once, as vectors in both layouts, each
+// value is converted once and taken through mean and deviation coordinate by coordinate, and all models' sums
+// are reduced over the warp together: at each level a lane hands half of its sums to its partner and keeps the others, so
+// N = 5 takes 8 exchanges of a binary64 where model after model takes 25, and a lane ends with one model.  Measured with
+// the shuffle (run-time N -> compiled): ResNet-18 N = 5 p = 1e-3 75.9 -> 60.9 us (with momentum 85.3 -> 79.0), N = 6 84.2 ->
+// 66.4, N = 8 103 -> 81; 2^25 coordinates, p = 1e-2: N = 2 135 -> 103, N = 3 235 -> 188; [P][N] ResNet-18 N = 5 119 -> 102, N = 8 706 ->
+// 113 (with the image's padding below).
+template <class T, int LAYOUT, bool WHOLE, int kN>
 __device__ __forceinline__ void consensus_warp(const ShuffleArgs &a, const unsigned char *image, int valid, uint32_t r1,
                                                uint32_t r_lo, uint32_t r_hi)
 {
     const int n_models = a.pop.N;
     const uint32_t lane = threadIdx.x & 31u;
+    constexpr int kOwn = kN ? kN : 1;
+    double own[kOwn] = {};   // the thread's sum for each model
     double mean[4] = {0.0, 0.0, 0.0, 0.0};
-    if (WHOLE || r1) {
+    if constexpr (kN != 0) {
+        if (WHOLE || r1) {
+            typename T::vec v[kOwn];   // [N][P]: four coordinates of a model; [P][N]: the group's values as they lie
+#pragma unroll
+            for (int k = 0; k < kOwn; ++k)
+                v[k] = reinterpret_cast<const typename T::vec *>(image)[LAYOUT == kLayoutNP ? k * blockDim.x + threadIdx.x : threadIdx.x * (pn_group_elems(kN, a.pn_pad) / 4u) + k];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                double x[kOwn], sum = 0.0;
+#pragma unroll
+                for (int n = 0; n < kOwn; ++n) {
+                    x[n] = static_cast<double>(T::to_float(LAYOUT == kLayoutNP ? T::get(v[n], c) : T::get(v[(c * kOwn + n) / 4], (c * kOwn + n) % 4)));
+                    sum += x[n];
+                }
+                const double q = sum * a.sq.inv_n;   // sum / N: the reciprocal's product, corrected by its remainder
+                const double m = fma(fma(-q, static_cast<double>(kOwn), sum), a.sq.inv_n, q);
+                if (WHOLE || c < valid) {   // padding beyond the tensor's end holds no coordinate
+#pragma unroll
+                    for (int n = 0; n < kOwn; ++n) {
+                        const double d = x[n] - m;
+                        own[n] = fma(d, d, own[n]);
+                    }
+                }
+            }
+        }
+    } else if (WHOLE || r1) {
         float x[4];
         for (int n = 0; n < n_models; ++n) {
             image_group<T, LAYOUT>(image, n_models, a.pn_pad, threadIdx.x, n, x);
@@ -592,6 +627,34 @@ __device__ __forceinline__ void consensus_warp(const ShuffleArgs &a, const unsig
     const uint32_t slot = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) % kSqSlots;
     for (uint32_t r = r_lo; r <= r_hi; ++r) {   // one trip unless the warp's groups lie in several ranges
         double *table = a.sq.slots + (static_cast<size_t>(slot) * a.sq.n_ranges + (r - 1)) * n_models;
+        if constexpr (kN != 0) {
+            double s[kN];
+#pragma unroll
+            for (int n = 0; n < kN; ++n) s[n] = WHOLE || r1 == r ? own[n] : 0.0;
+            int first = 0, count = kN;   // the lane holds the sums of models [first, first + count)
+            int width = kN;              // ... in s[0 .. width), the same on every lane
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                if (width > 1) {
+                    const int half = (width + 1) / 2;
+                    const bool upper = (lane & static_cast<uint32_t>(off)) != 0;
+#pragma unroll
+                    for (int i = 0; i < kN; ++i)
+                        if (i < half) {
+                            const double other = i + half < width ? s[i + half < kN ? i + half : 0] : 0.0;
+                            s[i] = (upper ? other : s[i]) + __shfl_xor_sync(0xFFFFFFFFu, upper ? s[i] : other, off);
+                        }
+                    first += upper ? half : 0;
+                    count = upper ? count - half : min(count, half);
+                    width = half;
+                } else {
+                    s[0] += __shfl_xor_sync(0xFFFFFFFFu, s[0], off);
+                }
+            }
+            constexpr uint32_t kCopies = kN > 4 ? 4u : (kN > 2 ? 8u : 16u);   // lanes that end with the same model
+            if (count > 0 && (lane & (kCopies - 1u)) == 0 && s[0] != 0.0) atomicAdd(table + first, s[0]);
+            continue;
+        }
         double keep = 0.0;   // lane l keeps the warp's sum of model l (mod 32)
         for (int n = 0; n < n_models; ++n) {
             double s = 0.0;
@@ -617,7 +680,7 @@ __device__ __forceinline__ void consensus_warp(const ShuffleArgs &a, const unsig
     }
 }
 
-template <class T, int LAYOUT>
+template <class T, int LAYOUT, int kN>
 __device__ __forceinline__ void consensus_tile(const ShuffleArgs &a, const unsigned char *image, const GroupInfo &gi, bool exists)
 {
     // this lane's range, counted from 1 (0: its group lies in none, or does not exist)
@@ -629,8 +692,8 @@ __device__ __forceinline__ void consensus_tile(const ShuffleArgs &a, const unsig
     const uint32_t r_hi = __reduce_max_sync(0xFFFFFFFFu, r1);
     if (r_hi == 0) return;
     const uint32_t r_lo = __reduce_min_sync(0xFFFFFFFFu, r1 ? r1 : 0xFFFFFFFFu);
-    if (__all_sync(0xFFFFFFFFu, r1 == r_hi && gi.valid == 4)) consensus_warp<T, LAYOUT, true>(a, image, 4, r1, r_hi, r_hi);
-    else consensus_warp<T, LAYOUT, false>(a, image, exists ? gi.valid : 0, r1, r_lo, r_hi);
+    if (__all_sync(0xFFFFFFFFu, r1 == r_hi && gi.valid == 4)) consensus_warp<T, LAYOUT, true, kN>(a, image, 4, r1, r_hi, r_hi);
+    else consensus_warp<T, LAYOUT, false, kN>(a, image, exists ? gi.valid : 0, r1, r_lo, r_hi);
 }
 
 #ifndef WASH_SERVING_ONLY   // a translation unit that only wants the copy and serving helpers above
@@ -641,14 +704,17 @@ __device__ __forceinline__ void consensus_tile(const ShuffleArgs &a, const unsig
 // the integer work of a launch that selects much hides behind the copies' flight instead of holding
 // the block's shared memory after them; it keeps a plan in registers across the wait, which the
 // lean flavour (48 registers, as many resident blocks as the shared memory allows) cannot afford.
-template <class TA, class TB, int LAYOUT, int G, bool STAT, bool EARLY>
-__global__ void __launch_bounds__(256, EARLY ? 3 : 5) shuffle_async_kernel(const __grid_constant__ ShuffleArgs a)
+// kN: the population size where it is compiled in (STAT, N = 2 .. 8), 0 = run-time N.  From N = 7 on the statistic does not
+// fit 48 registers (with them N = 8 takes 89 us for ResNet-18, with 64 81; N = 6 66 and 70).
+template <class TA, class TB, int LAYOUT, int G, bool STAT, bool EARLY, int kN>
+__global__ void __launch_bounds__(256, EARLY ? 3 : (kN > 6 ? 4 : 5)) shuffle_async_kernel(const __grid_constant__ ShuffleArgs a)
 {
+    if constexpr (kN != 0) __builtin_assume(a.pop.N == kN);
     let_next_start();
     await_previous();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr bool kHasB = TB::kCode != kDtypeNone;
-    const int n_models = a.pop.N;
+    const int n_models = kN ? kN : a.pop.N;
     const uint32_t T_ = blockDim.x;
     // G pairs of images of the two stacks, then the warps' lists, then the permutation columns
     const size_t group_elems = LAYOUT == kLayoutPN ? pn_group_elems(n_models, a.pn_pad) : 4u * static_cast<size_t>(n_models);
@@ -716,7 +782,7 @@ __global__ void __launch_bounds__(256, EARLY ? 3 : 5) shuffle_async_kernel(const
         if constexpr (STAT) {
 #pragma unroll
             for (int i = 0; i < G; ++i)
-                consensus_tile<TA, LAYOUT>(a, smem_raw + i * (a_bytes + b_bytes), gi[i], threadIdx.x < in_tile[i]);
+                consensus_tile<TA, LAYOUT, kN>(a, smem_raw + i * (a_bytes + b_bytes), gi[i], threadIdx.x < in_tile[i]);
         }
 #pragma unroll
         for (int i = 0; i < G; ++i) {
@@ -728,7 +794,7 @@ __global__ void __launch_bounds__(256, EARLY ? 3 : 5) shuffle_async_kernel(const
     publish_block_stats(a.stats, a.stats_direct ? nullptr : a.stat_slots, selected, moved);
 }
 
-template <class TA, class TB, int G>
+template <class TA, class TB, int G, int kN>
 cudaError_t launch_shuffle_async_tiles(const ShuffleArgs &args, const LaunchShape &shape, cudaStream_t stream)
 {
     constexpr bool kHasB = TB::kCode != kDtypeNone;
@@ -746,9 +812,15 @@ cudaError_t launch_shuffle_async_tiles(const ShuffleArgs &args, const LaunchShap
     const size_t smem = (per_thread * threads + 15) & ~static_cast<size_t>(15);
     const bool np = args.pop.layout == kLayoutNP;
     constexpr bool kEarlyBuilt = G == 1;   // the early flavour exists for one group per thread (what large populations get)
-    auto kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, false, false> : shuffle_async_kernel<TA, TB, kLayoutPN, G, false, false>;
-    if (args.sq.slots) kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, true, false> : shuffle_async_kernel<TA, TB, kLayoutPN, G, true, false>;
-    else if (args.early && kEarlyBuilt) kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, 1, false, true> : shuffle_async_kernel<TA, TB, kLayoutPN, 1, false, true>;
+    using Kernel = void (*)(ShuffleArgs);
+    Kernel kernel;
+    if constexpr (kN != 0) {   // built with the statistics only
+        kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, true, false, kN> : shuffle_async_kernel<TA, TB, kLayoutPN, G, true, false, kN>;
+    } else {
+        kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, false, false, 0> : shuffle_async_kernel<TA, TB, kLayoutPN, G, false, false, 0>;
+        if (args.sq.slots) kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, true, false, 0> : shuffle_async_kernel<TA, TB, kLayoutPN, G, true, false, 0>;
+        else if (args.early && kEarlyBuilt) kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, 1, false, true, 0> : shuffle_async_kernel<TA, TB, kLayoutPN, 1, false, true, 0>;
+    }
     KernelFit fit;
     cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), threads, smem, &fit);
     if (err != cudaSuccess) return err;
@@ -767,12 +839,23 @@ cudaError_t launch_shuffle_async_typed(const ShuffleArgs &args, const LaunchShap
     // takes two groups (measured on 2^27 coordinates, p = 1e-3: N = 4 0.84 -> 0.95 of the copy
     // bandwidth, N = 2 0.48 -> 0.56; four groups were slower than two for every N).
     // blocks_per_sm of wash_set_launch, when 1 or 2, overrides.
-    constexpr bool kHasB = TB::kCode != kDtypeNone;
-    const size_t per_group = static_cast<size_t>(args.pop.N) * (TA::kBytes * 4 + (kHasB ? TB::kBytes * 4 : 0));
-    int tiles = per_group <= 64 ? 2 : 1;
+    constexpr size_t kModelGroup = TA::kBytes * 4 + (TB::kCode != kDtypeNone ? TB::kBytes * 4 : 0);
+    int tiles = args.pop.N * kModelGroup <= 64 ? 2 : 1;
     if (shape.blocks_per_sm == 1 || shape.blocks_per_sm == 2) tiles = shape.blocks_per_sm;
-    if (tiles == 2) return launch_shuffle_async_tiles<TA, TB, 2>(args, shape, stream);
-    return launch_shuffle_async_tiles<TA, TB, 1>(args, shape, stream);
+    else if (args.sq.slots) {   // populations that have a kernel of their own
+        switch (args.pop.N) {
+        case 2: return launch_shuffle_async_tiles<TA, TB, 2 * kModelGroup <= 64 ? 2 : 1, 2>(args, shape, stream);
+        case 3: return launch_shuffle_async_tiles<TA, TB, 3 * kModelGroup <= 64 ? 2 : 1, 3>(args, shape, stream);
+        case 4: return launch_shuffle_async_tiles<TA, TB, 4 * kModelGroup <= 64 ? 2 : 1, 4>(args, shape, stream);
+        case 5: return launch_shuffle_async_tiles<TA, TB, 5 * kModelGroup <= 64 ? 2 : 1, 5>(args, shape, stream);
+        case 6: return launch_shuffle_async_tiles<TA, TB, 6 * kModelGroup <= 64 ? 2 : 1, 6>(args, shape, stream);
+        case 7: return launch_shuffle_async_tiles<TA, TB, 7 * kModelGroup <= 64 ? 2 : 1, 7>(args, shape, stream);
+        case 8: return launch_shuffle_async_tiles<TA, TB, 8 * kModelGroup <= 64 ? 2 : 1, 8>(args, shape, stream);
+        default: break;
+        }
+    }
+    if (tiles == 2) return launch_shuffle_async_tiles<TA, TB, 2, 0>(args, shape, stream);
+    return launch_shuffle_async_tiles<TA, TB, 1, 0>(args, shape, stream);
 }
 
 inline cudaError_t launch_shuffle_async(const ShuffleArgs &args, int a_dtype, int b_dtype, const LaunchShape &shape,

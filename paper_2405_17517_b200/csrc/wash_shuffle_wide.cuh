@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(64, 6) shuffle_wide_kernel(const __grid_consta
     cp_async_wait_all();
     if (LAYOUT == kLayoutPN) __syncthreads();   // a group's bytes were copied by threads of other warps
     else __syncwarp();
-    if constexpr (STAT) consensus_tile<TA, LAYOUT>(a, image_a, gi, threadIdx.x < in_block);
+    if constexpr (STAT) consensus_tile<TA, LAYOUT, 0>(a, image_a, gi, threadIdx.x < in_block);
 
     for (uint32_t first = 0; first < total; first += 32) {
         const uint32_t count = min(32u, total - first);

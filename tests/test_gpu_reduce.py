@@ -150,6 +150,31 @@ def test_consensus_distance(N, dtype, layout):
 
 
 @pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("dtype,opt", [("f32", None), ("bf16", None), ("bf16", "f32"), ("f32", "f32")])
+@pytest.mark.parametrize("N", [2, 3, 4, 5, 6, 7, 8, 9])
+def test_consensus_distance_for_each_compiled_population(N, dtype, opt, layout):
+    """Populations of 2 to 8 models have kernels of their own (9: the run-time one): ranges that meet inside a warp,
+    tensors that end inside a group, one range over many warps.  Sums of at most 4 * 10^4 binary64 terms in
+    another order differ by less than 4e4 * 2^-53 < 1e-11 relative."""
+    numel = [513, 2, 40_001, 1, 9, 127, 5000]
+    bounds = [0, 1, 3, 6, 7]
+    p = [0.2, 1.0, 0.01, 0.0, 0.5, 0.9, 0.3]
+    c = Case(N, numel, layout, dtype, opt, seed=N)
+    want = np.stack([oracle.consensus_sq(c.ora, c.host, lo, hi) for lo, hi in zip(bounds[:-1], bounds[1:])])
+    out = torch.zeros(len(bounds) - 1, N, dtype=torch.float64, device="cuda")
+    B.wash_shuffle_consensus(c.gpu.ctx, B.WASH_STACK_PARAMS if opt is None else B.WASH_STACK_BOTH, 4, 0.0, p, seed=2, stats=c.stats_dev, tensor_bounds=bounds, dev_sq_out=out)
+    stats = oracle.shuffle(c.ora, c.host, p, seed=2, step=4, stack2=c.host_opt)
+    c.assert_equal("N=%d layout=%d" % (N, layout))
+    assert np.allclose(out.cpu().numpy(), want, rtol=1e-11, atol=0)
+    assert c.gpu_stats() == tuple(stats)
+    alone = torch.zeros(N, dtype=torch.float64, device="cuda")
+    before = oracle.consensus_sq(c.ora, c.host, 1, 5)
+    B.wash_consensus_sq(c.gpu.ctx, B.WASH_STACK_PARAMS, 1, 5, alone)
+    assert np.allclose(alone.cpu().numpy(), before, rtol=1e-11, atol=0)
+    c.close()
+
+
+@pytest.mark.parametrize("layout", [0, 1])
 @pytest.mark.parametrize("N,dtype,opt_dtype,stacks", [(5, "f32", "f32", 2), (8, "bf16", "f32", 2), (13, "f32", None, 0),
                                                      (3, "f32", "bf16", 1), (40, "f32", None, 0), (2, "bf16", None, 0)])
 def test_consensus_distance_inside_the_streaming_shuffle(N, dtype, opt_dtype, stacks, layout):
