@@ -24,8 +24,8 @@
 //
 // The plan is bound by the integer pipes (a Philox block per 4 coordinates), send and receive by the
 // latency of a few dependent steps.  Five ResNet-50 models (25.6 M coordinates, 1.3e5 selected), parameters and
-// momentum: plan 32 -> 27 us, send 15, receive 8; a step 64.5 -> 49.7 us against a queue per warp, served 32 at a time, and
-// mask words fetched one tile after the other; N = 64, 3e5 coordinates at p = 0.05 70.7 -> 42.2 us.
+// momentum, launched back to back: plan 32 -> 21 us, a step 63.5 -> 45.1 us against a queue per warp, served 32 at a time, with
+// mask words fetched one tile after the other and kernels that do not overlap; N = 32, 5.6e5 selected 205 -> 167 us.
 #include "wash_device.cuh"
 #include "wash_launch.cuh"
 #include "wash_warp_tiles.cuh"
@@ -82,14 +82,20 @@ __device__ __forceinline__ void block_range(const ExchangeArgs &a, uint32_t *t0,
 }
 
 // The plan's block queue, as the sparse shuffle's: the coordinates its warps find, in any order (the
-// counts do not depend on it), drawn a thread each when the range is done or the queue full.
+// counts do not depend on it), drawn a thread each when a piece of the range is done or the queue full.
 constexpr uint32_t kPlanQueue = 1024;
+// The mask words of up to so many warp tiles stay in shared memory until their selected coordinates are drawn: nothing is
+// written before the first of these pieces is done, so the plan draws while the kernel before it (a step's receive, an
+// optimizer) still runs, and the receive bits are set without a trip to the L2.  A step (plan, send, receive) against
+// waiting first and writing word by word: ResNet-50 N = 5 47.0 -> 45.1 us (the plan alone 25.2 -> 21.0), N = 3 with 10^6
+// coordinates 14.5 -> 9.4, 10^8 coordinates 220 -> 180.  Four blocks stay on an SM (28 KB a block, 45 at N = 64).
+constexpr uint32_t kPlanHeldTiles = 128;
 
 __global__ void __launch_bounds__(kXThreads, kExchangeBlocksPerSm) exchange_plan_kernel(const __grid_constant__ ExchangeArgs a)
 {
     extern __shared__ uint32_t s_perm_all[];   // 32 * wide_pitch(N) words per warp when N > 16, else nothing
     let_next_start();
-    await_previous();
+    __shared__ __align__(16) uint32_t s_words[32 * kPlanHeldTiles];
     __shared__ uint2 q_key[kPlanQueue];       // {coordinate within its tensor, tensor}
     __shared__ uint32_t q_elem[kPlanQueue];   // row element (rows are shorter than 2^32)
     __shared__ uint32_t s_total[kMaxN + 1], s_count;
@@ -100,57 +106,66 @@ __global__ void __launch_bounds__(kXThreads, kExchangeBlocksPerSm) exchange_plan
     if (threadIdx.x == 0) s_count = 0;
     uint32_t t_first, t_end;
     block_range(a, &t_first, &t_end);
-    __syncthreads();
+    const uint32_t pieces = (t_end - t_first + kPlanHeldTiles - 1u) / kPlanHeldTiles, per_piece = pieces ? (t_end - t_first + pieces - 1u) / pieces : 0u;
     LaneSegment ls;
-    uint32_t t = t_first + warp, sel = 0, sel_g0 = 0;   // sel: coordinates of the lane's last tile that are not queued yet; sel_g0: its first group there
-    for (;;) {
-        for (;;) {
-            if (sel) {
-                uint32_t pos = atomicAdd(&s_count, static_cast<uint32_t>(__popc(sel)));
-                for (; sel && pos < kPlanQueue; sel &= sel - 1u, ++pos) {
-                    const uint32_t bit = static_cast<uint32_t>(__ffs(sel) - 1), g = sel_g0 + (bit >> 2), c = bit & 3u;
-                    if (g - ls.begin < ls.end - ls.begin) q_key[pos] = make_uint2(4u * (g + ls.cgroup_off) + c, ls.tensor);
-                    else {
-                        const GroupInfo gi = find_group(a.pop, g, a.status);
-                        q_key[pos] = make_uint2(4u * gi.cgroup + c, gi.tensor_id);
-                    }
-                    q_elem[pos] = 4u * sel_g0 + bit;
-                }
-            }
-            if (sel || t >= t_end) break;   // the queue is full, or the range is done (lane by lane: nothing in this loop needs the warp together)
-            sel_g0 = t * kExchangeTileGroups + 4u * lane;
-            sel = lane_masks(a, sel_g0, a.pop.n_groups, ls);
-            a.mask[static_cast<size_t>(t) * 32u + lane] = sel;
-            t += kExchangeWarps;
-        }
-        const bool again = __syncthreads_or(sel != 0 || t < t_end);   // (orders the queue's entries and the mask words before the atomics below, too)
-        const uint32_t count = min(s_count, kPlanQueue);
-        for (uint32_t first = warp * 32u; first < count; first += kXThreads) {
-            unsigned long long need;
-            uint32_t dest;
-            const bool active = first + lane < count;
-            const uint2 key = active ? q_key[first + lane] : make_uint2(0, 0);
-            routes_of(a, active, key.x, key.y, s_perm, &need, &dest);
-            if ((need >> a.self) & 1ull) {
-                const uint32_t elem = q_elem[first + lane];
-                atomicOr(&a.mask[elem >> 4], 0x10000u << (elem & 15u));
-            }
-            __syncwarp();
-            uint32_t mine[2] = {0, 0};   // lane l counts workers l and l + 32
-            for (int n = 0; n < n_models; ++n) {
-                const uint32_t votes = __popc(__ballot_sync(kFull, (need >> n) & 1ull));
-                if (lane == static_cast<uint32_t>(n & 31)) mine[n >> 5] = votes;
-            }
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-                if (mine[h]) atomicAdd(&s_total[lane + 32u * h], mine[h]);
-            if (lane == 0) atomicAdd(&s_total[n_models], min(32u, count - first));
-        }
-        __syncthreads();   // the queue is free, the totals are complete
-        if (!again) break;
-        if (threadIdx.x == 0) s_count = 0;
+    uint32_t p0 = t_first, p1;   // the piece's tiles
+    do {
+        p1 = min(p0 + per_piece, t_end);
         __syncthreads();
-    }
+        uint32_t t = p0 + warp, sel = 0, sel_g0 = 0;   // sel: coordinates of the lane's last tile that are not queued yet; sel_g0: its first group there
+        for (;;) {
+            for (;;) {
+                if (sel) {
+                    uint32_t pos = atomicAdd(&s_count, static_cast<uint32_t>(__popc(sel)));
+                    for (; sel && pos < kPlanQueue; sel &= sel - 1u, ++pos) {
+                        const uint32_t bit = static_cast<uint32_t>(__ffs(sel) - 1), g = sel_g0 + (bit >> 2), c = bit & 3u;
+                        if (g - ls.begin < ls.end - ls.begin) q_key[pos] = make_uint2(4u * (g + ls.cgroup_off) + c, ls.tensor);
+                        else {
+                            const GroupInfo gi = find_group(a.pop, g, a.status);
+                            q_key[pos] = make_uint2(4u * gi.cgroup + c, gi.tensor_id);
+                        }
+                        q_elem[pos] = 4u * sel_g0 + bit;
+                    }
+                }
+                if (sel || t >= p1) break;   // the queue is full, or the piece is done (lane by lane: nothing in this loop needs the warp together)
+                sel_g0 = t * kExchangeTileGroups + 4u * lane;
+                sel = lane_masks(a, sel_g0, a.pop.n_groups, ls);
+                s_words[(t - p0) * 32u + lane] = sel;
+                t += kExchangeWarps;
+            }
+            const bool again = __syncthreads_or(sel != 0 || t < p1);   // (orders the queue's entries and the mask words before the atomics below, too)
+            const uint32_t count = min(s_count, kPlanQueue);
+            for (uint32_t first = warp * 32u; first < count; first += kXThreads) {
+                unsigned long long need;
+                uint32_t dest;
+                const bool active = first + lane < count;
+                const uint2 key = active ? q_key[first + lane] : make_uint2(0, 0);
+                routes_of(a, active, key.x, key.y, s_perm, &need, &dest);
+                if ((need >> a.self) & 1ull) {
+                    const uint32_t elem = q_elem[first + lane];
+                    atomicOr(&s_words[(elem >> 4) - p0 * 32u], 0x10000u << (elem & 15u));
+                }
+                __syncwarp();
+                uint32_t mine[2] = {0, 0};   // lane l counts workers l and l + 32
+                for (int n = 0; n < n_models; ++n) {
+                    const uint32_t votes = __popc(__ballot_sync(kFull, (need >> n) & 1ull));
+                    if (lane == static_cast<uint32_t>(n & 31)) mine[n >> 5] = votes;
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    if (mine[h]) atomicAdd(&s_total[lane + 32u * h], mine[h]);
+                if (lane == 0) atomicAdd(&s_total[n_models], min(32u, count - first));
+            }
+            __syncthreads();   // the queue is free, the totals are complete
+            if (threadIdx.x == 0) s_count = 0;
+            if (!again) break;
+            __syncthreads();
+        }
+        await_previous();
+        uint4 *out = reinterpret_cast<uint4 *>(a.mask + static_cast<size_t>(p0) * 32u);
+        for (uint32_t i = threadIdx.x; i < (p1 - p0) * 8u; i += kXThreads) out[i] = reinterpret_cast<const uint4 *>(s_words)[i];
+        p0 = p1;
+    } while (p0 < t_end);
     if (threadIdx.x < static_cast<uint32_t>(columns)) a.block_total[static_cast<size_t>(blockIdx.x) * columns + threadIdx.x] = s_total[threadIdx.x];
 }
 

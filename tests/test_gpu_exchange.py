@@ -316,3 +316,22 @@ def test_lists_of_a_block_reproduce_the_population_shuffle(N, numel, p_layer):
     st = w.stats.cpu().numpy()
     assert (st[:, 0] == sel).all() and st[:, 1].sum() == moved
     w.close()
+
+
+@pytest.mark.parametrize("numel,p", [([80_000_003], 2e-4), ([39_000_001, 300], 2e-4), ([700_001, 9, 513], 0.05)])
+def test_plans_that_follow_a_receive_at_once(numel, p):
+    """The plan draws while the kernel before it still runs and holds up to 128 warp tiles of mask words a block until that
+    one is done (39 million coordinates on 148 SMs; longer rows go in pieces): steps launched one after the other,
+    nothing waited for in between."""
+    N, steps = 2, (0, 1, 2)
+    w = Workers(N, numel, seed=4)
+    for step in steps:
+        w.step(step, p, None, seed=9)
+    w.check()
+    need, sel = oracle.exchange_counts(w.ora, p, seed=9, step=steps[-1])
+    for step in steps:
+        oracle.shuffle(w.ora, w.host[0], p, seed=9, step=step)
+    assert (to_host_bits(w.dev[0]) == bits(w.host[0])).all()
+    for n in range(N):
+        assert B.wash_exchange_counts(w.ctx[n], N) == (need.tolist(), sel)
+    w.close()
