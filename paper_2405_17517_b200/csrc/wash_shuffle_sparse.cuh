@@ -12,13 +12,15 @@
 // the first of them.
 //
 // Two bounds.  The mask: one Philox block per 4 coordinates on the integer pipes (2^27 coordinates:
-// 80 us for the blocks alone, 86 us with the compares, this kernel 100 us at N = 2, p = 1e-4).  The
+// 80 us for the blocks alone, 86 us with the compares, this kernel 92 us at N = 2, p = 1e-4).  The
 // values: DRAM serves about 45e9 scattered 4-byte loads a second, 22e9 scattered stores and 20e9 pairs
 // of both (measured, one access per 800 bytes), so [N][P] cannot go below 1 us per 20 000 moved
-// values and stack: cfg4 (1.8e6 values in both stacks) 90 us by that figure, 81 us here -- neighbouring
-// coordinates of a model share DRAM pages.  With a queue per warp, served at the end of the warp's
-// range by a lane per coordinate, the same launches took (before -> now): cfg2 21.2 -> 16.4 us, cfg3
-// 70.9 -> 59.1, cfg4 89.1 -> 81.4, cfg1 8.2 -> 6.2, 2^27 coordinates N = 2 at p = 1e-3 119 -> 107 us.
+// values and stack: ResNet-50 N = 8, bf16 + fp32, p = 5e-3 (1.8e6 values in both stacks) 90 us by that figure, 77 us
+// here -- neighbouring coordinates of a model share DRAM pages.  With a queue per warp, served at the end of the warp's
+// range by a lane per coordinate, and launches that do not overlap, the same took (before -> now): that one 89.1 -> 77.1,
+// ResNet-18 N = 5 with momentum, p = 1e-3 21.0 -> 10.5, ResNet-50 N = 10 with momentum, p = 0.01 -> 0 70.8 -> 56.1, 2^27 coordinates N = 2
+// at p = 1e-3 119 -> 97.5 us.  Not for much selected in large [N][P] populations, where a set of 128 / N coordinates uses
+// half of a sector (N = 32, 2^25, p = 0.1 1855 -> 2740): WASH_MODE_AUTO streams from 2 % on there.
 #pragma once
 #include <cmath>
 #include "wash_device.cuh"
@@ -183,16 +185,22 @@ cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchSha
     if (err != cudaSuccess) return err;
     if (fit.occupancy < 1) return cudaErrorLaunchOutOfResources;
     const uint32_t resident = static_cast<uint32_t>(shape.sm_count > 0 ? shape.sm_count : 148) * static_cast<uint32_t>(fit.occupancy);
-    // Grid: enough blocks that one expects kSparsePerBlock selected coordinates, in several waves, so
-    // that one wave's (memory-bound) serving overlaps the next one's (multiply-bound) mask; but a warp
-    // keeps a few tiles, or a block's start, barriers and end weigh more than its mask, and a resident
-    // wave is the least.  Measured with 8 / 16 / 32 / 64 per block: cfg3 61.3 / 60.9 / 66.1 / 68.7 us, cfg4
-    // 82.3 / 82.3 / 86.2 / 96.3 us, 2^27 coordinates N = 2 at p = 1e-3 131 / 119 / 117 / 120 us; with 1 / 2 / 3 / 4 tiles a
-    // warp: five ResNet-50 models at p = 0.05 -> 0 60.7 / 51.2 / 49.7 / 51.2 us, eight of 2^25 at p = 0.01 98.2 / 98.6 /
-    // 101.7 / 104.0 us, [P][N] 69.6 / 53.3 / 49.3 / 49.2 us.
+    // Grid.  A block costs its start, its barriers and its end (about 1.5 us of a resident slot), so it takes as many tiles
+    // as it can; what ends that is the serving: several waves let one block's (memory-bound) serving overlap the
+    // next one's (multiply-bound) mask.  So: whole waves, as many as keep a block's expected selection at what [N][P]
+    // serves in 400 scattered values (300 in two stacks or more than 8 models), [P][N] in 300 coordinates, but not
+    // below kSparsePerBlock coordinates and 2 ([P][N] 3) tiles a warp.  Measured (blocks of 2 or 3 tiles a warp throughout ->
+    // this rule): N = 2, 2^27 coordinates, p = 3e-3 / 0.01 / 0.03 134 / 162 / 198 -> 106 / 124 / 183 us, 2^25, p = 0.01 41.2 -> 31.9; N = 3,
+    // 2.5e7, p = 3e-3 26.8 -> 20.9; ResNet-50 N = 5, p = 0.05 -> 0 44.9 -> 42.7; [P][N] N = 8, 2^25, p = 0.01 43.3 -> 36.7, N = 16, p = 3e-3
+    // 39.9 -> 31.7.  A larger load loses where values are many (400 instead of 300 for ResNet-50 N = 8 bf16 + fp32, p = 5e-3: 79.4
+    // against 77.1, N = 20, p = 2e-3 51.6 against 50.3), a broken wave where waves are few ([P][N] N = 8, 2^25: 1.4 waves
+    // 41.9, two 38.8).
+    const bool one_stack = TB::kCode == kDtypeNone;
     const double expected = static_cast<double>(args.expected_share) * 4.0 * static_cast<double>(args.group_hi - args.group_lo);
-    const double by_tiles = static_cast<double>(p.n_wtiles) / (kSparseWarps * (args.pop.layout == kLayoutNP ? 2 : 3));
-    uint32_t grid = static_cast<uint32_t>(fmin(expected / kSparsePerBlock, by_tiles));
+    const double by_tiles = static_cast<double>(p.n_wtiles) / (kSparseWarps * (np ? 2 : 3));
+    const double load = np ? (one_stack && args.pop.N <= 8 ? 400.0 : 300.0) / args.pop.N : 300.0;   // coordinates of a block, one stack
+    const double by_load = resident * ceil(expected * (one_stack ? 1.0 : 2.0) / load / resident);
+    uint32_t grid = static_cast<uint32_t>(fmin(fmin(expected / kSparsePerBlock, by_tiles), by_load));
     if (grid < resident) grid = resident;
     const uint32_t want = (p.n_wtiles + kSparseWarps - 1) / kSparseWarps;
     if (grid > want) grid = want;

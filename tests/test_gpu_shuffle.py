@@ -244,6 +244,22 @@ def test_last_layer_untouched_and_schedules_agree_with_oracle():
 
 
 @pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("N,numel,p,dtype,opt", [
+    (2, [9_000_001], [0.03], "f32", None),                       # several waves of blocks, loaded evenly
+    (3, [5_000_003, 30_000], [0.0005, 1.0], "f32", "f32"),       # one wave by the mean, a few blocks loaded far above it
+    (9, [2_000_001], [0.01], "bf16", None), (20, [1_000_001], [0.004], "f32", None)])
+def test_sparse_blocks_take_what_a_wave_leaves_them(N, numel, p, dtype, opt, layout):
+    c = Case(N, numel, layout, dtype, opt, seed=N)
+    B.wash_set_mode(c.gpu.ctx, B.WASH_MODE_SPARSE)
+    call = B.wash_shuffle if opt is None else B.wash_shuffle_both
+    call(c.gpu.ctx, 2, max(p), p, seed=3, stats=c.stats_dev)
+    want = oracle.shuffle(c.ora, c.host, p, seed=3, step=2, stack2=c.host_opt)
+    c.assert_equal("N=%d layout=%d" % (N, layout))
+    assert c.gpu_stats() == tuple(want)
+    c.close()
+
+
+@pytest.mark.parametrize("layout", [0, 1])
 @pytest.mark.parametrize("dtype,opt", [("f32", None), ("bf16", None), ("bf16", "f32")])
 @pytest.mark.parametrize("N", [2, 3, 4, 5, 6])
 def test_resident_warp_kernel_for_each_compiled_population(N, dtype, opt, layout):
