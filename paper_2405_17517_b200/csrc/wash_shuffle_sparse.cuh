@@ -19,8 +19,7 @@
 // here -- neighbouring coordinates of a model share DRAM pages.  With a queue per warp, served at the end of the warp's
 // range by a lane per coordinate, and launches that do not overlap, the same took (before -> now): that one 89.1 -> 77.1,
 // ResNet-18 N = 5 with momentum, p = 1e-3 21.0 -> 10.5, ResNet-50 N = 10 with momentum, p = 0.01 -> 0 70.8 -> 56.1, 2^27 coordinates N = 2
-// at p = 1e-3 119 -> 97.5 us.  Not for much selected in large [N][P] populations, where a set of 128 / N coordinates uses
-// half of a sector (N = 32, 2^25, p = 0.1 1855 -> 2740): WASH_MODE_AUTO streams from 2 % on there.
+// at p = 1e-3 119 -> 97.5 us.
 #pragma once
 #include <cmath>
 #include "wash_device.cuh"
@@ -33,6 +32,12 @@ namespace wash {
 constexpr int kSparseWarps = 4;
 constexpr int kSparseThreads = 32 * kSparseWarps;
 constexpr int kSparsePairs = 4;      // (coordinate, model) pairs a lane has in flight
+// Shares of the coordinates from which [N][P] is served a lane per coordinate (serve_row): pairs take 128 / N neighbouring
+// coordinates of a model side by side, half a sector at N = 32, a lane per coordinate 32, but all N values one
+// after the other.  fp32, pairs / rows: N = 8, 2^25, 10 % 331 / 323, 30 % 483 / 411 us; N = 16, 2^24, 10 % 375 / 390, 30 % 518 / 407; N = 20 30 %
+// 710 / 686; N = 24, 2^23, 2 % 146 / 177, 5 % 266 / 277; N = 28 2 % 173 / 216, 10 % 421 / 389; N = 32, 2^24, 1 % 266 / 265, 10 % 1417 / 901, all
+// 5830 / 1927; N = 5 30 % 338 / 421.
+constexpr float kRowsShare = 0.25f, kRowsShareLarge = 0.06f;   // 8 to 23 models, 24 and more
 constexpr double kSparsePerBlock = 16.0;   // selected coordinates a block expects, at least
 
 // entries of the queue: a permutation of up to 16 models stays in its entry (8 bytes), a larger one
@@ -44,11 +49,28 @@ struct SparseArgs {
     uint32_t n_wtiles;      // warp tiles in [group_lo, group_hi)
     uint32_t per_block, extra;   // tiles of a block: per_block, one more in the first `extra` blocks
     uint32_t in_set;        // coordinates whose N values a warp moves at a time: 32 * kSparsePairs / N
+    uint32_t column_offset; // ROWS: where the lanes' columns lie in shared memory
     uint32_t inverse;       // 2^16 / d, rounded up, for the division of a pair's number (below 128) by in_set ([N][P]) or N ([P][N])
 };
 
+// One stack's values of a lane's coordinate: all loaded into the lane's column of shared memory, then stored.
+template <class T, int LAYOUT, class PERM>
+__device__ __forceinline__ void serve_row(const PopView &pop, void *stack, uint32_t *column, long long elem, const PERM &source_of)
+{
+    const int n_models = pop.N;
+#pragma unroll 8
+    for (int n = 0; n < n_models; ++n) column[n * kSparseThreads] = T::load_elem(stack, elem_index<LAYOUT>(pop, n, elem));
+#pragma unroll 4
+    for (int n = 0; n < n_models; ++n) {
+        const uint32_t src = source_of(n);
+        if (src != static_cast<uint32_t>(n)) T::store_elem(stack, elem_index<LAYOUT>(pop, n, elem), column[src * kSparseThreads]);
+    }
+}
+
 // MIRROR: the moved values go to a second copy of the stacks as well (wash_step_host: the caller's buffers).
-template <class TA, class TB, int LAYOUT, bool MIRROR>
+// ROWS: a lane per coordinate loads all its values before it stores them (serve_rows), instead of a lane per (coordinate,
+// model) pair.
+template <class TA, class TB, int LAYOUT, bool MIRROR, bool ROWS>
 __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_sparse_kernel(const __grid_constant__ SparseArgs p)
 {
     let_next_start();
@@ -114,51 +136,64 @@ __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_spa
             }
         }
         __syncthreads();
-        // the lane's pairs of a set: [N][P] takes neighbouring coordinates of one model side by side,
-        // [P][N] the models of one coordinate
-        uint32_t pair_entry[kSparsePairs], pair_model[kSparsePairs];
-#pragma unroll
-        for (int k = 0; k < kSparsePairs; ++k) {
-            const uint32_t i = lane + 32u * k, outer = (i * p.inverse) >> 16;
-            const uint32_t inner = i - outer * (LAYOUT == kLayoutNP ? p.in_set : static_cast<uint32_t>(n_models));
-            pair_entry[k] = LAYOUT == kLayoutNP ? inner : outer;
-            pair_model[k] = LAYOUT == kLayoutNP ? outer : inner;
-            if (pair_model[k] >= static_cast<uint32_t>(n_models) || pair_entry[k] >= p.in_set) pair_entry[k] = 0xFFFFu;   // no pair
-        }
-        for (uint32_t first = warp * p.in_set; first < count; first += kSparseWarps * p.in_set) {
-            const uint32_t left = count - first;
-            uint32_t va[kSparsePairs], vb[kSparsePairs];
-            long long out[kSparsePairs];
+        if constexpr (ROWS) {
+            uint32_t *column = reinterpret_cast<uint32_t *>(smem_raw + p.column_offset) + threadIdx.x;
+            for (uint32_t e = threadIdx.x; e < count; e += kSparseThreads) {
+                const long long elem = block_elem + q_elem[e];
+                const uint2 packed = q_key[e];
+                const uint8_t *wide = reinterpret_cast<const uint8_t *>(q_wide + e * wide_pitch(n_models));
+                const auto source_of = [&](int n) -> uint32_t { return n_models <= 16 ? ((n < 8 ? packed.x : packed.y) >> (4 * (n & 7))) & 15u : wide[n]; };
+                serve_row<TA, LAYOUT>(a.pop, a.a, column, elem, source_of);
+                if constexpr (kHasB) serve_row<TB, LAYOUT>(a.pop, a.b, column, elem, source_of);
+                for (int n = 0; n < n_models; ++n) moved += source_of(n) != static_cast<uint32_t>(n) ? 1u : 0u;
+            }
+        } else {
+            // the lane's pairs of a set: [N][P] takes neighbouring coordinates of one model side by side,
+            // [P][N] the models of one coordinate
+            uint32_t pair_entry[kSparsePairs], pair_model[kSparsePairs];
 #pragma unroll
             for (int k = 0; k < kSparsePairs; ++k) {
-                out[k] = -1;
-                if (pair_entry[k] < left) {
-                    const uint32_t e = first + pair_entry[k], n = pair_model[k];
-                    uint32_t src;
-                    if (n_models <= 16) {
-                        const uint2 packed = q_key[e];
-                        src = ((n < 8 ? packed.x : packed.y) >> (4u * (n & 7u))) & 15u;
-                    } else src = reinterpret_cast<const uint8_t *>(q_wide + e * wide_pitch(n_models))[n];
-                    if (src != n) {
-                        const long long elem = block_elem + q_elem[e];
-                        const long long in = elem_index<LAYOUT>(a.pop, static_cast<int>(src), elem);
-                        out[k] = elem_index<LAYOUT>(a.pop, static_cast<int>(n), elem);
-                        va[k] = TA::load_elem(a.a, in);
-                        if constexpr (kHasB) vb[k] = TB::load_elem(a.b, in);
+                const uint32_t i = lane + 32u * k, outer = (i * p.inverse) >> 16;
+                const uint32_t inner = i - outer * (LAYOUT == kLayoutNP ? p.in_set : static_cast<uint32_t>(n_models));
+                pair_entry[k] = LAYOUT == kLayoutNP ? inner : outer;
+                pair_model[k] = LAYOUT == kLayoutNP ? outer : inner;
+                if (pair_model[k] >= static_cast<uint32_t>(n_models) || pair_entry[k] >= p.in_set) pair_entry[k] = 0xFFFFu;   // no pair
+            }
+            for (uint32_t first = warp * p.in_set; first < count; first += kSparseWarps * p.in_set) {
+                const uint32_t left = count - first;
+                uint32_t va[kSparsePairs], vb[kSparsePairs];
+                long long out[kSparsePairs];
+#pragma unroll
+                for (int k = 0; k < kSparsePairs; ++k) {
+                    out[k] = -1;
+                    if (pair_entry[k] < left) {
+                        const uint32_t e = first + pair_entry[k], n = pair_model[k];
+                        uint32_t src;
+                        if (n_models <= 16) {
+                            const uint2 packed = q_key[e];
+                            src = ((n < 8 ? packed.x : packed.y) >> (4u * (n & 7u))) & 15u;
+                        } else src = reinterpret_cast<const uint8_t *>(q_wide + e * wide_pitch(n_models))[n];
+                        if (src != n) {
+                            const long long elem = block_elem + q_elem[e];
+                            const long long in = elem_index<LAYOUT>(a.pop, static_cast<int>(src), elem);
+                            out[k] = elem_index<LAYOUT>(a.pop, static_cast<int>(n), elem);
+                            va[k] = TA::load_elem(a.a, in);
+                            if constexpr (kHasB) vb[k] = TB::load_elem(a.b, in);
+                        }
                     }
                 }
-            }
-            __syncwarp();   // every value of the set is loaded before the first is overwritten
+                __syncwarp();   // every value of the set is loaded before the first is overwritten
 #pragma unroll
-            for (int k = 0; k < kSparsePairs; ++k) {
-                if (out[k] < 0) continue;
-                TA::store_elem(a.a, out[k], va[k]);
-                if constexpr (kHasB) TB::store_elem(a.b, out[k], vb[k]);
-                if constexpr (MIRROR) {
-                    TA::store_elem(a.mirror_a, out[k], va[k]);
-                    if constexpr (kHasB) TB::store_elem(a.mirror_b, out[k], vb[k]);
+                for (int k = 0; k < kSparsePairs; ++k) {
+                    if (out[k] < 0) continue;
+                    TA::store_elem(a.a, out[k], va[k]);
+                    if constexpr (kHasB) TB::store_elem(a.b, out[k], vb[k]);
+                    if constexpr (MIRROR) {
+                        TA::store_elem(a.mirror_a, out[k], va[k]);
+                        if constexpr (kHasB) TB::store_elem(a.mirror_b, out[k], vb[k]);
+                    }
+                    ++moved;
                 }
-                ++moved;
             }
         }
         if (!again) break;
@@ -176,10 +211,15 @@ cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchSha
     SparseArgs p;
     p.s = args;
     p.n_wtiles = (args.group_hi - args.group_lo + kWarpTileGroups - 1) / kWarpTileGroups;
-    const size_t smem = sparse_queue_capacity(args.pop.N) * (12 + (args.pop.N > 16 ? 4 * static_cast<size_t>(wide_pitch(args.pop.N)) : 0));
+    size_t smem = sparse_queue_capacity(args.pop.N) * (12 + (args.pop.N > 16 ? 4 * static_cast<size_t>(wide_pitch(args.pop.N)) : 0));
     const bool np = args.pop.layout == kLayoutNP;
-    auto kernel = np ? shuffle_sparse_kernel<TA, TB, kLayoutNP, false> : shuffle_sparse_kernel<TA, TB, kLayoutPN, false>;
-    if (args.mirror_a) kernel = np ? shuffle_sparse_kernel<TA, TB, kLayoutNP, true> : shuffle_sparse_kernel<TA, TB, kLayoutPN, true>;
+    auto kernel = np ? shuffle_sparse_kernel<TA, TB, kLayoutNP, false, false> : shuffle_sparse_kernel<TA, TB, kLayoutPN, false, false>;
+    if (args.mirror_a) kernel = np ? shuffle_sparse_kernel<TA, TB, kLayoutNP, true, false> : shuffle_sparse_kernel<TA, TB, kLayoutPN, true, false>;
+    else if (np && args.expected_share >= (args.pop.N >= 24 ? kRowsShareLarge : args.pop.N >= 8 ? kRowsShare : 2.f)) {
+        kernel = shuffle_sparse_kernel<TA, TB, kLayoutNP, false, true>;
+        p.column_offset = static_cast<uint32_t>(smem);
+        smem += 4 * static_cast<size_t>(args.pop.N) * kSparseThreads;
+    }
     KernelFit fit;
     cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), kSparseThreads, smem, &fit);
     if (err != cudaSuccess) return err;
@@ -197,7 +237,9 @@ cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchSha
     // 41.9, two 38.8).
     const bool one_stack = TB::kCode == kDtypeNone;
     const double expected = static_cast<double>(args.expected_share) * 4.0 * static_cast<double>(args.group_hi - args.group_lo);
-    const double by_tiles = static_cast<double>(p.n_wtiles) / (kSparseWarps * (np ? 2 : 3));
+    double by_tiles = static_cast<double>(p.n_wtiles) / (kSparseWarps * (np ? 2 : 3));
+    // (one tile a warp where the queue would overflow: [P][N] N = 5, 2^25, p = 0.15 183 -> 172 us, [N][P] p = 0.1 194 -> 184)
+    if (expected > by_tiles * (np ? 0.75 : 1.0) * sparse_queue_capacity(args.pop.N)) by_tiles = static_cast<double>(p.n_wtiles) / kSparseWarps;
     const double load = np ? (one_stack && args.pop.N <= 8 ? 400.0 : 300.0) / args.pop.N : 300.0;   // coordinates of a block, one stack
     const double by_load = resident * ceil(expected * (one_stack ? 1.0 : 2.0) / load / resident);
     uint32_t grid = static_cast<uint32_t>(fmin(fmin(expected / kSparsePerBlock, by_tiles), by_load));
