@@ -203,13 +203,13 @@ uint64_t threshold_of(double p) { return static_cast<uint64_t>(std::floor(p * 42
 // Measured crossovers (2^24-2^25 coordinates):
 //   [N][P]  one stack   fp32 N = 2 18 %, 3 14 %, 4 15 %, 5 12 %, 8 6 %, 12 5 %, 16 4.7 %, 20 5 %, 32 2 %; bf16 18, 16, 19, 11, 15, 10, 7.5, 3, 1 %
 //           two stacks  fp32 N = 2 20 %, 5 6 %, 16 3 %, 32 1.8 %; bf16 + fp32 21, 5, 2.8, 1.3 %
-//   [P][N]  one stack   fp32 N = 2 14 %, 3 13 %, 4 15 %, 5 15 %, 8 17 %, 12 20 %, 16 40 %, 20 35 %, 32 above 50 %; bf16 13, 12, 19, 27, 28, 38, 48, 20, 33 %
+//   [P][N]  one stack   fp32 N = 2 14 %, 3 13 %, 4 15 %, 5 16 %, 6 21 %, 8 22 %, 12 23 %, 16 40 %, 20 35 %, 32 above 50 %; bf16 13, 12, 19, 27, 28, 38, 48, 20, 33 %
 //           two stacks  fp32 N = 2 23 %, 5 20 %, 16 and 32 above 50 %; bf16 + fp32 20, 30, above 50 %
 double sparse_share(int layout, int N, bool two_stacks, bool bf16)
 {
     if (layout == WASH_LAYOUT_NP) return std::fmin(0.18, (two_stacks ? 0.35 : 0.6) / N);
     if (N <= 3) return two_stacks ? 0.2 : 0.13;
-    if (N < 16) return two_stacks || bf16 ? 0.2 : 0.16;
+    if (N < 16) return two_stacks || bf16 || N > 5 ? 0.2 : 0.16;
     return bf16 && !two_stacks ? (N == 16 ? 0.4 : 0.2) : 0.4;
 }
 
@@ -251,6 +251,19 @@ int sync_table(wash_ctx *ctx, double p, const double *p_layer, cudaStream_t stre
     ctx->slot_used[slot] = true;
     ctx->seg_uploaded = true;
     return WASH_OK;
+}
+
+// [P][N]: a vector of padding after a group of the streaming kernels' shared-memory image, against bank conflicts.  It
+// pays where the groups are served densely, from half of the coordinates on, and lie a multiple of 128 bytes apart (64 in
+// two stacks); elsewhere the bytes it costs and the copies that are no longer one piece weigh more.  2^24 coordinates, padded /
+// not, at 22 / 40 / 70 / 100 %: fp32 N = 2 68 108 140 132 / 60 101 132 124 us; N = 8 179 215 297 306 / 161 206 397 298; N = 12 262 348 470 467 / 244
+// 323 457 438; N = 16 377 519 583 606 / 357 480 724 541; bf16 N = 8 189 196 288 280 / 188 193 277 263, N = 16 422 637 552 539 / 421 640 751
+// 553; two fp32 stacks of N = 4 170 205 243 212 / 152 178 313 281; bf16 + fp32 N = 10 439 642 551 535 / 418 616 512 514; fp32 N = 32, 2^23
+// coordinates, 25 / 60 % 404 761 / 358 692.
+uint32_t pn_pad(const wash_ctx *ctx, bool bf16, bool two_stacks, float share)
+{
+    if (ctx->layout != WASH_LAYOUT_PN || ctx->N > 16 || share < 0.5f) return 0u;
+    return ctx->N % (two_stacks ? 4 : bf16 ? 16 : 8) == 0 ? 4u : 0u;
 }
 
 // [P][N] with the distance to the consensus: every thread reads its whole group from the shared-memory image, so an
@@ -327,10 +340,8 @@ int shuffle_impl(wash_ctx *ctx, int which, uint64_t step, double p, const double
         }
         double coordinates = 0.0;
         for (int s = 0; s < ctx->n_seg; ++s) coordinates += static_cast<double>(ctx->seg_host[s].numel);
-        // [P][N], even N: the streaming kernel pads its shared-memory image against bank conflicts
-        // once a fifth of the coordinates is expected to be served from it
         args.expected_share = coordinates > 0.0 ? static_cast<float>(ctx->expected_selected / coordinates) : 0.f;
-        if (ctx->layout == WASH_LAYOUT_PN && !(ctx->N & 1)) args.pn_pad = ctx->expected_selected >= 0.2 * coordinates ? 4u : 0u;
+        args.pn_pad = pn_pad(ctx, a_dtype == wash::kDtypeBF16, b != nullptr, args.expected_share);
         // The streaming kernel's early flavour (permutations drawn while the copies are in flight, dense
         // serving for N > 16) costs registers and, for N > 16, three more permutation columns of shared
         // memory per thread: measured, it pays only for large populations of which most coordinates are

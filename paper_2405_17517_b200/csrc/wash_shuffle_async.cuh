@@ -15,10 +15,9 @@
 //           are copied by their own thread, bf16 vectors in 16-byte pairs by the two lanes that own them
 //   [P][N]: the block's T*4N elements are contiguous in global memory and are copied
 //           vector by vector, vector k*T + t by thread t; a group's 4N elements stay together
-//           and, when N is even and the launch expects to serve many coordinates, are followed
-//           by one vector of padding, so that a group spans an odd number of vectors and the
-//           lanes of a warp (one group each) fall into different shared-memory banks (at small
-//           p the image is hardly read and the padding would only cost bytes in flight):
+//           and, where the launch says so (pn_pad), are followed by one vector of padding, so that a
+//           group spans an odd number of vectors and the lanes of a warp (one group each) fall into
+//           different shared-memory banks:
 //           thread t's coordinate c of model n is element t*pn_group_elems + c*N + n.
 #pragma once
 #include "wash_device.cuh"

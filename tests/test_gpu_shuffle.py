@@ -243,6 +243,20 @@ def test_last_layer_untouched_and_schedules_agree_with_oracle():
     c.close()
 
 
+@pytest.mark.parametrize("p", [0.25, 0.6])
+@pytest.mark.parametrize("N,dtype,opt", [(2, "f32", None), (8, "f32", None), (16, "bf16", None), (16, "f32", None), (12, "f32", None),
+                                         (4, "f32", "f32"), (10, "bf16", "f32"), (20, "f32", None)])
+def test_coordinate_major_images_with_and_without_padding(N, dtype, opt, p):
+    """[P][N], below and above the share from which some populations' images are padded."""
+    c = Case(N, [30_001, 9, 2048], 1, dtype, opt, seed=N)
+    call = B.wash_shuffle if opt is None else B.wash_shuffle_both
+    call(c.gpu.ctx, 1, p, None, seed=6, stats=c.stats_dev)
+    want = oracle.shuffle(c.ora, c.host, p, seed=6, step=1, stack2=c.host_opt)
+    c.assert_equal("N=%d" % N)
+    assert c.gpu_stats() == tuple(want)
+    c.close()
+
+
 @pytest.mark.parametrize("layout", [0, 1])
 @pytest.mark.parametrize("N,numel,p,dtype,opt", [
     (2, [9_000_001], [0.03], "f32", None),                       # several waves of blocks, loaded evenly
