@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(64, 6) shuffle_wide_kernel(const __grid_consta
 // [P][N] with a group of all models of kWideSplitBytes and more: two threads to a group, the block's selected
 // coordinates in one list shared evenly by its warps.  Six blocks of 35 KB hold twice the warps that way,
 // each with half the copies, draws and moves.  N = 32, fp32, 2^23 coordinates, p = 0.03 / 0.1 / 0.25: 197 / 246 / 410 us by the kernel
-// above, 192 / 233 / 404; N = 24, bf16 + fp32, p = 0.25 436 / 386; N = 64, fp32, p = 0.1 632 / 542.  Smaller groups (N = 20, fp32, p = 0.1
+// above, 192 / 233 / 404 (both with a padded image at 0.25; without 357); N = 24, bf16 + fp32, p = 0.25 436 / 386; N = 64, fp32, p = 0.1 632 / 542.  Smaller groups (N = 20, fp32, p = 0.1
 // 145 / 165 us) and [N][P] (N = 20 200 / 202, N = 17 bf16 103 / 162) lose more by the block's barriers.
 constexpr size_t kWideSplitBytes = 512;
 constexpr uint32_t kWideRound = 16;   // coordinates of a warp's round
