@@ -335,7 +335,8 @@ __global__ void __launch_bounds__(64, 16) dense_pn_kernel(const __grid_constant_
             }
         }
         if constexpr (OP != kOpAverage) {
-            const uint32_t whole = __ballot_sync(0xFFFFFFFFu, valid == kElems);   // (orders the lanes' updates, too)
+            const uint32_t whole = __ballot_sync(0xFFFFFFFFu, valid == kElems);
+            __syncwarp();   // the units are copied by other lanes than those that updated them; a vote orders no memory accesses
             uint32_t unit = lane / N, j = lane - unit * N;
             for (uint32_t k = lane; k < 32u * N; k += 32) {
                 if ((whole >> unit) & 1u) stack[static_cast<size_t>(32u * u) * N + k] = image[(32u * u + unit) * pitch + j];

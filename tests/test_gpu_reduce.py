@@ -355,3 +355,19 @@ def test_host_step_into_pinned_buffers(N, numel, dtype, opt, p, layout):
         assert (v.numpy().view(bits(h).dtype) == bits(h)).all()
         assert b[0] == 0x55 and (b[-4:] == 0x55).all()
     c.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("N", [2, 4, 5, 6, 8, 10, 12, 16, 20, 24])
+def test_coordinate_major_updates_copied_by_other_lanes(N, dtype):
+    """[P][N]: a lane's updated units leave through other lanes of its warp: several units a lane, many warps, ragged
+    ends.  The definition fixes every rounding, so the bits are the oracle's."""
+    c = Case(N, [40_003, 9, 256, 5], B.WASH_LAYOUT_PN, dtype, seed=N + 90)
+    for alpha in (0.9, 0.25):
+        B.papa_ema(c.gpu.ctx, B.WASH_STACK_PARAMS, alpha)
+        oracle.papa_ema(c.ora, c.host, alpha)
+        c.assert_equal("ema N=%d %s" % (N, dtype))
+    B.papa_all(c.gpu.ctx, B.WASH_STACK_PARAMS)
+    oracle.papa_all(c.ora, c.host)
+    c.assert_equal("papa_all N=%d %s" % (N, dtype))
+    c.close()
