@@ -371,3 +371,25 @@ def test_coordinate_major_updates_copied_by_other_lanes(N, dtype):
     oracle.papa_all(c.ora, c.host)
     c.assert_equal("papa_all N=%d %s" % (N, dtype))
     c.close()
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("N,dtype", [(2, "f32"), (3, "bf16"), (5, "f32"), (8, "f32"), (9, "f32"), (20, "bf16")])
+def test_consensus_distance_of_a_model_that_has_diverged(N, dtype, layout):
+    """An infinite value makes the mean infinite: the other models are infinitely far from it, its own distance is not
+    a number (infinity less infinity), and a NaN takes every model's distance with it; other ranges stay finite."""
+    numel = [600, 2048, 700]
+    dense = W.flat_population(N, sum(numel), seed=N).copy()
+    dense[1, 77] = np.inf
+    dense[0, 600 + 2048 + 5] = np.nan
+    c = Case(N, numel, layout, dtype, dense=dense)
+    want = np.stack([oracle.consensus_sq(c.ora, c.host, t, t + 1) for t in range(3)])
+    assert np.isinf(np.delete(want[0], 1)).all() and np.isnan(want[0, 1]) and np.isfinite(want[1]).all() and np.isnan(want[2]).all()
+    alone = torch.zeros(3, N, dtype=torch.float64, device="cuda")
+    for t in range(3):
+        B.wash_consensus_sq(c.gpu.ctx, B.WASH_STACK_PARAMS, t, t + 1, alone[t])
+    fused = torch.zeros(3, N, dtype=torch.float64, device="cuda")
+    B.wash_shuffle_consensus(c.gpu.ctx, B.WASH_STACK_PARAMS, 0, 0.3, None, seed=1, tensor_bounds=[0, 1, 2, 3], dev_sq_out=fused)
+    for got in (alone, fused):      # 2048 binary64 terms in another order: below 2048 * 2^-53 relative
+        assert np.allclose(got.cpu().numpy(), want, rtol=1e-12, atol=0, equal_nan=True)
+    c.close()
