@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(1024) sq_flush_kernel(double *slots, int count
         *hi = 0.0;
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, d);
-        if (lane == 0) out[j] += s;
+        if (lane == 0) atomicAdd(out + j, s);   // contexts on other streams may add to the same array
     }
 }
 

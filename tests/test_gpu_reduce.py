@@ -393,3 +393,24 @@ def test_consensus_distance_of_a_model_that_has_diverged(N, dtype, layout):
     for got in (alone, fused):      # 2048 binary64 terms in another order: below 2048 * 2^-53 relative
         assert np.allclose(got.cpu().numpy(), want, rtol=1e-12, atol=0, equal_nan=True)
     c.close()
+
+
+def test_consensus_distances_of_two_contexts_on_two_streams_add_up():
+    """Shards (contexts of their own) on streams of their own that add to one array: no term is lost.  Two models at -1 and
+    1: every coordinate adds 1 to each, exactly."""
+    numel, calls = [256], 400
+    stack = torch.ones(2, 256, device="cuda")
+    stack[1] = -1.0
+    shards = [B.Population(2, numel, B.WASH_LAYOUT_NP, 0) for _ in range(2)]
+    for s in shards:
+        s.bind(B.WASH_STACK_PARAMS, stack)
+    out = torch.zeros(2, dtype=torch.float64, device="cuda")
+    streams = [torch.cuda.Stream() for _ in shards]
+    torch.cuda.synchronize()
+    for _ in range(calls):
+        for s, stream in zip(shards, streams):
+            B.wash_consensus_sq(s.ctx, B.WASH_STACK_PARAMS, 0, 1, out, stream)
+    torch.cuda.synchronize()
+    assert (out.cpu().numpy() == 2.0 * calls * 256).all()
+    for s in shards:
+        s.close()
