@@ -157,7 +157,8 @@ int wash_layer_probs(int32_t L, double p, int32_t schedule, double *out);
  * coordinates are not written.
  *   step   < 2^56, the training step; seed: any 64-bit value.
  *   stats  DEVICE-accessible pointer (device memory or mapped pinned host memory) to a
- *          wash_stats the kernel atomically adds to; may be NULL.
+ *          wash_stats the kernel atomically adds to (counters in host memory cost one more
+ *          small kernel); may be NULL.
  * Errors: WASH_ERR_ARG (p out of range / NaN, step too large), WASH_ERR_STATE (stack
  * not bound), WASH_ERR_UNSUPPORTED, WASH_ERR_CUDA. */
 int wash_shuffle(wash_ctx *ctx, uint64_t step, double p, const double *p_layer,

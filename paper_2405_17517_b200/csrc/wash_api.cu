@@ -465,7 +465,7 @@ int wash_create_segments(wash_ctx **out, int32_t N, int32_t n_segments, const in
     if (err != cudaSuccess) { delete ctx; return cuda_fail(err, "cudaDeviceGetAttribute"); }
     ctx->shape.sm_count = sm_count;
     const size_t seg_bytes = sizeof(SegEntry) * static_cast<size_t>(n_segments);
-    const size_t slot_bytes = sizeof(wash::StatSlot) * wash::kStatSlots + sizeof(double) * wash::kSqSlots * wash::kMaxSqRanges * static_cast<size_t>(N);
+    const size_t slot_bytes = sizeof(wash::StatSlot) * (wash::kStatSlots + 1) + sizeof(double) * wash::kSqSlots * wash::kMaxSqRanges * static_cast<size_t>(N);
     if ((err = cudaMalloc(&ctx->seg_dev, seg_bytes)) != cudaSuccess ||
         (err = cudaMalloc(&ctx->tile_first_dev, sizeof(uint32_t) * ctx->n_tiles)) != cudaSuccess ||
         (err = cudaMalloc(&ctx->status_dev, sizeof(uint32_t))) != cudaSuccess ||
@@ -490,7 +490,7 @@ int wash_create_segments(wash_ctx **out, int32_t N, int32_t n_segments, const in
         release(ctx);
         return cuda_fail(err, "table upload");
     }
-    ctx->sq_slots_dev = reinterpret_cast<double *>(ctx->stat_slots_dev + wash::kStatSlots);
+    ctx->sq_slots_dev = reinterpret_cast<double *>(ctx->stat_slots_dev + wash::kStatSlots + 1);
     *out = ctx;
     return WASH_OK;
 }

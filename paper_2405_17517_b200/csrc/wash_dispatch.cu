@@ -54,6 +54,18 @@ __global__ void __launch_bounds__(kStatSlots) flush_stats_kernel(StatSlot *slots
     }
 }
 
+// Adds a launch's two counters, gathered on the device, to the caller's in host memory and zeroes them again.
+__global__ void __launch_bounds__(32) hand_over_stats_kernel(StatSlot *total, unsigned long long *stats)
+{
+    let_next_start();
+    await_previous();
+    if (threadIdx.x != 0 || total->selected == 0) return;
+    atomicAdd(stats, total->selected);
+    atomicAdd(stats + 1, total->moved);
+    total->selected = 0;
+    total->moved = 0;
+}
+
 // Adds the kSqSlots partial copies of the [range][model] table of squared distances into the
 // caller's array and leaves the slots zeroed for the next launch.  A warp per entry, a lane per two
 // copies (a thread that went through the copies of an entry one after the other took 64 round trips).
@@ -162,10 +174,23 @@ static cudaError_t launch_shuffle_kernel(const ShuffleArgs &args, int a_dtype, i
 cudaError_t launch_shuffle(const ShuffleArgs &args, int a_dtype, int b_dtype, int mode,
                            const LaunchShape &shape, cudaStream_t stream, bool *supported)
 {
+    // Counters in host memory: an atomic crosses PCIe and takes about a microsecond, one after the other, and a launch has
+    // hundreds of blocks that report (2^20 coordinates, N = 3: 437 us, 16 us with counters on the device; sparse 949 us).  Such a
+    // launch counts into the spare slot on the device, and one more kernel hands the two sums over.
+    ShuffleArgs call = args;
+    cudaPointerAttributes where;
+    bool hand_over = false;
+    if (args.stats) {
+        if (cudaPointerGetAttributes(&where, args.stats) != cudaSuccess) cudaGetLastError();
+        else hand_over = where.type != cudaMemoryTypeDevice;
+        if (hand_over) call.stats = &args.stat_slots[kStatSlots].selected;   // {selected, moved}
+    }
     bool flush = false;
-    cudaError_t err = launch_shuffle_kernel(args, a_dtype, b_dtype, mode, shape, stream, supported, &flush);
-    if (err != cudaSuccess || !*supported || !flush) return err;
-    return launch_chained(flush_stats_kernel, 1, kStatSlots, 0, stream, args.stat_slots, args.stats);
+    cudaError_t err = launch_shuffle_kernel(call, a_dtype, b_dtype, mode, shape, stream, supported, &flush);
+    if (err != cudaSuccess || !*supported) return err;
+    if (flush && (err = launch_chained(flush_stats_kernel, 1, kStatSlots, 0, stream, call.stat_slots, call.stats)) != cudaSuccess) return err;
+    if (hand_over) err = launch_chained(hand_over_stats_kernel, 1, 32, 0, stream, call.stat_slots + kStatSlots, args.stats);
+    return err;
 }
 
 cudaError_t launch_reduce(const ReduceArgs &args, int op, int dtype, int out_dtype, const LaunchShape &shape,

@@ -26,7 +26,8 @@ static_assert(sizeof(SegEntry) == 32, "SegEntry must stay 32 bytes");
 
 // Statistics are gathered in kStatSlots partial sums before they reach the caller's two
 // counters: per-block atomics on one address were measured to cost about 1 ns each and
-// to dominate the kernel once most blocks have a selected coordinate.
+// to dominate the kernel once most blocks have a selected coordinate.  One more slot gathers the sums of a launch whose
+// counters lie in host memory.
 constexpr int kStatSlots = 256;
 struct StatSlot {
     unsigned long long selected, moved;
@@ -81,7 +82,7 @@ struct ShuffleArgs {
     PhiloxKeys keys;              // from the seed
     uint32_t step_lo, step_hi8;   // step & 0xFFFFFFFF, (step >> 32) << 8
     unsigned long long *stats;    // device-accessible {selected, moved} or nullptr
-    StatSlot *stat_slots;         // device, kStatSlots zeroed entries (left zeroed by every launch)
+    StatSlot *stat_slots;         // device, kStatSlots + 1 zeroed entries (left zeroed by every launch)
     bool stats_direct = false;    // few blocks report: they add to `stats` themselves (kernels that need a flush kernel otherwise)
     uint32_t *status;             // device status word
     SqArgs sq;                    // consensus distance of the first stack (streaming kernel only)

@@ -29,7 +29,7 @@ constexpr long long kMaxRowElems = WASH_NOALLOC_MAX_ROW_ELEMS;
 constexpr size_t kMaxTiles = static_cast<size_t>(kMaxRowElems / 4) >> wash::kTileShift;
 constexpr size_t kSegBytes = sizeof(SegEntry) * kMaxTensors;          // 32 KiB
 constexpr size_t kTileBytes = sizeof(uint32_t) * kMaxTiles;           // 256 KiB
-constexpr size_t kSlotBytes = sizeof(wash::StatSlot) * wash::kStatSlots;   // 8 KiB
+constexpr size_t kSlotBytes = sizeof(wash::StatSlot) * (wash::kStatSlots + 1);   // 8 KiB
 constexpr size_t kScratchBytes = kSegBytes + kTileBytes + kSlotBytes;
 
 // The scratch itself.  In host code this name is only a handle for the runtime's symbol

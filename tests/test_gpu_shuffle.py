@@ -553,3 +553,47 @@ def test_calls_that_follow_each_other_at_once(captured):
     assert (to_host_bits(c.dev_opt) == bits(c.host_opt)).all()
     assert c.gpu_stats() == tuple(tot)
     c.close()
+
+
+@pytest.mark.parametrize("mode", [B.WASH_MODE_STREAM, B.WASH_MODE_SPARSE], ids=["stream", "sparse"])
+@pytest.mark.parametrize("N,p", [(2, 0.02), (5, 0.01), (8, 0.001), (20, 0.001), (20, 0.5)])
+def test_counters_in_mapped_host_memory(N, p, mode):
+    """The counts are the oracle's, call after call, and a launch does not pay an atomic over PCIe (a microsecond each) per
+    reporting block: with counters in pinned memory it takes no more than three times as long as with counters on the
+    device, plus 50 us (one more kernel and a few such atomics; with one per block it was 430 us and more)."""
+    numel = [400_001, 300]
+    c = Case(N, numel, seed=N)
+    B.wash_set_mode(c.gpu.ctx, mode)
+    pinned = torch.zeros(2, dtype=torch.int64).pin_memory()
+    want = np.zeros(2, dtype=np.int64)
+    for step in range(2):
+        B.wash_shuffle(c.gpu.ctx, step, p, None, seed=3, stats=pinned)
+        want += np.array(oracle.shuffle(c.ora, c.host, p, seed=3, step=step), dtype=np.int64)
+    c.assert_equal("N=%d" % N)
+    assert (pinned.numpy() == want).all()
+
+    def us(stats):
+        best = 1e9
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for i in range(10):
+                B.wash_shuffle(c.gpu.ctx, i, p, None, seed=3, stats=stats)
+            b.record()
+            b.synchronize()
+            best = min(best, 100.0 * a.elapsed_time(b))
+        return best
+    on_device, in_host_memory = us(c.stats_dev), us(pinned)
+    assert in_host_memory < 3 * on_device + 50, (in_host_memory, on_device)
+    c.close()
+
+
+def test_counters_in_mapped_host_memory_without_a_context():
+    for N, p in ((3, 0.02), (8, 0.001)):
+        c = Case(N, [300_001, 9], seed=N)
+        pinned = torch.zeros(2, dtype=torch.int64).pin_memory()
+        B.wash_shuffle_noalloc(N, c.numel, 0, B.WASH_F32, c.dev, c.dev.numel(), 5, p, None, seed=2, stats=pinned)
+        want = oracle.shuffle(c.ora, c.host, p, seed=2, step=5)
+        c.assert_equal("N=%d" % N)
+        assert tuple(pinned.tolist()) == tuple(want)
+        c.close()
