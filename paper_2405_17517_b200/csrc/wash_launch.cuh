@@ -17,7 +17,15 @@ namespace wash {
 // writes visible -- and let_next_start() at its beginning.  A kernel of another library before or
 // after ours, or a copy between two kernels, is ordered as always.
 __device__ __forceinline__ void await_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Called by the last blocks only: a release takes the launch unit about a nanosecond, a block after the other, which is more than
+// a block of the one-trip streaming kernel takes of the memory: five models, 2^24 coordinates, p = 1e-4 53 us without, 70 with a
+// release in every block, 51 from the last kReleasing.  A block that ends without it counts as released, so the next kernel
+// starts no later; no more blocks than these are resident at a time.
+constexpr unsigned kReleasing = 148 * 32;
+__device__ __forceinline__ void let_next_start()
+{
+    if (gridDim.x - blockIdx.x <= kReleasing) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 template <class... Params, class... Args>
 cudaError_t launch_chained(void (*kernel)(Params...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, const Args &...args)

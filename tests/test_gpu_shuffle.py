@@ -597,3 +597,34 @@ def test_counters_in_mapped_host_memory_without_a_context():
         c.assert_equal("N=%d" % N)
         assert tuple(pinned.tolist()) == tuple(want)
         c.close()
+
+
+@pytest.mark.parametrize("N,dtype,opt", [(5, "f32", None), (3, "bf16", "f32"), (10, "bf16", None)])
+def test_streaming_is_not_bound_by_the_launch_of_its_blocks(N, dtype, opt):
+    """A long row, few coordinates selected: the kernel reads the stacks once.  A copy of them (which reads and writes) is the
+    measure: half of its time is the bound, 0.50-0.52 was measured, 0.67-0.70 when every block released the next kernel."""
+    P = 1 << 24
+    pop = B.Population(N, [P], B.WASH_LAYOUT_NP, 0)
+    stacks = []
+    for role, dt in ((B.WASH_STACK_PARAMS, dtype), (B.WASH_STACK_OPT, opt)):
+        if dt:
+            stacks.append(torch.zeros(N * P, dtype=torch.float32 if dt == "f32" else torch.bfloat16, device="cuda"))
+            pop.bind(role, stacks[-1])
+    spare = [torch.empty_like(s) for s in stacks]
+    step = B.wash_shuffle_both if opt else B.wash_shuffle
+
+    def us(call):
+        best = 1e9
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for i in range(10):
+                call(i)
+            b.record()
+            b.synchronize()
+            best = min(best, 100.0 * a.elapsed_time(b))
+        return best
+    copied = us(lambda i: [d.copy_(s) for d, s in zip(spare, stacks)])
+    shuffled = us(lambda i: step(pop.ctx, i, 1e-4, None, seed=1))
+    assert shuffled < 0.61 * copied, (shuffled, copied)
+    pop.close()
