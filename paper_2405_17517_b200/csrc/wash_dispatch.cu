@@ -22,8 +22,8 @@ uint64_t launch_count() { return g_launches.load(std::memory_order_relaxed); }
 // compare-and-swap loops and cost this one-block kernel 20 us when 256 threads contended.)
 __global__ void __launch_bounds__(kStatSlots) flush_stats_kernel(StatSlot *slots, unsigned long long *stats)
 {
-    let_next_start();
     await_previous();
+    let_next_start();
     __shared__ unsigned long long part[2][kStatSlots / 32];
     unsigned long long sel = slots[threadIdx.x].selected, mov = slots[threadIdx.x].moved;
     if (sel) {
@@ -57,8 +57,8 @@ __global__ void __launch_bounds__(kStatSlots) flush_stats_kernel(StatSlot *slots
 // Adds a launch's two counters, gathered on the device, to the caller's in host memory and zeroes them again.
 __global__ void __launch_bounds__(32) hand_over_stats_kernel(StatSlot *total, unsigned long long *stats)
 {
-    let_next_start();
     await_previous();
+    let_next_start();
     if (threadIdx.x != 0 || total->selected == 0) return;
     atomicAdd(stats, total->selected);
     atomicAdd(stats + 1, total->moved);
@@ -71,8 +71,8 @@ __global__ void __launch_bounds__(32) hand_over_stats_kernel(StatSlot *total, un
 // copies (a thread that went through the copies of an entry one after the other took 64 round trips).
 __global__ void __launch_bounds__(1024) sq_flush_kernel(double *slots, int count, double *out)
 {
-    let_next_start();
     await_previous();
+    let_next_start();
     static_assert(kSqSlots == 64, "two copies per lane");
     const int lane = threadIdx.x & 31;
     for (int j = threadIdx.x >> 5; j < count; j += blockDim.x >> 5) {

@@ -14,14 +14,20 @@ namespace wash {
 // wait until the kernel before it in the stream has drained, its blocks may start as that one's
 // last blocks run.  In return every kernel calls await_previous() before it touches anything that an
 // earlier kernel may write or read -- which waits until the kernels before it are complete and their
-// writes visible -- and let_next_start() at its beginning.  A kernel of another library before or
-// after ours, or a copy between two kernels, is ordered as always.
-__device__ __forceinline__ void await_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// Called by the last blocks only: a release takes the launch unit about a nanosecond, a block after the other, which is more than
-// a block of the one-trip streaming kernel takes of the memory: five models, 2^24 coordinates, p = 1e-4 53 us without, 70 with a
-// release in every block, 51 from the last kReleasing.  A block that ends without it counts as released, so the next kernel
-// starts no later; no more blocks than these are resident at a time.
+// writes visible.  A kernel of another library launched in the ordinary way, or a copy, is ordered as always; one that is
+// itself launched as a programmatic dependent has to wait, too, before it reads a stack (include/wash.h says so).
+//
+// let_next_start() allows the next kernel's blocks to be placed.  Two rules for where it is called:
+//   after await_previous(): called before, a chain of short launches piles up, kernel after kernel resident and waiting, and the
+//     blocks of the one whose turn comes sit several to an SM (EMA of 16 bf16 models, 2^17 coordinates, back to back
+//     7.2 us without programmatic launches, 13.9 released first, 6.4 released after the wait; 20 models, [P][N] 8.3, 20.6, 10.2).
+//     Kernels whose work before the wait is what the overlap is for say so themselves.
+//   by the last blocks only: a release takes the launch unit about a nanosecond, a block after the other, which is more than
+//     a block of the one-trip streaming kernel takes of the memory: five models, 2^24 coordinates, p = 1e-4 53 us without, 70
+//     with a release in every block, 51 from the last kReleasing.  A block that ends without it counts as released, so the
+//     next kernel starts no later; no more blocks than these are resident at a time.
 constexpr unsigned kReleasing = 148 * 32;
+__device__ __forceinline__ void await_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_start()
 {
     if (gridDim.x - blockIdx.x <= kReleasing) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -76,8 +76,8 @@ __device__ __forceinline__ void store_average(const ReduceArgs &a, uint64_t unit
 template <class T, class TOUT, int OP, int N>
 __global__ void __launch_bounds__(256) regs_np_kernel(const __grid_constant__ ReduceArgs a)
 {
-    let_next_start();
     await_previous();
+    let_next_start();
     constexpr int kElems = Unit<T>::kElems;
     const uint64_t unit = a.group_lo / Unit<T>::kGroups + static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (unit * Unit<T>::kGroups >= a.group_hi) return;
@@ -125,8 +125,8 @@ __global__ void __launch_bounds__(256) regs_np_kernel(const __grid_constant__ Re
 template <class T, class TOUT, int OP>
 __global__ void __launch_bounds__(64, 20) staged_np_kernel(const __grid_constant__ ReduceArgs a, int per_thread)
 {
-    let_next_start();
     await_previous();
+    let_next_start();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr int kElems = Unit<T>::kElems;
     const int n_models = a.pop.N;
@@ -209,8 +209,8 @@ __global__ void __launch_bounds__(64, 20) staged_np_kernel(const __grid_constant
 template <class T, class TOUT, int OP, int kN>
 __global__ void __launch_bounds__(64, 16) dense_pn_kernel(const __grid_constant__ ReduceArgs a, int per_thread)
 {
-    let_next_start();
     await_previous();
+    let_next_start();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr int kElems = Unit<T>::kElems;
     const uint32_t N = kN ? kN : static_cast<uint32_t>(a.pop.N), pitch = N | 1u;

@@ -732,8 +732,8 @@ template <class TA, class TB, int LAYOUT, int G, bool STAT, bool EARLY, int kN>
 __global__ void __launch_bounds__(256, EARLY ? 3 : (kN > 6 ? 4 : 5)) shuffle_async_kernel(const __grid_constant__ ShuffleArgs a)
 {
     if constexpr (kN != 0) __builtin_assume(a.pop.N == kN);
-    let_next_start();
     await_previous();
+    let_next_start();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr bool kHasB = TB::kCode != kDtypeNone;
     const int n_models = kN ? kN : a.pop.N;

@@ -131,8 +131,8 @@ template <class TA, class TB, int LAYOUT, int G, int kN>
 __global__ void __launch_bounds__(32, G == 2 ? 32 : 28) shuffle_loop_kernel(const __grid_constant__ ShuffleArgs a)
 {
     if constexpr (kN != 0) __builtin_assume(a.pop.N == kN);
-    let_next_start();
     await_previous();
+    let_next_start();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr bool kHasB = TB::kCode != kDtypeNone;
     constexpr uint32_t T_ = 32;   // the launch has one warp per block

@@ -38,6 +38,12 @@ constexpr int kSparsePairs = 4;      // (coordinate, model) pairs a lane has in 
 // 710 / 686; N = 24, 2^23, 2 % 146 / 177, 5 % 266 / 277; N = 28 2 % 173 / 216, 10 % 421 / 389; N = 32, 2^24, 1 % 266 / 265, 10 % 1417 / 901, all
 // 5830 / 1927; N = 5 30 % 338 / 421.
 constexpr float kRowsShare = 0.25f, kRowsShareLarge = 0.06f;   // 8 to 23 models, 24 and more
+// Selected values per coordinate (of all models and stacks) up to which the next kernel may start at once: while masks
+// are most of the time, the next launch of this kernel draws its own beside this one's last; where values are, its waiting blocks
+// are in the way.  Back to back, released early / after the wait: N = 2, 2^23 coordinates, p = 1e-3 (0.002) 7.4 / 9.1 us, ResNet-18 N = 5 with
+// momentum (0.01) 10.5 / 12.7, N = 5, 2^23, p = 0.01 (0.05) 10.2 / 12.4, ResNet-50 N = 5, p = 0.05 -> 0 (0.12) 42.7 / 45.6; N = 20, 2^20, p = 0.01 (0.2)
+// 9.2 / 7.2, N = 32, 2^20, p = 0.01 (0.32) 23.5 / 16.6, N = 5, 2^20, p = 0.1 (0.5) 8.7 / 6.0.
+constexpr double kReleaseShare = 0.15;
 constexpr double kSparsePerBlock = 16.0;   // selected coordinates a block expects, at least
 
 // entries of the queue: a permutation of up to 16 models stays in its entry (8 bytes), a larger one
@@ -48,6 +54,7 @@ struct SparseArgs {
     ShuffleArgs s;
     uint32_t n_wtiles;      // warp tiles in [group_lo, group_hi)
     uint32_t per_block, extra;   // tiles of a block: per_block, one more in the first `extra` blocks
+    bool release_early;     // the next kernel may start with this one's masks
     uint32_t in_set;        // coordinates whose N values a warp moves at a time: 32 * kSparsePairs / N
     uint32_t column_offset; // ROWS: where the lanes' columns lie in shared memory
     uint32_t inverse;       // 2^16 / d, rounded up, for the division of a pair's number (below 128) by in_set ([N][P]) or N ([P][N])
@@ -73,7 +80,7 @@ __device__ __forceinline__ void serve_row(const PopView &pop, void *stack, uint3
 template <class TA, class TB, int LAYOUT, bool MIRROR, bool ROWS>
 __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_sparse_kernel(const __grid_constant__ SparseArgs p)
 {
-    let_next_start();
+    if (p.release_early) let_next_start();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ uint32_t s_count;
     constexpr bool kHasB = TB::kCode != kDtypeNone;
@@ -120,6 +127,7 @@ __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_spa
         const bool again = __syncthreads_or(sel != 0 || t < t_end);   // (orders the queue's entries, too)
         const uint32_t count = min(s_count, capacity);
         await_previous();   // the masks read nothing but the tables; the stacks come now
+        if (!p.release_early) let_next_start();
         if (n_models <= 16) {
             for (uint32_t e = threadIdx.x; e < count; e += kSparseThreads) {
                 const uint2 key = q_key[e];
@@ -248,6 +256,7 @@ cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchSha
     if (grid > want) grid = want;
     p.per_block = p.n_wtiles / grid;
     p.extra = p.n_wtiles % grid;
+    p.release_early = static_cast<double>(args.expected_share) * args.pop.N * (one_stack ? 1 : 2) <= kReleaseShare;
     p.in_set = 32u * kSparsePairs / static_cast<uint32_t>(args.pop.N);
     const uint32_t divisor = args.pop.layout == kLayoutNP ? p.in_set : static_cast<uint32_t>(args.pop.N);
     p.inverse = (65536u + divisor - 1u) / divisor;

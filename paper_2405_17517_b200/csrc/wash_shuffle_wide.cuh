@@ -36,8 +36,8 @@ __device__ __forceinline__ void move_value(const ShuffleArgs &a, const unsigned 
 template <class TA, class TB, int LAYOUT, bool STAT>
 __global__ void __launch_bounds__(64, 6) shuffle_wide_kernel(const __grid_constant__ ShuffleArgs a)
 {
-    let_next_start();
     await_previous();
+    let_next_start();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr bool kHasB = TB::kCode != kDtypeNone;
     const int n_models = a.pop.N;
@@ -129,8 +129,8 @@ constexpr uint32_t kWideRound = 16;   // coordinates of a warp's round
 template <class TA, class TB>
 __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_constant__ ShuffleArgs a)
 {
-    let_next_start();
     await_previous();
+    let_next_start();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ uint32_t s_count;
     constexpr int LAYOUT = kLayoutPN;
