@@ -81,6 +81,12 @@ __device__ __forceinline__ void block_range(const ExchangeArgs &a, uint32_t *t0,
     *t1 = static_cast<uint32_t>((static_cast<uint64_t>(blockIdx.x) + 1) * a.n_wtiles / a.n_blocks);
 }
 
+// A short row, a tile a warp: its three kernels leave room on the SMs and are bound by their starts, so each releases the next at
+// once; on a long row waiting blocks are in the way of the running ones.  Plan, send and receive, all released at once / all after
+// the wait / the plan alone at once: 2^17 coordinates, N = 20, p = 0.1 16.9 / 23.2 / 23.4 us; 2^20, N = 32, p = 0.1 39.2 / 40.5 / 58.5; 2^24,
+// p = 0.01, N = 5 40.9 / 37.5, N = 64 166 / 134.
+__device__ __forceinline__ bool short_row(const ExchangeArgs &a) { return a.n_wtiles <= a.n_blocks * static_cast<uint32_t>(kExchangeWarps); }
+
 // The plan's block queue, as the sparse shuffle's: the coordinates its warps find, in any order (the
 // counts do not depend on it), drawn a thread each when a piece of the range is done or the queue full.
 constexpr uint32_t kPlanQueue = 1024;
@@ -105,9 +111,7 @@ __global__ void __launch_bounds__(kXThreads, kExchangeBlocksPerSm) exchange_plan
     if (threadIdx.x == 0) s_count = 0;
     uint32_t t_first, t_end;
     block_range(a, &t_first, &t_end);
-    // The send may be placed beside a plan that leaves room on the SMs (a short row: a tile a warp), else after the wait: 2^17
-    // coordinates, N = 20, p = 0.1, plan, send and receive released early / late 17 / 23 us; 2^24, p = 0.01, N = 5 40.9 / 37.5, N = 64 167 / 134.
-    const bool release_early = t_end - t_first <= static_cast<uint32_t>(kExchangeWarps);
+    const bool release_early = short_row(a);
     if (release_early) let_next_start();
     const uint32_t pieces = (t_end - t_first + kPlanHeldTiles - 1u) / kPlanHeldTiles, per_piece = pieces ? (t_end - t_first + pieces - 1u) / pieces : 0u;
     LaneSegment ls;
@@ -231,8 +235,10 @@ __device__ __forceinline__ uint32_t fill_list(const ExchangeArgs &a, CoordList &
 
 __global__ void __launch_bounds__(kXThreads) exchange_send_kernel(const __grid_constant__ ExchangeArgs a)
 {
+    const bool release_early = short_row(a);
+    if (release_early) let_next_start();
     await_previous();
-    let_next_start();
+    if (!release_early) let_next_start();
     extern __shared__ uint32_t s_perm_all[];
     __shared__ CoordList list;
     __shared__ uint32_t s_base[kMaxN], s_votes[kExchangeWarps][kMaxN];
@@ -309,8 +315,10 @@ __global__ void __launch_bounds__(kXThreads) exchange_send_kernel(const __grid_c
 
 __global__ void __launch_bounds__(kXThreads) exchange_receive_kernel(const __grid_constant__ ExchangeArgs a)
 {
+    const bool release_early = short_row(a);
+    if (release_early) let_next_start();
     await_previous();
-    let_next_start();
+    if (!release_early) let_next_start();
     __shared__ CoordList list;
     __shared__ uint32_t s_part[kExchangeWarps];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
