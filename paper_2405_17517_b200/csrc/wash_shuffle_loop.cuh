@@ -24,7 +24,8 @@
 // swap chains and row addresses then need no loop control or multiplications (run-time N -> compiled in: N = 2,
 // 2^27 coordinates p = 1e-2 236 -> 216 us, 1e-3 205 -> 195; 2^25 coordinates: N = 2 [P][N] p = 0.1 94.0 -> 81.0, N = 3
 // p = 1e-2 85.4 -> 82.4 (bf16 78.6 -> 70.4), N = 4 bf16 88.9 -> 79.9, N = 5 144.7 -> 137.9; N = 3, 2^20 7.49 -> 7.07).
-// Larger populations move more bytes for the same control.
+// Larger populations move more bytes for the same control.  The narrow form (two groups a lane) likewise: 2^27 coordinates,
+// p = 1e-4, N = 2 174 -> 170, bf16 205 -> 169, N = 3 257 -> 248, bf16 223 -> 198; N = 5 bf16, 2^24, 34.9 -> 32.7.
 //
 // An image of a stage is the one-trip kernel's block image with T = 32 (the block is one warp,
 // so every helper of that kernel -- copies, serving, padding rule -- is used as it is).
@@ -287,7 +288,13 @@ cudaError_t launch_shuffle_loop_typed(const ShuffleArgs &args, const LaunchShape
     // (A forced launch may bring groups of any size: beyond kLoopFourMaxGroupBytes four of them leave too few warps.)
     const size_t per_group = static_cast<size_t>(args.pop.N) * 4 * (TA::kBytes + TB::kBytes);
     if (args.expected_share < kLoopNarrowShare || per_group > kLoopFourMaxGroupBytes)
-        return launch_shuffle_loop_tiles<TA, TB, 2, 0>(args, shape, stream);
+        switch (args.pop.N) {
+        case 2: return launch_shuffle_loop_tiles<TA, TB, 2, 2>(args, shape, stream);
+        case 3: return launch_shuffle_loop_tiles<TA, TB, 2, 3>(args, shape, stream);
+        case 4: return launch_shuffle_loop_tiles<TA, TB, 2, 4>(args, shape, stream);
+        case 5: return launch_shuffle_loop_tiles<TA, TB, 2, 5>(args, shape, stream);
+        default: return launch_shuffle_loop_tiles<TA, TB, 2, 0>(args, shape, stream);
+        }
     switch (args.pop.N) {
     case 2: return launch_shuffle_loop_tiles<TA, TB, 4, 2>(args, shape, stream);
     case 3: return launch_shuffle_loop_tiles<TA, TB, 4, 3>(args, shape, stream);
