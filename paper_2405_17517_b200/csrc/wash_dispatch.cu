@@ -129,6 +129,8 @@ cudaError_t launch_philox_probe(unsigned long long n_blocks, uint64_t seed, uint
 // to kLoopMaxGroupBytes while at most kLoopMaxShare is expected to be selected; larger groups only where serving, which it
 // does once per four groups of a lane, weighs most against its fewer resident warps.  Its time over the one-trip
 // kernel's, 2^24 coordinates, at 0.3 / 0.5 / 1 / 2 / 5 / 8 / 12 %:
+//   32-48     bf16 [P][N], whose values are picked out of the image two bytes at a time: N = 4 at 15 / 20 / 30 % .91 1.08 1.09, N = 5 at
+//             10 / 13 / 20 / 30 % .82 .99 1.27 1.29, N = 6 .96 1.11 1.43 1.44
 //   64 bytes  fp32 N = 4  [N][P] .97 .89 .81 .83 .94 1.01 1.06   [P][N] .97 .87 .72 .66 .75 .87 .94   (two stacks of N = 2 alike)
 //             bf16 N = 8  [N][P] .94 .80 .65 .70 .76 .77 .87     [P][N] .97 .89 .78 .71 .91 1.11 1.23
 //   80        fp32 N = 5  [N][P] .89 .90 .89 .91 1.01 1.09 1.16  [P][N] .88 .87 .78 .73 .80 .92 1.05
@@ -139,7 +141,7 @@ cudaError_t launch_philox_probe(unsigned long long n_blocks, uint64_t seed, uint
 static bool resident_warps_pay(size_t per_group, int layout, bool bf16, bool two_stacks, float share)
 {
     const bool np = layout == kLayoutNP, one_bf16 = bf16 && !two_stacks;
-    if (per_group <= kLoopMaxGroupBytes) return share <= kLoopMaxShare;
+    if (per_group <= kLoopMaxGroupBytes) return share <= (one_bf16 && !np && per_group >= 32 ? 5.2f / per_group : kLoopMaxShare);
     if (per_group <= 64) return share >= 0.003f && share <= (one_bf16 ? (np ? 0.12f : 0.06f) : (np ? 0.07f : 0.12f));
     if (per_group > 96) return false;
     if (two_stacks) return !np && share >= 0.008f && share <= 0.03f;
