@@ -50,6 +50,9 @@ constexpr double kSparsePerBlock = 16.0;   // selected coordinates a block expec
 // takes wide_pitch(N) words beside it
 __host__ __device__ constexpr uint32_t sparse_queue_capacity(int n_models) { return n_models <= 32 ? 512u : 256u; }
 
+// list of a warp of the form for dense selections: a tile's 512 coordinates and what the tile before left
+constexpr uint32_t kWarpList = 512 + 32;
+
 struct SparseArgs {
     ShuffleArgs s;
     uint32_t n_wtiles;      // warp tiles in [group_lo, group_hi)
@@ -212,6 +215,105 @@ __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_spa
     publish_block_stats(a.stats, a.stats_direct ? nullptr : a.stat_slots, selected, moved);
 }
 
+// Where much is selected: a warp by itself, without the block's barriers.  It lists a tile's selected coordinates in order behind
+// the few left over from the tile before and serves them 32 at a time, a lane per coordinate (serve_row), so that
+// one warp's mask, another's loads and a third one's stores run beside each other all the time.
+template <class TA, class TB, int LAYOUT>
+__global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_sparse_warps_kernel(const __grid_constant__ SparseArgs p)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    constexpr bool kHasB = TB::kCode != kDtypeNone;
+    const ShuffleArgs &a = p.s;
+    const int n_models = a.pop.N;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    // [a list per warp: row elements, counted from the first of the warp's range][a column of N words per thread][N > 16: 32 permutations per warp]
+    uint32_t *list = reinterpret_cast<uint32_t *>(smem_raw) + warp * kWarpList;
+    uint32_t *columns = reinterpret_cast<uint32_t *>(smem_raw) + kSparseWarps * kWarpList;
+    uint32_t *column = columns + threadIdx.x, *s_perm = columns + n_models * kSparseThreads + warp * 32u * wide_pitch(n_models);
+
+    const uint64_t range = blockIdx.x * kSparseWarps + warp, ranges = static_cast<uint64_t>(gridDim.x) * kSparseWarps;
+    const uint32_t t_first = static_cast<uint32_t>(range * p.n_wtiles / ranges), t_end = static_cast<uint32_t>((range + 1) * p.n_wtiles / ranges);
+    const uint32_t first_group = a.group_lo + t_first * kWarpTileGroups;
+    uint32_t selected = 0, moved = 0, length = 0;
+    LaneSegment ls, served;
+    bool waited = false;
+    for (uint32_t t = t_first; t < t_end; ++t) {
+        const uint32_t g0 = a.group_lo + t * kWarpTileGroups + 4u * lane;
+        uint32_t sel = lane_masks(a, g0, a.group_hi, ls), in_tile = 0;
+        uint32_t pos = length + warp_exclusive_scan(__popc(sel), &in_tile);
+        for (; sel; sel &= sel - 1u, ++pos) list[pos] = 4u * (g0 - first_group) + static_cast<uint32_t>(__ffs(sel) - 1);
+        length += in_tile;
+        __syncwarp();
+        if (length < 32u && t + 1 < t_end) continue;
+        if (!waited) {   // the masks read nothing but the tables; the stacks come now
+            await_previous();
+            let_next_start();
+            waited = true;
+        }
+        uint32_t done = 0;
+        while (length - done >= 32u || (t + 1 == t_end && done < length)) {
+            const uint32_t count = min(32u, length - done);
+            const bool active = lane < count;
+            const long long elem = 4ll * first_group + list[done + min(lane, count - 1u)];
+            const uint32_t g = static_cast<uint32_t>(elem >> 2);
+            if (g - served.begin >= served.end - served.begin) lane_segment_load(a, g, a.group_hi, served);
+            const uint32_t coord = 4u * (g + served.cgroup_off) + static_cast<uint32_t>(elem & 3);
+            __syncwarp();
+            uint64_t packed = 0;
+            if (n_models > 16) draw_permutations_by_warp(s_perm, n_models, count, coord, served.tensor, a.step_lo, a.step_hi8, a.keys);
+            else if (active) packed = draw_permutation_packed(n_models, coord, served.tensor, a.step_lo, a.step_hi8, a.keys);
+            if (active) {
+                const uint8_t *wide = reinterpret_cast<const uint8_t *>(s_perm + lane * wide_pitch(n_models));
+                const auto source_of = [&](int n) -> uint32_t { return n_models <= 16 ? static_cast<uint32_t>(packed >> (4 * n)) & 15u : wide[n]; };
+                serve_row<TA, LAYOUT>(a.pop, a.a, column, elem, source_of);
+                if constexpr (kHasB) serve_row<TB, LAYOUT>(a.pop, a.b, column, elem, source_of);
+                for (int n = 0; n < n_models; ++n) moved += source_of(n) != static_cast<uint32_t>(n) ? 1u : 0u;
+                ++selected;
+            }
+            __syncwarp();
+            done += count;
+        }
+        const uint32_t rest = length - done;   // fewer than 32: to the front of the list
+        const uint32_t keep = lane < rest ? list[done + lane] : 0u;
+        __syncwarp();
+        if (lane < rest) list[lane] = keep;
+        length = rest;
+        __syncwarp();
+    }
+    if (!waited) {   // a block's end without the wait would let later kernels pass the one before this
+        await_previous();
+        let_next_start();
+    }
+    publish_block_stats(a.stats, a.stats_direct ? nullptr : a.stat_slots, selected, moved);
+}
+
+// Which selections shuffle_sparse_warps_kernel serves.  Time by pairs (by rows of the block's queue: r) / by warps:
+//   [P][N], one stack: a lane takes a coordinate's N neighbouring values itself, so where most of them move the queue's
+//     reading per pair is what it saves.  2^24 coordinates, fp32: N = 3 20 % 77 / 86, 30 % 110 / 105, all 258 / 228; 4 15 % 78 / 75, 2^27 10 %
+//     450 / 430; 5 20 % 106 / 120, 30 % 147 / 145, 50 % 210 / 187; 8 20 % 138 / 133, all 511 / 368; 10 30 % 251 / 231; 12 30 % 283 / 293,
+//     50 % 422 / 393; 14 (2^23) 50 % 254 / 288, all 440 / 388; 16 all 954 / 1197.  N = 2 2^24 10 % 44 / 43, 20 % 59 / 64, 30 % 90 / 83,
+//     2^27 8 % 272 / 256, 10 % 343 / 289, 20 % 470 / 440.
+//     bf16: N = 2 10 % 43 / 40, 3 15 % 56 / 57, 5 20 % 93 / 98, 30 % 136 / 118, 8 30 % 184 / 203, 50 % 281 / 223, 10 50 % 358 / 361, all 646 / 449.
+//     Two stacks by pairs throughout (N = 7 all 281 / 294, N = 5 407 / 403).
+//   [N][P]: from 18 models on in between, where pairs fill a fraction of a sector and rows wait for the block; with the shared
+//     memory held to kWarpsCarveout so that the L1 keeps the sectors that neighbouring coordinates share (N = 20, 15 %, 2^23 333 us without, 280
+//     with; 32 509 / 407; a larger L1 yet loses resident warps, 270 and 435).  N = 18 6 % 192 / 197, 15 % 244 / 235, 30 % r 308 / 281;
+//     20 15 % 280 / 280, 30 % r 346 / 284, 50 % r 390 / 368; 24 6 % 295 / 260, 15 % r 363 / 301, 50 % r 454 / 448; 32 6 % r 402 / 348,
+//     30 % r 557 / 489, 50 % r 627 / 673; 48 6 % r 582 / 534, 15 % r 763 / 692, 30 % r 817 / 934; 64 15 % r 1019 / 958, 30 % r 1109 / 1410;
+//     bf16 + fp32 20 15 % 599 / 450, 24 30 % r 638 / 540.
+constexpr int kWarpsCarveout = 132 * 100 / 228;   // per cent of the largest shared memory
+inline bool sparse_by_warps(const ShuffleArgs &args, bool bf16, bool two_stacks)
+{
+    const int N = args.pop.N;
+    const float share = args.expected_share;
+    if (args.pop.layout == kLayoutNP) return N >= 18 && share >= (N < 40 ? 0.05f : 0.025f) && share < (N < 40 ? 0.4f : 0.12f);
+    if (two_stacks) return false;
+    if (bf16) return N <= 12 && share >= (N <= 3 ? 0.1f : N <= 6 ? 0.25f : N <= 9 ? 0.4f : 0.7f);
+    if (N == 2 && args.pop.n_groups >= 1u << 24) return share >= 0.08f;
+    if (N == 4 || N == 8) return share >= 0.15f;   // a coordinate's values are whole 16-byte pieces
+    return N <= 15 && share >= (N <= 3 ? 0.25f : N <= 10 ? 0.3f : N <= 12 ? 0.4f : 0.7f);
+}
+
 template <class TA, class TB>
 cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchShape &shape, cudaStream_t stream)
 {
@@ -227,6 +329,24 @@ cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchSha
         kernel = shuffle_sparse_kernel<TA, TB, kLayoutNP, false, true>;
         p.column_offset = static_cast<uint32_t>(smem);
         smem += 4 * static_cast<size_t>(args.pop.N) * kSparseThreads;
+    }
+    if (!args.mirror_a && sparse_by_warps(args, TA::kBytes == 2, TB::kCode != kDtypeNone)) {
+        auto by_warps = np ? shuffle_sparse_warps_kernel<TA, TB, kLayoutNP> : shuffle_sparse_warps_kernel<TA, TB, kLayoutPN>;
+        smem = 4 * kSparseWarps * static_cast<size_t>(kWarpList) + 4 * static_cast<size_t>(args.pop.N) * kSparseThreads +
+               (args.pop.N > 16 ? 4 * static_cast<size_t>(wide_pitch(args.pop.N)) * kSparseThreads : 0);
+        KernelFit fit;
+        cudaError_t err = kernel_fit(reinterpret_cast<const void *>(by_warps), kSparseThreads, smem, &fit);
+        if (err == cudaSuccess && np) err = cudaFuncSetAttribute(reinterpret_cast<const void *>(by_warps), cudaFuncAttributePreferredSharedMemoryCarveout, kWarpsCarveout);
+        if (err != cudaSuccess) return err;
+        if (fit.occupancy < 1) return cudaErrorLaunchOutOfResources;
+        // four waves, as far as a warp keeps two tiles: ranges that select unequally even out
+        const uint32_t wave = static_cast<uint32_t>(shape.sm_count > 0 ? shape.sm_count : 148) * static_cast<uint32_t>(fit.occupancy);
+        uint32_t grid = p.n_wtiles / (2 * kSparseWarps);
+        if (grid > 4 * wave) grid = 4 * wave;
+        if (grid < wave) grid = wave;
+        const uint32_t want = (p.n_wtiles + kSparseWarps - 1) / kSparseWarps;
+        if (grid > want) grid = want;
+        return launch_chained(by_warps, grid, kSparseThreads, smem, stream, p);
     }
     KernelFit fit;
     cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), kSparseThreads, smem, &fit);

@@ -653,3 +653,22 @@ def test_short_launches_that_follow_each_other_stay_spread_over_the_gpu():
         apart = us(lambda: (B.papa_ema(c.gpu.ctx, 0, 0.9), scratch.zero_())) - us(lambda: scratch.zero_())
         assert chained < 1.3 * apart + 1.0, (N, chained, apart)
         c.close()
+
+
+@pytest.mark.parametrize("N,layout,numel,p,dtype,opt", [
+    (2, 1, [70_001, 9], 0.3, "f32", None), (3, 1, [511], 1.0, "f32", None), (4, 1, [2_000_003, 33], 0.16, "f32", None), (5, 1, [512, 7], 0.9, "bf16", None),
+    (8, 1, [100_003], 0.45, "bf16", None), (10, 1, [513, 60_001], 0.31, "f32", None), (12, 1, [30_001, 1, 5], 1.0, "bf16", None), (15, 1, [40_001], 0.8, "f32", None),
+    (18, 0, [200_001, 31], 0.06, "f32", None), (20, 0, [2_047, 90_001], 0.2, "bf16", "f32"), (32, 0, [100_003], 0.39, "bf16", None), (33, 0, [65_537, 9], 0.1, "f32", "f32"),
+    (64, 0, [70_003], 0.026, "f32", None), (64, 0, [511], 0.1, "bf16", "bf16")])
+def test_sparse_warps_that_serve_by_themselves(N, layout, numel, p, dtype, opt):
+    """Dense selections of the sparse kernel, a warp's list from tile to tile: lists of a full tile and none, ranges that
+    end inside a tile and a tensor, more warps than tiles, permutations packed and in shared memory; also twice in a row."""
+    c = Case(N, numel, layout, dtype, opt, seed=N + 3)
+    B.wash_set_mode(c.gpu.ctx, B.WASH_MODE_SPARSE)
+    want = np.zeros(2, dtype=np.int64)
+    for step in (0, 1):
+        (B.wash_shuffle_both if opt else B.wash_shuffle)(c.gpu.ctx, step, p, None, seed=21, stats=c.stats_dev)
+        want += np.array(oracle.shuffle(c.ora, c.host, p, seed=21, step=step, stack2=c.host_opt), dtype=np.int64)
+    c.assert_equal("N=%d layout=%d p=%g" % (N, layout, p))
+    assert c.gpu_stats() == tuple(want)
+    c.close()
