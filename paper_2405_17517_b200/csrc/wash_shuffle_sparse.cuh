@@ -47,8 +47,9 @@ constexpr double kReleaseShare = 0.15;
 constexpr double kSparsePerBlock = 16.0;   // selected coordinates a block expects, at least
 
 // entries of the queue: a permutation of up to 16 models stays in its entry (8 bytes), a larger one
-// takes wide_pitch(N) words beside it
-__host__ __device__ constexpr uint32_t sparse_queue_capacity(int n_models) { return n_models <= 32 ? 512u : 256u; }
+// takes wide_pitch(N) words beside it.  Half as many from 29 models on: eight blocks would leave the L1 28 KB and the sectors that
+// neighbouring coordinates share would not stay (6.3e6 coordinates, 1 %: N = 28 85 us, 29 113, 33 with 256 entries 97).
+__host__ __device__ constexpr uint32_t sparse_queue_capacity(int n_models) { return n_models <= 28 ? 512u : 256u; }
 
 // list of a warp of the form for dense selections: a tile's 512 coordinates and what the tile before left
 constexpr uint32_t kWarpList = 512 + 32;
