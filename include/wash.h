@@ -62,12 +62,13 @@ enum wash_mode {
     WASH_MODE_SPARSE = 1, /* draws the mask first; touches only selected coordinates          */
     WASH_MODE_AUTO = 2             /* SPARSE when the call's probabilities select, in expectation,
                                       less than a share of the coordinates that depends on layout,
-                                      N and the number of stacks, else STREAM.  [N][padded_P]:
-                                      60 % / N for one stack, 35 % / N for two, 18 % at most;
-                                      [padded_P][N]: 13 % to 40 %, growing with N (the measured
-                                      crossovers on B200: in the second layout the N values of a
-                                      coordinate share a DRAM access; a small population leaves
-                                      the streaming kernels bound by issue slots)                */
+                                      N, the number of stacks and their type, else STREAM.
+                                      [N][padded_P]: 18 % (N = 2) falling to 2 %; two stacks 20 %
+                                      falling to 1.8 %.  [padded_P][N]: 13 % to 50 %, two stacks
+                                      20 % to 60 % (the measured crossovers on B200: in the second
+                                      layout the N values of a coordinate share a DRAM access; a
+                                      small population leaves the streaming kernels bound by issue
+                                      slots)                                                     */
 };
 
 #define WASH_MAX_N 64            /* largest population                                     */

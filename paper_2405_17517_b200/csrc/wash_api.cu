@@ -200,17 +200,28 @@ uint64_t threshold_of(double p) { return static_cast<uint64_t>(std::floor(p * 42
 // WASH_MODE_AUTO: the expected share of selected coordinates up to which the sparse kernel is launched.  Serving a
 // coordinate costs it a scattered DRAM access and store per model and stack in [N][P], a few neighbouring ones for
 // all N models in [P][N]; the streaming kernels pay for the stack's bytes and, in small populations, for issue slots.
-// Measured crossovers (2^24-2^25 coordinates):
-//   [N][P]  one stack   fp32 N = 2 18 %, 3 14 %, 4 15 %, 5 12 %, 8 6 %, 12 5 %, 16 4.7 %, 20 5 %, 32 2 %; bf16 18, 16, 19, 11, 15, 10, 7.5, 3, 1 %
-//           two stacks  fp32 N = 2 20 %, 5 6 %, 16 3 %, 32 1.8 %; bf16 + fp32 21, 5, 2.8, 1.3 %
-//   [P][N]  one stack   fp32 N = 2 14 %, 3 13 %, 4 15 %, 5 16 %, 6 21 %, 8 22 %, 12 23 %, 16 40 %, 20 35 %, 32 above 50 %; bf16 13, 12, 19, 27, 28, 38, 48, 20, 33 %
-//           two stacks  fp32 N = 2 23 %, 5 20 %, 16 and 32 above 50 %; bf16 + fp32 20, 30, above 50 %
+// The share at which their times meet (1.5e7 coordinates, 7e6 from N = 20 on, 4e6 at 64; "to 50 %": within 5 % of each other
+// or better up to there), by N:
+//   [N][P]  one stack   fp32  2: 13 %, 3: 16, 4: 16, 5: 14, 6: 12, 8: 5.5, 10: 5.5, 12: 5, 16: 4.5, 20: 4, 24: 3.5, 32: 4, 64: 2.7
+//                       bf16  2: 13, 3: 20, 4: 18, 5: 8, 6: 8 (then level to 20), 8: 8, 10: 8, 12: 6.2, 16: 6.3, 20: 2.7, 24: 2, 32: 3, 64: 1.7
+//           two stacks  fp32  2: 30, 3: 12, 4: 6, 5: 5, 6: 4.5, 8: 3.8, 10: 3.4, 12: 3.2, 16: 3, 20: 3.2, 24: 3, 32: 3, 64: 2;
+//                bf16 + fp32  2: 20, 3: 25, 4: 9, 5: 5, 6: 4.5, 8: 3.5, 10: 3, 12: 3, 16: 2.5, 20: 2.8, 24: 2.3, 32: 2.5, 64: 1.6
+//   [P][N]  one stack   fp32  2: 13, 3: 17, 4: to 50, 5: 18, 6: 18, 8: to 50, 10: 16, 12: 22, 16: to 50, 20: 30, 24: 45, 32: to 50, 64: 100
+//                       bf16  2: 14, 3: 18, 4 to 8: to 50, 10 and 12: 40, 16: to 50, 20 and 24: 20, 32: 25, 64: to 50
+//           two stacks  fp32  2: to 50, 3: 20, 4: 20, 5: 25, 6: 35, 8: 90, 10: 60, 12: 80, 20: 55, 16 and from 24 on: 100;
+//                bf16 + fp32  2: 20, 3: 30, 4: 30, 5: 35, 6: 45, 8: 70, 10: 60, 12: 70, 20: 60, 16 and from 24 on: 100
 double sparse_share(int layout, int N, bool two_stacks, bool bf16)
 {
-    if (layout == WASH_LAYOUT_NP) return std::fmin(0.18, (two_stacks ? 0.35 : 0.6) / N);
-    if (N <= 3) return two_stacks ? 0.2 : 0.13;
-    if (N < 16) return two_stacks || bf16 || N > 5 ? 0.2 : 0.16;
-    return bf16 && !two_stacks ? (N == 16 ? 0.4 : 0.2) : 0.4;
+    if (layout == WASH_LAYOUT_NP) {
+        if (two_stacks) return N <= 3 ? (N == 2 ? 0.2 : 0.12) : N > 32 ? 0.018 : std::fmax(0.27 / N, 0.025);
+        if (bf16) return N <= 4 ? 0.18 : N <= 7 ? 0.08 : N <= 16 ? 0.06 : 0.02;
+        return std::fmax(std::fmin(0.6 / N, 0.17), 0.027);
+    }
+    if (two_stacks) return N <= 4 ? 0.2 : N <= 7 ? 0.3 : 0.6;
+    if (bf16) return N <= 3 ? 0.15 : N <= 8 ? 0.5 : N <= 12 ? 0.4 : N <= 16 ? 0.5 : N <= 32 ? 0.2 : 0.45;
+    if (N <= 3) return 0.13;
+    if (N == 4 || N == 8) return 0.5;   // a coordinate's values are whole 16-byte pieces
+    return N <= 12 ? 0.18 : N <= 16 ? 0.5 : N <= 24 ? 0.3 : 0.5;
 }
 
 // Brings the device copy of the segment table up to date with the call's
