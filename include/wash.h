@@ -23,6 +23,11 @@
  *     them.  The context owns only its small tables.
  *   - `stream` is a cudaStream_t passed as void* (NULL = the default stream).  Kernel
  *     launches are asynchronous on it; argument errors are reported before any launch.
+ *     Kernels of this library release their programmatic dependents while they still have stores
+ *     to do: a kernel that is launched as one (programmatic stream serialization) behind a call
+ *     of this library must wait (griddepcontrol.wait, cudaGridDependencySynchronize) before it reads
+ *     a stack, also where it takes the weights for constant and would fetch them early.
+ *     Launches of the ordinary kind and copies need nothing.
  *     Calls on one context must be issued on one stream at a time (the context's
  *     tables are rewritten in stream order when the probabilities change).
  *   - Randomness is a pure function of (seed, step, tensor index, coordinate index)
@@ -129,11 +134,12 @@ int wash_set_mode(wash_ctx *ctx, int32_t mode);
  * blocks_per_sm, the kernel of a streaming shuffle (0: by the rules below; the dense
  * operators and WASH_MODE_SPARSE ignore it).  blocks_per_sm = 1 or 2 fixes the number of groups a thread takes
  * (default: 2 when a group of all models is at most 64 bytes, else 1); blocks_per_sm = -2 / -3
- * forces the streaming kernel's lean / early flavour (early draws the permutations while the
+ * forces the streaming kernel's lean / early flavour (lean: not the early one; from 0.3 % selected on that is, for more than 16
+ * models, the kernel of their own named below; early draws the permutations while the
  * stack's copies are in flight and serves populations of more than 16 models densely; by
  * default it is launched for N > 16 when the call's probabilities select 70 % or more; from
  * 0.3 % to there populations of more than 16 models have a kernel of their own);
- * blocks_per_sm = -4 / -5 forces (N <= 16) / excludes the streaming kernel for small groups (a
+ * blocks_per_sm = -4 / -5 forces (N <= 16; ignored above) / excludes the streaming kernel for small groups (a
  * resident grid of warps walking tiles through two shared-memory stages; by default
  * it is launched when a group of all models of both stacks is at most 48 bytes and the
  * call's probabilities select at most 30 %, and for groups of up to 96 bytes where serving
@@ -242,7 +248,7 @@ enum wash_step_ops { WASH_OP_SHUFFLE = 1, WASH_OP_EMA = 2, WASH_OP_AVERAGE = 4 }
  * device stacks must be bound; they serve as staging and hold the results too.
  * A step that only shuffles and moves few values stores them into the host buffers as the
  * kernels run, when the buffers are pinned and mapped, and does not copy the stacks back.
- * Populations of 2^20 coordinates per model and more are processed in eight coordinate
+ * Populations of 2^20 coordinates per model and more are processed in eight to 32 coordinate
  * ranges on two internal copy streams, so that the copy in of one range, the kernels on
  * the previous one and the copy out of the one before overlap; the result is the same. */
 int wash_step_host(wash_ctx *ctx, int32_t ops, void *host_params, void *host_opt, void *host_avg,

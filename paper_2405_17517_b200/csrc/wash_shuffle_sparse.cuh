@@ -11,12 +11,12 @@
 // The exchange is in place: a warp loads all values of its set of coordinates before it stores
 // the first of them.
 //
-// Two bounds.  The mask: one Philox block per 4 coordinates on the integer pipes (2^27 coordinates:
+// Two costs.  The mask: one Philox block per 4 coordinates on the integer pipes (2^27 coordinates:
 // 80 us for the blocks alone, 86 us with the compares, this kernel 92 us at N = 2, p = 1e-4).  The
-// values: DRAM serves about 45e9 scattered 4-byte loads a second, 22e9 scattered stores and 20e9 pairs
-// of both (measured, one access per 800 bytes), so [N][P] cannot go below 1 us per 20 000 moved
-// values and stack: ResNet-50 N = 8, bf16 + fp32, p = 5e-3 (1.8e6 values in both stacks) 90 us by that figure, 77 us
-// here -- neighbouring coordinates of a model share DRAM pages.  With a queue per warp, served at the end of the warp's
+// values: DRAM serves about 45e9 isolated 4-byte loads a second, 22e9 stores and 20e9 pairs
+// of both (measured, one access per 800 bytes), 1 us per 20 000 moved values and stack.  That is the rate of isolated accesses
+// and no bound for denser ones, which share DRAM pages and sectors: ResNet-50 N = 8, bf16 + fp32, p = 5e-3 (1.8e6 values in
+// both stacks) would take 90 us by it and takes 77.  With a queue per warp, served at the end of the warp's
 // range by a lane per coordinate, and launches that do not overlap, the same took (before -> now): that one 89.1 -> 77.1,
 // ResNet-18 N = 5 with momentum, p = 1e-3 21.0 -> 10.5, ResNet-50 N = 10 with momentum, p = 0.01 -> 0 70.8 -> 56.1, 2^27 coordinates N = 2
 // at p = 1e-3 119 -> 97.5 us.
@@ -79,7 +79,7 @@ __device__ __forceinline__ void serve_row(const PopView &pop, void *stack, uint3
 }
 
 // MIRROR: the moved values go to a second copy of the stacks as well (wash_step_host: the caller's buffers).
-// ROWS: a lane per coordinate loads all its values before it stores them (serve_rows), instead of a lane per (coordinate,
+// ROWS: a lane per coordinate loads all its values before it stores them (serve_row), instead of a lane per (coordinate,
 // model) pair.
 template <class TA, class TB, int LAYOUT, bool MIRROR, bool ROWS>
 __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_sparse_kernel(const __grid_constant__ SparseArgs p)
