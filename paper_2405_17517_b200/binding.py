@@ -129,7 +129,10 @@ def _stream(stream) -> Optional[int]:
         if _current_raw_stream is None:
             import torch
             torch.cuda.init()
-            _current_raw_stream = (torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+            try:
+                _current_raw_stream = (torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+            except AttributeError:      # not part of torch's public interface
+                _current_raw_stream = (lambda d: torch.cuda.current_stream(d).cuda_stream, torch.cuda.current_device)
         raw, device = _current_raw_stream
         return raw(device()) or None
     if isinstance(stream, int):

@@ -141,15 +141,6 @@ __device__ __forceinline__ char *group_vec_ptr(void *base, const PopView &pop, u
     return static_cast<char *>(base) + e * T::kBytes;
 }
 
-// raw bits of (model n, coordinate c of the group) out of the group's N vectors
-template <class T, int LAYOUT, int CAP>
-__device__ __forceinline__ uint32_t group_value(const typename T::vec (&v)[CAP], int n_models, int n, int c)
-{
-    if (LAYOUT == kLayoutNP) return T::get(v[n], c);
-    const int f = c * n_models + n;
-    return T::get(v[f >> 2], f & 3);
-}
-
 // ---- statistics -----------------------------------------------------------------------
 // Called by every thread of the block at the end of a shuffle kernel.  Warp sums go to
 // shared memory and a block that selected anything adds its sums to slot (blockIdx mod

@@ -414,3 +414,28 @@ def test_consensus_distances_of_two_contexts_on_two_streams_add_up():
     assert (out.cpu().numpy() == 2.0 * calls * 256).all()
     for s in shards:
         s.close()
+
+
+@pytest.mark.parametrize("pinned", [True, False, "params only", "unaligned"])
+def test_host_step_stores_moved_values_only_into_buffers_that_are_all_mapped(pinned):
+    """The two ways of a shuffling step over host buffers differ in their kernels: storing the moved values as they are served is
+    one launch (the sparse kernel), copying the stacks back one of the streaming kernel and one for its counters (eight
+    models, this size).  Both buffers pinned: stored; one of them or none, or one at an address that is no multiple of its
+    elements' size: copied.  The results are the same."""
+    N, p = 8, 0.01
+    c = Case(N, [400_001, 9], 0, "f32", "f32", seed=5)
+    views = []
+    for k, h in enumerate((c.host, c.host_opt)):
+        raw = torch.empty(h.nbytes + 16, dtype=torch.uint8, pin_memory=pinned is True or pinned == "unaligned" or (pinned == "params only" and k == 0))
+        at = 2 if pinned == "unaligned" and k == 1 else 0
+        raw[at:at + h.nbytes] = torch.from_numpy(h.reshape(-1).view(np.uint8))
+        views.append((raw, at))
+    before = B.wash_launch_count()
+    got = B.wash_step_host(c.gpu.ctx, B.WASH_OP_SHUFFLE, views[0][0].data_ptr() + views[0][1], views[1][0].data_ptr() + views[1][1], None, 3, p, None, 17)
+    launches = B.wash_launch_count() - before
+    assert got == tuple(oracle.shuffle(c.ora, c.host, p, seed=17, step=3, stack2=c.host_opt))
+    c.assert_equal("device stacks")
+    for (raw, at), h in zip(views, (c.host, c.host_opt)):
+        assert (raw[at:at + h.nbytes].numpy() == h.reshape(-1).view(np.uint8)).all()
+    assert launches == (1 if pinned is True else 2), launches
+    c.close()

@@ -291,18 +291,20 @@ def test_resident_warp_kernel_for_each_compiled_population(N, dtype, opt, layout
     c.close()
 
 
-@pytest.mark.parametrize("dtype", ["f32", "bf16"])
-@pytest.mark.parametrize("N", [2, 4])
-def test_resident_warp_kernel_with_a_padded_coordinate_major_image(N, dtype):
-    """[P][N] with an even N and a quarter of the coordinates selected: the shared-memory image is
-    padded against bank conflicts while the small-group streaming kernel is still the one launched
-    (forced here for N = 4 in fp32, whose groups it does not take by default)."""
-    c = Case(N, [300_007, 12, 40_000], 1, dtype, None, seed=90 + N)
+@pytest.mark.parametrize("N,dtype,opt", [(2, "f32", None), (2, "bf16", None), (4, "f32", None), (4, "bf16", None),
+                                         (8, "f32", None), (16, "bf16", None), (4, "f32", "f32")])
+@pytest.mark.parametrize("p", [0.25, 0.6])
+def test_resident_warp_kernel_with_a_padded_coordinate_major_image(N, dtype, opt, p):
+    """[P][N]: from half of the coordinates on the shared-memory image is padded against bank conflicts where a group is a
+    multiple of 128 bytes (64 in two stacks): N = 8 in fp32, 16 in bf16, two fp32 stacks of N = 4 at p = 0.6; the
+    small-group streaming kernel, forced here, fetches and serves a padded image by a path of its own."""
+    c = Case(N, [300_007, 12, 40_000], 1, dtype, opt, seed=90 + N)
     B.wash_set_launch(c.gpu.ctx, 0, -4)
+    shuffle = B.wash_shuffle_both if opt else B.wash_shuffle
     tot = [0, 0]
     for step in (0, 1):
-        B.wash_shuffle(c.gpu.ctx, step, 0.25, None, seed=5, stats=c.stats_dev)
-        s = oracle.shuffle(c.ora, c.host, 0.25, seed=5, step=step)
+        shuffle(c.gpu.ctx, step, p, None, seed=5, stats=c.stats_dev)
+        s = oracle.shuffle(c.ora, c.host, p, seed=5, step=step, stack2=c.host_opt)
         tot[0] += s[0]; tot[1] += s[1]
         c.assert_equal("N=%d %s step=%d" % (N, dtype, step))
     assert c.gpu_stats() == tuple(tot)
