@@ -7,9 +7,9 @@
 //
 // The unit of work is 16 bytes of every model: 4 coordinates in fp32, 8 in bf16 (tensors start on
 // multiples of 8 elements, so a unit never straddles two).  [N][P] keeps a unit's N vectors in registers
-// where N is small (unrolled per N); larger populations and [P][N] stage them in shared memory by
-// cp.async with N a run-time value, sum them from there and, for the operators that write the stack,
-// read them once more from there.
+// where N is small (unrolled per N), [P][N] the 4N values of a group of four coordinates (pn_in_registers says which N);
+// larger populations stage them in shared memory by cp.async, sum them from there and, for the operators that write the
+// stack, read them once more from there.
 // Bound: HBM, except bf16 [P][N], which has two values a word to widen, round and check for NaN and is bound
 // by issue slots (N = 32 249 us where the bytes take 164).  Before, a thread held four coordinates of every model (8-byte
 // vectors in bf16, values of [P][N] picked out of registers), and populations not in a list of unrolled sizes went
@@ -116,6 +116,54 @@ __global__ void __launch_bounds__(256) regs_np_kernel(const __grid_constant__ Re
 #pragma unroll
             for (int q = 0; q < kElems; ++q)
                 if (q < valid) T::store_elem(out, q, T::from_float(OP == kOpPapaAll ? m[q] : __fadd_rn(__fmul_rn(a.alpha, Unit<T>::get(v[n], q)), m[q])));
+        }
+    }
+}
+
+// [P][N], small N: a thread per group of four coordinates, its 4N contiguous values in registers.
+template <class T, class TOUT, int OP, int N>
+__global__ void __launch_bounds__(256) regs_pn_kernel(const __grid_constant__ ReduceArgs a)
+{
+    await_previous();
+    let_next_start();
+    const uint64_t g = a.group_lo + static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (g >= a.group_hi) return;
+    constexpr int kVec = 4 * T::kBytes;
+    char *group = group_vec_ptr<T, kLayoutPN>(a.stack, a.pop, g, 0);
+    typename T::vec v[N];   // element f of the group = (coordinate f / N, model f % N)
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = T::load_group(group + j * kVec);
+    const int valid = find_group(a.pop, static_cast<uint32_t>(g), a.status).valid;
+    if (valid == 0) return;
+    float m[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        m[c] = T::to_float(T::get(v[c * N / 4], c * N % 4));
+#pragma unroll
+        for (int n = 1; n < N; ++n) m[c] = __fadd_rn(m[c], T::to_float(T::get(v[(c * N + n) / 4], (c * N + n) % 4)));
+        m[c] = __fdiv_rn(m[c], static_cast<float>(N));
+        if (OP == kOpEma) m[c] = __fmul_rn(a.one_minus_alpha, m[c]);
+    }
+    const long long e0 = 4ll * static_cast<long long>(g);
+    if constexpr (OP == kOpAverage) {
+        if (valid == 4) TOUT::store_group(static_cast<char *>(a.out) + e0 * TOUT::kBytes, TOUT::pack_floats(m[0], m[1], m[2], m[3]));
+        else {
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                if (c < valid) TOUT::store_elem(a.out, e0 + c, TOUT::from_float(m[c]));
+        }
+    } else {
+        const auto updated = [&](int f) -> float {
+            return OP == kOpPapaAll ? m[f / N] : __fadd_rn(__fmul_rn(a.alpha, T::to_float(T::get(v[f / 4], f % 4))), m[f / N]);
+        };
+        if (valid == 4) {
+#pragma unroll
+            for (int j = 0; j < N; ++j)
+                T::store_group(group + j * kVec, T::pack_floats(updated(4 * j), updated(4 * j + 1), updated(4 * j + 2), updated(4 * j + 3)));
+        } else {   // a tensor's ragged end: its padding is not written
+#pragma unroll
+            for (int f = 0; f < 3 * N; ++f)
+                if (f < valid * N) T::store_elem(group, f, T::from_float(updated(f)));
         }
     }
 }
@@ -369,9 +417,10 @@ cudaError_t launch_dense(K kernel, const ReduceArgs &args, uint64_t units, int p
 // [N][P]: the largest population whose vectors are kept in registers.  Measured (registers / staged): average,
 // fp32, N = 3 78 / 82 us, N = 10 162 / 164, N = 20 (ResNet-18) 136 / 139; EMA, fp32, N = 5 71 / 74, N = 10 309 / 313, 131072 coordinates of
 // N = 16 4.6 / 6.1, N = 32 equal; EMA, bf16, 2^25 coordinates N = 2 49 / 59, ResNet-50
-// N = 5 94 / 87, N = 8 156 / 133 (few resident warps); PAPA-all, bf16, N = 8 129 / 132.
+// N = 5 94 / 87, N = 8 156 / 133 (few resident warps); PAPA-all, bf16, N = 8 129 / 132; average, bf16, 3 * 2^23 coordinates, fp32 out N = 26 200 us in
+// registers, 28 275, 32 293, 33 253 staged.
 template <class T>
-constexpr int regs_max_models(int op) { return op == kOpAverage ? 32 : (T::kBytes == 4 ? 16 : (op == kOpEma ? 3 : 8)); }
+constexpr int regs_max_models(int op) { return op == kOpAverage ? (T::kBytes == 4 ? 32 : 26) : (T::kBytes == 4 ? 16 : (op == kOpEma ? 3 : 8)); }
 
 template <class T, class TOUT, int OP, int N>
 cudaError_t launch_regs_n(const ReduceArgs &args, uint64_t units, const LaunchShape &shape, cudaStream_t stream)
@@ -384,6 +433,33 @@ cudaError_t launch_regs_n(const ReduceArgs &args, uint64_t units, const LaunchSh
     return launch_chained(regs_np_kernel<T, TOUT, OP, N>, static_cast<unsigned>(grid), threads, 0, stream, args);
 }
 
+// [P][N]: the populations that are kept in registers instead of staged.  Staging pays for copies that leave in 16-byte pieces of
+// whole lines where a lane's registers would be read with gaps (N = 8: 128 bytes from lane to lane), and costs a trip
+// through shared memory, which the bytes of a small group do not hide.  Staged / registers, 3 * 2^23 coordinates, fp32:
+//   average  N = 2 60 / 44, 4 90 / 72, 6 127 / 102, 7 128 / 122, 8 137 / 185, 9 149 / 152, 10 178 / 169 us (bf16 out 4 89 / 65, 7 132 / 116)
+//   EMA      N = 2 76 / 60, 4 133 / 128, 5 158 / 167, 8 238 / 402
+//   PAPA-all N = 2 75 / 60, 3 91.3 / 90.9, 4 131 / 137
+template <class T>
+constexpr bool pn_in_registers(int op, int N)
+{
+    return T::kBytes == 4 && N <= (op == kOpAverage ? 7 : op == kOpEma ? 4 : 3);
+}
+constexpr int kPnRegsMax = 7;
+
+template <class T, class TOUT, int OP, int N>
+cudaError_t launch_regs_pn_n(const ReduceArgs &args, const LaunchShape &shape, cudaStream_t stream)
+{
+    if constexpr (N < kPnRegsMax)
+        if (args.pop.N > N) return launch_regs_pn_n<T, TOUT, OP, N + 1>(args, shape, stream);
+    if constexpr (pn_in_registers<T>(OP, N)) {
+        const unsigned threads = shape.threads > 0 ? static_cast<unsigned>(shape.threads) : 256u;
+        const uint64_t grid = (static_cast<uint64_t>(args.group_hi - args.group_lo) + threads - 1) / threads;
+        if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+        return launch_chained(regs_pn_kernel<T, TOUT, OP, N>, static_cast<unsigned>(grid), threads, 0, stream, args);
+    }
+    return cudaErrorInvalidValue;   // pn_in_registers decided otherwise
+}
+
 template <class T, class TOUT, int OP>
 cudaError_t launch_reduce_typed(const ReduceArgs &args, const LaunchShape &shape, cudaStream_t stream)
 {
@@ -391,14 +467,10 @@ cudaError_t launch_reduce_typed(const ReduceArgs &args, const LaunchShape &shape
     if (units == 0) return cudaSuccess;
     const int N = args.pop.N;
     if (args.pop.layout == kLayoutPN) {
+        if (pn_in_registers<T>(OP, N)) return launch_regs_pn_n<T, TOUT, OP, 2>(args, shape, stream);
         const int per_thread = units_per_thread(N);
         const size_t bytes = static_cast<size_t>(N | 1) * 16;
-        if constexpr (Unit<T>::kElems == 4) {
-            switch (N) {
-            case 2: return launch_dense(dense_pn_kernel<T, TOUT, OP, 2>, args, units, per_thread, bytes, shape, stream);
-            case 3: return launch_dense(dense_pn_kernel<T, TOUT, OP, 3>, args, units, per_thread, bytes, shape, stream);
-            }
-        } else {
+        if constexpr (Unit<T>::kElems == 8) {
             switch (N) {
             case 2: return launch_dense(dense_pn_kernel<T, TOUT, OP, 2>, args, units, per_thread, bytes, shape, stream);
             case 3: return launch_dense(dense_pn_kernel<T, TOUT, OP, 3>, args, units, per_thread, bytes, shape, stream);

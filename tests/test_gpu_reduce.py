@@ -439,3 +439,25 @@ def test_host_step_stores_moved_values_only_into_buffers_that_are_all_mapped(pin
         assert (raw[at:at + h.nbytes].numpy() == h.reshape(-1).view(np.uint8)).all()
     assert launches == (1 if pinned is True else 2), launches
     c.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("N", range(2, 14))
+def test_coordinate_major_populations_in_registers_or_staged(N, dtype):
+    """[P][N] on both sides of the rule that keeps small populations in registers: tensors that end after 1 to 7 elements
+    of their last eight, one that is shorter than a group, several blocks; both types of the average.  The same operations
+    in the same order as the oracle's: the same bits, the padding of rows and of the average untouched."""
+    c = Case(N, [1, 2053, 7, 1030, 4, 70_003, 8], B.WASH_LAYOUT_PN, dtype, seed=N + 110)
+    B.papa_ema(c.gpu.ctx, B.WASH_STACK_PARAMS, 0.3)
+    oracle.papa_ema(c.ora, c.host, 0.3)
+    c.assert_equal("ema")
+    for tdt, ndt, code in ((torch.float32, np.float32, B.WASH_F32), (torch.bfloat16, np.uint16, B.WASH_BF16)):
+        out = torch.full((c.P,), 7.0, dtype=tdt, device="cuda")
+        want = np.full(c.P, 7.0, dtype=np.float32) if ndt is np.float32 else np.full(c.P, 0x40E0, dtype=np.uint16)
+        B.population_average(c.gpu.ctx, B.WASH_STACK_PARAMS, out, code)
+        oracle.population_average(c.ora, c.host, want)
+        assert (to_host_bits(out) == bits(want)).all()
+    B.papa_all(c.gpu.ctx, B.WASH_STACK_PARAMS)
+    oracle.papa_all(c.ora, c.host)
+    c.assert_equal("papa_all")
+    c.close()
