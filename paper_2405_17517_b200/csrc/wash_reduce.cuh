@@ -439,12 +439,16 @@ cudaError_t launch_regs_n(const ReduceArgs &args, uint64_t units, const LaunchSh
 //   average  N = 2 60 / 44, 4 90 / 72, 6 127 / 102, 7 128 / 122, 8 137 / 185, 9 149 / 152, 10 178 / 169 us (bf16 out 4 89 / 65, 7 132 / 116)
 //   EMA      N = 2 76 / 60, 4 133 / 128, 5 158 / 167, 8 238 / 402
 //   PAPA-all N = 2 75 / 60, 3 91.3 / 90.9, 4 131 / 137
+// bf16, whose staged sums are carried from vector to vector from 9 models on (fp32 out / bf16 out):
+//   average  N = 2 42 / 36 and 37 / 34, 3 39 / 40 and 34 / 36, 4 51 / 45 and 44 / 40, 6 68 / 57 and 61 / 51, 7 66 / 65, 8 82 / 98 and 86 / 96, 9 115 / 83 and
+//            136 / 76, 10 117 / 92 and 136 / 85, 12 122 / 112 and 134 / 108;  EMA N = 2 47 / 35, 3 57 / 67;  PAPA-all N = 2 44 / 32, 3 49 / 65
 template <class T>
 constexpr bool pn_in_registers(int op, int N)
 {
-    return T::kBytes == 4 && N <= (op == kOpAverage ? 7 : op == kOpEma ? 4 : 3);
+    if (T::kBytes == 2) return op == kOpAverage ? N <= 12 && N != 3 && N != 8 : N == 2;
+    return N <= (op == kOpAverage ? 7 : op == kOpEma ? 4 : 3);
 }
-constexpr int kPnRegsMax = 7;
+constexpr int kPnRegsMax = 12;
 
 template <class T, class TOUT, int OP, int N>
 cudaError_t launch_regs_pn_n(const ReduceArgs &args, const LaunchShape &shape, cudaStream_t stream)
@@ -470,14 +474,13 @@ cudaError_t launch_reduce_typed(const ReduceArgs &args, const LaunchShape &shape
         if (pn_in_registers<T>(OP, N)) return launch_regs_pn_n<T, TOUT, OP, 2>(args, shape, stream);
         const int per_thread = units_per_thread(N);
         const size_t bytes = static_cast<size_t>(N | 1) * 16;
-        if constexpr (Unit<T>::kElems == 8) {
-            switch (N) {
-            case 2: return launch_dense(dense_pn_kernel<T, TOUT, OP, 2>, args, units, per_thread, bytes, shape, stream);
-            case 3: return launch_dense(dense_pn_kernel<T, TOUT, OP, 3>, args, units, per_thread, bytes, shape, stream);
-            case 4: return launch_dense(dense_pn_kernel<T, TOUT, OP, 4>, args, units, per_thread, bytes, shape, stream);
-            case 5: return launch_dense(dense_pn_kernel<T, TOUT, OP, 5>, args, units, per_thread, bytes, shape, stream);
-            case 6: return launch_dense(dense_pn_kernel<T, TOUT, OP, 6>, args, units, per_thread, bytes, shape, stream);
-            case 7: return launch_dense(dense_pn_kernel<T, TOUT, OP, 7>, args, units, per_thread, bytes, shape, stream);
+        if constexpr (Unit<T>::kElems == 8) {   // what pn_in_registers leaves of the populations below a vector's elements
+            if (N == 3) return launch_dense(dense_pn_kernel<T, TOUT, OP, 3>, args, units, per_thread, bytes, shape, stream);
+            if constexpr (OP != kOpAverage) switch (N) {
+                case 4: return launch_dense(dense_pn_kernel<T, TOUT, OP, 4>, args, units, per_thread, bytes, shape, stream);
+                case 5: return launch_dense(dense_pn_kernel<T, TOUT, OP, 5>, args, units, per_thread, bytes, shape, stream);
+                case 6: return launch_dense(dense_pn_kernel<T, TOUT, OP, 6>, args, units, per_thread, bytes, shape, stream);
+                case 7: return launch_dense(dense_pn_kernel<T, TOUT, OP, 7>, args, units, per_thread, bytes, shape, stream);
             }
         }
         return launch_dense(dense_pn_kernel<T, TOUT, OP, 0>, args, units, per_thread, bytes, shape, stream);
