@@ -137,9 +137,10 @@ __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_co
     constexpr bool kHasB = TB::kCode != kDtypeNone;
     const int n_models = a.pop.N;
     const uint32_t groups = blockDim.x / 2u, lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    // (pn_pad is 0 for these populations; left out of the kernel, the same one took 977 us for N = 32, 2^25 coordinates, p = 0.1, 963 with it)
     // the images of the two stacks, the block's list {coordinate within its tensor, tensor} and where it lies (group * 4 +
     // coordinate slot), kWideRound permutations per warp
-    const uint32_t group_elems = pn_group_elems(n_models, 0u);   // (populations of more than 16 models are not padded)
+    const uint32_t group_elems = pn_group_elems(n_models, a.pn_pad);
     unsigned char *image_a = smem_raw, *image_b = image_a + group_elems * groups * TA::kBytes;
     uint2 *s_key = reinterpret_cast<uint2 *>(image_b + (kHasB ? group_elems * groups * TB::kBytes : 0));
     uint32_t *s_perm = reinterpret_cast<uint32_t *>(s_key + 4 * groups) + warp * kWideRound * wide_pitch(n_models);
@@ -147,8 +148,8 @@ __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_co
 
     const uint64_t g_block = a.group_lo + static_cast<uint64_t>(blockIdx.x) * groups;
     const uint32_t in_block = static_cast<uint32_t>(min(static_cast<uint64_t>(groups), a.group_hi - g_block));
-    async_fetch<TA, LAYOUT>(smem_addr(image_a), a.a, a.pop, g_block, in_block, n_models, 0u);
-    if constexpr (kHasB) async_fetch<TB, LAYOUT>(smem_addr(image_b), a.b, a.pop, g_block, in_block, n_models, 0u);
+    async_fetch<TA, LAYOUT>(smem_addr(image_a), a.a, a.pop, g_block, in_block, n_models, a.pn_pad);
+    if constexpr (kHasB) async_fetch<TB, LAYOUT>(smem_addr(image_b), a.b, a.pop, g_block, in_block, n_models, a.pn_pad);
     if (threadIdx.x == 0) s_count = 0;
     __syncthreads();
 
@@ -222,7 +223,7 @@ cudaError_t launch_shuffle_wide_typed(const ShuffleArgs &call, const LaunchShape
     const size_t per_thread = group_elems * (TA::kBytes + (kHasB ? TB::kBytes : 0)) + 4 + 4 * wide_pitch(args.pop.N);
     if (args.pop.layout == kLayoutPN && !args.sq.slots && 4 * static_cast<size_t>(args.pop.N) * (TA::kBytes + TB::kBytes) >= kWideSplitBytes) {
         // the images, the list (keys and places of every coordinate) and kWideRound permutations per warp
-        const size_t per_group = 4 * static_cast<size_t>(args.pop.N) * (TA::kBytes + (kHasB ? TB::kBytes : 0)) + 4 * 8 + 4 + 4 * wide_pitch(args.pop.N);
+        const size_t per_group = group_elems * (TA::kBytes + (kHasB ? TB::kBytes : 0)) + 4 * 8 + 4 + 4 * wide_pitch(args.pop.N);
         const uint32_t groups = per_group * 64 > 44 * 1024 ? 32 : 64;   // five blocks and more on an SM
         const size_t smem = (per_group * groups + 15) & ~static_cast<size_t>(15);
         KernelFit fit;
