@@ -8,7 +8,9 @@ namespace wash {
 
 // ---- Philox4x32-10 (Salmon et al., SC'11) ------------------------------------------
 // Ten rounds of two 32x32->64 multiplies; the key advances by the two Weyl constants
-// after every round (the ten keys come ready-made from the host: PhiloxKeys).
+// after every round (the ten keys come ready-made from the host: PhiloxKeys).  A multiply is written as a 64-bit product: as
+// __umulhi and a 32-bit product the masks of 2^27 coordinates take 84.7 us, so 82.3.  Not the multiplies alone bound it: hoisting what the
+// groups of a tensor share (two of 20) or taking neighbouring groups' first product by addition changes nothing.
 struct Philox4 {
     uint32_t x, y, z, w;
 };
@@ -18,12 +20,11 @@ __device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint3
     constexpr uint32_t kMul0 = 0xD2511F53u, kMul1 = 0xCD9E8D57u;
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        const uint32_t hi0 = __umulhi(kMul0, c0), lo0 = kMul0 * c0;
-        const uint32_t hi1 = __umulhi(kMul1, c2), lo1 = kMul1 * c2;
-        c0 = hi1 ^ c1 ^ keys.k[2 * r];
-        c2 = hi0 ^ c3 ^ keys.k[2 * r + 1];
-        c1 = lo1;
-        c3 = lo0;
+        const uint64_t p0 = static_cast<uint64_t>(kMul0) * c0, p1 = static_cast<uint64_t>(kMul1) * c2;
+        c0 = static_cast<uint32_t>(p1 >> 32) ^ c1 ^ keys.k[2 * r];
+        c2 = static_cast<uint32_t>(p0 >> 32) ^ c3 ^ keys.k[2 * r + 1];
+        c1 = static_cast<uint32_t>(p1);
+        c3 = static_cast<uint32_t>(p0);
     }
     return Philox4{c0, c1, c2, c3};
 }
