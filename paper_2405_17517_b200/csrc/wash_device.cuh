@@ -168,8 +168,13 @@ __device__ __forceinline__ void publish_block_stats(unsigned long long *stats, S
 }
 
 // The same for a resident grid of one-warp blocks, without the flush kernel: the last block to
-// report to a slot moves the slot's totals on and zeroes the slot.  Two levels, because a few
-// thousand blocks that end together would queue up at one address (1-2 ns each).
+// report to a slot moves the slot's total on and zeroes the slot.  Two levels, because a few
+// thousand blocks that end together would queue up at one address (1-2 ns each).  A slot's counters and the number
+// of blocks that have reported share one 64-bit word, so that a block reports with a single atomic and the last one reads
+// the total out of its return value: with a word for each, a fence between them and two exchanges to fetch the totals, the end
+// of a launch took three trips to the L2 more.
+//   bits 0..7 blocks (at most 32 a SM: 19 to a slot), 8..33 selected, 34..63 moved: a slot's share of the 2^33
+//   coordinates a row may have is 2^25, moved 16 times as much (the kernel takes populations of up to 16 models).
 __device__ __forceinline__ void publish_warp_stats(unsigned long long *stats, StatSlot *slots, uint32_t selected, uint32_t moved)
 {
     if (!stats) return;
@@ -177,16 +182,12 @@ __device__ __forceinline__ void publish_warp_stats(unsigned long long *stats, St
     moved = __reduce_add_sync(0xFFFFFFFFu, moved);
     if (threadIdx.x != 0) return;
     StatSlot *slot = slots + blockIdx.x % kStatSlots;
-    if (selected) {
-        atomicAdd(&slot->selected, static_cast<unsigned long long>(selected));
-        atomicAdd(&slot->moved, static_cast<unsigned long long>(moved));
-    }
-    __threadfence();
     const unsigned long long sharers = (gridDim.x - blockIdx.x % kStatSlots + kStatSlots - 1) / kStatSlots;
-    if (atomicAdd(&slot->blocks, 1ull) + 1ull != sharers) return;
-    __threadfence();
-    slot->blocks = 0;
-    const unsigned long long s = atomicExch(&slot->selected, 0ull), m = atomicExch(&slot->moved, 0ull);
+    const unsigned long long mine = 1ull | (static_cast<unsigned long long>(selected) << 8) | (static_cast<unsigned long long>(moved) << 34);
+    const unsigned long long total = atomicAdd(&slot->report, mine) + mine;
+    if ((total & 255ull) != sharers) return;
+    slot->report = 0;
+    const unsigned long long s = (total >> 8) & ((1ull << 26) - 1ull), m = total >> 34;
     if (s) {
         atomicAdd(stats, s);
         atomicAdd(stats + 1, m);

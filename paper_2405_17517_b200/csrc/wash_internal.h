@@ -31,7 +31,7 @@ static_assert(sizeof(SegEntry) == 32, "SegEntry must stay 32 bytes");
 constexpr int kStatSlots = 256;
 struct StatSlot {
     unsigned long long selected, moved;
-    unsigned long long blocks;   // resident-warp streaming kernel: blocks that have reported
+    unsigned long long report;   // resident-warp streaming kernel: blocks that have reported and their counters (publish_warp_stats)
     unsigned long long reserved;
 };
 

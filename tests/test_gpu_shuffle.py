@@ -674,3 +674,19 @@ def test_sparse_warps_that_serve_by_themselves(N, layout, numel, p, dtype, opt):
     c.assert_equal("N=%d layout=%d p=%g" % (N, layout, p))
     assert c.gpu_stats() == tuple(want)
     c.close()
+
+
+@pytest.mark.parametrize("N,tiles", [(2, 1), (2, 300), (2, 148 * 22 - 1), (2, 148 * 22), (2, 148 * 22 + 1), (3, 1500), (3, 2400)])
+def test_resident_warps_with_one_tile_and_with_more(N, tiles):
+    """As many warps as tiles, where masks are drawn before the wait for the kernel before, and one tile more; the counters,
+    a word per slot, over calls that follow each other at once."""
+    c = Case(N, [512 * tiles - 3], 0, seed=N)
+    B.wash_set_launch(c.gpu.ctx, 0, -4)
+    want = np.zeros(2, dtype=np.int64)
+    for step in range(4):
+        B.wash_shuffle(c.gpu.ctx, step, 0.05, None, seed=3, stats=c.stats_dev)
+    for step in range(4):
+        want += np.array(oracle.shuffle(c.ora, c.host, 0.05, seed=3, step=step), dtype=np.int64)
+    c.assert_equal("N=%d tiles=%d" % (N, tiles))
+    assert c.gpu_stats() == tuple(want)
+    c.close()
