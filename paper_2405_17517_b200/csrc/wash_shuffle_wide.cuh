@@ -33,6 +33,33 @@ __device__ __forceinline__ void move_value(const ShuffleArgs &a, const unsigned 
     if constexpr (kHasB) TB::store_elem(a.b, out, image_value<TB, LAYOUT>(image_b, n_models, a.pn_pad, t_owner, static_cast<int>(src), static_cast<int>(c)));
 }
 
+// Values of selected coordinates of a [P][N] image, four models to a thread (N a multiple of 4): model n of coordinate l takes the value of
+// model byte n of perm + l * wide_pitch(N).  A word of the permutation, four values of the image and one store where a lane per (coordinate,
+// model) pair read a byte, a value and stored 4 bytes; the issue slots of the moves, not the memory, were what kept the kernels from
+// it.  Fixed points are stored, too (sectors are then written whole; alone that gave N = 32, p = 0.1 236 -> 226).  [P][N], pairs -> quads:
+// shuffle_wide_kernel N = 20 fp32, 2^23 coordinates, p = 0.1 / 0.3 / 0.6 141 / 243 / 388 -> 127 / 201 / 297 us, N = 32 bf16 173 / 329 / 551 -> 151 / 256 /
+// 405; shuffle_wide_pn_kernel N = 32 fp32 p = 0.01 / 0.1 / 0.6 170 / 234 / 693 -> 163 / 209 / 546, N = 64 346 / 544 / 1726 -> 334 / 491 / 1308.
+template <class TA, class TB>
+__device__ __forceinline__ uint32_t move_quads(const ShuffleArgs &a, const unsigned char *image_a, const unsigned char *image_b, uint64_t g_block,
+                                               const uint32_t *s_perm, const uint8_t *s_entry, uint32_t count, uint32_t thread, uint32_t threads)
+{
+    constexpr bool kHasB = TB::kCode != kDtypeNone;
+    const uint32_t n_models = static_cast<uint32_t>(a.pop.N), quads = n_models / 4u, group_elems = pn_group_elems(a.pop.N, a.pn_pad);
+    uint32_t moved = 0;
+    for (uint32_t i = thread; i < count * quads; i += threads) {
+        const uint32_t l = (4u * i * a.pair_inverse) >> 20, q = i - l * quads;
+        const uint32_t src = s_perm[l * wide_pitch(a.pop.N) + q], entry = s_entry[l], g = entry >> 2, c = entry & 3u;
+        const uint32_t from = g * group_elems + c * n_models;
+        const long long out = (4ll * static_cast<long long>(g_block + g) + c) * n_models + 4u * q;
+        const uint32_t s0 = from + (src & 255u), s1 = from + ((src >> 8) & 255u), s2 = from + ((src >> 16) & 255u), s3 = from + (src >> 24);
+        TA::store_group(static_cast<char *>(a.a) + out * TA::kBytes, TA::pack(TA::load_elem(image_a, s0), TA::load_elem(image_a, s1), TA::load_elem(image_a, s2), TA::load_elem(image_a, s3)));
+        if constexpr (kHasB)
+            TB::store_group(static_cast<char *>(a.b) + out * TB::kBytes, TB::pack(TB::load_elem(image_b, s0), TB::load_elem(image_b, s1), TB::load_elem(image_b, s2), TB::load_elem(image_b, s3)));
+        moved += __popc(__vcmpne4(src, 0x03020100u + q * 0x04040404u)) >> 3;
+    }
+    return moved;
+}
+
 template <class TA, class TB, int LAYOUT, bool STAT>
 __global__ void __launch_bounds__(64, 6) shuffle_wide_kernel(const __grid_constant__ ShuffleArgs a)
 {
@@ -91,7 +118,10 @@ __global__ void __launch_bounds__(64, 6) shuffle_wide_kernel(const __grid_consta
         const uint32_t count = min(32u, total - first);
         if (first) draw(first, count);
         if (lane < count) ++selected;
-        if (LAYOUT == kLayoutPN || count <= kWidePairsMax) {
+        if (LAYOUT == kLayoutPN && n_models % 4 == 0) {
+            const size_t skip = static_cast<size_t>(warp_base) * group_elems;
+            moved += move_quads<TA, TB>(a, image_a + skip * TA::kBytes, image_b + skip * TB::kBytes, g_block + warp_base, s_perm, list + first, count, lane, 32u);
+        } else if (LAYOUT == kLayoutPN || count <= kWidePairsMax) {
             // a lane per (coordinate, model) pair, the models of a coordinate side by side
             const uint32_t pairs = count * static_cast<uint32_t>(n_models);
             for (uint32_t base = 0; base < pairs; base += 32) {
@@ -125,7 +155,11 @@ __global__ void __launch_bounds__(64, 6) shuffle_wide_kernel(const __grid_consta
 // above, 192 / 233 / 404 (both with a padded image at 0.25; without 357); N = 24, bf16 + fp32, p = 0.25 436 / 386; N = 64, fp32, p = 0.1 632 / 542.  Smaller groups (N = 20, fp32, p = 0.1
 // 145 / 165 us) and [N][P] (N = 20 200 / 202, N = 17 bf16 103 / 162) lose more by the block's barriers.
 constexpr size_t kWideSplitBytes = 512;
-constexpr uint32_t kWideRound = 16;   // coordinates of a warp's round
+// Coordinates whose permutations a warp of that kernel draws together.  The chain of swaps costs a warp the same for one coordinate and for
+// 32, so few warps with many coordinates each take fewer instructions than an even share for all, and a longer way to the first
+// move.  N = 32 fp32, 2^23, p = 0.1 / 0.3: an even share 226 / 407 us (by pairs), 16 209 / 349, 32 221 / 364.  The moves are dealt to all threads.
+constexpr uint32_t kWideChunk = 16;
+
 template <class TA, class TB>
 __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_constant__ ShuffleArgs a)
 {
@@ -139,12 +173,12 @@ __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_co
     const uint32_t groups = blockDim.x / 2u, lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     // (pn_pad is 0 for these populations; left out of the kernel, the same one took 977 us for N = 32, 2^25 coordinates, p = 0.1, 963 with it)
     // the images of the two stacks, the block's list {coordinate within its tensor, tensor} and where it lies (group * 4 +
-    // coordinate slot), kWideRound permutations per warp
+    // coordinate slot), as many permutations as the block has groups
     const uint32_t group_elems = pn_group_elems(n_models, a.pn_pad);
     unsigned char *image_a = smem_raw, *image_b = image_a + group_elems * groups * TA::kBytes;
     uint2 *s_key = reinterpret_cast<uint2 *>(image_b + (kHasB ? group_elems * groups * TB::kBytes : 0));
-    uint32_t *s_perm = reinterpret_cast<uint32_t *>(s_key + 4 * groups) + warp * kWideRound * wide_pitch(n_models);
-    uint8_t *s_entry = reinterpret_cast<uint8_t *>(reinterpret_cast<uint32_t *>(s_key + 4 * groups) + warps * kWideRound * wide_pitch(n_models));
+    uint32_t *s_perm = reinterpret_cast<uint32_t *>(s_key + 4 * groups);
+    uint8_t *s_entry = reinterpret_cast<uint8_t *>(s_perm + groups * wide_pitch(n_models));
 
     const uint64_t g_block = a.group_lo + static_cast<uint64_t>(blockIdx.x) * groups;
     const uint32_t in_block = static_cast<uint32_t>(min(static_cast<uint64_t>(groups), a.group_hi - g_block));
@@ -176,39 +210,42 @@ __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_co
     }
     __syncthreads();
     const uint32_t total = s_count;
-    // a round gives every warp up to kWideRound coordinates, as evenly as they go
-    uint32_t mine = 0, count = 0;
-    auto deal = [&](uint32_t first) {
-        const uint32_t left = total - first, share = min(kWideRound, (left + warps - 1u) / warps);
-        mine = first + warp * share;
-        count = mine < total ? min(share, total - mine) : 0u;
-        if (count) {
-            const uint2 key = s_key[mine + min(lane, count - 1u)];
-            draw_permutations_by_warp(s_perm, n_models, count, key.x, key.y, a.step_lo, a.step_hi8, a.keys);
+    // a round: the permutations of up to `groups` coordinates, kWideChunk at a time by a warp
+    auto draw = [&](uint32_t first) {
+        const uint32_t in_round = min(groups, total - first);
+        for (uint32_t at = ((warp + blockIdx.x) % warps) * kWideChunk; at < in_round; at += warps * kWideChunk) {
+            const uint32_t count = min(kWideChunk, in_round - at);
+            const uint2 key = s_key[first + at + min(lane, count - 1u)];
+            draw_permutations_by_warp(s_perm + at * wide_pitch(n_models), n_models, count, key.x, key.y, a.step_lo, a.step_hi8, a.keys);
         }
-        return share * warps;
+        return in_round;
     };
     // the first round's permutations are drawn while the copies are in flight
-    uint32_t step = total ? deal(0) : 0u;
+    uint32_t in_round = draw(0);
     cp_async_wait_all();
     __syncthreads();   // a group's bytes were copied by threads of other warps
-    for (uint32_t first = 0; first < total; first += step) {
-        if (first) step = deal(first);
-        if (lane < count) ++selected;
-        // a lane per (coordinate, model) pair, the models of a coordinate side by side
-        const uint32_t pairs = count * static_cast<uint32_t>(n_models);
-        for (uint32_t i = lane; i < pairs; i += 32) {
-            const uint32_t l = (i * a.pair_inverse) >> 20, n = i - l * static_cast<uint32_t>(n_models);
-            const uint32_t src = reinterpret_cast<const uint8_t *>(s_perm + l * wide_pitch(n_models))[n];
-            if (src == n) continue;
-            const uint32_t entry = s_entry[mine + l], g = entry >> 2, c = entry & 3u;
-            const long long out = elem_index<LAYOUT>(a.pop, static_cast<int>(n), 4ll * static_cast<long long>(g_block + g) + c);
-            const uint32_t from = g * group_elems + c * static_cast<uint32_t>(n_models) + src;
-            TA::store_elem(a.a, out, TA::load_elem(image_a, from));
-            if constexpr (kHasB) TB::store_elem(a.b, out, TB::load_elem(image_b, from));
-            ++moved;
+    if (threadIdx.x == 0) selected = total;
+    for (uint32_t first = 0; first < total;) {
+        if (n_models % 4 == 0) moved += move_quads<TA, TB>(a, image_a, image_b, g_block, s_perm, s_entry + first, in_round, threadIdx.x, blockDim.x);
+        else {
+            // a lane per (coordinate, model) pair, the models of a coordinate side by side
+            for (uint32_t i = threadIdx.x; i < in_round * static_cast<uint32_t>(n_models); i += blockDim.x) {
+                const uint32_t l = (i * a.pair_inverse) >> 20, n = i - l * static_cast<uint32_t>(n_models);
+                const uint32_t src = reinterpret_cast<const uint8_t *>(s_perm + l * wide_pitch(n_models))[n];
+                if (src == n) continue;
+                const uint32_t entry = s_entry[first + l], g = entry >> 2, c = entry & 3u;
+                const long long out = elem_index<LAYOUT>(a.pop, static_cast<int>(n), 4ll * static_cast<long long>(g_block + g) + c);
+                const uint32_t from = g * group_elems + c * static_cast<uint32_t>(n_models) + src;
+                TA::store_elem(a.a, out, TA::load_elem(image_a, from));
+                if constexpr (kHasB) TB::store_elem(a.b, out, TB::load_elem(image_b, from));
+                ++moved;
+            }
         }
-        __syncwarp();   // the permutations are overwritten by the next round
+        first += in_round;
+        if (first >= total) break;
+        __syncthreads();   // the permutations are overwritten by the next round
+        in_round = draw(first);
+        __syncthreads();
     }
     publish_block_stats(a.stats, a.stats_direct ? nullptr : a.stat_slots, selected, moved);
 }
@@ -222,7 +259,7 @@ cudaError_t launch_shuffle_wide_typed(const ShuffleArgs &call, const LaunchShape
     const size_t group_elems = 4 * static_cast<size_t>(args.pop.N) + (args.pop.layout == kLayoutPN ? args.pn_pad : 0);
     const size_t per_thread = group_elems * (TA::kBytes + (kHasB ? TB::kBytes : 0)) + 4 + 4 * wide_pitch(args.pop.N);
     if (args.pop.layout == kLayoutPN && !args.sq.slots && 4 * static_cast<size_t>(args.pop.N) * (TA::kBytes + TB::kBytes) >= kWideSplitBytes) {
-        // the images, the list (keys and places of every coordinate) and kWideRound permutations per warp
+        // the images, the list (keys and places of every coordinate) and a permutation per group
         const size_t per_group = group_elems * (TA::kBytes + (kHasB ? TB::kBytes : 0)) + 4 * 8 + 4 + 4 * wide_pitch(args.pop.N);
         const uint32_t groups = per_group * 64 > 44 * 1024 ? 32 : 64;   // five blocks and more on an SM
         const size_t smem = (per_group * groups + 15) & ~static_cast<size_t>(15);

@@ -690,3 +690,19 @@ def test_resident_warps_with_one_tile_and_with_more(N, tiles):
     c.assert_equal("N=%d tiles=%d" % (N, tiles))
     assert c.gpu_stats() == tuple(want)
     c.close()
+
+
+@pytest.mark.parametrize("N,numel,p,dtype,opt", [
+    (20, [30_001], 0.1, "bf16", None), (24, [9_001, 2], 0.5, "f32", None), (28, [253, 4, 3000], 0.9, "f32", None), (32, [40_009], 0.02, "f32", None),
+    (32, [16_390], 0.3, "bf16", "f32"), (36, [8_191], 0.6, "f32", "f32"), (48, [10_003], 0.4, "bf16", None), (60, [5_001], 0.2, "f32", "bf16"), (64, [4_099], 0.65, "f32", None), (47, [6_001], 0.5, "f32", None)])
+def test_wide_populations_coordinate_major(N, numel, p, dtype, opt):
+    """[P][N], N > 16: four models to a thread, the block's permutations drawn by some of its warps in one and in several
+    rounds, one and two threads to a group, and a population that is no multiple of four."""
+    c = Case(N, numel, 1, dtype, opt, seed=N)
+    for step in (0, 1):
+        (B.wash_shuffle_both if opt else B.wash_shuffle)(c.gpu.ctx, step, p, None, seed=8, stats=c.stats_dev)
+    want = np.array(oracle.shuffle(c.ora, c.host, p, seed=8, step=0, stack2=c.host_opt), dtype=np.int64)
+    want += np.array(oracle.shuffle(c.ora, c.host, p, seed=8, step=1, stack2=c.host_opt), dtype=np.int64)
+    c.assert_equal("N=%d p=%g" % (N, p))
+    assert c.gpu_stats() == tuple(want)
+    c.close()
