@@ -51,6 +51,24 @@ constexpr double kSparsePerBlock = 16.0;   // selected coordinates a block expec
 // neighbouring coordinates share would not stay (6.3e6 coordinates, 1 %: N = 28 85 us, 29 113, 33 with 256 entries 97).
 __host__ __device__ constexpr uint32_t sparse_queue_capacity(int n_models) { return n_models <= 28 ? 512u : 256u; }
 
+// A scattered value of a stack.  HALF_LINE: the L2 is asked to fetch 64 bytes around it instead of the 128 it fetches otherwise
+// (it does not go below 64).  Where accesses are dense enough for the bytes to count, and not the memory's pages alone, that
+// is a third of the loads' time: 2^21 loads of 4 bytes, one in 800 / 200 / 80 bytes 45 / 40 / 28 us, with 64 bytes 41 / 26 / 22.
+template <class T, bool HALF_LINE>
+__device__ __forceinline__ uint32_t load_scattered(const void *stack, long long idx)
+{
+    if constexpr (!HALF_LINE) return T::load_elem(stack, idx);
+    const void *p = static_cast<const char *>(stack) + idx * T::kBytes;
+    uint32_t v;
+    if constexpr (T::kBytes == 4) asm volatile("ld.global.L2::64B.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    else {
+        uint16_t h;
+        asm volatile("ld.global.L2::64B.u16 %0, [%1];" : "=h"(h) : "l"(p) : "memory");
+        v = h;
+    }
+    return v;
+}
+
 // list of a warp of the form for dense selections: a tile's 512 coordinates and what the tile before left
 constexpr uint32_t kWarpList = 512 + 32;
 
@@ -65,12 +83,12 @@ struct SparseArgs {
 };
 
 // One stack's values of a lane's coordinate: all loaded into the lane's column of shared memory, then stored.
-template <class T, int LAYOUT, class PERM>
+template <class T, int LAYOUT, bool HALF_LINE, class PERM>
 __device__ __forceinline__ void serve_row(const PopView &pop, void *stack, uint32_t *column, long long elem, const PERM &source_of)
 {
     const int n_models = pop.N;
 #pragma unroll 8
-    for (int n = 0; n < n_models; ++n) column[n * kSparseThreads] = T::load_elem(stack, elem_index<LAYOUT>(pop, n, elem));
+    for (int n = 0; n < n_models; ++n) column[n * kSparseThreads] = load_scattered<T, HALF_LINE>(stack, elem_index<LAYOUT>(pop, n, elem));
 #pragma unroll 4
     for (int n = 0; n < n_models; ++n) {
         const uint32_t src = source_of(n);
@@ -81,7 +99,7 @@ __device__ __forceinline__ void serve_row(const PopView &pop, void *stack, uint3
 // MIRROR: the moved values go to a second copy of the stacks as well (wash_step_host: the caller's buffers).
 // ROWS: a lane per coordinate loads all its values before it stores them (serve_row), instead of a lane per (coordinate,
 // model) pair.
-template <class TA, class TB, int LAYOUT, bool MIRROR, bool ROWS>
+template <class TA, class TB, int LAYOUT, bool MIRROR, bool ROWS, bool HALF_LINE>
 __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_sparse_kernel(const __grid_constant__ SparseArgs p)
 {
     if (p.release_early) let_next_start();
@@ -155,8 +173,8 @@ __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_spa
                 const uint2 packed = q_key[e];
                 const uint8_t *wide = reinterpret_cast<const uint8_t *>(q_wide + e * wide_pitch(n_models));
                 const auto source_of = [&](int n) -> uint32_t { return n_models <= 16 ? ((n < 8 ? packed.x : packed.y) >> (4 * (n & 7))) & 15u : wide[n]; };
-                serve_row<TA, LAYOUT>(a.pop, a.a, column, elem, source_of);
-                if constexpr (kHasB) serve_row<TB, LAYOUT>(a.pop, a.b, column, elem, source_of);
+                serve_row<TA, LAYOUT, HALF_LINE>(a.pop, a.a, column, elem, source_of);
+                if constexpr (kHasB) serve_row<TB, LAYOUT, HALF_LINE>(a.pop, a.b, column, elem, source_of);
                 for (int n = 0; n < n_models; ++n) moved += source_of(n) != static_cast<uint32_t>(n) ? 1u : 0u;
             }
         } else {
@@ -189,8 +207,8 @@ __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_spa
                             const long long elem = block_elem + q_elem[e];
                             const long long in = elem_index<LAYOUT>(a.pop, static_cast<int>(src), elem);
                             out[k] = elem_index<LAYOUT>(a.pop, static_cast<int>(n), elem);
-                            va[k] = TA::load_elem(a.a, in);
-                            if constexpr (kHasB) vb[k] = TB::load_elem(a.b, in);
+                            va[k] = load_scattered<TA, HALF_LINE>(a.a, in);
+                            if constexpr (kHasB) vb[k] = load_scattered<TB, HALF_LINE>(a.b, in);
                         }
                     }
                 }
@@ -219,7 +237,7 @@ __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_spa
 // Where much is selected: a warp by itself, without the block's barriers.  It lists a tile's selected coordinates in order behind
 // the few left over from the tile before and serves them 32 at a time, a lane per coordinate (serve_row), so that
 // one warp's mask, another's loads and a third one's stores run beside each other all the time.
-template <class TA, class TB, int LAYOUT>
+template <class TA, class TB, int LAYOUT, bool HALF_LINE>
 __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_sparse_warps_kernel(const __grid_constant__ SparseArgs p)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -266,8 +284,8 @@ __global__ void __launch_bounds__(kSparseThreads, 32 / kSparseWarps) shuffle_spa
             if (active) {
                 const uint8_t *wide = reinterpret_cast<const uint8_t *>(s_perm + lane * wide_pitch(n_models));
                 const auto source_of = [&](int n) -> uint32_t { return n_models <= 16 ? static_cast<uint32_t>(packed >> (4 * n)) & 15u : wide[n]; };
-                serve_row<TA, LAYOUT>(a.pop, a.a, column, elem, source_of);
-                if constexpr (kHasB) serve_row<TB, LAYOUT>(a.pop, a.b, column, elem, source_of);
+                serve_row<TA, LAYOUT, HALF_LINE>(a.pop, a.a, column, elem, source_of);
+                if constexpr (kHasB) serve_row<TB, LAYOUT, HALF_LINE>(a.pop, a.b, column, elem, source_of);
                 for (int n = 0; n < n_models; ++n) moved += source_of(n) != static_cast<uint32_t>(n) ? 1u : 0u;
                 ++selected;
             }
@@ -315,24 +333,43 @@ inline bool sparse_by_warps(const ShuffleArgs &args, bool bf16, bool two_stacks)
     return N <= 15 && share >= (N <= 3 ? 0.25f : N <= 10 ? 0.3f : N <= 12 ? 0.4f : 0.7f);
 }
 
+// Whether the loads of values ask for 64 bytes.  128 bytes are the better request where a line's other half holds a selected
+// coordinate as well, which is then fetched for nothing; and where masks and not values are most of the time the two are alike and the
+// plain load costs fewer instructions (ResNet-18 N = 5 with momentum, p = 1e-3: 10.6 -> 10.9 us).  128 / 64 bytes, 2^24 coordinates,
+//   [N][P] fp32: N = 2 two stacks, 5 % (1.6 to a line) 48.8 / 43.1, 10 % 66.0 / 65.9; 5 2 % 45.4 / 42.1, 5 % 81.3 / 76.3, 15 % 111 / 128; 8 2 % 81.8 / 75.7,
+//     6 % 149 / 149; 16 (2^23) 2 % 96.2 / 92.3, 6 % 169 / 181; 32 5 % (by warps) 339 / 306;  bf16: N = 8 2 % (1.3 to a line) 62.2 / 59.3, 6 % 92 / 107;
+//     32 (2^23) 2 % 149 / 158
+//   [P][N] fp32, two stacks: N = 3 5 % (0.5 to a line) 54.7 / 48.9, 30 % (3.2) 141 / 146; 5 10 % (0.6) 118 / 104, 30 % 206 / 216; 8 10 % 132 / 119.
+// ResNet-50 N = 8, bf16 + fp32, p = 5e-3: 77.2 -> 71.3 us, N = 5, p = 0.05 -> 0 46.8 -> 44.9.
+inline bool fetch_half_lines(const ShuffleArgs &args, int elem_bytes, bool two_stacks)
+{
+    const int N = args.pop.N;
+    const float per_line = args.expected_share * 128.f / static_cast<float>(args.pop.layout == kLayoutNP ? elem_bytes : elem_bytes * N);
+    const float most = args.pop.layout == kLayoutPN ? 1.f : N <= 5 || sparse_by_warps(args, elem_bytes == 2, two_stacks) ? 2.f : N <= 16 ? 1.5f : 1.2f;
+    return per_line < most && args.expected_share * N * (two_stacks ? 2 : 1) >= 0.02f;
+}
+
 template <class TA, class TB>
 cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchShape &shape, cudaStream_t stream)
 {
     if (args.group_hi <= args.group_lo) return cudaSuccess;
     SparseArgs p;
     p.s = args;
+    const bool half = fetch_half_lines(args, TA::kBytes, TB::kCode != kDtypeNone);
     p.n_wtiles = (args.group_hi - args.group_lo + kWarpTileGroups - 1) / kWarpTileGroups;
     size_t smem = sparse_queue_capacity(args.pop.N) * (12 + (args.pop.N > 16 ? 4 * static_cast<size_t>(wide_pitch(args.pop.N)) : 0));
     const bool np = args.pop.layout == kLayoutNP;
-    auto kernel = np ? shuffle_sparse_kernel<TA, TB, kLayoutNP, false, false> : shuffle_sparse_kernel<TA, TB, kLayoutPN, false, false>;
-    if (args.mirror_a) kernel = np ? shuffle_sparse_kernel<TA, TB, kLayoutNP, true, false> : shuffle_sparse_kernel<TA, TB, kLayoutPN, true, false>;
+    auto kernel = np ? shuffle_sparse_kernel<TA, TB, kLayoutNP, false, false, false> : shuffle_sparse_kernel<TA, TB, kLayoutPN, false, false, false>;
+    if (half) kernel = np ? shuffle_sparse_kernel<TA, TB, kLayoutNP, false, false, true> : shuffle_sparse_kernel<TA, TB, kLayoutPN, false, false, true>;
+    if (args.mirror_a) kernel = np ? shuffle_sparse_kernel<TA, TB, kLayoutNP, true, false, false> : shuffle_sparse_kernel<TA, TB, kLayoutPN, true, false, false>;
     else if (np && args.expected_share >= (args.pop.N >= 24 ? kRowsShareLarge : args.pop.N >= 8 ? kRowsShare : 2.f)) {
-        kernel = shuffle_sparse_kernel<TA, TB, kLayoutNP, false, true>;
+        kernel = half ? shuffle_sparse_kernel<TA, TB, kLayoutNP, false, true, true> : shuffle_sparse_kernel<TA, TB, kLayoutNP, false, true, false>;
         p.column_offset = static_cast<uint32_t>(smem);
         smem += 4 * static_cast<size_t>(args.pop.N) * kSparseThreads;
     }
     if (!args.mirror_a && sparse_by_warps(args, TA::kBytes == 2, TB::kCode != kDtypeNone)) {
-        auto by_warps = np ? shuffle_sparse_warps_kernel<TA, TB, kLayoutNP> : shuffle_sparse_warps_kernel<TA, TB, kLayoutPN>;
+        auto by_warps = np ? shuffle_sparse_warps_kernel<TA, TB, kLayoutNP, false> : shuffle_sparse_warps_kernel<TA, TB, kLayoutPN, false>;
+        if (half && np) by_warps = shuffle_sparse_warps_kernel<TA, TB, kLayoutNP, true>;
         smem = 4 * kSparseWarps * static_cast<size_t>(kWarpList) + 4 * static_cast<size_t>(args.pop.N) * kSparseThreads +
                (args.pop.N > 16 ? 4 * static_cast<size_t>(wide_pitch(args.pop.N)) * kSparseThreads : 0);
         KernelFit fit;

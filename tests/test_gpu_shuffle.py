@@ -706,3 +706,21 @@ def test_wide_populations_coordinate_major(N, numel, p, dtype, opt):
     c.assert_equal("N=%d p=%g" % (N, p))
     assert c.gpu_stats() == tuple(want)
     c.close()
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("N,p,dtype,opt", [(2, 0.03, "f32", None), (5, 0.004, "f32", "f32"), (8, 0.01, "bf16", "f32"), (16, 0.02, "bf16", None), (20, 0.05, "f32", None),
+                                           (32, 0.001, "f32", "bf16"), (64, 0.004, "bf16", None), (3, 0.0004, "f32", None), (5, 0.0002, "f32", "f32")])
+def test_sparse_loads_of_half_lines_and_half_waves(N, p, dtype, opt, layout):
+    """Selections for which the sparse kernel's loads ask for 64 bytes (pairs, rows and warps that serve by themselves), and those
+    rare enough for half a wave of blocks; three steps in a row, the second drawing while the first still serves."""
+    numel = [700_001, 9, 120_000] if N <= 16 else [150_001, 9]
+    c = Case(N, numel, layout, dtype, opt, seed=N)
+    B.wash_set_mode(c.gpu.ctx, B.WASH_MODE_SPARSE)
+    want = np.zeros(2, dtype=np.int64)
+    for step in range(3):
+        (B.wash_shuffle_both if opt else B.wash_shuffle)(c.gpu.ctx, step, p, None, seed=17, stats=c.stats_dev)
+        want += np.array(oracle.shuffle(c.ora, c.host, p, seed=17, step=step, stack2=c.host_opt), dtype=np.int64)
+    c.assert_equal("N=%d p=%g layout=%d" % (N, p, layout))
+    assert c.gpu_stats() == tuple(want)
+    c.close()
