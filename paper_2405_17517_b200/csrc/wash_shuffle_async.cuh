@@ -284,6 +284,38 @@ __device__ __forceinline__ uint32_t dense_bytes_write(const ShuffleArgs &a, cons
     return moved;
 }
 
+// two or four neighbouring values, stored together
+template <class T, int COUNT>
+__device__ __forceinline__ void store_neighbours(char *p, const uint32_t (&v)[COUNT])
+{
+    if constexpr (COUNT == 4) T::store_group(p, T::pack(v[0], v[1], v[2], v[3]));
+    else if constexpr (T::kBytes == 4) *reinterpret_cast<uint2 *>(p) = make_uint2(v[0], v[1]);
+    else *reinterpret_cast<uint32_t *>(p) = v[0] | (v[1] << 16);
+}
+
+// COUNT neighbouring models' values of a coordinate in [P][N], stored together: model n + q takes the value of model nibble q of perm.
+// Fixed points are stored, too.  A lane serves a coordinate, so a store of one value is 32 scattered writes for the L2, which
+// bound dealt serving: 2^24 coordinates, by single values -> by four (N a multiple of 4) or two (other even N), N = 8 bf16, p = 0.2 180 ->
+// 120 us, two fp32 stacks, p = 0.4 449 -> 272; N = 12 bf16, p = 0.03 142 -> 114; N = 16 fp32, p = 0.1 210 -> 197, 0.4 481 -> 323, bf16 + fp32, p = 0.1 504 ->
+// 307, 0.4 1196 -> 500; by two N = 6 bf16, p = 0.1 102 -> 77, N = 14 two fp32 stacks, p = 0.4 900 -> 596.  N = 2 stays by single
+// values (two fp32 stacks, p = 0.03 57 -> 63 us by two).
+template <class TA, class TB, int COUNT>
+__device__ __forceinline__ uint32_t move_neighbours(const ShuffleArgs &a, const unsigned char *image_a, const unsigned char *image_b,
+                                                    uint32_t img0, uint32_t perm, int n, long long out0)
+{
+    uint32_t va[COUNT], vb[COUNT], moved = 0;
+#pragma unroll
+    for (int q = 0; q < COUNT; ++q) {
+        const uint32_t src = (perm >> (4 * q)) & 15u;
+        moved += src != static_cast<uint32_t>(n + q) ? 1u : 0u;
+        va[q] = TA::load_elem(image_a, img0 + src);
+        if constexpr (TB::kCode != kDtypeNone) vb[q] = TB::load_elem(image_b, img0 + src);
+    }
+    store_neighbours<TA, COUNT>(static_cast<char *>(a.a) + (out0 + n) * TA::kBytes, va);
+    if constexpr (TB::kCode != kDtypeNone) store_neighbours<TB, COUNT>(static_cast<char *>(a.b) + (out0 + n) * TB::kBytes, vb);
+    return moved;
+}
+
 // The moves of one selected coordinate (coordinate c of the group of block thread t_owner): model n
 // takes the value of model pi(n), nibble n of `perm` (N <= 16) or byte n of the column s_perm.
 template <class TA, class TB, int LAYOUT>
@@ -301,6 +333,14 @@ __device__ __forceinline__ void move_coordinate(const ShuffleArgs &a, const unsi
     const long long out0 = LAYOUT == kLayoutNP ? e : e * n_models;
     const uint32_t img_step = LAYOUT == kLayoutNP ? T_ * 4u : 1u;
     const uint32_t img0 = LAYOUT == kLayoutNP ? t_owner * 4u + c : t_owner * pn_group_elems(n_models, a.pn_pad) + c * n_models;
+    if (LAYOUT == kLayoutPN && n_models <= 16 && n_models % 4 == 0) {
+        for (int n = 0; n < n_models; n += 4, perm >>= 16) moved += move_neighbours<TA, TB, 4>(a, image_a, image_b, img0, static_cast<uint32_t>(perm), n, out0);
+        return;
+    }
+    if (LAYOUT == kLayoutPN && n_models <= 16 && n_models % 2 == 0 && n_models != 2) {
+        for (int n = 0; n < n_models; n += 2, perm >>= 8) moved += move_neighbours<TA, TB, 2>(a, image_a, image_b, img0, static_cast<uint32_t>(perm), n, out0);
+        return;
+    }
     long long out = out0;
     uint64_t rest = perm;   // nibble n on top of the low end when model n's turn comes
     for (int n = 0; n < n_models; ++n, out += out_step, rest >>= 4) {

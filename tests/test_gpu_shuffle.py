@@ -724,3 +724,19 @@ def test_sparse_loads_of_half_lines_and_half_waves(N, p, dtype, opt, layout):
     c.assert_equal("N=%d p=%g layout=%d" % (N, p, layout))
     assert c.gpu_stats() == tuple(want)
     c.close()
+
+
+@pytest.mark.parametrize("code", [-4, -5], ids=["resident", "one-trip"])
+@pytest.mark.parametrize("dtype,opt", [("f32", None), ("bf16", None), ("f32", "bf16"), ("bf16", "f32"), ("f32", "f32")])
+@pytest.mark.parametrize("N", [2, 4, 6, 8, 10, 14, 16])
+def test_neighbouring_models_stored_together(N, dtype, opt, code):
+    """[P][N], dealt serving: two or four models' values with one store (N even, N a multiple of 4), fixed points
+    among them, counted as not moved; also in tensors that end inside a group."""
+    c = Case(N, [9001, 3, 130, 2046], 1, dtype, opt, seed=N)
+    B.wash_set_launch(c.gpu.ctx, 0, code)
+    p_layer = [0.1, 1.0, 0.45, 0.25]
+    (B.wash_shuffle_both if opt else B.wash_shuffle)(c.gpu.ctx, 4, 0.0, p_layer, seed=5, stats=c.stats_dev)
+    want = oracle.shuffle(c.ora, c.host, p_layer, seed=5, step=4, stack2=c.host_opt)
+    c.assert_equal("N=%d %s/%s" % (N, dtype, opt))
+    assert c.gpu_stats() == tuple(want)
+    c.close()
