@@ -1097,9 +1097,10 @@ int wash_check(wash_ctx *ctx, void *stream_v)
     if (err != cudaSuccess) return cuda_fail(err, "reading the status word");
     if (status) {
         cudaMemsetAsync(ctx->status_dev, 0, sizeof(uint32_t), stream);
-        return fail(WASH_ERR_DEVICE_CHECK, "device status 0x%x:%s%s", status,
+        return fail(WASH_ERR_DEVICE_CHECK, "device status 0x%x:%s%s%s", status,
                     (status & 1u) ? " a group outside its segment table;" : "",
-                    (status & 4u) ? " an exchange step needed more slots than the staging buffers hold;" : "");
+                    (status & 4u) ? " an exchange step needed more slots than the staging buffers hold;" : "",
+                    (status & 8u) ? " a block's copies did not arrive;" : "");
     }
     return WASH_OK;
 }

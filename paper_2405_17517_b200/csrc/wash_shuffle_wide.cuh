@@ -160,13 +160,35 @@ constexpr size_t kWideSplitBytes = 512;
 // move.  N = 32 fp32, 2^23, p = 0.1 / 0.3: an even share 226 / 407 us (by pairs), 16 209 / 349, 32 221 / 364.  The moves are dealt to all threads.
 constexpr uint32_t kWideChunk = 16;
 
-template <class TA, class TB>
+// A copy of the block's contiguous bytes by one thread (16-byte aligned, a multiple of 16 bytes), reported to an mbarrier.
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_t bytes, uint32_t barrier)
+{
+    asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes), "r"(barrier) : "memory");
+}
+// Waits for the barrier's first phase, but not for ever.
+__device__ __forceinline__ bool bulk_copies_done(uint32_t barrier)
+{
+    for (uint32_t i = 0; i < (1u << 20); ++i) {
+        uint32_t done;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(done) : "r"(barrier) : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+
+// BULK: the block's bytes come by one bulk copy a stack instead of 16 bytes a thread at a time (a sixth of the kernel's instructions).
+// Which launches: those whose blocks have 64 groups, and larger groups with 32.  Time by 16 bytes over time by bulk copies, 2^22 - 2^23 coordinates, p = 0.01 /
+// 0.03 / 0.1 / 0.3 / 0.6; blocks of 64 groups N = 32 fp32 (512 bytes) 1.04 1.09 1.12 1.09 1.07, N = 24 bf16 + fp32 (576) 1.14 1.17 1.13 1.17 1.13; of 32 groups
+// N = 24 fp32 twice (768) 1.02 0.74 0.83 1.14 1.11, N = 48 fp32 (768) 0.80 0.75 0.87 1.11 1.08, N = 32 fp32 twice (1024) 1.03 0.88 0.96 1.18 1.12, N = 64 fp32 (1024) 1.10 1.23
+// 1.19 1.11 1.07, N = 48 bf16 + fp32 (1152) 1.21 1.33 1.31 1.20 1.13, N = 64 fp32 twice (2048) 1.22 1.37 1.32 1.19 1.12.  N = 32 fp32, 2^25, p = 0.1 813 -> 707 us.
+template <class TA, class TB, bool BULK>
 __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_constant__ ShuffleArgs a)
 {
     await_previous();
     let_next_start();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ uint32_t s_count;
+    __shared__ __align__(8) unsigned long long s_barrier;
     constexpr int LAYOUT = kLayoutPN;
     constexpr bool kHasB = TB::kCode != kDtypeNone;
     const int n_models = a.pop.N;
@@ -182,9 +204,22 @@ __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_co
 
     const uint64_t g_block = a.group_lo + static_cast<uint64_t>(blockIdx.x) * groups;
     const uint32_t in_block = static_cast<uint32_t>(min(static_cast<uint64_t>(groups), a.group_hi - g_block));
-    async_fetch<TA, LAYOUT>(smem_addr(image_a), a.a, a.pop, g_block, in_block, n_models, a.pn_pad);
-    if constexpr (kHasB) async_fetch<TB, LAYOUT>(smem_addr(image_b), a.b, a.pop, g_block, in_block, n_models, a.pn_pad);
-    if (threadIdx.x == 0) s_count = 0;
+    const uint32_t barrier = smem_addr(&s_barrier);
+    if constexpr (BULK) {
+        if (threadIdx.x == 0) {
+            s_count = 0;
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barrier) : "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            const uint32_t bytes_a = in_block * 4u * n_models * TA::kBytes, bytes_b = kHasB ? in_block * 4u * n_models * TB::kBytes : 0u;
+            asm volatile("{\n\t.reg .b64 s;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 s, [%0], %1;\n\t}" ::"r"(barrier), "r"(bytes_a + bytes_b) : "memory");
+            bulk_copy(smem_addr(image_a), group_vec_ptr<TA, LAYOUT>(a.a, a.pop, g_block, 0), bytes_a, barrier);
+            if constexpr (kHasB) bulk_copy(smem_addr(image_b), group_vec_ptr<TB, LAYOUT>(a.b, a.pop, g_block, 0), bytes_b, barrier);
+        }
+    } else {
+        async_fetch<TA, LAYOUT>(smem_addr(image_a), a.a, a.pop, g_block, in_block, n_models, a.pn_pad);
+        if constexpr (kHasB) async_fetch<TB, LAYOUT>(smem_addr(image_b), a.b, a.pop, g_block, in_block, n_models, a.pn_pad);
+        if (threadIdx.x == 0) s_count = 0;
+    }
     __syncthreads();
 
     uint32_t selected = 0, moved = 0;
@@ -222,8 +257,14 @@ __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_co
     };
     // the first round's permutations are drawn while the copies are in flight
     uint32_t in_round = draw(0);
-    cp_async_wait_all();
-    __syncthreads();   // a group's bytes were copied by threads of other warps
+    if constexpr (BULK) {
+        if (!bulk_copies_done(barrier)) {   // (not seen) report and move nothing; the block stays for its copies once more as long
+            if (a.status) atomicOr(a.status, 8u);
+            bulk_copies_done(barrier);
+            return;
+        }
+    } else cp_async_wait_all();
+    __syncthreads();   // a group's bytes were copied, its permutations drawn by threads of other warps
     if (threadIdx.x == 0) selected = total;
     for (uint32_t first = 0; first < total;) {
         if (n_models % 4 == 0) moved += move_quads<TA, TB>(a, image_a, image_b, g_block, s_perm, s_entry + first, in_round, threadIdx.x, blockDim.x);
@@ -263,14 +304,18 @@ cudaError_t launch_shuffle_wide_typed(const ShuffleArgs &call, const LaunchShape
         const size_t per_group = group_elems * (TA::kBytes + (kHasB ? TB::kBytes : 0)) + 4 * 8 + 4 + 4 * wide_pitch(args.pop.N);
         const uint32_t groups = per_group * 64 > 44 * 1024 ? 32 : 64;   // five blocks and more on an SM
         const size_t smem = (per_group * groups + 15) & ~static_cast<size_t>(15);
+        // a bulk copy takes multiples of 16 bytes: groups come in pairs (rows and ranges are whole units of 8 elements) and have 8 N bytes at least
+        const size_t group_bytes = 4 * static_cast<size_t>(args.pop.N) * (TA::kBytes + TB::kBytes);
+        const bool bulk = args.pn_pad == 0 && ((args.group_lo | args.group_hi) & 1u) == 0 && (groups == 64 || group_bytes > 1024 || (group_bytes == 1024 && !kHasB));
+        auto kernel = bulk ? shuffle_wide_pn_kernel<TA, TB, true> : shuffle_wide_pn_kernel<TA, TB, false>;
         KernelFit fit;
-        cudaError_t err = kernel_fit(reinterpret_cast<const void *>(shuffle_wide_pn_kernel<TA, TB>), 2 * static_cast<int>(groups), smem, &fit);
+        cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), 2 * static_cast<int>(groups), smem, &fit);
         if (err != cudaSuccess) return err;
         if (fit.occupancy < 1) return cudaErrorLaunchOutOfResources;
         const uint64_t grid = (static_cast<uint64_t>(args.group_hi - args.group_lo) + groups - 1) / groups;
         if (grid == 0) return cudaSuccess;
         if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-        return launch_chained(shuffle_wide_pn_kernel<TA, TB>, static_cast<unsigned>(grid), 2 * groups, smem, stream, args);
+        return launch_chained(kernel, static_cast<unsigned>(grid), 2 * groups, smem, stream, args);
     }
     int threads = shape.threads > 0 ? (shape.threads >= 64 ? 64 : 32) : 64;
     while (threads > 32 && per_thread * threads > 44 * 1024) threads >>= 1;   // five blocks and more on an SM
