@@ -26,7 +26,16 @@
 
 namespace wash {
 
-constexpr uint32_t kDenseMinSelected = 64;   // selected coordinates of a warp's 128 from which every lane serves its own group
+// Selected coordinates of a warp's 128 from which every lane serves its own group.  Later in [P][N] where the dealt coordinates' values are
+// stored together (move_neighbours): dense / dealt at 45 / 55 / 70 / 85 / 100 % selected, 2^23 coordinates, N = 2 fp32 1.15 1.09 0.98 0.83 0.84, N = 8 fp32 1.06 1.10
+// 1.07 0.92 0.91, N = 16 bf16 1.11 1.24 1.20 0.99 0.99, N = 10 two fp32 stacks 1.03 1.34 1.15 0.98 0.86; never with two stacks of a multiple of four models from 8 on, N = 8
+// two fp32 stacks 1.17 1.83 1.87 1.63 1.65, N = 16 bf16 + fp32 1.23 2.06 2.16 1.89 1.82.
+template <int LAYOUT, bool TWO_STACKS>
+__device__ __forceinline__ uint32_t dense_min_selected(int n_models)
+{
+    if (LAYOUT == kLayoutNP || n_models % 2 != 0) return 64;
+    return TWO_STACKS && n_models >= 8 && n_models % 4 == 0 ? 129 : 100;
+}
 
 template <int BYTES>
 __device__ __forceinline__ void cp_async(uint32_t dst_smem, const void *src)
@@ -385,7 +394,7 @@ __device__ __forceinline__ void plan_tile(const ShuffleArgs &a, uint8_t *s_list,
     if (!__any_sync(0xFFFFFFFFu, sel != 0)) return;   // most warps have nothing selected at small p
     const uint32_t mine = __popc(sel);
     const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, mine);
-    if (total >= kDenseMinSelected && __all_sync(0xFFFFFFFFu, sel == 0 || gi.valid == 4)) {
+    if (total >= dense_min_selected<kLayoutNP, false>(n_models) && __all_sync(0xFFFFFFFFu, sel == 0 || gi.valid == 4)) {   // (the early flavour: N > 16)
         pl.mode = kServeDense;
         if (sel) {
             if (n_models <= 16) dense_draw<uint64_t>(a, sel, gi, pl.perm, selected, moved);
@@ -550,7 +559,7 @@ __device__ __forceinline__ void serve_tile(const ShuffleArgs &a, const unsigned 
         serve_few<TA, TB, LAYOUT>(a, image_a, image_b, g_block, sel, gi, selected, moved);
         return;
     }
-    if (n_models <= 16 && total >= kDenseMinSelected && __all_sync(0xFFFFFFFFu, sel == 0 || gi.valid == 4)) {
+    if (n_models <= 16 && total >= dense_min_selected<LAYOUT, TB::kCode != kDtypeNone>(n_models) && __all_sync(0xFFFFFFFFu, sel == 0 || gi.valid == 4)) {
         if (sel) {
             if (n_models <= 8) serve_group_dense<TA, TB, LAYOUT, uint32_t>(a, image_a, image_b, g_block, sel, gi, selected, moved);
             else serve_group_dense<TA, TB, LAYOUT, uint64_t>(a, image_a, image_b, g_block, sel, gi, selected, moved);

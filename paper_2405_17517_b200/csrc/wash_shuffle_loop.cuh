@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(32, G == 2 ? 32 : 28) shuffle_loop_kernel(cons
         if (!__any_sync(0xFFFFFFFFu, sel != 0)) continue;
         const unsigned char *images = smem_raw + stage * stage_bytes;
         const uint32_t count = __reduce_add_sync(0xFFFFFFFFu, __popc(sel));
-        if (count >= kDenseMinSelected * G) {
+        if (count >= dense_min_selected<LAYOUT, kHasB>(n_models) * G) {
             // every lane serves its own groups, those that are whole; the others go to the list below
 #pragma unroll 1
             for (int i = 0; i < G; ++i) {

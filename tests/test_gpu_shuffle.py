@@ -731,10 +731,11 @@ def test_sparse_loads_of_half_lines_and_half_waves(N, p, dtype, opt, layout):
 @pytest.mark.parametrize("N", [2, 4, 6, 8, 10, 14, 16])
 def test_neighbouring_models_stored_together(N, dtype, opt, code):
     """[P][N], dealt serving: two or four models' values with one store (N even, N a multiple of 4), fixed points
-    among them, counted as not moved; also in tensors that end inside a group."""
-    c = Case(N, [9001, 3, 130, 2046], 1, dtype, opt, seed=N)
+    among them, counted as not moved; in tensors that end inside a group, and up to the selection that is served densely or, with
+    two stacks of 8 models and more, is not."""
+    c = Case(N, [9001, 3, 130, 2046, 3001], 1, dtype, opt, seed=N)
     B.wash_set_launch(c.gpu.ctx, 0, code)
-    p_layer = [0.1, 1.0, 0.45, 0.25]
+    p_layer = [0.1, 1.0, 0.45, 0.25, 0.9]
     (B.wash_shuffle_both if opt else B.wash_shuffle)(c.gpu.ctx, 4, 0.0, p_layer, seed=5, stats=c.stats_dev)
     want = oracle.shuffle(c.ora, c.host, p_layer, seed=5, step=4, stack2=c.host_opt)
     c.assert_equal("N=%d %s/%s" % (N, dtype, opt))
