@@ -44,6 +44,8 @@ constexpr int kSlots = 4;   // pinned staging slots for table uploads
 // Expected share of selected coordinates from which the streaming kernel's early flavour is launched (N > 16) instead of the
 // wide kernel.  2^24 coordinates, fp32, N = 32, wide / early at 50 / 70 / 100 %: [N][P] 559 / 647, 693 / 690, 895 / 665 us; [P][N] 659 / 960, 838 / 867,
 // 1092 / 848; N = 17 crosses at 60 %, N = 64 and two stacks at 70-90 %.
+// Not in [P][N] with a multiple of four models, whose moves the wide kernels make four at a time: 2^22 coordinates, 70 / 100 %, N = 20 fp32 169 / 239, 212 / 220,
+// N = 32 301 / 503, 389 / 427, N = 64 bf16 + fp32 1021 / 2729, 1302 / 2245.
 constexpr double kEarlyShare = 0.7;
 // wash_step_host: up to this expected selection the moved values are stored into the caller's mapped buffers, above it the
 // stacks are copied back.  A scattered store over PCIe took 0.87 ns a value ([P][N]: the N values of a coordinate share one), the
@@ -197,6 +199,9 @@ void *mapped_host(void *ptr, size_t bytes, int dtype)
 // floor(p * 2^32) for p in [0, 1]; the product is exact in binary64
 uint64_t threshold_of(double p) { return static_cast<uint64_t>(std::floor(p * 4294967296.0)); }
 
+// [P][N]: whether the streaming kernels store neighbouring models' values together
+bool stored_together(int layout, int N) { return layout == WASH_LAYOUT_PN && N % (N <= 16 ? 2 : 4) == 0; }
+
 // WASH_MODE_AUTO: the expected share of selected coordinates up to which the sparse kernel is launched.  Serving a
 // coordinate costs it a scattered DRAM access and store per model and stack in [N][P], a few neighbouring ones for
 // all N models in [P][N]; the streaming kernels pay for the stack's bytes and, in small populations, for issue slots.
@@ -206,10 +211,11 @@ uint64_t threshold_of(double p) { return static_cast<uint64_t>(std::floor(p * 42
 //                       bf16  2: 13, 3: 20, 4: 18, 5: 8, 6: 8 (then level to 20), 8: 8, 10: 8, 12: 6.2, 16: 6.3, 20: 2.7, 24: 2, 32: 3, 64: 1.7
 //           two stacks  fp32  2: 30, 3: 12, 4: 6, 5: 5, 6: 4.5, 8: 3.8, 10: 3.4, 12: 3.2, 16: 3, 20: 3.2, 24: 3, 32: 3, 64: 2;
 //                bf16 + fp32  2: 20, 3: 25, 4: 9, 5: 5, 6: 4.5, 8: 3.5, 10: 3, 12: 3, 16: 2.5, 20: 2.8, 24: 2.3, 32: 2.5, 64: 1.6
-//   [P][N]  one stack   fp32  2: 13, 3: 17, 4: to 50, 5: 18, 6: 18, 8: to 50, 10: 16, 12: 22, 16: to 50, 20: 30, 24: 45, 32: to 50, 64: 100
-//                       bf16  2: 14, 3: 18, 4 to 8: to 50, 10 and 12: 40, 16: to 50, 20 and 24: 20, 32: 25, 64: to 50
-//           two stacks  fp32  2: to 50, 3: 20, 4: 20, 5: 25, 6: 35, 8: 90, 10: 60, 12: 80, 20: 55, 16 and from 24 on: 100;
-//                bf16 + fp32  2: 20, 3: 30, 4: 30, 5: 35, 6: 45, 8: 70, 10: 60, 12: 70, 20: 60, 16 and from 24 on: 100
+//   [P][N]  one stack   fp32  2: 14, 3: 17, 4: 35, 5: 18, 6: 19, 8: 20, 10: 15, 12: 16, 16: 16, 20: 17, 24: 20, 28: 22, 32: 22, 33: 36, 48: 36, 64: 45
+//                       bf16  2: 18, 3: 18, 4: 42, 5: to 50, 6: 35, 8: 19, 9: 37, 10: 19, 12: 17, 16: 17, 20 to 32: 13, 33: 16, 48: 17, 64: 15
+//           two stacks  fp32  2: 35, 3: 20, 4: 22, 5: 25, 6: 23, 8: 28, 10: 27, 12: 27, 14: 32, 16: 37, 20: 27, 24: 33, 28: 33, 32: 65, 48: 55, 64: 100;
+//                bf16 + fp32  2: 18, 3: 30, 4: 20, 5: 35, 6: 20, 8: 22, 10: 25, 12: 22, 14: 40, 16: 32, 20: 27, 24: 27, 28: 33, 32: 50, 48: 40, 64: 100
+// (576 cells of [P][N], 6 to 65 %: AUTO on the slower kernel by more than 6 % in 9.)
 double sparse_share(int layout, int N, bool two_stacks, bool bf16)
 {
     if (layout == WASH_LAYOUT_NP) {
@@ -217,11 +223,15 @@ double sparse_share(int layout, int N, bool two_stacks, bool bf16)
         if (bf16) return N <= 4 ? 0.18 : N <= 7 ? 0.08 : N <= 16 ? 0.06 : 0.02;
         return std::fmax(std::fmin(0.6 / N, 0.17), 0.027);
     }
-    if (two_stacks) return N <= 4 ? 0.2 : N <= 7 ? 0.3 : 0.6;
-    if (bf16) return N <= 3 ? 0.15 : N <= 8 ? 0.5 : N <= 12 ? 0.4 : N <= 16 ? 0.5 : N <= 32 ? 0.2 : 0.45;
+    if (stored_together(layout, N)) {
+        if (two_stacks) return N <= 12 ? 0.24 : N <= 16 ? 0.34 : N <= 24 ? 0.28 : N <= 28 ? 0.36 : N < 64 ? 0.55 : 1.0;
+        if (bf16) return N == 2 ? 0.17 : N == 4 ? 0.42 : N == 6 ? 0.35 : N <= 16 ? 0.18 : N <= 32 ? 0.135 : N < 64 ? 0.17 : 0.15;
+        return N == 2 ? 0.13 : N == 4 ? 0.35 : N <= 8 ? 0.2 : N <= 16 ? 0.16 : N <= 24 ? 0.18 : N <= 32 ? 0.22 : N < 64 ? 0.36 : 0.45;
+    }
+    if (two_stacks) return N <= 4 ? 0.2 : N <= 7 ? 0.3 : N <= 16 ? 0.6 : 0.48;
+    if (bf16) return N <= 3 ? 0.15 : N <= 8 ? 0.5 : N <= 12 ? 0.37 : N <= 16 ? 0.5 : N <= 32 ? 0.2 : 0.17;
     if (N <= 3) return 0.13;
-    if (N == 4 || N == 8) return 0.5;   // a coordinate's values are whole 16-byte pieces
-    return N <= 12 ? 0.18 : N <= 16 ? 0.5 : N <= 24 ? 0.3 : 0.5;
+    return N <= 12 ? 0.18 : N <= 16 ? 0.5 : N <= 24 ? 0.3 : 0.36;
 }
 
 // Brings the device copy of the segment table up to date with the call's
@@ -357,7 +367,7 @@ int shuffle_impl(wash_ctx *ctx, int which, uint64_t step, double p, const double
         // serving for N > 16) costs registers and, for N > 16, three more permutation columns of shared
         // memory per thread: measured, it pays only for large populations of which most coordinates are
         // served (kEarlyShare).
-        args.early = ctx->N > 16 && ctx->expected_selected >= kEarlyShare * coordinates;
+        args.early = ctx->N > 16 && ctx->expected_selected >= kEarlyShare * coordinates && !stored_together(ctx->layout, ctx->N);
         if (ctx->shape.blocks_per_sm == -2) args.early = false;   // tuning override (wash_set_launch)
         if (ctx->shape.blocks_per_sm == -3) args.early = true;
         if (sq) {   // the statistic is gathered by the streaming kernel only
