@@ -10,6 +10,7 @@
 // after the other and moved its N values in a loop, all after the wait.  N = 32, fp32, 2^24 coordinates, [P][N],
 // p = 0.01 / 0.03 / 0.1: 376 / 500 / 681 -> 334 / 373 / 482 us (reading and writing alone 331 / 338 / 361); [N][P] 415 / 599 / 753 ->
 // 408 / 544 / 632 us; N = 20, bf16 + fp32, [P][N], p = 0.25: 1221 -> 678 us.
+// [P][N] since then (move_quads, bulk copies), 2^23 coordinates: 169 / 191 / 233 -> 157 / 163 / 185 us.
 #pragma once
 #define WASH_SERVING_ONLY
 #include "wash_shuffle_async.cuh"
@@ -153,7 +154,8 @@ __global__ void __launch_bounds__(64, 6) shuffle_wide_kernel(const __grid_consta
 // coordinates in one list shared evenly by its warps.  Six blocks of 35 KB hold twice the warps that way,
 // each with half the copies, draws and moves.  N = 32, fp32, 2^23 coordinates, p = 0.03 / 0.1 / 0.25: 197 / 246 / 410 us by the kernel
 // above, 192 / 233 / 404 (both with a padded image at 0.25; without 357); N = 24, bf16 + fp32, p = 0.25 436 / 386; N = 64, fp32, p = 0.1 632 / 542.  Smaller groups (N = 20, fp32, p = 0.1
-// 145 / 165 us) and [N][P] (N = 20 200 / 202, N = 17 bf16 103 / 162) lose more by the block's barriers.
+// 145 / 165 us) and [N][P] (N = 20 200 / 202, N = 17 bf16 103 / 162) lose more by the block's barriers;
+// as they do with four models a thread (from 256 bytes on: N = 17 fp32, p = 0.1 121 / 134, N = 24 fp32 155 / 173, N = 32 bf16 151 / 171).
 constexpr size_t kWideSplitBytes = 512;
 // Coordinates whose permutations a warp of that kernel draws together.  The chain of swaps costs a warp the same for one coordinate and for
 // 32, so few warps with many coordinates each take fewer instructions than an even share for all, and a longer way to the first
