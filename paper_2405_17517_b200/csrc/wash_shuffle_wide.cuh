@@ -14,6 +14,7 @@
 #pragma once
 #define WASH_SERVING_ONLY
 #include "wash_shuffle_async.cuh"
+#include "wash_bulk_copy.cuh"
 
 namespace wash {
 
@@ -162,22 +163,6 @@ constexpr size_t kWideSplitBytes = 512;
 // move.  N = 32 fp32, 2^23, p = 0.1 / 0.3: an even share 226 / 407 us (by pairs), 16 209 / 349, 32 221 / 364.  The moves are dealt to all threads.
 constexpr uint32_t kWideChunk = 16;
 
-// A copy of the block's contiguous bytes by one thread (16-byte aligned, a multiple of 16 bytes), reported to an mbarrier.
-__device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_t bytes, uint32_t barrier)
-{
-    asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes), "r"(barrier) : "memory");
-}
-// Waits for the barrier's first phase, but not for ever.
-__device__ __forceinline__ bool bulk_copies_done(uint32_t barrier)
-{
-    for (uint32_t i = 0; i < (1u << 20); ++i) {
-        uint32_t done;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(done) : "r"(barrier) : "memory");
-        if (done) return true;
-    }
-    return false;
-}
-
 // BULK: the block's bytes come by one bulk copy a stack instead of 16 bytes a thread at a time (a sixth of the kernel's instructions).
 // Which launches: those whose blocks have 64 groups, and larger groups with 32.  Time by 16 bytes over time by bulk copies, 2^22 - 2^23 coordinates, p = 0.01 /
 // 0.03 / 0.1 / 0.3 / 0.6; blocks of 64 groups N = 32 fp32 (512 bytes) 1.04 1.09 1.12 1.09 1.07, N = 24 bf16 + fp32 (576) 1.14 1.17 1.13 1.17 1.13; of 32 groups
@@ -210,10 +195,9 @@ __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_co
     if constexpr (BULK) {
         if (threadIdx.x == 0) {
             s_count = 0;
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barrier) : "memory");
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             const uint32_t bytes_a = in_block * 4u * n_models * TA::kBytes, bytes_b = kHasB ? in_block * 4u * n_models * TB::kBytes : 0u;
-            asm volatile("{\n\t.reg .b64 s;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 s, [%0], %1;\n\t}" ::"r"(barrier), "r"(bytes_a + bytes_b) : "memory");
+            bulk_barrier_init(barrier);
+            bulk_barrier_expect(barrier, bytes_a + bytes_b);
             bulk_copy(smem_addr(image_a), group_vec_ptr<TA, LAYOUT>(a.a, a.pop, g_block, 0), bytes_a, barrier);
             if constexpr (kHasB) bulk_copy(smem_addr(image_b), group_vec_ptr<TB, LAYOUT>(a.b, a.pop, g_block, 0), bytes_b, barrier);
         }
@@ -259,14 +243,17 @@ __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_co
     };
     // the first round's permutations are drawn while the copies are in flight
     uint32_t in_round = draw(0);
+    // (a group's bytes were copied, its permutations drawn by threads of other warps: both forms end with a barrier)
     if constexpr (BULK) {
-        if (!bulk_copies_done(barrier)) {   // (not seen) report and move nothing; the block stays for its copies once more as long
-            if (a.status) atomicOr(a.status, 8u);
-            bulk_copies_done(barrier);
+        if (!block_copies_done(barrier, kBulkTries)) {   // (not seen) report and move nothing; the block stays for its copies once more as long
+            if (threadIdx.x == 0 && a.status) atomicOr(a.status, 8u);
+            bulk_copies_done(barrier, kBulkTries);
             return;
         }
-    } else cp_async_wait_all();
-    __syncthreads();   // a group's bytes were copied, its permutations drawn by threads of other warps
+    } else {
+        cp_async_wait_all();
+        __syncthreads();
+    }
     if (threadIdx.x == 0) selected = total;
     for (uint32_t first = 0; first < total;) {
         if (n_models % 4 == 0) moved += move_quads<TA, TB>(a, image_a, image_b, g_block, s_perm, s_entry + first, in_round, threadIdx.x, blockDim.x);
