@@ -381,7 +381,8 @@ int wash_exchange_counts(wash_ctx *ctx, uint64_t *host_need, uint64_t *host_sele
  *
  * Device-side checks: the kernel is given no status word, so a group that falls outside
  * the tables (which this call builds itself from numel) would be skipped without a report;
- * there is no wash_check for this entry point. */
+ * there is no wash_check for this entry point.  Kernels that could give up a wait, and would report it
+ * there, are not launched: large groups in [padded_P][N] take the copies that cannot. */
 int wash_shuffle_noalloc(int32_t N, int32_t n_tensors, const int64_t *numel, int32_t layout,
                          int32_t dtype, void *dev_stack, int64_t n_elems, uint64_t step, double p,
                          const double *p_layer, uint64_t seed, int32_t device, void *stream,
@@ -393,7 +394,9 @@ const char *wash_noalloc_last_error(void);
 /* ---- diagnostics ------------------------------------------------------------------ */
 
 /* Waits for `stream` and returns WASH_ERR_DEVICE_CHECK if a kernel recorded an
- * inconsistency (an index outside its table) since the last check, else WASH_OK. */
+ * inconsistency since the last check, else WASH_OK.  wash_last_error() names which: an index outside its
+ * table, an exchange step that needed more slots than the staging buffers hold, a block of the streaming
+ * shuffle whose copies did not arrive (none of its values was moved). */
 int wash_check(wash_ctx *ctx, void *stream);
 
 /* Message for the calling thread's most recent error (never NULL). */

@@ -95,6 +95,15 @@ struct ShuffleArgs {
     float expected_share = 0.f;   // share of the coordinates the call's probabilities select, in expectation (sizes the sparse kernel's grid)
 };
 
+// Whether the blocks of shuffle_wide_pn_kernel fetch their bytes by bulk copies (its comment has the measurements).  Only where a
+// wait that is given up can be reported: without a status word (wash_shuffle_noalloc) the block would stay as it was, and nobody would know.
+// A bulk copy takes multiples of 16 bytes: groups come in pairs (rows and ranges are whole units of 8 elements) and have 8 N bytes at least.
+inline bool copies_in_bulk(const ShuffleArgs &args, uint32_t groups, size_t group_bytes, bool two_stacks)
+{
+    if (!args.status || args.pn_pad != 0 || ((args.group_lo | args.group_hi) & 1u) != 0) return false;
+    return groups == 64 || group_bytes > 1024 || (group_bytes == 1024 && !two_stacks);
+}
+
 struct ReduceArgs {
     PopView pop;
     void *stack;                  // device stack (read; written by EMA / papa_all)

@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_co
     // (a group's bytes were copied, its permutations drawn by threads of other warps: both forms end with a barrier)
     if constexpr (BULK) {
         if (!block_copies_done(barrier, kBulkTries)) {   // (not seen) report and move nothing; the block stays for its copies once more as long
-            if (threadIdx.x == 0 && a.status) atomicOr(a.status, 8u);
+            if (threadIdx.x == 0) atomicOr(a.status, 8u);
             bulk_copies_done(barrier, kBulkTries);
             return;
         }
@@ -293,10 +293,8 @@ cudaError_t launch_shuffle_wide_typed(const ShuffleArgs &call, const LaunchShape
         const size_t per_group = group_elems * (TA::kBytes + (kHasB ? TB::kBytes : 0)) + 4 * 8 + 4 + 4 * wide_pitch(args.pop.N);
         const uint32_t groups = per_group * 64 > 44 * 1024 ? 32 : 64;   // five blocks and more on an SM
         const size_t smem = (per_group * groups + 15) & ~static_cast<size_t>(15);
-        // a bulk copy takes multiples of 16 bytes: groups come in pairs (rows and ranges are whole units of 8 elements) and have 8 N bytes at least
         const size_t group_bytes = 4 * static_cast<size_t>(args.pop.N) * (TA::kBytes + TB::kBytes);
-        const bool bulk = args.pn_pad == 0 && ((args.group_lo | args.group_hi) & 1u) == 0 && (groups == 64 || group_bytes > 1024 || (group_bytes == 1024 && !kHasB));
-        auto kernel = bulk ? shuffle_wide_pn_kernel<TA, TB, true> : shuffle_wide_pn_kernel<TA, TB, false>;
+        auto kernel = copies_in_bulk(args, groups, group_bytes, kHasB) ? shuffle_wide_pn_kernel<TA, TB, true> : shuffle_wide_pn_kernel<TA, TB, false>;
         KernelFit fit;
         cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), 2 * static_cast<int>(groups), smem, &fit);
         if (err != cudaSuccess) return err;

@@ -1,0 +1,17 @@
+// The rules by which launches choose their kernels, for tests without a GPU.
+#include "wash_internal.h"
+
+extern "C" {
+
+int rule_copies_in_bulk(int has_status, unsigned pn_pad, unsigned group_lo, unsigned group_hi, unsigned groups, unsigned long long group_bytes, int two_stacks)
+{
+    uint32_t word = 0;
+    wash::ShuffleArgs args = {};
+    args.status = has_status ? &word : nullptr;
+    args.pn_pad = pn_pad;
+    args.group_lo = group_lo;
+    args.group_hi = group_hi;
+    return wash::copies_in_bulk(args, groups, group_bytes, two_stacks != 0) ? 1 : 0;
+}
+
+}

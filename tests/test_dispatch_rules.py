@@ -1,0 +1,30 @@
+"""Rules by which launches choose their kernels (csrc/wash_internal.h), compiled for the host and evaluated over their ranges."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+from paper_2405_17517_b200 import build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    lib = str(tmp_path_factory.mktemp("rules") / "rules.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build._nvcc()))), "include")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-I", build.CSRC, "-I", cuda, os.path.join(HERE, "dispatch_rules.cpp"), "-o", lib], check=True)
+    return ctypes.CDLL(lib)
+
+
+@pytest.mark.parametrize("two_stacks", [0, 1])
+@pytest.mark.parametrize("group_bytes", [512, 576, 768, 1024, 1152, 2048])
+def test_bulk_copies_only_where_they_can_be_reported_and_fit(rules, group_bytes, two_stacks):
+    """A launch without a status word never takes copies whose wait can be given up; neither do odd ranges or padded images, whose
+    bytes are no multiples of 16 or not contiguous."""
+    def bulk(has_status=1, pad=0, lo=0, hi=1000, groups=32):
+        return rules.rule_copies_in_bulk(has_status, pad, lo, hi, groups, ctypes.c_ulonglong(group_bytes), two_stacks)
+    assert not bulk(has_status=0) and not bulk(has_status=0, groups=64)
+    assert not bulk(pad=4) and not bulk(lo=3) and not bulk(hi=999)
+    assert bulk(groups=64)

@@ -75,6 +75,21 @@ def test_two_calls_in_a_row_match_the_context_based_shuffle():
         assert (int(stats[0]), int(stats[1])) == (sel, moved)
 
 
+@pytest.mark.parametrize("N,numel,bf16,p", [(32, [40_009, 5], False, 0.1), (64, [9_001, 130, 3], True, 0.3), (64, [12_003], False, 0.02), (47, [6_001], False, 0.5)])
+def test_large_groups_coordinate_major(N, numel, bf16, p):
+    """[padded_P][N], groups of 512 bytes and more: the context's call fetches them by bulk copies, this one does not; the same bits."""
+    code = B.WASH_BF16 if bf16 else B.WASH_F32
+    stack, P, host, off = _make(N, numel, 1, bf16, seed=N)
+    want, want_stats = _reference(N, numel, 1, code, stack, 6, p, None, 21)
+    stats = torch.zeros(2, dtype=torch.int64, device="cuda")
+    B.wash_shuffle_noalloc(N, numel, 1, code, stack, stack.numel(), 6, p, None, 21, 0, None, stats)
+    torch.cuda.synchronize()
+    assert torch.equal(_bits(stack), _bits(want)) and torch.equal(stats, want_stats)
+    host = np.ascontiguousarray(host)
+    assert tuple(stats.tolist()) == oracle.shuffle(oracle.Population(N, numel, off, P, 1), host, p, seed=21, step=6)
+    assert (_bits(stack).cpu().numpy().view(np.uint16 if bf16 else np.uint32) == (host if bf16 else host.view(np.uint32))).all()
+
+
 def test_a_capturing_stream_is_refused_and_nothing_is_recorded():
     """The call copies its tables from host arrays that are gone when it returns, so it must
     not be recorded into a graph: a stream in capture mode gets WASH_ERR_STATE."""
