@@ -22,8 +22,9 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_
     asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes), "r"(barrier) : "memory");
 }
 
-// Waits for the barrier's first phase, but not for ever: `tries` trials.
-constexpr uint32_t kBulkTries = 1u << 20;
+// Waits for the barrier's first phase, but not for ever: `tries` trials.  A trial that sees nothing arrive returns after 7850 clocks, so
+// kBulkTries are a second (1.05 s at 1.965 GHz); copies take microseconds.
+constexpr uint32_t kBulkTries = 1u << 18;
 __device__ __forceinline__ bool bulk_copies_done(uint32_t barrier, uint32_t tries)
 {
     for (uint32_t i = 0; i < tries; ++i) {
