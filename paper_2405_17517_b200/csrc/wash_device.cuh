@@ -173,8 +173,8 @@ __device__ __forceinline__ void publish_block_stats(unsigned long long *stats, S
 // of blocks that have reported share one 64-bit word, so that a block reports with a single atomic and the last one reads
 // the total out of its return value: with a word for each, a fence between them and two exchanges to fetch the totals, the end
 // of a launch took three trips to the L2 more.
-//   bits 0..7 blocks (at most 32 a SM: 19 to a slot), 8..33 selected, 34..63 moved: a slot's share of the 2^33
-//   coordinates a row may have is 2^25, moved 16 times as much (the kernel takes populations of up to 16 models).
+//   bits 0..7 blocks, 8..33 selected, 34..63 moved (at most 16 times as many: the kernel takes populations of up to 16 models);
+//   report_grid chooses a grid of which no slot gets more than these hold.
 __device__ __forceinline__ void publish_warp_stats(unsigned long long *stats, StatSlot *slots, uint32_t selected, uint32_t moved)
 {
     if (!stats) return;

@@ -95,6 +95,17 @@ struct ShuffleArgs {
     float expected_share = 0.f;   // share of the coordinates the call's probabilities select, in expectation (sizes the sparse kernel's grid)
 };
 
+// Blocks of the resident-warp streaming kernel: those that are resident, as far as there are tiles for them -- and, where a device has few
+// SMs, so many that the counters of a slot fit the fields they are reported in (publish_warp_stats): fewer than 256 blocks and fewer than
+// 2^26 selected coordinates to a slot.  A row has fewer than 2^33 coordinates; one slot in kStatSlots gets ceil(grid / kStatSlots) of the grid's equal
+// shares, which is at most 2 / 257 of the row for a grid of kStatSlots blocks or more and could be all of it for smaller ones.
+inline uint32_t report_grid(uint64_t n_tiles, uint64_t resident)
+{
+    constexpr uint64_t kLeast = kStatSlots, kMost = 255ull * kStatSlots;
+    const uint64_t grid = resident < kLeast ? kLeast : resident > kMost ? kMost : resident;
+    return static_cast<uint32_t>(n_tiles < grid ? n_tiles : grid);
+}
+
 // Whether the blocks of shuffle_wide_pn_kernel fetch their bytes by bulk copies (its comment has the measurements).  Only where a
 // wait that is given up can be reported: without a status word (wash_shuffle_noalloc) the block would stay as it was, and nobody would know.
 // A bulk copy takes multiples of 16 bytes: groups come in pairs (rows and ranges are whole units of 8 elements) and have 8 N bytes at least.

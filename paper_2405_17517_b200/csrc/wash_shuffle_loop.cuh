@@ -285,8 +285,7 @@ cudaError_t launch_shuffle_loop_tiles(const ShuffleArgs &args, const LaunchShape
     const uint64_t n_tiles = (static_cast<uint64_t>(args.group_hi - args.group_lo) + per_tile - 1) / per_tile;
     if (n_tiles == 0) return cudaSuccess;
     const uint64_t resident = static_cast<uint64_t>(shape.sm_count > 0 ? shape.sm_count : 148) * fit.occupancy;
-    const uint64_t grid = n_tiles < resident ? n_tiles : resident;
-    return launch_chained(kernel, static_cast<unsigned>(grid), 32, smem, stream, args);
+    return launch_chained(kernel, report_grid(n_tiles, resident), 32, smem, stream, args);
 }
 
 template <class TA, class TB>

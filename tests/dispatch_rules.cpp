@@ -14,4 +14,7 @@ int rule_copies_in_bulk(int has_status, unsigned pn_pad, unsigned group_lo, unsi
     return wash::copies_in_bulk(args, groups, group_bytes, two_stacks != 0) ? 1 : 0;
 }
 
+unsigned rule_report_grid(unsigned long long n_tiles, unsigned long long resident) { return wash::report_grid(n_tiles, resident); }
+int rule_stat_slots() { return wash::kStatSlots; }
+
 }

@@ -28,3 +28,19 @@ def test_bulk_copies_only_where_they_can_be_reported_and_fit(rules, group_bytes,
     assert not bulk(has_status=0) and not bulk(has_status=0, groups=64)
     assert not bulk(pad=4) and not bulk(lo=3) and not bulk(hi=999)
     assert bulk(groups=64)
+
+
+@pytest.mark.parametrize("tile", [256, 512], ids=["two groups a lane", "four"])
+def test_no_slot_is_reported_more_than_its_fields_hold(rules, tile):
+    """The resident-warp kernel's packed report (8 bits of blocks, 26 of selected coordinates) on devices of 1 to 592 SMs, from one
+    block an SM on, for rows up to the longest there are and everything selected; blocks take the tiles round-robin."""
+    rules.rule_report_grid.argtypes = [ctypes.c_ulonglong, ctypes.c_ulonglong]
+    slots = rules.rule_stat_slots()
+    for n_tiles in (1, slots - 1, slots, slots + 1, 4736, 1 << 20, (1 << 33) // tile):
+        for resident in [sms * blocks for sms in (1, 2, 7, 16, 37, 74, 148, 296, 592) for blocks in range(1, 33)]:
+            grid = rules.rule_report_grid(n_tiles, resident)
+            assert 1 <= grid <= n_tiles and grid >= min(resident, n_tiles)
+            blocks = range(0, grid, slots)            # of the fullest slot: its first block takes every grid-th tile from 0 on
+            assert len(blocks) < 256
+            coordinates = sum((n_tiles - b + grid - 1) // grid for b in blocks) * tile
+            assert coordinates < 1 << 26 and 16 * coordinates < 1 << 30
