@@ -95,6 +95,27 @@ struct ShuffleArgs {
     float expected_share = 0.f;   // share of the coordinates the call's probabilities select, in expectation (sizes the sparse kernel's grid)
 };
 
+// Whether the sparse kernels' loads of values ask for 64 bytes of a line instead of all 128 (load_scattered).  128 bytes are the better
+// request where a line's other half holds a selected coordinate as well, which is then fetched for nothing, and where masks and not
+// values are most of the time the two are alike and the plain load costs fewer instructions.  Time with 64 bytes over time with 128, stacks of 400 MB:
+//   [N][P], 1 / 2 / 4 / 6 % selected (10 %): fp32 N = 3 1.01 1.00 .98 .97 (1.01), 5 .98 .93 .92 .96 (1.07), 8 .97 .93 .96 1.01, 16 .98 .97 1.01 1.07, 24 1.00 1.02
+//     1.09, 48 .99 1.04, 64 1.03 1.05;  bf16 8 .98 .95 1.06 1.16, 16 .96 .99 1.12, 24 1.00 1.07, 48 1.03 1.16;  two fp32 stacks 2 1.02 1.02 .92 .88 (.91), 3 .99 .92 .90 .92 (.99), 8 1.00 .98
+//     .99 1.02, 24 .97 .99 1.08;  bf16 + fp32, in either order 3 1.00 .93 .90 .96 (1.05), 5 .96 .94 .97 1.02, 8 .98 .98 1.01 1.06, 12 1.00 .99 1.03, 24 .98 1.02 1.10, 32 .98 1.02
+//     1.12;  by warps (shuffle_sparse_warps_kernel), 6 / 10 % fp32 24 .92 .95, 64 .94 .97, bf16 24 .97 .99, bf16 + fp32 .94 .96.
+//     Few values, .002 to .003 of a coordinate's: 1.00 to 1.03 up to .03 values a coordinate (N = 5 two stacks, p = 2e-3 1.03), from .04 on .97 to 1.00.
+//   [P][N], one stack: 1.00 to 1.03 throughout.  Two stacks, 1 / 2 / 4 / 6 / 10 %: fp32 N = 3 1.01 .98 .93 .90 .93, 5 1.00 .99 .97 .95 .90, 8 1.00 1.01 .98 .96 .94, 12 1.01 1.02 .99
+//     .98 .99, 16 1.00 1.02 1.03 1.02 1.02, 32 1.01 1.02 1.01; bf16 + fp32 3 1.00 .99 .95 .91 .98, 5 1.01 .98 .95 .92 .94, 24 1.00 1.01 1.02 1.02 1.03.
+// ResNet-50 N = 8, bf16 + fp32, p = 5e-3: 77.2 -> 71.3 us, N = 5, p = 0.05 -> 0 46.8 -> 44.9.
+inline bool fetch_half_lines(const ShuffleArgs &args, bool by_warps, int bytes_a, int bytes_b)
+{
+    const int N = args.pop.N;
+    const bool two_stacks = bytes_b != 0;
+    const float elem = two_stacks ? 0.5f * static_cast<float>(bytes_a + bytes_b) : static_cast<float>(bytes_a);   // the stacks are asked alike
+    const float values = args.expected_share * static_cast<float>(N), per_line = args.expected_share * 128.f / elem;
+    if (args.pop.layout == kLayoutPN) return two_stacks && N <= 12 && values >= 0.06f && per_line < static_cast<float>(N);
+    return values >= 0.035f && per_line < (by_warps ? 4.f : N <= 3 ? 3.f : N <= 5 ? 2.f : N <= 16 ? 1.5f : N <= 32 ? 0.7f : 0.f);
+}
+
 // Blocks of the resident-warp streaming kernel: those that are resident, as far as there are tiles for them -- and, where a device has few
 // SMs, so many that the counters of a slot fit the fields they are reported in (publish_warp_stats): fewer than 256 blocks and fewer than
 // 2^26 selected coordinates to a slot.  A row has fewer than 2^33 coordinates; one slot in kStatSlots gets ceil(grid / kStatSlots) of the grid's equal

@@ -333,29 +333,14 @@ inline bool sparse_by_warps(const ShuffleArgs &args, bool bf16, bool two_stacks)
     return N <= 15 && share >= (N <= 3 ? 0.25f : N <= 10 ? 0.3f : N <= 12 ? 0.4f : 0.7f);
 }
 
-// Whether the loads of values ask for 64 bytes.  128 bytes are the better request where a line's other half holds a selected
-// coordinate as well, which is then fetched for nothing; and where masks and not values are most of the time the two are alike and the
-// plain load costs fewer instructions (ResNet-18 N = 5 with momentum, p = 1e-3: 10.6 -> 10.9 us).  128 / 64 bytes, 2^24 coordinates,
-//   [N][P] fp32: N = 2 two stacks, 5 % (1.6 to a line) 48.8 / 43.1, 10 % 66.0 / 65.9; 5 2 % 45.4 / 42.1, 5 % 81.3 / 76.3, 15 % 111 / 128; 8 2 % 81.8 / 75.7,
-//     6 % 149 / 149; 16 (2^23) 2 % 96.2 / 92.3, 6 % 169 / 181; 32 5 % (by warps) 339 / 306;  bf16: N = 8 2 % (1.3 to a line) 62.2 / 59.3, 6 % 92 / 107;
-//     32 (2^23) 2 % 149 / 158
-//   [P][N] fp32, two stacks: N = 3 5 % (0.5 to a line) 54.7 / 48.9, 30 % (3.2) 141 / 146; 5 10 % (0.6) 118 / 104, 30 % 206 / 216; 8 10 % 132 / 119.
-// ResNet-50 N = 8, bf16 + fp32, p = 5e-3: 77.2 -> 71.3 us, N = 5, p = 0.05 -> 0 46.8 -> 44.9.
-inline bool fetch_half_lines(const ShuffleArgs &args, int elem_bytes, bool two_stacks)
-{
-    const int N = args.pop.N;
-    const float per_line = args.expected_share * 128.f / static_cast<float>(args.pop.layout == kLayoutNP ? elem_bytes : elem_bytes * N);
-    const float most = args.pop.layout == kLayoutPN ? 1.f : N <= 5 || sparse_by_warps(args, elem_bytes == 2, two_stacks) ? 2.f : N <= 16 ? 1.5f : 1.2f;
-    return per_line < most && args.expected_share * N * (two_stacks ? 2 : 1) >= 0.02f;
-}
-
 template <class TA, class TB>
 cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchShape &shape, cudaStream_t stream)
 {
     if (args.group_hi <= args.group_lo) return cudaSuccess;
     SparseArgs p;
     p.s = args;
-    const bool half = fetch_half_lines(args, TA::kBytes, TB::kCode != kDtypeNone);
+    const bool by_warp = sparse_by_warps(args, TA::kBytes == 2, TB::kCode != kDtypeNone);
+    const bool half = fetch_half_lines(args, by_warp, TA::kBytes, TB::kBytes);
     p.n_wtiles = (args.group_hi - args.group_lo + kWarpTileGroups - 1) / kWarpTileGroups;
     size_t smem = sparse_queue_capacity(args.pop.N) * (12 + (args.pop.N > 16 ? 4 * static_cast<size_t>(wide_pitch(args.pop.N)) : 0));
     const bool np = args.pop.layout == kLayoutNP;
@@ -367,7 +352,7 @@ cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchSha
         p.column_offset = static_cast<uint32_t>(smem);
         smem += 4 * static_cast<size_t>(args.pop.N) * kSparseThreads;
     }
-    if (!args.mirror_a && sparse_by_warps(args, TA::kBytes == 2, TB::kCode != kDtypeNone)) {
+    if (!args.mirror_a && by_warp) {
         auto by_warps = np ? shuffle_sparse_warps_kernel<TA, TB, kLayoutNP, false> : shuffle_sparse_warps_kernel<TA, TB, kLayoutPN, false>;
         if (half && np) by_warps = shuffle_sparse_warps_kernel<TA, TB, kLayoutNP, true>;
         smem = 4 * kSparseWarps * static_cast<size_t>(kWarpList) + 4 * static_cast<size_t>(args.pop.N) * kSparseThreads +

@@ -14,6 +14,15 @@ int rule_copies_in_bulk(int has_status, unsigned pn_pad, unsigned group_lo, unsi
     return wash::copies_in_bulk(args, groups, group_bytes, two_stacks != 0) ? 1 : 0;
 }
 
+int rule_fetch_half_lines(int layout, int n_models, float share, int by_warps, int bytes_a, int bytes_b)
+{
+    wash::ShuffleArgs args = {};
+    args.pop.layout = layout;
+    args.pop.N = n_models;
+    args.expected_share = share;
+    return wash::fetch_half_lines(args, by_warps != 0, bytes_a, bytes_b) ? 1 : 0;
+}
+
 unsigned rule_report_grid(unsigned long long n_tiles, unsigned long long resident) { return wash::report_grid(n_tiles, resident); }
 int rule_stat_slots() { return wash::kStatSlots; }
 

@@ -44,3 +44,18 @@ def test_no_slot_is_reported_more_than_its_fields_hold(rules, tile):
             assert len(blocks) < 256
             coordinates = sum((n_tiles - b + grid - 1) // grid for b in blocks) * tile
             assert coordinates < 1 << 26 and 16 * coordinates < 1 << 30
+
+
+def test_half_lines_are_asked_for_alike_in_either_order_of_the_stacks(rules):
+    """Both stacks of a launch take one form of load, so bf16 weights with fp32 momentum and fp32 weights with bf16 momentum
+    get the same one; a single stack in [P][N], whose loads never gained, and rare values get the plain load."""
+    def half(layout, N, share, a, b, by_warps=0):
+        return rules.rule_fetch_half_lines(layout, N, ctypes.c_float(share), by_warps, a, b)
+    shares = [10.0 ** (-4 + 0.05 * k) for k in range(81)]
+    for layout in (0, 1):
+        for N in range(2, 65):
+            for by_warps in (0, 1):
+                assert [half(layout, N, s, 2, 4, by_warps) for s in shares] == [half(layout, N, s, 4, 2, by_warps) for s in shares]
+            assert not any(half(1, N, s, e, 0) for s in shares for e in (2, 4))
+            assert not any(half(layout, N, s, a, b) for s in shares if s * N < 0.03 for a, b in ((4, 0), (2, 0), (4, 4), (2, 4)))
+    assert half(0, 8, 0.005, 2, 4) and half(0, 5, 0.025, 4, 0)
