@@ -116,6 +116,25 @@ inline bool fetch_half_lines(const ShuffleArgs &args, bool by_warps, int bytes_a
     return values >= 0.035f && per_line < (by_warps ? 4.f : N <= 3 ? 3.f : N <= 5 ? 2.f : N <= 16 ? 1.5f : N <= 32 ? 0.7f : 0.f);
 }
 
+// Whether half a wave of blocks serves a sparse launch of `n_wtiles` warp tiles whose values would be `by_load` blocks' (launch_shuffle_sparse_typed
+// has the units).  Launches that follow each other at once gain by it: a launch's masks are drawn beside the serving of the one before, which a
+// whole wave leaves no room, and 16 warps draw masks at nearly the rate of 32.  A launch behind a kernel that releases nothing early, an
+// optimizer's in a training loop, gains nothing and waits for blocks that serve twice as much.  us, whole -> half: call after call | behind an elementwise
+// kernel on other data | behind one on the stacks (chains less the chains without the shuffle):
+//   ResNet-18 N = 5, p = 3e-4 10.2 -> 9.1 | 12.5 -> 12.4 | 13.5 -> 13.4;  with momentum, p = 1e-3 (0.32 of a wave) 10.9 -> 9.5 | 14.3 -> 16.1 | 14.1 -> 14.8
+//   N = 2, 2^23 coordinates, p = 1e-3 8.0 -> 7.2 | 10.2 -> 10.2 | 10.2 -> 10.2;  N = 10, 2^23, 5e-4 8.9 -> 7.4 | 10.5 -> 10.6 | 11.2 -> 11.2;  N = 16 bf16, 2^23, 5e-4 9.3 ->
+//   7.6 | 12.3 -> 12.3 | 14.0 -> 14.2;  N = 5, 2^24, 1e-3 14.2 -> 13.5 | 18.4 -> 18.4 | 18.0 -> 18.3;  [P][N] N = 8, 2^24, 1e-3 13.9 -> 13.1 | 16.5 -> 17.1 | 17.6 -> 17.8
+// So ResNet-18 with momentum, 0.32 of a wave, loses behind other kernels up to what it gains; from 0.4 on more, as rows of more than 16 tiles a warp do, and
+// populations of 48 models, whose coordinate is a block's work for a while, lose both ways (N = 20, 2^22, 1e-3 6.9 -> 6.6 | 10.2 -> 10.3 | 9.6 -> 9.6):
+//   N = 5 with momentum, 2^24, 1e-3 (0.47) 14.3 -> 13.4 | 20.3 -> 22.4 | 18.7 -> 20.9;  N = 3, 2^25, 3e-4 (28 tiles) 25.1 -> 24.4 | 28.7 -> 30.2 | 29.2 -> 30.3
+//   N = 48, 2^21, 1e-3 8.0 -> 8.4 | 10.7 -> 12.1 | 9.7 -> 10.5;  [P][N], 3e-3 6.8 -> 7.2 | 8.2 -> 8.3 | 8.0 -> 8.9
+// Five eighths to seven eighths of a wave gain less and lose as much (ResNet-18 with momentum 0.75: 11.4 | 14.3 | 14.2).  Waves and a half lose (N = 3 two
+// stacks, p = 5e-3, 1.5 waves 20.7, two 18.9).
+inline bool half_wave_serves(int n_models, double by_load, uint32_t resident, uint32_t n_wtiles)
+{
+    return n_models <= 32 && by_load <= 0.4 * resident && n_wtiles <= 32ull * resident;   // 16 tiles for each of the 4 warps of resident / 2 blocks
+}
+
 // Blocks of the resident-warp streaming kernel: those that are resident, as far as there are tiles for them -- and, where a device has few
 // SMs, so many that the counters of a slot fit the fields they are reported in (publish_warp_stats): fewer than 256 blocks and fewer than
 // 2^26 selected coordinates to a slot.  A row has fewer than 2^33 coordinates; one slot in kStatSlots gets ceil(grid / kStatSlots) of the grid's equal

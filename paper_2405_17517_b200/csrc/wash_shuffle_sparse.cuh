@@ -386,10 +386,6 @@ cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchSha
     // 39.9 -> 31.7.  A larger load loses where values are many (400 instead of 300 for ResNet-50 N = 8 bf16 + fp32, p = 5e-3: 79.4
     // against 77.1, N = 20, p = 2e-3 51.6 against 50.3), a broken wave where waves are few ([P][N] N = 8, 2^25: 1.4 waves
     // 41.9, two 38.8).
-    // Half a wave where that serves everything and the next kernel is released at once: its masks are then drawn beside this one's
-    // serving instead of after it, and 16 warps draw masks at 0.98 of the rate of 32.  A whole wave leaves the next one no room.  ResNet-18
-    // N = 5 with momentum, p = 1e-3 (half a wave takes up to 60 coordinates a block): 10.6 -> 9.1 us; 2^24 coordinates, p = 1e-3, N = 5 two stacks 14.2 ->
-    // 12.9, [P][N] N = 8 14.8 -> 13.0.  Waves and a half lose (N = 3 two stacks, p = 5e-3, 1.5 waves 20.7, two 18.9).
     const bool one_stack = TB::kCode == kDtypeNone;
     const double expected = static_cast<double>(args.expected_share) * 4.0 * static_cast<double>(args.group_hi - args.group_lo);
     double by_tiles = static_cast<double>(p.n_wtiles) / (kSparseWarps * (np ? 2 : 3));
@@ -399,7 +395,7 @@ cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchSha
     p.release_early = static_cast<double>(args.expected_share) * args.pop.N * (one_stack ? 1 : 2) <= kReleaseShare;
     const double by_load = expected * (one_stack ? 1.0 : 2.0) / load;
     uint32_t grid = static_cast<uint32_t>(fmin(fmin(expected / kSparsePerBlock, by_tiles), resident * ceil(by_load / resident)));
-    if (grid < resident) grid = p.release_early && by_load <= resident / 2 ? resident / 2 : resident;
+    if (grid < resident) grid = p.release_early && half_wave_serves(args.pop.N, by_load, resident, p.n_wtiles) ? resident / 2 : resident;
     const uint32_t want = (p.n_wtiles + kSparseWarps - 1) / kSparseWarps;
     if (grid > want) grid = want;
     p.per_block = p.n_wtiles / grid;

@@ -23,6 +23,8 @@ int rule_fetch_half_lines(int layout, int n_models, float share, int by_warps, i
     return wash::fetch_half_lines(args, by_warps != 0, bytes_a, bytes_b) ? 1 : 0;
 }
 
+int rule_half_wave_serves(int n_models, double by_load, unsigned resident, unsigned n_wtiles) { return wash::half_wave_serves(n_models, by_load, resident, n_wtiles) ? 1 : 0; }
+
 unsigned rule_report_grid(unsigned long long n_tiles, unsigned long long resident) { return wash::report_grid(n_tiles, resident); }
 int rule_stat_slots() { return wash::kStatSlots; }
 

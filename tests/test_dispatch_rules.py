@@ -59,3 +59,11 @@ def test_half_lines_are_asked_for_alike_in_either_order_of_the_stacks(rules):
             assert not any(half(1, N, s, e, 0) for s in shares for e in (2, 4))
             assert not any(half(layout, N, s, a, b) for s in shares if s * N < 0.03 for a, b in ((4, 0), (2, 0), (4, 4), (2, 4)))
     assert half(0, 8, 0.005, 2, 4) and half(0, 5, 0.025, 4, 0)
+
+
+def test_half_a_wave_only_where_it_does_not_lose_more_than_it_gains(rules):
+    """Up to 32 models, 0.4 of a wave's values and 16 tiles a warp (1184 resident blocks)."""
+    def half(N, by_load, n_wtiles):
+        return rules.rule_half_wave_serves(N, ctypes.c_double(by_load), 1184, n_wtiles)
+    assert half(5, 374.0, 21_914) and half(32, 0.0, 37_888)
+    assert not half(33, 1.0, 100) and not half(5, 474.0, 21_914) and not half(5, 1.0, 37_889)

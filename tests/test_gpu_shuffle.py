@@ -711,9 +711,9 @@ def test_wide_populations_coordinate_major(N, numel, p, dtype, opt):
 @pytest.mark.parametrize("layout", [0, 1])
 @pytest.mark.parametrize("N,p,dtype,opt", [(2, 0.03, "f32", None), (5, 0.004, "f32", "f32"), (8, 0.01, "bf16", "f32"), (16, 0.02, "bf16", None), (20, 0.05, "f32", None),
                                            (32, 0.001, "f32", "bf16"), (64, 0.004, "bf16", None), (3, 0.0004, "f32", None), (5, 0.0002, "f32", "f32")])
-def test_sparse_loads_of_half_lines_and_half_waves(N, p, dtype, opt, layout):
-    """Selections for which the sparse kernel's loads ask for 64 bytes (pairs, rows and warps that serve by themselves), and those
-    rare enough for half a wave of blocks; three steps in a row, the second drawing while the first still serves."""
+def test_sparse_loads_of_half_lines(N, p, dtype, opt, layout):
+    """Selections about which the sparse kernel's loads ask for 64 bytes (pairs, rows and warps that serve by themselves) and
+    two that are too rare for it; three steps in a row, the second drawing while the first still serves."""
     numel = [700_001, 9, 120_000] if N <= 16 else [150_001, 9]
     c = Case(N, numel, layout, dtype, opt, seed=N)
     B.wash_set_mode(c.gpu.ctx, B.WASH_MODE_SPARSE)
@@ -722,6 +722,46 @@ def test_sparse_loads_of_half_lines_and_half_waves(N, p, dtype, opt, layout):
         (B.wash_shuffle_both if opt else B.wash_shuffle)(c.gpu.ctx, step, p, None, seed=17, stats=c.stats_dev)
         want += np.array(oracle.shuffle(c.ora, c.host, p, seed=17, step=step, stack2=c.host_opt), dtype=np.int64)
     c.assert_equal("N=%d p=%g layout=%d" % (N, p, layout))
+    assert c.gpu_stats() == tuple(want)
+    c.close()
+
+
+def _half_wave_row(at_least_blocks_over=1.5):
+    """Coordinates for which a launch of a warp tile (512 coordinates) a warp would take more blocks of four warps than half a wave
+    holds (eight blocks an SM are a wave)."""
+    half = 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    return int(at_least_blocks_over * half) * 4 * 512 + 3
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("N,p,dtype,opt", [(2, 1e-3, "f32", None), (3, 4e-4, "bf16", None), (5, 2e-4, "f32", "f32"), (8, 3e-4, "bf16", "f32"), (16, 2e-4, "f32", None), (20, 2e-4, "bf16", None), (40, 1e-4, "bf16", None)])
+def test_sparse_half_a_wave_of_blocks(N, p, dtype, opt, layout):
+    """Selections rare enough for half a wave of blocks, in rows that would fill more (N = 40: the whole wave), three steps in a row: the
+    second draws its masks beside the first one's serving."""
+    c = Case(N, [_half_wave_row(), 5, 2047], layout, dtype, opt, seed=N)
+    B.wash_set_mode(c.gpu.ctx, B.WASH_MODE_SPARSE)
+    want = np.zeros(2, dtype=np.int64)
+    for step in range(3):
+        (B.wash_shuffle_both if opt else B.wash_shuffle)(c.gpu.ctx, step, p, None, seed=23, stats=c.stats_dev)
+        want += np.array(oracle.shuffle(c.ora, c.host, p, seed=23, step=step, stack2=c.host_opt), dtype=np.int64)
+    c.assert_equal("N=%d p=%g layout=%d" % (N, p, layout))
+    assert c.gpu_stats() == tuple(want)
+    c.close()
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("N", [2, 5, 16])
+def test_sparse_half_a_wave_with_everything_selected_in_one_place(N, layout):
+    """A schedule that is rare on the whole, and selects in one tensor what fills the queue (512 entries) of the block whose range it is
+    several times over."""
+    c = Case(N, [_half_wave_row() // 2, 1900, _half_wave_row() // 2], layout, "f32", "f32", seed=N)
+    B.wash_set_mode(c.gpu.ctx, B.WASH_MODE_SPARSE)
+    p_layer = [1e-5, 1.0, 1e-5]
+    want = np.zeros(2, dtype=np.int64)
+    for step in range(2):
+        B.wash_shuffle_both(c.gpu.ctx, step, 0.0, p_layer, seed=29, stats=c.stats_dev)
+        want += np.array(oracle.shuffle(c.ora, c.host, p_layer, seed=29, step=step, stack2=c.host_opt), dtype=np.int64)
+    c.assert_equal("N=%d layout=%d" % (N, layout))
     assert c.gpu_stats() == tuple(want)
     c.close()
 
