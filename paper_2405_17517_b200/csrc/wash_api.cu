@@ -199,9 +199,6 @@ void *mapped_host(void *ptr, size_t bytes, int dtype)
 // floor(p * 2^32) for p in [0, 1]; the product is exact in binary64
 uint64_t threshold_of(double p) { return static_cast<uint64_t>(std::floor(p * 4294967296.0)); }
 
-// [P][N]: whether the streaming kernels store neighbouring models' values together
-bool stored_together(int layout, int N) { return layout == WASH_LAYOUT_PN && N % (N <= 16 ? 2 : 4) == 0; }
-
 // WASH_MODE_AUTO: the expected share of selected coordinates up to which the sparse kernel is launched.  Serving a
 // coordinate costs it a scattered DRAM access and store per model and stack in [N][P], a few neighbouring ones for
 // all N models in [P][N]; the streaming kernels pay for the stack's bytes and, in small populations, for issue slots.
@@ -223,7 +220,7 @@ double sparse_share(int layout, int N, bool two_stacks, bool bf16)
         if (bf16) return N <= 4 ? 0.18 : N <= 7 ? 0.08 : N <= 16 ? 0.06 : 0.02;
         return std::fmax(std::fmin(0.6 / N, 0.17), 0.027);
     }
-    if (stored_together(layout, N)) {
+    if (N == 2 || wash::stored_together(layout, N) > 1) {
         if (two_stacks) return N <= 12 ? 0.24 : N <= 16 ? 0.34 : N <= 24 ? 0.28 : N <= 28 ? 0.36 : N < 64 ? 0.55 : 1.0;
         if (bf16) return N == 2 ? 0.17 : N == 4 ? 0.42 : N == 6 ? 0.35 : N <= 16 ? 0.18 : N <= 32 ? 0.135 : N < 64 ? 0.17 : 0.15;
         return N == 2 ? 0.13 : N == 4 ? 0.35 : N <= 8 ? 0.2 : N <= 16 ? 0.16 : N <= 24 ? 0.18 : N <= 32 ? 0.22 : N < 64 ? 0.36 : 0.45;
@@ -367,7 +364,7 @@ int shuffle_impl(wash_ctx *ctx, int which, uint64_t step, double p, const double
         // serving for N > 16) costs registers and, for N > 16, three more permutation columns of shared
         // memory per thread: measured, it pays only for large populations of which most coordinates are
         // served (kEarlyShare).
-        args.early = ctx->N > 16 && ctx->expected_selected >= kEarlyShare * coordinates && !stored_together(ctx->layout, ctx->N);
+        args.early = ctx->N > 16 && ctx->expected_selected >= kEarlyShare * coordinates && wash::stored_together(ctx->layout, ctx->N) == 1;
         if (ctx->shape.blocks_per_sm == -2) args.early = false;   // tuning override (wash_set_launch)
         if (ctx->shape.blocks_per_sm == -3) args.early = true;
         if (sq) {   // the statistic is gathered by the streaming kernel only

@@ -11,6 +11,13 @@ constexpr int kDtypeF32 = 0, kDtypeBF16 = 1, kDtypeNone = -1;
 constexpr int kLayoutNP = 0, kLayoutPN = 1;
 constexpr int kModeStream = 0, kModeSparse = 1;
 
+// Values of a selected coordinate that the streaming kernels store with one instruction: neighbouring models' in [P][N]
+// (move_neighbours up to 16 models, move_quads above); 1: every value by itself.
+__host__ __device__ constexpr int stored_together(int layout, int n_models)
+{
+    return layout != kLayoutPN || n_models == 2 ? 1 : n_models % 4 == 0 ? 4 : n_models % 2 == 0 && n_models <= 16 ? 2 : 1;
+}
+
 // One row of a stack is cut into groups of 4 consecutive elements; a group never
 // straddles two tensors because tensors start on multiples of 8 elements.
 struct SegEntry {

@@ -30,10 +30,10 @@ namespace wash {
 // stored together (move_neighbours): dense / dealt at 45 / 55 / 70 / 85 / 100 % selected, 2^23 coordinates, N = 2 fp32 1.15 1.09 0.98 0.83 0.84, N = 8 fp32 1.06 1.10
 // 1.07 0.92 0.91, N = 16 bf16 1.11 1.24 1.20 0.99 0.99, N = 10 two fp32 stacks 1.03 1.34 1.15 0.98 0.86; never with two stacks of a multiple of four models from 8 on, N = 8
 // two fp32 stacks 1.17 1.83 1.87 1.63 1.65, N = 16 bf16 + fp32 1.23 2.06 2.16 1.89 1.82.
-template <int LAYOUT, bool TWO_STACKS>
+template <int LAYOUT, bool TWO_STACKS, bool TOGETHER>
 __device__ __forceinline__ uint32_t dense_min_selected(int n_models)
 {
-    if (LAYOUT == kLayoutNP || n_models % 2 != 0) return 64;
+    if (!TOGETHER) return LAYOUT == kLayoutPN && n_models == 2 ? 100 : 64;
     return TWO_STACKS && n_models >= 8 && n_models % 4 == 0 ? 129 : 100;
 }
 
@@ -327,7 +327,7 @@ __device__ __forceinline__ uint32_t move_neighbours(const ShuffleArgs &a, const 
 
 // The moves of one selected coordinate (coordinate c of the group of block thread t_owner): model n
 // takes the value of model pi(n), nibble n of `perm` (N <= 16) or byte n of the column s_perm.
-template <class TA, class TB, int LAYOUT>
+template <class TA, class TB, int LAYOUT, bool TOGETHER>
 __device__ __forceinline__ void move_coordinate(const ShuffleArgs &a, const unsigned char *image_a, const unsigned char *image_b,
                                                 const uint8_t *s_perm, uint64_t perm, uint32_t t_owner, uint32_t c, uint64_t g_block,
                                                 uint32_t &moved)
@@ -342,11 +342,11 @@ __device__ __forceinline__ void move_coordinate(const ShuffleArgs &a, const unsi
     const long long out0 = LAYOUT == kLayoutNP ? e : e * n_models;
     const uint32_t img_step = LAYOUT == kLayoutNP ? T_ * 4u : 1u;
     const uint32_t img0 = LAYOUT == kLayoutNP ? t_owner * 4u + c : t_owner * pn_group_elems(n_models, a.pn_pad) + c * n_models;
-    if (LAYOUT == kLayoutPN && n_models <= 16 && n_models % 4 == 0) {
+    if (TOGETHER && stored_together(LAYOUT, n_models) == 4) {
         for (int n = 0; n < n_models; n += 4, perm >>= 16) moved += move_neighbours<TA, TB, 4>(a, image_a, image_b, img0, static_cast<uint32_t>(perm), n, out0);
         return;
     }
-    if (LAYOUT == kLayoutPN && n_models <= 16 && n_models % 2 == 0 && n_models != 2) {
+    if (TOGETHER) {
         for (int n = 0; n < n_models; n += 2, perm >>= 8) moved += move_neighbours<TA, TB, 2>(a, image_a, image_b, img0, static_cast<uint32_t>(perm), n, out0);
         return;
     }
@@ -394,7 +394,7 @@ __device__ __forceinline__ void plan_tile(const ShuffleArgs &a, uint8_t *s_list,
     if (!__any_sync(0xFFFFFFFFu, sel != 0)) return;   // most warps have nothing selected at small p
     const uint32_t mine = __popc(sel);
     const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, mine);
-    if (total >= dense_min_selected<kLayoutNP, false>(n_models) && __all_sync(0xFFFFFFFFu, sel == 0 || gi.valid == 4)) {   // (the early flavour: N > 16)
+    if (total >= dense_min_selected<kLayoutNP, false, false>(n_models) && __all_sync(0xFFFFFFFFu, sel == 0 || gi.valid == 4)) {
         pl.mode = kServeDense;
         if (sel) {
             if (n_models <= 16) dense_draw<uint64_t>(a, sel, gi, pl.perm, selected, moved);
@@ -447,7 +447,7 @@ __device__ __forceinline__ void apply_tile(const ShuffleArgs &a, const unsigned 
         }
         return;
     }
-    if (lane < pl.total) move_coordinate<TA, TB, LAYOUT>(a, image_a, image_b, s_perm, pl.perm[0], warp_base + (pl.entry >> 2), pl.entry & 3u, g_block, moved);
+    if (lane < pl.total) move_coordinate<TA, TB, LAYOUT, false>(a, image_a, image_b, s_perm, pl.perm[0], warp_base + (pl.entry >> 2), pl.entry & 3u, g_block, moved);
     const uint8_t *list = s_list + (threadIdx.x >> 5) * 128;
     for (uint32_t first = 32; first < pl.total; first += 32) {   // further rounds: draw and move
         const bool active = first + lane < pl.total;
@@ -459,7 +459,7 @@ __device__ __forceinline__ void apply_tile(const ShuffleArgs &a, const unsigned 
         uint64_t perm = 0;
         if (n_models <= 16) perm = draw_permutation_packed(n_models, 4u * cgroup + c, tensor, a.step_lo, a.step_hi8, a.keys);
         else draw_permutation_u8(s_perm, T_, n_models, 4u * cgroup + c, tensor, a.step_lo, a.step_hi8, a.keys);
-        move_coordinate<TA, TB, LAYOUT>(a, image_a, image_b, s_perm, perm, warp_base + owner, c, g_block, moved);
+        move_coordinate<TA, TB, LAYOUT, false>(a, image_a, image_b, s_perm, perm, warp_base + owner, c, g_block, moved);
         ++selected;
     }
     __syncwarp();   // the warp's list is rewritten by the next tile
@@ -544,7 +544,7 @@ __device__ __forceinline__ void serve_few(const ShuffleArgs &a, const unsigned c
     }
 }
 
-template <class TA, class TB, int LAYOUT>
+template <class TA, class TB, int LAYOUT, bool TOGETHER>
 __device__ __forceinline__ void serve_tile(const ShuffleArgs &a, const unsigned char *image_a, const unsigned char *image_b,
                                            uint8_t *s_list, uint8_t *s_perm, uint64_t g_block,
                                            uint32_t sel, const GroupInfo &gi, uint32_t &selected, uint32_t &moved)
@@ -559,7 +559,7 @@ __device__ __forceinline__ void serve_tile(const ShuffleArgs &a, const unsigned 
         serve_few<TA, TB, LAYOUT>(a, image_a, image_b, g_block, sel, gi, selected, moved);
         return;
     }
-    if (n_models <= 16 && total >= dense_min_selected<LAYOUT, TB::kCode != kDtypeNone>(n_models) && __all_sync(0xFFFFFFFFu, sel == 0 || gi.valid == 4)) {
+    if ((TOGETHER || n_models <= 16) && total >= dense_min_selected<LAYOUT, TB::kCode != kDtypeNone, TOGETHER>(n_models) && __all_sync(0xFFFFFFFFu, sel == 0 || gi.valid == 4)) {
         if (sel) {
             if (n_models <= 8) serve_group_dense<TA, TB, LAYOUT, uint32_t>(a, image_a, image_b, g_block, sel, gi, selected, moved);
             else serve_group_dense<TA, TB, LAYOUT, uint64_t>(a, image_a, image_b, g_block, sel, gi, selected, moved);
@@ -586,9 +586,9 @@ __device__ __forceinline__ void serve_tile(const ShuffleArgs &a, const unsigned 
         const uint32_t tensor = __shfl_sync(0xFFFFFFFFu, gi.tensor_id, owner);
         if (!active) continue;
         uint64_t perm = 0;
-        if (n_models <= 16) perm = draw_permutation_packed(n_models, 4u * cgroup + c, tensor, a.step_lo, a.step_hi8, a.keys);
+        if (TOGETHER || n_models <= 16) perm = draw_permutation_packed(n_models, 4u * cgroup + c, tensor, a.step_lo, a.step_hi8, a.keys);
         else draw_permutation_u8(s_perm, T_, n_models, 4u * cgroup + c, tensor, a.step_lo, a.step_hi8, a.keys);
-        move_coordinate<TA, TB, LAYOUT>(a, image_a, image_b, s_perm, perm, warp_base + owner, c, g_block, moved);
+        move_coordinate<TA, TB, LAYOUT, TOGETHER>(a, image_a, image_b, s_perm, perm, warp_base + owner, c, g_block, moved);
         ++selected;
     }
     __syncwarp();   // the warp's list is rewritten by the next tile
@@ -777,7 +777,7 @@ __device__ __forceinline__ void consensus_tile(const ShuffleArgs &a, const unsig
 // lean flavour (48 registers, as many resident blocks as the shared memory allows) cannot afford.
 // kN: the population size where it is compiled in (STAT, N = 2 .. 8), 0 = run-time N.  From N = 7 on the statistic does not
 // fit 48 registers (with them N = 8 takes 89 us for ResNet-18, with 64 81; N = 6 66 and 70).
-template <class TA, class TB, int LAYOUT, int G, bool STAT, bool EARLY, int kN>
+template <class TA, class TB, int LAYOUT, int G, bool STAT, bool EARLY, int kN, bool TOGETHER>
 __global__ void __launch_bounds__(256, EARLY ? 3 : (kN > 6 ? 4 : 5)) shuffle_async_kernel(const __grid_constant__ ShuffleArgs a)
 {
     if constexpr (kN != 0) __builtin_assume(a.pop.N == kN);
@@ -858,7 +858,7 @@ __global__ void __launch_bounds__(256, EARLY ? 3 : (kN > 6 ? 4 : 5)) shuffle_asy
 #pragma unroll
         for (int i = 0; i < G; ++i) {
             const unsigned char *image_a = smem_raw + i * (a_bytes + b_bytes);
-            serve_tile<TA, TB, LAYOUT>(a, image_a, image_a + a_bytes, s_list, s_perm,
+            serve_tile<TA, TB, LAYOUT, TOGETHER>(a, image_a, image_a + a_bytes, s_list, s_perm,
                                        g_first + static_cast<uint64_t>(i) * T_, sel[i], gi[i], selected, moved);
         }
     }
@@ -886,11 +886,14 @@ cudaError_t launch_shuffle_async_tiles(const ShuffleArgs &args, const LaunchShap
     using Kernel = void (*)(ShuffleArgs);
     Kernel kernel;
     if constexpr (kN != 0) {   // built with the statistics only
-        kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, true, false, kN> : shuffle_async_kernel<TA, TB, kLayoutPN, G, true, false, kN>;
+        kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, true, false, kN, false> : shuffle_async_kernel<TA, TB, kLayoutPN, G, true, false, kN, (stored_together(kLayoutPN, kN) > 1)>;
     } else {
-        kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, false, false, 0> : shuffle_async_kernel<TA, TB, kLayoutPN, G, false, false, 0>;
-        if (args.sq.slots) kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, true, false, 0> : shuffle_async_kernel<TA, TB, kLayoutPN, G, true, false, 0>;
-        else if (args.early && kEarlyBuilt) kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, 1, false, true, 0> : shuffle_async_kernel<TA, TB, kLayoutPN, 1, false, true, 0>;
+        const bool together = args.pop.N <= 16 && stored_together(args.pop.layout, args.pop.N) > 1;
+        kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, false, false, 0, false>
+                    : together ? shuffle_async_kernel<TA, TB, kLayoutPN, G, false, false, 0, true> : shuffle_async_kernel<TA, TB, kLayoutPN, G, false, false, 0, false>;
+        if (args.sq.slots) kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, true, false, 0, false>
+                                       : together ? shuffle_async_kernel<TA, TB, kLayoutPN, G, true, false, 0, true> : shuffle_async_kernel<TA, TB, kLayoutPN, G, true, false, 0, false>;
+        else if (args.early && kEarlyBuilt) kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, 1, false, true, 0, false> : shuffle_async_kernel<TA, TB, kLayoutPN, 1, false, true, 0, false>;
     }
     KernelFit fit;
     cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), threads, smem, &fit);

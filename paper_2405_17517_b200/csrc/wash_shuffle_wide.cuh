@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(64, 6) shuffle_wide_kernel(const __grid_consta
         const uint32_t count = min(32u, total - first);
         if (first) draw(first, count);
         if (lane < count) ++selected;
-        if (LAYOUT == kLayoutPN && n_models % 4 == 0) {
+        if (stored_together(LAYOUT, n_models) == 4) {
             const size_t skip = static_cast<size_t>(warp_base) * group_elems;
             moved += move_quads<TA, TB>(a, image_a + skip * TA::kBytes, image_b + skip * TB::kBytes, g_block + warp_base, s_perm, list + first, count, lane, 32u);
         } else if (LAYOUT == kLayoutPN || count <= kWidePairsMax) {
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_co
     }
     if (threadIdx.x == 0) selected = total;
     for (uint32_t first = 0; first < total;) {
-        if (n_models % 4 == 0) moved += move_quads<TA, TB>(a, image_a, image_b, g_block, s_perm, s_entry + first, in_round, threadIdx.x, blockDim.x);
+        if (stored_together(LAYOUT, n_models) == 4) moved += move_quads<TA, TB>(a, image_a, image_b, g_block, s_perm, s_entry + first, in_round, threadIdx.x, blockDim.x);
         else {
             // a lane per (coordinate, model) pair, the models of a coordinate side by side
             for (uint32_t i = threadIdx.x; i < in_round * static_cast<uint32_t>(n_models); i += blockDim.x) {

@@ -25,6 +25,8 @@ int rule_fetch_half_lines(int layout, int n_models, float share, int by_warps, i
 
 int rule_half_wave_serves(int n_models, double by_load, unsigned resident, unsigned n_wtiles) { return wash::half_wave_serves(n_models, by_load, resident, n_wtiles) ? 1 : 0; }
 
+int rule_stored_together(int layout, int n_models) { return wash::stored_together(layout, n_models); }
+
 unsigned rule_report_grid(unsigned long long n_tiles, unsigned long long resident) { return wash::report_grid(n_tiles, resident); }
 int rule_stat_slots() { return wash::kStatSlots; }
 

@@ -67,3 +67,12 @@ def test_half_a_wave_only_where_it_does_not_lose_more_than_it_gains(rules):
         return rules.rule_half_wave_serves(N, ctypes.c_double(by_load), 1184, n_wtiles)
     assert half(5, 374.0, 21_914) and half(32, 0.0, 37_888)
     assert not half(33, 1.0, 100) and not half(5, 474.0, 21_914) and not half(5, 1.0, 37_889)
+
+
+def test_which_populations_store_neighbouring_values_together(rules):
+    """[P][N]: four models' values where the population is a multiple of four, two where it is even, up to 16 models, but not two
+    models; the kernels' code paths, WASH_MODE_AUTO's table and the early flavour all go by this."""
+    assert rules.rule_stored_together(1, 2) == 1
+    for N in range(3, 65):
+        want = 4 if N % 4 == 0 else 2 if N % 2 == 0 and N <= 16 else 1
+        assert rules.rule_stored_together(1, N) == want and rules.rule_stored_together(0, N) == 1
