@@ -180,6 +180,7 @@ cudaError_t launch_shuffle(const ShuffleArgs &args, int a_dtype, int b_dtype, in
     // hundreds of blocks that report (2^20 coordinates, N = 3: 437 us, 16 us with counters on the device; sparse 949 us).  Such a
     // launch counts into the spare slot on the device, and one more kernel hands the two sums over.
     ShuffleArgs call = args;
+    call.dense_from = dense_threshold(args.pop.N, b_dtype != kDtypeNone, a_dtype == kDtypeF32 && b_dtype != kDtypeBF16);
     cudaPointerAttributes where;
     bool hand_over = false;
     if (args.stats) {

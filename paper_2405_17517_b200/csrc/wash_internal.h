@@ -18,6 +18,17 @@ __host__ __device__ constexpr int stored_together(int layout, int n_models)
     return layout != kLayoutPN || n_models == 2 ? 1 : n_models % 4 == 0 ? 4 : n_models % 2 == 0 && n_models <= 16 ? 2 : 1;
 }
 
+// How a streaming kernel serves what a warp has selected.  The forms are kernels of their own: the code of one costs the populations
+// of another up to 12 % (N = 7 bf16, p = 0.4 176 us alone, 198 with the code that stores values together; 4 % by the choice at run time).
+//   kServeByCount      values one by one, densely from half of a warp's coordinates on: [N][P], odd populations, more than 16 models
+//   kServeByThreshold  values one by one, densely from a threshold on (dense_threshold): two models in [P][N]
+//   kServeTogether     neighbouring models' values together, densely from a threshold on: even populations from 4 to 16 models in [P][N]
+constexpr int kServeByCount = 0, kServeByThreshold = 1, kServeTogether = 2;
+__host__ __device__ constexpr int serve_form(int layout, int n_models)
+{
+    return layout != kLayoutPN || n_models > 16 ? kServeByCount : n_models == 2 ? kServeByThreshold : stored_together(layout, n_models) > 1 ? kServeTogether : kServeByCount;
+}
+
 // One row of a stack is cut into groups of 4 consecutive elements; a group never
 // straddles two tensors because tensors start on multiples of 8 elements.
 struct SegEntry {
@@ -96,6 +107,7 @@ struct ShuffleArgs {
     bool measure_only = false;    // with sq: nothing is selected
     uint32_t pn_pad = 0;          // streaming kernel, [P][N]: elements of padding after a group in the shared-memory image (0 or 4)
     uint32_t pair_inverse = 0;    // streaming kernel, N > 16: 2^20 / N, rounded up (i / N = i * pair_inverse >> 20 for i < 2080; set by its launcher)
+    uint64_t dense_from = 1ull << 33;   // streaming kernels, even populations of up to 16 models in [P][N]: threshold from which a tensor is served densely (dense_threshold)
     bool early = false;           // streaming kernel: the flavour that draws permutations while the copies are in flight
     void *mirror_a = nullptr;     // sparse kernel: a second copy of each stack (mapped host memory) that receives the moved values, too
     void *mirror_b = nullptr;
@@ -140,6 +152,23 @@ inline bool fetch_half_lines(const ShuffleArgs &args, bool by_warps, int bytes_a
 inline bool half_wave_serves(int n_models, double by_load, uint32_t resident, uint32_t n_wtiles)
 {
     return n_models <= 32 && by_load <= 0.4 * resident && n_wtiles <= 32ull * resident;   // 16 tiles for each of the 4 warps of resident / 2 blocks
+}
+
+// [P][N], even populations of up to 16 models: the threshold from which every lane serves its own group (serve_group_dense) instead of
+// coordinates dealt to the lanes, whose values are stored together from 4 models on.  It is the tensor's threshold that decides, not what a
+// warp happens to have selected: warps of both kinds beside each other take longer than those of either (N = 2 fp32, 2^24 coordinates, p = 0.8, from 100 selected of
+// a warp's 128 on 165 us, all dense 130, all dealt 161; two fp32 stacks 278, 212, 262).  Time dense over time dealt at 45 / 55 / 65 / 75 / 80 / 85 / 90 / 100 %:
+//   one stack   fp32 N = 2 1.19 1.00 .97 .87 .81 .80 .80 .80, 4 1.43 1.20 1.16 1.04 .96 .95 .95 .96, 6 1.42 1.16 1.12 1.00 .93 .91 .91 .90, 8 2.40 1.20 1.15 1.03 .98 .96 .96 .96, 10
+//               1.59 1.29 1.25 1.10 1.01 1.00 1.00 1.00, 12 1.65 1.33 1.29 1.13 1.04 1.04 1.03 1.04, 14 as 10, 16 2.81 1.36 1.33 1.18 1.10 1.08 1.07 1.07;  bf16 2 1.20 1.00 .97
+//               .88 .82 .81 .81 .80, 4 1.36 1.14 1.10 .99 .92 .91 .91 .91, 8 1.61 1.31 1.25 1.10 1.00 .98 .98 .98, 10 to 16 as fp32
+//   two stacks  fp32 N = 2 1.15 .98 .95 .86 .80 .79 .79 .77, 4 1.99 1.14 1.22 1.11 1.10 1.08 1.07 1.14, 6 1.27 1.17 1.11 .99 1.00 .99 .93 .94, 8 3.20 1.96 1.92 1.78 1.71 1.66 1.65 1.58, 10 1.56 1.42
+//               1.28 1.16 1.13 1.08 1.02 .92, 12 2.40 1.81 1.79 1.65 1.62 1.57 1.51 1.51, 14 1.61 1.47 1.33 1.18 1.12 1.07 1.02 .95, 16 3.16 2.01 1.98 1.87 1.78 1.75 1.72 1.59;  bf16 + fp32 4 1.86 1.12 1.13
+//               1.02 .95 .93 .94 .94, 6 1.30 1.12 1.21 1.02 .99 1.00 .98 .97, 8 to 16 by fours 1.3 to 3.6, 10 1.22 1.24 1.14 1.07 1.04 1.03 .99 .95, 14 1.34 1.24 1.13 1.02 .99 .96 .92 .86
+inline uint64_t dense_threshold(int n_models, bool two_stacks, bool all_f32)
+{
+    float share = n_models == 2 ? 0.56f : n_models <= 8 ? 0.78f : !two_stacks ? 0.85f : all_f32 ? 0.88f : 0.79f;
+    if (n_models % 4 == 0 && (two_stacks ? n_models > 4 || all_f32 : n_models > 8)) share = 2.f;   // never
+    return static_cast<uint64_t>(share * 4294967296.f);
 }
 
 // Blocks of the resident-warp streaming kernel: those that are resident, as far as there are tiles for them -- and, where a device has few

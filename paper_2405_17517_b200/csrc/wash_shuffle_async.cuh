@@ -26,16 +26,7 @@
 
 namespace wash {
 
-// Selected coordinates of a warp's 128 from which every lane serves its own group.  Later in [P][N] where the dealt coordinates' values are
-// stored together (move_neighbours): dense / dealt at 45 / 55 / 70 / 85 / 100 % selected, 2^23 coordinates, N = 2 fp32 1.15 1.09 0.98 0.83 0.84, N = 8 fp32 1.06 1.10
-// 1.07 0.92 0.91, N = 16 bf16 1.11 1.24 1.20 0.99 0.99, N = 10 two fp32 stacks 1.03 1.34 1.15 0.98 0.86; never with two stacks of a multiple of four models from 8 on, N = 8
-// two fp32 stacks 1.17 1.83 1.87 1.63 1.65, N = 16 bf16 + fp32 1.23 2.06 2.16 1.89 1.82.
-template <int LAYOUT, bool TWO_STACKS, bool TOGETHER>
-__device__ __forceinline__ uint32_t dense_min_selected(int n_models)
-{
-    if (!TOGETHER) return LAYOUT == kLayoutPN && n_models == 2 ? 100 : 64;
-    return TWO_STACKS && n_models >= 8 && n_models % 4 == 0 ? 129 : 100;
-}
+constexpr uint32_t kDenseMinSelected = 64;   // selected coordinates of a warp's 128 from which every lane serves its own group (even populations in [P][N]: dense_threshold)
 
 template <int BYTES>
 __device__ __forceinline__ void cp_async(uint32_t dst_smem, const void *src)
@@ -394,7 +385,7 @@ __device__ __forceinline__ void plan_tile(const ShuffleArgs &a, uint8_t *s_list,
     if (!__any_sync(0xFFFFFFFFu, sel != 0)) return;   // most warps have nothing selected at small p
     const uint32_t mine = __popc(sel);
     const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, mine);
-    if (total >= dense_min_selected<kLayoutNP, false, false>(n_models) && __all_sync(0xFFFFFFFFu, sel == 0 || gi.valid == 4)) {
+    if (total >= kDenseMinSelected && __all_sync(0xFFFFFFFFu, sel == 0 || gi.valid == 4)) {
         pl.mode = kServeDense;
         if (sel) {
             if (n_models <= 16) dense_draw<uint64_t>(a, sel, gi, pl.perm, selected, moved);
@@ -544,10 +535,11 @@ __device__ __forceinline__ void serve_few(const ShuffleArgs &a, const unsigned c
     }
 }
 
-template <class TA, class TB, int LAYOUT, bool TOGETHER>
+// much: the threshold of the lane's group is one from which the population is served densely (dense_threshold); not looked at in kServeByCount.
+template <class TA, class TB, int LAYOUT, int FORM>
 __device__ __forceinline__ void serve_tile(const ShuffleArgs &a, const unsigned char *image_a, const unsigned char *image_b,
                                            uint8_t *s_list, uint8_t *s_perm, uint64_t g_block,
-                                           uint32_t sel, const GroupInfo &gi, uint32_t &selected, uint32_t &moved)
+                                           uint32_t sel, const GroupInfo &gi, bool much, uint32_t &selected, uint32_t &moved)
 {
     const int n_models = a.pop.N;
     const uint32_t T_ = blockDim.x;
@@ -559,7 +551,8 @@ __device__ __forceinline__ void serve_tile(const ShuffleArgs &a, const unsigned 
         serve_few<TA, TB, LAYOUT>(a, image_a, image_b, g_block, sel, gi, selected, moved);
         return;
     }
-    if ((TOGETHER || n_models <= 16) && total >= dense_min_selected<LAYOUT, TB::kCode != kDtypeNone, TOGETHER>(n_models) && __all_sync(0xFFFFFFFFu, sel == 0 || gi.valid == 4)) {
+    constexpr bool kByCount = FORM == kServeByCount;
+    if ((!kByCount || (n_models <= 16 && total >= kDenseMinSelected)) && __all_sync(0xFFFFFFFFu, sel == 0 || (gi.valid == 4 && (kByCount || much)))) {
         if (sel) {
             if (n_models <= 8) serve_group_dense<TA, TB, LAYOUT, uint32_t>(a, image_a, image_b, g_block, sel, gi, selected, moved);
             else serve_group_dense<TA, TB, LAYOUT, uint64_t>(a, image_a, image_b, g_block, sel, gi, selected, moved);
@@ -586,9 +579,9 @@ __device__ __forceinline__ void serve_tile(const ShuffleArgs &a, const unsigned 
         const uint32_t tensor = __shfl_sync(0xFFFFFFFFu, gi.tensor_id, owner);
         if (!active) continue;
         uint64_t perm = 0;
-        if (TOGETHER || n_models <= 16) perm = draw_permutation_packed(n_models, 4u * cgroup + c, tensor, a.step_lo, a.step_hi8, a.keys);
+        if (!kByCount || n_models <= 16) perm = draw_permutation_packed(n_models, 4u * cgroup + c, tensor, a.step_lo, a.step_hi8, a.keys);
         else draw_permutation_u8(s_perm, T_, n_models, 4u * cgroup + c, tensor, a.step_lo, a.step_hi8, a.keys);
-        move_coordinate<TA, TB, LAYOUT, TOGETHER>(a, image_a, image_b, s_perm, perm, warp_base + owner, c, g_block, moved);
+        move_coordinate<TA, TB, LAYOUT, FORM == kServeTogether>(a, image_a, image_b, s_perm, perm, warp_base + owner, c, g_block, moved);
         ++selected;
     }
     __syncwarp();   // the warp's list is rewritten by the next tile
@@ -777,7 +770,7 @@ __device__ __forceinline__ void consensus_tile(const ShuffleArgs &a, const unsig
 // lean flavour (48 registers, as many resident blocks as the shared memory allows) cannot afford.
 // kN: the population size where it is compiled in (STAT, N = 2 .. 8), 0 = run-time N.  From N = 7 on the statistic does not
 // fit 48 registers (with them N = 8 takes 89 us for ResNet-18, with 64 81; N = 6 66 and 70).
-template <class TA, class TB, int LAYOUT, int G, bool STAT, bool EARLY, int kN, bool TOGETHER>
+template <class TA, class TB, int LAYOUT, int G, bool STAT, bool EARLY, int kN, int FORM>
 __global__ void __launch_bounds__(256, EARLY ? 3 : (kN > 6 ? 4 : 5)) shuffle_async_kernel(const __grid_constant__ ShuffleArgs a)
 {
     if constexpr (kN != 0) __builtin_assume(a.pop.N == kN);
@@ -808,13 +801,16 @@ __global__ void __launch_bounds__(256, EARLY ? 3 : (kN > 6 ? 4 : 5)) shuffle_asy
 
     uint32_t selected = 0, moved = 0;
     uint32_t sel[G];
+    bool much[G];
     GroupInfo gi[G];
 #pragma unroll
     for (int i = 0; i < G; ++i) {
         sel[i] = 0;
+        much[i] = false;
         gi[i] = GroupInfo{0, 0, 0, 0};
         if (threadIdx.x < in_tile[i]) {
             gi[i] = find_group(a.pop, static_cast<uint32_t>(g_first + static_cast<uint64_t>(i) * T_ + threadIdx.x), a.status);
+            much[i] = gi[i].thr >= a.dense_from;
             if (gi[i].thr != 0 && gi[i].valid != 0 && !(STAT && a.measure_only)) {
                 // word < thr with thr in [0, 2^32]: a 32-bit compare; a threshold of 2^32 selects
                 // whatever the word is, so the block is not drawn at all
@@ -858,8 +854,8 @@ __global__ void __launch_bounds__(256, EARLY ? 3 : (kN > 6 ? 4 : 5)) shuffle_asy
 #pragma unroll
         for (int i = 0; i < G; ++i) {
             const unsigned char *image_a = smem_raw + i * (a_bytes + b_bytes);
-            serve_tile<TA, TB, LAYOUT, TOGETHER>(a, image_a, image_a + a_bytes, s_list, s_perm,
-                                       g_first + static_cast<uint64_t>(i) * T_, sel[i], gi[i], selected, moved);
+            serve_tile<TA, TB, LAYOUT, FORM>(a, image_a, image_a + a_bytes, s_list, s_perm,
+                                       g_first + static_cast<uint64_t>(i) * T_, sel[i], gi[i], much[i], selected, moved);
         }
     }
     publish_block_stats(a.stats, a.stats_direct ? nullptr : a.stat_slots, selected, moved);
@@ -886,14 +882,17 @@ cudaError_t launch_shuffle_async_tiles(const ShuffleArgs &args, const LaunchShap
     using Kernel = void (*)(ShuffleArgs);
     Kernel kernel;
     if constexpr (kN != 0) {   // built with the statistics only
-        kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, true, false, kN, false> : shuffle_async_kernel<TA, TB, kLayoutPN, G, true, false, kN, (stored_together(kLayoutPN, kN) > 1)>;
+        kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, true, false, kN, kServeByCount> : shuffle_async_kernel<TA, TB, kLayoutPN, G, true, false, kN, serve_form(kLayoutPN, kN)>;
     } else {
-        const bool together = args.pop.N <= 16 && stored_together(args.pop.layout, args.pop.N) > 1;
-        kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, false, false, 0, false>
-                    : together ? shuffle_async_kernel<TA, TB, kLayoutPN, G, false, false, 0, true> : shuffle_async_kernel<TA, TB, kLayoutPN, G, false, false, 0, false>;
-        if (args.sq.slots) kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, true, false, 0, false>
-                                       : together ? shuffle_async_kernel<TA, TB, kLayoutPN, G, true, false, 0, true> : shuffle_async_kernel<TA, TB, kLayoutPN, G, true, false, 0, false>;
-        else if (args.early && kEarlyBuilt) kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, 1, false, true, 0, false> : shuffle_async_kernel<TA, TB, kLayoutPN, 1, false, true, 0, false>;
+        const int form = serve_form(args.pop.layout, args.pop.N);
+        kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, false, false, 0, kServeByCount> : shuffle_async_kernel<TA, TB, kLayoutPN, G, false, false, 0, kServeByCount>;
+        if (form == kServeTogether) kernel = shuffle_async_kernel<TA, TB, kLayoutPN, G, false, false, 0, kServeTogether>;
+        if constexpr (G == 2)   // (what two models get)
+            if (form == kServeByThreshold) kernel = shuffle_async_kernel<TA, TB, kLayoutPN, G, false, false, 0, kServeByThreshold>;
+        if (args.sq.slots) {
+            kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, G, true, false, 0, kServeByCount> : shuffle_async_kernel<TA, TB, kLayoutPN, G, true, false, 0, kServeByCount>;
+            if (form == kServeTogether) kernel = shuffle_async_kernel<TA, TB, kLayoutPN, G, true, false, 0, kServeTogether>;
+        } else if (args.early && kEarlyBuilt) kernel = np ? shuffle_async_kernel<TA, TB, kLayoutNP, 1, false, true, 0, kServeByCount> : shuffle_async_kernel<TA, TB, kLayoutPN, 1, false, true, 0, kServeByCount>;
     }
     KernelFit fit;
     cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), threads, smem, &fit);

@@ -128,7 +128,7 @@ __device__ __forceinline__ uint32_t list_selected(uint16_t *list, uint32_t sel)
 
 // kN: the population size where it is compiled in (the helpers read it from the arguments: the assumption reaches
 // them), 0 = run-time N.
-template <class TA, class TB, int LAYOUT, int G, int kN, bool TOGETHER>
+template <class TA, class TB, int LAYOUT, int G, int kN, int FORM>
 __global__ void __launch_bounds__(32, G == 2 ? 32 : 28) shuffle_loop_kernel(const __grid_constant__ ShuffleArgs a)
 {
     if constexpr (kN != 0) __builtin_assume(a.pop.N == kN);
@@ -231,7 +231,8 @@ __global__ void __launch_bounds__(32, G == 2 ? 32 : 28) shuffle_loop_kernel(cons
         if (!__any_sync(0xFFFFFFFFu, sel != 0)) continue;
         const unsigned char *images = smem_raw + stage * stage_bytes;
         const uint32_t count = __reduce_add_sync(0xFFFFFFFFu, __popc(sel));
-        if (count >= dense_min_selected<LAYOUT, kHasB, TOGETHER>(n_models) * G) {
+        const uint64_t thr = static_cast<uint64_t>(sc.thr_lo) | (static_cast<uint64_t>(sc.thr_hi) << 32);   // of the lane's last group
+        if (FORM == kServeByCount ? count >= kDenseMinSelected * G : __all_sync(0xFFFFFFFFu, sel == 0 || thr >= a.dense_from) != 0) {
             // every lane serves its own groups, those that are whole; the others go to the list below
 #pragma unroll 1
             for (int i = 0; i < G; ++i) {
@@ -259,7 +260,7 @@ __global__ void __launch_bounds__(32, G == 2 ? 32 : 28) shuffle_loop_kernel(cons
             }
             const uint64_t perm = draw_permutation_packed(n_models, 4u * cgroup + c, tensor, a.step_lo, a.step_hi8, a.keys);
             const unsigned char *image_a = images + i * (a_bytes + b_bytes);
-            move_coordinate<TA, TB, LAYOUT, TOGETHER>(a, image_a, image_a + a_bytes, nullptr, perm, owner, c, g - owner, moved);
+            move_coordinate<TA, TB, LAYOUT, FORM == kServeTogether>(a, image_a, image_a + a_bytes, nullptr, perm, owner, c, g - owner, moved);
             ++selected;
         }
         __syncwarp();   // the stage is overwritten by the copies the next trip starts
@@ -276,10 +277,10 @@ cudaError_t launch_shuffle_loop_tiles(const ShuffleArgs &args, const LaunchShape
     const size_t image = group_elems * (TA::kBytes + (kHasB ? TB::kBytes : 0)) * 32;
     const size_t smem = (2 * G * image + 2 * 32 * 4 * G + 15) & ~static_cast<size_t>(15);
     const bool np = args.pop.layout == kLayoutNP;
-    constexpr bool kTogether = kN != 0 && stored_together(kLayoutPN, kN) > 1;   // (a population that is compiled in)
-    auto kernel = np ? shuffle_loop_kernel<TA, TB, kLayoutNP, G, kN, false> : shuffle_loop_kernel<TA, TB, kLayoutPN, G, kN, kTogether>;
+    constexpr int kForm = kN != 0 ? serve_form(kLayoutPN, kN) : kServeByCount;   // (of a population that is compiled in)
+    auto kernel = np ? shuffle_loop_kernel<TA, TB, kLayoutNP, G, kN, kServeByCount> : shuffle_loop_kernel<TA, TB, kLayoutPN, G, kN, kForm>;
     if constexpr (kN == 0)
-        if (stored_together(args.pop.layout, args.pop.N) > 1) kernel = shuffle_loop_kernel<TA, TB, kLayoutPN, G, 0, true>;
+        if (serve_form(args.pop.layout, args.pop.N) == kServeTogether) kernel = shuffle_loop_kernel<TA, TB, kLayoutPN, G, 0, kServeTogether>;
     KernelFit fit;
     cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), 32, smem, &fit);
     if (err != cudaSuccess) return err;

@@ -76,3 +76,15 @@ def test_which_populations_store_neighbouring_values_together(rules):
     for N in range(3, 65):
         want = 4 if N % 4 == 0 else 2 if N % 2 == 0 and N <= 16 else 1
         assert rules.rule_stored_together(1, N) == want and rules.rule_stored_together(0, N) == 1
+
+
+def test_tensors_are_served_densely_late_or_never_in_even_populations(rules):
+    """A threshold of up to 2^32 is reached (by everything selected at the latest) or none is: populations of a multiple of four from 12
+    models on in one stack, from 8 on in two."""
+    rules.rule_dense_threshold.restype = ctypes.c_ulonglong
+    for N in range(2, 17, 2):
+        for two_stacks in (0, 1):
+            for all_f32 in (0, 1):
+                at = rules.rule_dense_threshold(N, two_stacks, all_f32) / 2.0 ** 32
+                never = N % 4 == 0 and (N >= 12 or (two_stacks and (N >= 8 or all_f32)))
+                assert at > 1.0 if never else 0.5 < at < 0.9

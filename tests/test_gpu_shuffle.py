@@ -781,3 +781,18 @@ def test_neighbouring_models_stored_together(N, dtype, opt, code):
     c.assert_equal("N=%d %s/%s" % (N, dtype, opt))
     assert c.gpu_stats() == tuple(want)
     c.close()
+
+
+@pytest.mark.parametrize("code", [-4, -5], ids=["resident", "one-trip"])
+@pytest.mark.parametrize("N,dtype,opt", [(2, "f32", None), (2, "bf16", "f32"), (4, "bf16", None), (4, "bf16", "f32"), (6, "f32", "f32"), (8, "f32", None), (10, "bf16", None), (14, "f32", "bf16")])
+def test_dense_serving_by_the_tensors_threshold(N, dtype, opt, code):
+    """[P][N], even populations: neighbouring tensors on both sides of the threshold from which a tensor is served densely (0.56 of the coordinates for two
+    models, 0.78 to 0.87 above), small ones, so that warps hold groups of both, ragged ones, and one whose threshold is reached by none of its words."""
+    c = Case(N, [130, 7, 1021, 64, 300, 5003, 12, 260, 900, 33, 2050], 1, dtype, opt, seed=N)
+    B.wash_set_launch(c.gpu.ctx, 0, code)
+    p_layer = [0.55, 0.57, 0.5, 0.79, 0.77, 0.9, 1.0, 0.86, 0.88, 0.0, 0.8]
+    (B.wash_shuffle_both if opt else B.wash_shuffle)(c.gpu.ctx, 3, 0.0, p_layer, seed=11, stats=c.stats_dev)
+    want = oracle.shuffle(c.ora, c.host, p_layer, seed=11, step=3, stack2=c.host_opt)
+    c.assert_equal("N=%d %s/%s" % (N, dtype, opt))
+    assert c.gpu_stats() == tuple(want)
+    c.close()
