@@ -461,3 +461,21 @@ def test_coordinate_major_populations_in_registers_or_staged(N, dtype):
     oracle.papa_all(c.ora, c.host)
     c.assert_equal("papa_all")
     c.close()
+
+
+@pytest.mark.parametrize("p_layer", [[0.7, 0.75, 0.9, 0.7], [1.0, 1.0, 1.0, 1.0]], ids=["most", "all"])
+@pytest.mark.parametrize("N,dtype,opt", [(20, "f32", None), (24, "bf16", "f32"), (32, "f32", "f32"), (40, "bf16", None), (64, "f32", None), (18, "f32", None)])
+def test_consensus_of_large_populations_of_which_most_is_selected(N, dtype, opt, p_layer):
+    """[P][N], more than 16 models and 70 % and more selected: a multiple of four takes the kernel for such populations, which moves four
+    models' values at once, others the early flavour's share; stacks and distances as ever."""
+    numel = [1021, 6, 4099, 130]
+    c = Case(N, numel, B.WASH_LAYOUT_PN, dtype, opt, seed=N)
+    bounds = [0, 2, 4]
+    want_sq = np.stack([oracle.consensus_sq(c.ora, c.host, lo, hi) for lo, hi in zip(bounds[:-1], bounds[1:])])
+    out = torch.zeros((2, N), dtype=torch.float64, device="cuda")
+    B.wash_shuffle_consensus(c.gpu.ctx, B.WASH_STACK_PARAMS if opt is None else B.WASH_STACK_BOTH, 2, 0.0, p_layer, seed=6, stats=c.stats_dev, tensor_bounds=bounds, dev_sq_out=out)
+    want = oracle.shuffle(c.ora, c.host, p_layer, seed=6, step=2, stack2=c.host_opt)
+    c.assert_equal("N=%d" % N)
+    assert c.gpu_stats() == tuple(want)
+    assert np.allclose(out.cpu().numpy(), want_sq, rtol=1e-12, atol=0)   # binary64 sums of positive terms in another order: (terms) 2^-53
+    c.close()
