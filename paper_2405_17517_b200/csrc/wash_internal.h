@@ -102,17 +102,19 @@ struct ShuffleArgs {
     unsigned long long *stats;    // device-accessible {selected, moved} or nullptr
     StatSlot *stat_slots;         // device, kStatSlots + 1 zeroed entries (left zeroed by every launch)
     bool stats_direct = false;    // few blocks report: they add to `stats` themselves (kernels that need a flush kernel otherwise)
+    uint32_t dense_from = 0xFFFFFFFFu;   // streaming kernels, even populations of up to 16 models in [P][N]: half the threshold from which a tensor is served densely (dense_threshold)
     uint32_t *status;             // device status word
     SqArgs sq;                    // consensus distance of the first stack (streaming kernel only)
     bool measure_only = false;    // with sq: nothing is selected
     uint32_t pn_pad = 0;          // streaming kernel, [P][N]: elements of padding after a group in the shared-memory image (0 or 4)
     uint32_t pair_inverse = 0;    // streaming kernel, N > 16: 2^20 / N, rounded up (i / N = i * pair_inverse >> 20 for i < 2080; set by its launcher)
-    uint64_t dense_from = 1ull << 33;   // streaming kernels, even populations of up to 16 models in [P][N]: threshold from which a tensor is served densely (dense_threshold)
     bool early = false;           // streaming kernel: the flavour that draws permutations while the copies are in flight
     void *mirror_a = nullptr;     // sparse kernel: a second copy of each stack (mapped host memory) that receives the moved values, too
     void *mirror_b = nullptr;
     float expected_share = 0.f;   // share of the coordinates the call's probabilities select, in expectation (sizes the sparse kernel's grid)
 };
+// A launch with more than 288 bytes of arguments costs the host 0.35 us more (3.4 -> 3.75 us a call with 296).
+static_assert(sizeof(ShuffleArgs) <= 288, "ShuffleArgs must stay within 288 bytes");
 
 // Whether the sparse kernels' loads of values ask for 64 bytes of a line instead of all 128 (load_scattered).  128 bytes are the better
 // request where a line's other half holds a selected coordinate as well, which is then fetched for nothing, and where masks and not
@@ -164,11 +166,11 @@ inline bool half_wave_serves(int n_models, double by_load, uint32_t resident, ui
 //   two stacks  fp32 N = 2 1.15 .98 .95 .86 .80 .79 .79 .77, 4 1.99 1.14 1.22 1.11 1.10 1.08 1.07 1.14, 6 1.27 1.17 1.11 .99 1.00 .99 .93 .94, 8 3.20 1.96 1.92 1.78 1.71 1.66 1.65 1.58, 10 1.56 1.42
 //               1.28 1.16 1.13 1.08 1.02 .92, 12 2.40 1.81 1.79 1.65 1.62 1.57 1.51 1.51, 14 1.61 1.47 1.33 1.18 1.12 1.07 1.02 .95, 16 3.16 2.01 1.98 1.87 1.78 1.75 1.72 1.59;  bf16 + fp32 4 1.86 1.12 1.13
 //               1.02 .95 .93 .94 .94, 6 1.30 1.12 1.21 1.02 .99 1.00 .98 .97, 8 to 16 by fours 1.3 to 3.6, 10 1.22 1.24 1.14 1.07 1.04 1.03 .99 .95, 14 1.34 1.24 1.13 1.02 .99 .96 .92 .86
-inline uint64_t dense_threshold(int n_models, bool two_stacks, bool all_f32)
+inline uint32_t dense_threshold(int n_models, bool two_stacks, bool all_f32)   // (half of it: it may be 2^32)
 {
-    float share = n_models == 2 ? 0.56f : n_models <= 8 ? 0.78f : !two_stacks ? 0.85f : all_f32 ? 0.88f : 0.79f;
-    if (n_models % 4 == 0 && (two_stacks ? n_models > 4 || all_f32 : n_models > 8)) share = 2.f;   // never
-    return static_cast<uint64_t>(share * 4294967296.f);
+    const float share = n_models == 2 ? 0.56f : n_models <= 8 ? 0.78f : !two_stacks ? 0.85f : all_f32 ? 0.88f : 0.79f;
+    if (n_models % 4 == 0 && (two_stacks ? n_models > 4 || all_f32 : n_models > 8)) return 0xFFFFFFFFu;   // never
+    return static_cast<uint32_t>(share * 2147483648.f);
 }
 
 // Blocks of the resident-warp streaming kernel: those that are resident, as far as there are tiles for them -- and, where a device has few

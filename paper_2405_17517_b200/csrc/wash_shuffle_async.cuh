@@ -810,7 +810,7 @@ __global__ void __launch_bounds__(256, EARLY ? 3 : (kN > 6 ? 4 : 5)) shuffle_asy
         gi[i] = GroupInfo{0, 0, 0, 0};
         if (threadIdx.x < in_tile[i]) {
             gi[i] = find_group(a.pop, static_cast<uint32_t>(g_first + static_cast<uint64_t>(i) * T_ + threadIdx.x), a.status);
-            much[i] = gi[i].thr >= a.dense_from;
+            much[i] = static_cast<uint32_t>(gi[i].thr >> 1) >= a.dense_from;
             if (gi[i].thr != 0 && gi[i].valid != 0 && !(STAT && a.measure_only)) {
                 // word < thr with thr in [0, 2^32]: a 32-bit compare; a threshold of 2^32 selects
                 // whatever the word is, so the block is not drawn at all

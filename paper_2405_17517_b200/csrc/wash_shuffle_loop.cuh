@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(32, G == 2 ? 32 : 28) shuffle_loop_kernel(cons
         if (!__any_sync(0xFFFFFFFFu, sel != 0)) continue;
         const unsigned char *images = smem_raw + stage * stage_bytes;
         const uint32_t count = __reduce_add_sync(0xFFFFFFFFu, __popc(sel));
-        const uint64_t thr = static_cast<uint64_t>(sc.thr_lo) | (static_cast<uint64_t>(sc.thr_hi) << 32);   // of the lane's last group
+        const uint32_t thr = (sc.thr_lo >> 1) | (sc.thr_hi << 31);   // half the threshold of the lane's last group
         if (FORM == kServeByCount ? count >= kDenseMinSelected * G : __all_sync(0xFFFFFFFFu, sel == 0 || thr >= a.dense_from) != 0) {
             // every lane serves its own groups, those that are whole; the others go to the list below
 #pragma unroll 1

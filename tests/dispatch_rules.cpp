@@ -27,7 +27,7 @@ int rule_half_wave_serves(int n_models, double by_load, unsigned resident, unsig
 
 int rule_stored_together(int layout, int n_models) { return wash::stored_together(layout, n_models); }
 
-unsigned long long rule_dense_threshold(int n_models, int two_stacks, int all_f32) { return wash::dense_threshold(n_models, two_stacks != 0, all_f32 != 0); }
+unsigned rule_dense_threshold(int n_models, int two_stacks, int all_f32) { return wash::dense_threshold(n_models, two_stacks != 0, all_f32 != 0); }
 
 unsigned rule_report_grid(unsigned long long n_tiles, unsigned long long resident) { return wash::report_grid(n_tiles, resident); }
 int rule_stat_slots() { return wash::kStatSlots; }

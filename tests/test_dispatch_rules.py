@@ -79,12 +79,12 @@ def test_which_populations_store_neighbouring_values_together(rules):
 
 
 def test_tensors_are_served_densely_late_or_never_in_even_populations(rules):
-    """A threshold of up to 2^32 is reached (by everything selected at the latest) or none is: populations of a multiple of four from 12
+    """A threshold of up to 2^32 (half of it is compared) is reached (by everything selected at the latest) or none is: populations of a multiple of four from 12
     models on in one stack, from 8 on in two."""
-    rules.rule_dense_threshold.restype = ctypes.c_ulonglong
+    rules.rule_dense_threshold.restype = ctypes.c_uint32
     for N in range(2, 17, 2):
         for two_stacks in (0, 1):
             for all_f32 in (0, 1):
-                at = rules.rule_dense_threshold(N, two_stacks, all_f32) / 2.0 ** 32
+                at = rules.rule_dense_threshold(N, two_stacks, all_f32) / 2.0 ** 31
                 never = N % 4 == 0 and (N >= 12 or (two_stacks and (N >= 8 or all_f32)))
                 assert at > 1.0 if never else 0.5 < at < 0.9
