@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_co
     await_previous();
     let_next_start();
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ uint32_t s_count;
+    __shared__ uint32_t s_count, s_gave_up;
     __shared__ __align__(8) unsigned long long s_barrier;
     constexpr int LAYOUT = kLayoutPN;
     constexpr bool kHasB = TB::kCode != kDtypeNone;
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_co
     const uint32_t barrier = smem_addr(&s_barrier);
     if constexpr (BULK) {
         if (threadIdx.x == 0) {
-            s_count = 0;
+            s_count = s_gave_up = 0;
             const uint32_t bytes_a = in_block * 4u * n_models * TA::kBytes, bytes_b = kHasB ? in_block * 4u * n_models * TB::kBytes : 0u;
             bulk_barrier_init(barrier);
             bulk_barrier_expect(barrier, bytes_a + bytes_b);
@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_co
     uint32_t in_round = draw(0);
     // (a group's bytes were copied, its permutations drawn by threads of other warps: both forms end with a barrier)
     if constexpr (BULK) {
-        if (!block_copies_done(barrier, kBulkTries)) {   // (not seen) report and move nothing; the block stays for its copies once more as long
+        if (!block_copies_done(barrier, kBulkTries, &s_gave_up)) {   // (not seen) report and move nothing; the block stays for its copies once more as long
             if (threadIdx.x == 0) atomicOr(a.status, 8u);
             bulk_copies_done(barrier, kBulkTries);
             return;

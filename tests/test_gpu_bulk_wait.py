@@ -25,6 +25,7 @@ def probe(tmp_path_factory):
 @pytest.mark.parametrize("arrive,first_warp,others,want", [(1, 64, 64, 1),    # all see the copies
                                                            (1, 0, 64, 0),     # one warp gives up, the others see them
                                                            (1, 64, 0, 0),
+                                                           (1, 0, 0, 0),      # all give up
                                                            (0, 8, 8, 0)])     # nothing arrives: the wait ends
 def test_every_thread_gets_one_answer(probe, threads, arrive, first_warp, others, want):
     torch.cuda.init()
