@@ -184,13 +184,31 @@ inline uint32_t report_grid(uint64_t n_tiles, uint64_t resident)
     return static_cast<uint32_t>(n_tiles < grid ? n_tiles : grid);
 }
 
-// Whether the blocks of shuffle_wide_pn_kernel fetch their bytes by bulk copies (its comment has the measurements).  Only where a
-// wait that is given up can be reported: without a status word (wash_shuffle_noalloc) the block would stay as it was, and nobody would know.
-// A bulk copy takes multiples of 16 bytes: groups come in pairs (rows and ranges are whole units of 8 elements) and have 8 N bytes at least.
-inline bool copies_in_bulk(const ShuffleArgs &args, uint32_t groups, size_t group_bytes, bool two_stacks)
+// Whether the blocks of shuffle_wide_pn_kernel fetch their bytes by bulk copies.  Only where a wait that is given up can be reported: without a
+// status word (wash_shuffle_noalloc) the block would stay as it was, and nobody would know.  A bulk copy takes multiples of 16 bytes: groups come
+// in pairs (rows and ranges are whole units of 8 elements) and have 8 N bytes at least.
+// Time with bulk copies over time with 16 bytes (bf16: 8) a thread at a time, by bytes of a block's images (32 groups, 64 for N <= 39 in fp32 and like sizes), 1 / 3 /
+// 10 / 30 % selected, stacks of 0.4 GB, and of 3 GB:
+//   one stack    fp32  22 KB (N = 44) .92 .84 .85 .90, 1.34 1.41 .85 .90;  25 KB (48) .94 .85 .84 .90, 1.30 1.24 .85 .90;  27 KB (52) .91 .83 .84 .90, 1.18 .83 .84 .90;  29 KB (56) .93 .84
+//                .84 .90, 1.13 1.21 .84 .90;  30 KB (58 to 60) .88 .82 .85, .88 .82 .85;  33 KB (32, 64) .95 .91 .88 .90, .97 .92 .87 .90;  37 KB (36) .91 .87 .86 .90, the same
+//   two stacks   bf16 + fp32  22 KB (28) .93 .87 .89 .85, 1.42 1.55 1.33 .84;  25 KB (32) .91 .85 .83 .84, 1.27 1.40 .87 .83;  28 KB (36) .89 .82 .83 .84, 1.12 1.26 .84 .83;  31 KB (40) .85 .77 .77
+//                .84, .89 1.09 .96 .83;  32 to 34 KB (42 to 44, 22) .86 .78 .79 .84, .88 .79 to 1.03 .79 .83;  37 KB (24, 48) .85 .80 .82 .85, .86 .82 .82 .84
+//                fp32 twice  25 KB (24) .96 .94 .96 .87, 1.33 1.61 1.42 .87;  33 KB (32) .95 .89 .86 .85, .99 1.22 1.00 .85;  34 and 35 KB (33, 34; 17) .96 .90 .86 .84, .99 1.16 .88 .85;  35 KB and
+//                more of 32 groups (35, 36) .93 .84 .82 .85, .95 .84 to 1.04 .84 .85;  37 to 41 KB of 64 groups (18, 20) .96 .95 .94 .89, .99 to 1.18 1.12 .95 .88;  49 and 65 KB (48, 64) .86 .76 .76 .84, the same
+//                bf16 twice  20 KB (40) .68 .71 .75, 1.15 1.20 .69 .73;  25 KB (48) .70 .65 .68 .80, .95 .65 to 1.03 .67 .80;  33 KB (32, 64) .68 .65 .68 .80, the same
+// So they pay where much is selected, for large blocks, and in stacks of up to half a GB (400 MB: .63 to 1.00 in all of 420 cells); small blocks of
+// which little is selected lose in stacks of 0.8 to 1.6 GB and more, for a reason that is not known.  N = 32 fp32, 2^25 coordinates, p = 0.1 813 -> 707 us.
+inline bool copies_in_bulk(const ShuffleArgs &args, uint32_t groups, int bytes_a, int bytes_b)
 {
     if (!args.status || args.pn_pad != 0 || ((args.group_lo | args.group_hi) & 1u) != 0) return false;
-    return groups == 64 || group_bytes > 1024 || (group_bytes == 1024 && !two_stacks);
+    const uint32_t group_bytes = 4u * static_cast<uint32_t>(args.pop.N * (bytes_a + bytes_b)), image = groups * group_bytes;
+    const float share = args.expected_share;
+    if (static_cast<uint64_t>(args.group_hi - args.group_lo) * group_bytes <= 500000000u) return true;
+    if (bytes_a != 4 && bytes_b != 4) return share >= 0.08f || image >= 24000u;
+    if (share >= 0.2f) return true;
+    if (bytes_b == 0) return image >= 29500u;
+    if (bytes_a != bytes_b) return image >= 32000u;
+    return share >= 0.08f ? image >= 33000u : group_bytes >= 1120u;
 }
 
 struct ReduceArgs {

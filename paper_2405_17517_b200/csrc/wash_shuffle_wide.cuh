@@ -163,11 +163,8 @@ constexpr size_t kWideSplitBytes = 512;
 // move.  N = 32 fp32, 2^23, p = 0.1 / 0.3: an even share 226 / 407 us (by pairs), 16 209 / 349, 32 221 / 364.  The moves are dealt to all threads.
 constexpr uint32_t kWideChunk = 16;
 
-// BULK: the block's bytes come by one bulk copy a stack instead of 16 bytes a thread at a time (a sixth of the kernel's instructions).
-// Which launches: those whose blocks have 64 groups, and larger groups with 32.  Time by 16 bytes over time by bulk copies, 2^22 - 2^23 coordinates, p = 0.01 /
-// 0.03 / 0.1 / 0.3 / 0.6; blocks of 64 groups N = 32 fp32 (512 bytes) 1.04 1.09 1.12 1.09 1.07, N = 24 bf16 + fp32 (576) 1.14 1.17 1.13 1.17 1.13; of 32 groups
-// N = 24 fp32 twice (768) 1.02 0.74 0.83 1.14 1.11, N = 48 fp32 (768) 0.80 0.75 0.87 1.11 1.08, N = 32 fp32 twice (1024) 1.03 0.88 0.96 1.18 1.12, N = 64 fp32 (1024) 1.10 1.23
-// 1.19 1.11 1.07, N = 48 bf16 + fp32 (1152) 1.21 1.33 1.31 1.20 1.13, N = 64 fp32 twice (2048) 1.22 1.37 1.32 1.19 1.12.  N = 32 fp32, 2^25, p = 0.1 813 -> 707 us.
+// BULK: the block's bytes come by one bulk copy a stack instead of 16 bytes a thread at a time, which are a sixth of the kernel's instructions
+// (copies_in_bulk chooses).
 template <class TA, class TB, bool BULK>
 __global__ void __launch_bounds__(128, 6) shuffle_wide_pn_kernel(const __grid_constant__ ShuffleArgs a)
 {
@@ -293,8 +290,7 @@ cudaError_t launch_shuffle_wide_typed(const ShuffleArgs &call, const LaunchShape
         const size_t per_group = group_elems * (TA::kBytes + (kHasB ? TB::kBytes : 0)) + 4 * 8 + 4 + 4 * wide_pitch(args.pop.N);
         const uint32_t groups = per_group * 64 > 44 * 1024 ? 32 : 64;   // five blocks and more on an SM
         const size_t smem = (per_group * groups + 15) & ~static_cast<size_t>(15);
-        const size_t group_bytes = 4 * static_cast<size_t>(args.pop.N) * (TA::kBytes + TB::kBytes);
-        auto kernel = copies_in_bulk(args, groups, group_bytes, kHasB) ? shuffle_wide_pn_kernel<TA, TB, true> : shuffle_wide_pn_kernel<TA, TB, false>;
+        auto kernel = copies_in_bulk(args, groups, TA::kBytes, TB::kBytes) ? shuffle_wide_pn_kernel<TA, TB, true> : shuffle_wide_pn_kernel<TA, TB, false>;
         KernelFit fit;
         cudaError_t err = kernel_fit(reinterpret_cast<const void *>(kernel), 2 * static_cast<int>(groups), smem, &fit);
         if (err != cudaSuccess) return err;

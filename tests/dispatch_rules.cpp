@@ -3,7 +3,7 @@
 
 extern "C" {
 
-int rule_copies_in_bulk(int has_status, unsigned pn_pad, unsigned group_lo, unsigned group_hi, unsigned groups, unsigned long long group_bytes, int two_stacks)
+int rule_copies_in_bulk(int has_status, unsigned pn_pad, unsigned group_lo, unsigned group_hi, unsigned groups, int n_models, int bytes_a, int bytes_b, float share)
 {
     uint32_t word = 0;
     wash::ShuffleArgs args = {};
@@ -11,7 +11,9 @@ int rule_copies_in_bulk(int has_status, unsigned pn_pad, unsigned group_lo, unsi
     args.pn_pad = pn_pad;
     args.group_lo = group_lo;
     args.group_hi = group_hi;
-    return wash::copies_in_bulk(args, groups, group_bytes, two_stacks != 0) ? 1 : 0;
+    args.pop.N = n_models;
+    args.expected_share = share;
+    return wash::copies_in_bulk(args, groups, bytes_a, bytes_b) ? 1 : 0;
 }
 
 int rule_fetch_half_lines(int layout, int n_models, float share, int by_warps, int bytes_a, int bytes_b)

@@ -18,16 +18,22 @@ def rules(tmp_path_factory):
     return ctypes.CDLL(lib)
 
 
-@pytest.mark.parametrize("two_stacks", [0, 1])
-@pytest.mark.parametrize("group_bytes", [512, 576, 768, 1024, 1152, 2048])
-def test_bulk_copies_only_where_they_can_be_reported_and_fit(rules, group_bytes, two_stacks):
+@pytest.mark.parametrize("bytes_a,bytes_b", [(4, 0), (2, 0), (4, 4), (2, 4), (4, 2), (2, 2)])
+@pytest.mark.parametrize("N", [17, 24, 32, 40, 48, 56, 60, 64])
+def test_bulk_copies_only_where_they_can_be_reported_and_fit(rules, N, bytes_a, bytes_b):
     """A launch without a status word never takes copies whose wait can be given up; neither do odd ranges or padded images, whose
-    bytes are no multiples of 16 or not contiguous."""
-    def bulk(has_status=1, pad=0, lo=0, hi=1000, groups=32):
-        return rules.rule_copies_in_bulk(has_status, pad, lo, hi, groups, ctypes.c_ulonglong(group_bytes), two_stacks)
-    assert not bulk(has_status=0) and not bulk(has_status=0, groups=64)
-    assert not bulk(pad=4) and not bulk(lo=3) and not bulk(hi=999)
-    assert bulk(groups=64)
+    bytes are no multiples of 16 or not contiguous.  Where they fit, a larger selection or a larger block never turns them off, and the
+    stacks' order does not matter."""
+    def bulk(has_status=1, pad=0, lo=0, hi=1 << 26, groups=32, share=0.5, a=bytes_a, b=bytes_b):
+        return rules.rule_copies_in_bulk(has_status, pad, lo, hi, groups, N, a, b, ctypes.c_float(share))
+    for share in (0.005, 0.1, 0.5, 1.0):
+        assert not bulk(has_status=0, share=share) and not bulk(has_status=0, groups=64, share=share)
+        assert not bulk(pad=4, share=share) and not bulk(lo=3, share=share) and not bulk(hi=999, share=share) and bulk(hi=1000, share=share)
+        assert bulk(groups=32, share=share) <= bulk(groups=64, share=share)
+        if bytes_b:
+            assert bulk(share=share) == bulk(share=share, a=bytes_b, b=bytes_a)
+    taken = [bulk(share=s) for s in (0.003, 0.01, 0.05, 0.1, 0.19, 0.21, 0.6, 1.0)]
+    assert taken == sorted(taken) and taken[-1] == 1
 
 
 @pytest.mark.parametrize("tile", [256, 512], ids=["two groups a lane", "four"])
