@@ -137,8 +137,9 @@ int wash_set_mode(wash_ctx *ctx, int32_t mode);
  * forces the streaming kernel's lean / early flavour (lean: not the early one; from 0.3 % selected on that is, for more than 16
  * models, the kernel of their own named below; early draws the permutations while the
  * stack's copies are in flight and serves populations of more than 16 models densely; by
- * default it is launched for N > 16 when the call's probabilities select 70 % or more; from
- * 0.3 % to there populations of more than 16 models have a kernel of their own);
+ * default it is launched for N > 16 when the call's probabilities select 70 % or more, but not in
+ * [padded_P][N] with a multiple of four models; from 0.3 % on, to there or throughout, populations of
+ * more than 16 models have a kernel of their own);
  * blocks_per_sm = -4 / -5 forces (N <= 16; ignored above) / excludes the streaming kernel for small groups (a
  * resident grid of warps walking tiles through two shared-memory stages; by default
  * it is launched when a group of all models of both stacks is at most 48 bytes and the

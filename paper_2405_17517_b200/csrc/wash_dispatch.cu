@@ -158,7 +158,8 @@ static cudaError_t launch_shuffle_kernel(const ShuffleArgs &args, int a_dtype, i
     // Three streaming kernels.  Small groups of all models (both stacks) go to the resident-warp kernel, whose
     // instruction count per group is a fraction of the one-trip kernel's (resident_warps_pay); larger
     // groups, the consensus statistic and the early flavour stay with the one-trip kernel; populations of more
-    // than 16 models have a one-trip kernel of their own from kWideMinShare on, until the early flavour takes over.
+    // than 16 models have a one-trip kernel of their own from kWideMinShare on, until the early flavour takes over
+    // (in [P][N] with a multiple of four models it does not).
     // blocks_per_sm of wash_set_launch: -4 forces the resident-warp kernel, -5 the one-trip kernel.
     const size_t elem_a = a_dtype == kDtypeF32 ? 4 : a_dtype == kDtypeBF16 ? 2 : 0, elem_b = b_dtype == kDtypeF32 ? 4 : b_dtype == kDtypeBF16 ? 2 : 0;
     const size_t per_group = static_cast<size_t>(args.pop.N) * 4 * (elem_a + elem_b);

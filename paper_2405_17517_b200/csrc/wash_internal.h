@@ -107,7 +107,7 @@ struct ShuffleArgs {
     SqArgs sq;                    // consensus distance of the first stack (streaming kernel only)
     bool measure_only = false;    // with sq: nothing is selected
     uint32_t pn_pad = 0;          // streaming kernel, [P][N]: elements of padding after a group in the shared-memory image (0 or 4)
-    uint32_t pair_inverse = 0;    // streaming kernel, N > 16: 2^20 / N, rounded up (i / N = i * pair_inverse >> 20 for i < 2080; set by its launcher)
+    uint32_t pair_inverse = 0;    // streaming kernel, N > 16: 2^20 / N, rounded up (i / N = i * pair_inverse >> 20 for i < 2^14, and i is at most 64 N; set by its launcher)
     bool early = false;           // streaming kernel: the flavour that draws permutations while the copies are in flight
     void *mirror_a = nullptr;     // sparse kernel: a second copy of each stack (mapped host memory) that receives the moved values, too
     void *mirror_b = nullptr;

@@ -363,7 +363,7 @@ __device__ __forceinline__ void move_coordinate(const ShuffleArgs &a, const unsi
 //          32 at a time: with a few selected coordinates per warp (p around 0.01-0.1) one round
 //          serves them all, instead of one divergent pass per coordinate slot; the plan draws the
 //          first round's permutations, later rounds draw theirs when they are served;
-//   dense  half of the warp's coordinates or more selected (and every such group whole): dealing
+//   dense  half of the warp's coordinates or more selected (and every such group whole; even populations in [P][N]: dense_threshold): dealing
 //          would take two rounds or more, in each of which a lane draws one permutation and stores
 //          4-byte values; every lane serving its own group costs less from there on.
 // Both are called by all threads of the block.

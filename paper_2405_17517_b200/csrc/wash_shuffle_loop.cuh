@@ -179,7 +179,10 @@ __global__ void __launch_bounds__(32, G == 2 ? 32 : 28) shuffle_loop_kernel(cons
     // A launch of one tile a warp draws its masks, which need nothing but the tables, before it waits for the kernel before it.
     // (With several tiles the copies of the first come first: they hide the masks.)  With the counters' single report
     // (publish_warp_stats), call after call, p = 0.01: N = 3, 2^20 coordinates 7.1 -> 4.3 us, 2^17 5.6 -> 4.1; N = 2, 2^20 8.0 -> 4.2; several tiles a
-    // warp, by the report alone: N = 2, 2^22 12.5 -> 10.9, N = 5, 2^21 11.0 -> 9.4.
+    // warp, by the report alone: N = 2, 2^22 12.5 -> 10.9, N = 5, 2^21 11.0 -> 9.4.  Of these the early masks are the part that takes a kernel of this library
+    // before it.  Neither / the report alone / both, call after call | behind an elementwise kernel of another library on other data | on the stacks
+    // (the device's time, the host ahead): N = 3, 2^20 7.2 5.5 3.7 | 7.6 6.1 6.0 | 6.2 4.1 4.1;  2^17 5.7 4.0 2.8 | 5.1 4.1 4.1 | 4.1 3.1 3.7;  N = 2, 2^20 8.0 6.4 4.1 | 6.2 4.2 4.2 |
+    // 6.2 5.3 4.6.
     const bool one_trip = n_tiles <= gridDim.x;
     if (!one_trip) {
         await_previous();

@@ -16,7 +16,7 @@
 // values: DRAM serves about 45e9 isolated 4-byte loads a second, 22e9 stores and 20e9 pairs
 // of both (measured, one access per 800 bytes), 1 us per 20 000 moved values and stack.  That is the rate of isolated accesses
 // and no bound for denser ones, which share DRAM pages and sectors: ResNet-50 N = 8, bf16 + fp32, p = 5e-3 (1.8e6 values in
-// both stacks) would take 90 us by it and takes 77.  With a queue per warp, served at the end of the warp's
+// both stacks) would take 90 us by it and takes 70.  With a queue per warp, served at the end of the warp's
 // range by a lane per coordinate, and launches that do not overlap, the same took (before -> now): that one 89.1 -> 77.1,
 // ResNet-18 N = 5 with momentum, p = 1e-3 21.0 -> 10.5, ResNet-50 N = 10 with momentum, p = 0.01 -> 0 70.8 -> 56.1, 2^27 coordinates N = 2
 // at p = 1e-3 119 -> 97.5 us.
@@ -385,7 +385,7 @@ cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchSha
     // 2.5e7, p = 3e-3 26.8 -> 20.9; ResNet-50 N = 5, p = 0.05 -> 0 44.9 -> 42.7; [P][N] N = 8, 2^25, p = 0.01 43.3 -> 36.7, N = 16, p = 3e-3
     // 39.9 -> 31.7.  A larger load loses where values are many (400 instead of 300 for ResNet-50 N = 8 bf16 + fp32, p = 5e-3: 79.4
     // against 77.1, N = 20, p = 2e-3 51.6 against 50.3), a broken wave where waves are few ([P][N] N = 8, 2^25: 1.4 waves
-    // 41.9, two 38.8).
+    // 41.9, two 38.8).  Half a wave where that serves everything and the next kernel is released at once (half_wave_serves).
     const bool one_stack = TB::kCode == kDtypeNone;
     const double expected = static_cast<double>(args.expected_share) * 4.0 * static_cast<double>(args.group_hi - args.group_lo);
     double by_tiles = static_cast<double>(p.n_wtiles) / (kSparseWarps * (np ? 2 : 3));
