@@ -151,9 +151,13 @@ inline bool fetch_half_lines(const ShuffleArgs &args, bool by_warps, int bytes_a
 //   N = 48, 2^21, 1e-3 8.0 -> 8.4 | 10.7 -> 12.1 | 9.7 -> 10.5;  [P][N], 3e-3 6.8 -> 7.2 | 8.2 -> 8.3 | 8.0 -> 8.9
 // Five eighths to seven eighths of a wave gain less and lose as much (ResNet-18 with momentum 0.75: 11.4 | 14.3 | 14.2).  Waves and a half lose (N = 3 two
 // stacks, p = 5e-3, 1.5 waves 20.7, two 18.9).
-inline bool half_wave_serves(int n_models, double by_load, uint32_t resident, uint32_t n_wtiles)
+// More than 32 models with few values a block gain, call after call: N = 64 bf16, 3e-4 (100 values) [N][P] 7.8 -> 7.3, [P][N] 6.8 -> 5.9; [P][N], whose values are neighbours,
+// 1e-3 (340) 7.7 -> 6.9; N = 48 above has 170 in [N][P] and 510 in [P][N].  `expected` coordinates in `stacks` stacks.
+inline bool half_wave_serves(int layout, int n_models, int stacks, double expected, double by_load, uint32_t resident, uint32_t n_wtiles)
 {
-    return n_models <= 32 && by_load <= 0.4 * resident && n_wtiles <= 32ull * resident;   // 16 tiles for each of the 4 warps of resident / 2 blocks
+    const double values = expected * n_models * stacks / (0.5 * resident);   // of a block
+    if (n_models > 32 && values > (layout == kLayoutNP ? 128.0 : 400.0)) return false;
+    return by_load <= 0.4 * resident && n_wtiles <= 32ull * resident;   // 16 tiles for each of the 4 warps of resident / 2 blocks
 }
 
 // [P][N], even populations of up to 16 models: the threshold from which every lane serves its own group (serve_group_dense) instead of

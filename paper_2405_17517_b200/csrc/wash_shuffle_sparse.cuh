@@ -395,7 +395,7 @@ cudaError_t launch_shuffle_sparse_typed(const ShuffleArgs &args, const LaunchSha
     p.release_early = static_cast<double>(args.expected_share) * args.pop.N * (one_stack ? 1 : 2) <= kReleaseShare;
     const double by_load = expected * (one_stack ? 1.0 : 2.0) / load;
     uint32_t grid = static_cast<uint32_t>(fmin(fmin(expected / kSparsePerBlock, by_tiles), resident * ceil(by_load / resident)));
-    if (grid < resident) grid = p.release_early && half_wave_serves(args.pop.N, by_load, resident, p.n_wtiles) ? resident / 2 : resident;
+    if (grid < resident) grid = p.release_early && half_wave_serves(args.pop.layout, args.pop.N, one_stack ? 1 : 2, expected, by_load, resident, p.n_wtiles) ? resident / 2 : resident;
     const uint32_t want = (p.n_wtiles + kSparseWarps - 1) / kSparseWarps;
     if (grid > want) grid = want;
     p.per_block = p.n_wtiles / grid;

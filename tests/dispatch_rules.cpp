@@ -25,7 +25,10 @@ int rule_fetch_half_lines(int layout, int n_models, float share, int by_warps, i
     return wash::fetch_half_lines(args, by_warps != 0, bytes_a, bytes_b) ? 1 : 0;
 }
 
-int rule_half_wave_serves(int n_models, double by_load, unsigned resident, unsigned n_wtiles) { return wash::half_wave_serves(n_models, by_load, resident, n_wtiles) ? 1 : 0; }
+int rule_half_wave_serves(int layout, int n_models, int stacks, double expected, double by_load, unsigned resident, unsigned n_wtiles)
+{
+    return wash::half_wave_serves(layout, n_models, stacks, expected, by_load, resident, n_wtiles) ? 1 : 0;
+}
 
 int rule_stored_together(int layout, int n_models) { return wash::stored_together(layout, n_models); }
 

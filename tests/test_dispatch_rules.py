@@ -68,11 +68,13 @@ def test_half_lines_are_asked_for_alike_in_either_order_of_the_stacks(rules):
 
 
 def test_half_a_wave_only_where_it_does_not_lose_more_than_it_gains(rules):
-    """Up to 32 models, 0.4 of a wave's values and 16 tiles a warp (1184 resident blocks)."""
-    def half(N, by_load, n_wtiles):
-        return rules.rule_half_wave_serves(N, ctypes.c_double(by_load), 1184, n_wtiles)
-    assert half(5, 374.0, 21_914) and half(32, 0.0, 37_888)
-    assert not half(33, 1.0, 100) and not half(5, 474.0, 21_914) and not half(5, 1.0, 37_889)
+    """0.4 of a wave's values and 16 tiles a warp (1184 resident blocks); with more than 32 models few values a block."""
+    def half(N, by_load, n_wtiles, layout=0, stacks=1, expected=0.0):
+        return rules.rule_half_wave_serves(layout, N, stacks, ctypes.c_double(expected), ctypes.c_double(by_load), 1184, n_wtiles)
+    assert half(5, 374.0, 21_914, stacks=2, expected=11_220.0) and half(32, 0.0, 37_888, expected=1e6)
+    assert not half(5, 474.0, 21_914) and not half(5, 1.0, 37_889)
+    assert half(64, 200.0, 6_000, expected=937.0) and half(64, 10.0, 6_000, layout=1, expected=3_125.0)
+    assert not half(48, 333.0, 4_069, expected=2_083.0) and not half(48, 21.0, 4_069, layout=1, expected=6_250.0) and not half(64, 200.0, 6_000, stacks=2, expected=937.0)
 
 
 def test_which_populations_store_neighbouring_values_together(rules):

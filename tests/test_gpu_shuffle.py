@@ -736,7 +736,7 @@ def _half_wave_row(at_least_blocks_over=1.5):
 @pytest.mark.parametrize("layout", [0, 1])
 @pytest.mark.parametrize("N,p,dtype,opt", [(2, 1e-3, "f32", None), (3, 4e-4, "bf16", None), (5, 2e-4, "f32", "f32"), (8, 3e-4, "bf16", "f32"), (16, 2e-4, "f32", None), (20, 2e-4, "bf16", None), (40, 1e-4, "bf16", None)])
 def test_sparse_half_a_wave_of_blocks(N, p, dtype, opt, layout):
-    """Selections rare enough for half a wave of blocks, in rows that would fill more (N = 40: the whole wave), three steps in a row: the
+    """Selections rare enough for half a wave of blocks, in rows that would fill more, three steps in a row: the
     second draws its masks beside the first one's serving."""
     c = Case(N, [_half_wave_row(), 5, 2047], layout, dtype, opt, seed=N)
     B.wash_set_mode(c.gpu.ctx, B.WASH_MODE_SPARSE)
